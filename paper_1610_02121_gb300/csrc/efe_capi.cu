@@ -79,6 +79,7 @@ struct efe_handle {
   int64_t nnz = 0;
   int32_t* ec_col = nullptr;
   double *mec = nullptr, *hec_kin = nullptr, *hec = nullptr;
+  double* mecD = nullptr;     // M^ec D^-1 (row pattern, FP64)
   int64_t *ec_cptr = nullptr, *ec_cidx = nullptr;
   int64_t nseg = 0;
   int64_t *seg_start = nullptr, *seg_end = nullptr, *row_seg_ptr = nullptr;
@@ -527,7 +528,7 @@ int apply_H_generic(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, i
   }
   if (h->nE > 0) {
     launch_spmm_nodes<T>(h->n_tn, h->t_nodes, h->t_ptr, h->t_col, h->hecT, 1.0, Xe, ldxe, Wc, ldw, N, st);
-    launch_spmm_segments<T>(h->nseg, h->seg_start, h->seg_end, h->ec_col, h->hec, nullptr, Xc, ldx, h->part, N, st);
+    launch_spmm_segments<T>(h->nseg, h->seg_start, h->seg_end, h->ec_col, h->hec, Xc, ldx, h->part, N, st);
     launch_seg_reduce((int)h->nE, h->row_seg_ptr, h->part, 1.0, nullptr, 0, 0.0, We, ldwe, N, st);
     launch_gemm_nn(h->nE, N, (int)h->nE, 1.0, h->Hee, h->nE, Xe, ldxe, 1.0, We, ldwe, st);
     CKL();
@@ -552,7 +553,7 @@ int minv_core(efe_handle* h, T* Wc, int64_t ldw, const double* We, int64_t ldwe,
       return EFE_OK;
     }
   }
-  launch_spmm_segments<T>(h->nseg, h->seg_start, h->seg_end, h->ec_col, h->mec, h->Dinv, Wc, ldw, h->part, N, st);
+  launch_spmm_segments<T>(h->nseg, h->seg_start, h->seg_end, h->ec_col, h->mecD, Wc, ldw, h->part, N, st);
   launch_seg_reduce((int)h->nE, h->row_seg_ptr, h->part, -1.0, We, ldwe, 1.0, h->rb, N, N, st);
   launch_gemm_nn(h->nE, N, (int)h->nE, 1.0, h->Sinv, h->nE, h->rb, N, 0.0, h->xe, N, st);
   launch_spmm_nodes<T>(h->n_tn, h->t_nodes, h->t_ptr, h->t_col, h->mecT, -1.0, h->xe, N, Wc, ldw, N, st);
@@ -574,8 +575,7 @@ int apply_M_impl(efe_handle* h, const double* X, int64_t ldx, int N, double* Y, 
   } else if (h->nE > 0) {
     launch_spmm_nodes<double>(h->n_tn, h->t_nodes, h->t_ptr, h->t_col, h->mecT, 1.0, X + nn * ldx, ldx, Y, ldy, N, st);
     launch_row_scale<double>(nn, h->mask, Y, ldy, Y, ldy, N, st);
-    launch_spmm_segments<double>(h->nseg, h->seg_start, h->seg_end, h->ec_col, h->mec, nullptr, X, ldx, h->part, N,
-                                 st);
+    launch_spmm_segments<double>(h->nseg, h->seg_start, h->seg_end, h->ec_col, h->mec, X, ldx, h->part, N, st);
     launch_seg_reduce((int)h->nE, h->row_seg_ptr, h->part, 1.0, nullptr, 0, 0.0, Y + nn * ldy, ldy, N, st);
     launch_gemm_nn(h->nE, N, (int)h->nE, 1.0, h->Mee, h->nE, X + nn * ldx, ldx, 1.0, Y + nn * ldy, ldy, st);
   }
@@ -1248,6 +1248,10 @@ int efe_create(const efe_mesh_desc* mesh, const efe_atoms_desc* atoms, const efe
     TRY(dalloc(h, &h->mecT32, h->nnz));
     TRY(dalloc(h, &h->hecT32, h->nnz));
     TRY(dalloc(h, &h->hec32, h->nnz));
+    // M^ec D^-1, formed once: scaling inside the Schur residual's rows product cost
+    // an FP64 multiply and a gather per entry and column
+    TRY(dalloc(h, &h->mecD, h->nnz));
+    launch_col_scale(h->nnz, h->mec, h->Dinv, h->ec_col, h->mecD, 0);
     launch_permute(h->nnz, h->mec, h->t_perm, h->mecT, 0);
     launch_to_f32(h->mecT, h->mecT32, h->nnz, 0);
     TRY(dalloc(h, &h->mec2, h->nnz));
@@ -2507,7 +2511,7 @@ extern "C" int efe_apply_M_noalloc(efe_handle* h, const double* X, int64_t ldx, 
     launch_spmm_nodes<double>(h->n_tn, h->t_nodes, h->t_ptr, h->t_col, h->mecT, 1.0, X + nn * ldx, ldx, Y, ldy, N, st);
     launch_row_scale<double>(nn, h->mask, Y, ldy, Y, ldy, N, st);
     // every partial is written before it is read: nothing to clear
-    launch_spmm_segments<double>(h->nseg, h->seg_start, h->seg_end, h->ec_col, h->mec, nullptr, X, ldx, part, N, st);
+    launch_spmm_segments<double>(h->nseg, h->seg_start, h->seg_end, h->ec_col, h->mec, X, ldx, part, N, st);
     launch_seg_reduce((int)h->nE, h->row_seg_ptr, part, 1.0, nullptr, 0, 0.0, Y + nn * ldy, ldy, N, st);
     launch_gemm_nn(h->nE, N, (int)h->nE, 1.0, h->Mee, h->nE, X + nn * ldx, ldx, 1.0, Y + nn * ldy, ldy, st);
   }

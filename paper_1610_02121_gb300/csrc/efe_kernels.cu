@@ -7,6 +7,7 @@
 // (Sec. IV.D) and the scaled three-term recurrence -- and the FP64 dense kernels
 // of Cholesky-QR and Rayleigh-Ritz.  No FP atomics anywhere: every reduction
 // has a fixed order, so results are bitwise reproducible run to run.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -15,6 +16,8 @@
 
 #include "efe_func.h"
 #include "efe_kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace efe {
 
@@ -89,6 +92,12 @@ __global__ void k_permute(int64_t n, const double* __restrict__ src, const int64
                           double* __restrict__ dst) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) dst[i] = src[perm[i]];
+}
+
+__global__ void k_col_scale(int64_t n, const double* __restrict__ v, const double* __restrict__ scale,
+                            const int32_t* __restrict__ col, double* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) out[i] = v[i] * scale[col[i]];
 }
 
 __global__ void k_to_f32(const double* __restrict__ s, float* __restrict__ d, int64_t n) {
@@ -183,22 +192,54 @@ __global__ void k_spmm_nodes(int64_t nrows, const int32_t* __restrict__ rnode, c
   }
 }
 
-template <typename T>
-__global__ void k_spmm_segments(const int64_t* __restrict__ seg_start, const int64_t* __restrict__ seg_end,
-                                const int32_t* __restrict__ col, const double* __restrict__ val,
-                                const double* __restrict__ scale, const T* __restrict__ Xc, int64_t ldx,
-                                double* __restrict__ part, int N) {
-  const int64_t seg = blockIdx.x;
+// part[seg][c] = sum_{q in seg} val[q] Xc[col[q]][c] in FP64.  A CTA takes one
+// segment (up to 2048 entries of a row) and CX columns; its 256 / CX thread rows
+// take every (256 / CX)-th entry, four loads in flight each, and their sums are
+// added in fixed order.  What bounds it is the latency of the entry -> row chain
+// when one thread walks a segment alone, and the FP64 pipe (one FMA per entry and
+// column) once enough threads share it; where the segments are fewer than the SMs
+// a cluster of CL CTAs shares one (an SM retires about two FP64 FMAs a clock: 4 us
+// for one segment and 8 columns).  Per launch: 8 vectors on 15 segments 585 us with
+// one thread per column, 28 with thread rows, 11.3 with the cluster; 12 vectors on
+// 190 segments 641 -> 18.5 us.
+constexpr int SEG_T = 256;
+constexpr int SEG_CL = 4;
+template <typename T, int CX, int CL>
+__global__ void __launch_bounds__(SEG_T) k_spmm_segments(const int64_t* __restrict__ seg_start,
+                                                         const int64_t* __restrict__ seg_end,
+                                                         const int32_t* __restrict__ col,
+                                                         const double* __restrict__ val, const T* __restrict__ Xc,
+                                                         int64_t ldx, double* __restrict__ part, int N) {
+  constexpr int LY = SEG_T / CX;
+  __shared__ double red[LY][CX];
+  __shared__ double csum[CX];
+  const int tx = threadIdx.x % CX, ty = threadIdx.x / CX;
+  const int64_t seg = blockIdx.x / CL;
+  const int rank = blockIdx.x % CL;
   const int64_t q0 = seg_start[seg], q1 = seg_end[seg];
-  for (int c = threadIdx.x; c < N; c += blockDim.x) {
-    double s = 0.0;
-    for (int64_t q = q0; q < q1; ++q) {
-      const int64_t g = col[q];
-      const double v = scale ? val[q] * scale[g] : val[q];
-      s = fma(v, (double)Xc[g * ldx + c], s);
-    }
-    part[seg * N + c] = s;
+  const int c = blockIdx.y * CX + tx;
+  double s = 0.0;
+  if (c < N) {
+#pragma unroll 8
+    for (int64_t q = q0 + rank * LY + ty; q < q1; q += LY * CL) s = fma(val[q], (double)Xc[(int64_t)col[q] * ldx + c], s);
   }
+  red[ty][tx] = s;
+  __syncthreads();
+  double t = 0.0;
+  if (ty == 0) {
+#pragma unroll
+    for (int k = 0; k < LY; ++k) t += red[k][tx];
+    csum[tx] = t;
+  }
+  if constexpr (CL > 1) {
+    // the cluster's sums in rank order, read over distributed shared memory
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    if (rank == 0 && ty == 0)
+      for (int r = 1; r < CL; ++r) t += cl.map_shared_rank(csum, r)[tx];
+    cl.sync();
+  }
+  if (rank == 0 && ty == 0 && c < N) part[seg * N + c] = t;
 }
 
 // ---------------------------------------------------------------------------
@@ -336,7 +377,6 @@ __global__ void __launch_bounds__(256) k_spmm_segments_narrow(const int64_t* __r
                                                               const int64_t* __restrict__ seg_end,
                                                               const int32_t* __restrict__ col,
                                                               const double* __restrict__ val,
-                                                              const double* __restrict__ scale,
                                                               const T* __restrict__ Xc, int64_t ldx,
                                                               double* __restrict__ part, int N) {
   __shared__ double red[8][SPMM_NARROW];
@@ -346,7 +386,7 @@ __global__ void __launch_bounds__(256) k_spmm_segments_narrow(const int64_t* __r
   double s[SPMM_NARROW] = {0.0, 0.0, 0.0, 0.0};
   for (int64_t q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
     const int64_t g = col[q];
-    const double v = scale ? val[q] * scale[g] : val[q];
+    const double v = val[q];
 #pragma unroll
     for (int c = 0; c < SPMM_NARROW; ++c)
       if (c < N) s[c] = fma(v, (double)Xc[g * ldx + c], s[c]);
@@ -877,54 +917,89 @@ __global__ void k_spmm_nodes_df(int64_t nrows, const int32_t* __restrict__ rnode
 }
 
 // Rows product over function groups (the items of k_grp_rows): part[item][k][c]
-// = sum over the item's nodes of coef[k][node] Xc[node][c], FP64 Xc, double-float
-// sums over the whole item
-__global__ void __launch_bounds__(GRP_CT) k_grp_rows_df(const int4* __restrict__ items, const int64_t* __restrict__ ec_ptr,
-                                                       const int32_t* __restrict__ ec_col, const float2* __restrict__ coef,
-                                                       const double* __restrict__ Xc, int64_t ldx, double* __restrict__ part,
-                                                       int N) {
-  __shared__ int64_t nd[GRP_CHUNK];
-  __shared__ float2 cf[GRP_KMAX][GRP_CHUNK];
-  __shared__ int64_t rowp[GRP_KMAX];
-  const int4 it = items[blockIdx.x];
+// = sum over the item's nodes of coef[k][node] Xc[node][c], FP64 Xc, one
+// double-float sum over the whole item in node order.  One thread per (function,
+// column): CX columns x 8 functions per CTA.  The sums are serial chains of
+// length 1024, so everything else is kept off them: all threads fetch and cut the
+// next 64 nodes' rows into float pairs in shared memory (two buffers) while the
+// chains run on the current ones.  With one thread per column for all functions
+// each step of the chain carried a gathered load, its cut and k_g double-float
+// updates, and blocks of fewer than 128 columns left the other threads idle.  Per
+// launch, before -> now: 12 vectors on 76 items 600 -> 46 us, 135 vectors on 319
+// items 713 -> 271 us, 640 vectors 1433 -> 878 us (the FP32 pipe's 14 operations
+// per function, node and column take about 0.1 and 0.45 ms).  Same sums, bit for bit.
+template <int CX>
+__global__ void __launch_bounds__(CX * GRP_KMAX) k_grp_rows_df(const int4* __restrict__ items,
+                                                              const int64_t* __restrict__ ec_ptr,
+                                                              const int32_t* __restrict__ ec_col,
+                                                              const float2* __restrict__ coef,
+                                                              const double* __restrict__ Xc, int64_t ldx,
+                                                              double* __restrict__ part, int N) {
+  constexpr int NT = CX * GRP_KMAX, RPT = GRP_CHUNK * CX / NT;   // threads; chunk rows per thread
+  __shared__ float2 xs[2][GRP_CHUNK][CX];
+  __shared__ float2 cf[2][GRP_KMAX][GRP_CHUNK];
+  const int4 it = items[blockIdx.x];   // first function, functions, node positions [j0, j1)
   const int f0 = it.x, kg = it.y, j0 = it.z, j1 = it.w;
-  const int c = blockIdx.y * GRP_CT + threadIdx.x;
-  if (threadIdx.x < kg) rowp[threadIdx.x] = ec_ptr[f0 + threadIdx.x];
-  float S[GRP_KMAX], C[GRP_KMAX];
+  const int tid = threadIdx.x, tx = tid % CX, k = tid / CX;
+  const int c = blockIdx.y * CX + tx;
+  const int32_t* cols = ec_col + ec_ptr[f0];
+  constexpr int CPT = GRP_KMAX * GRP_CHUNK / NT;   // coefficients per thread
+  const float2* cr[CPT];
 #pragma unroll
-  for (int k = 0; k < GRP_KMAX; ++k) {
-    S[k] = 0.f;
-    C[k] = 0.f;
+  for (int u = 0; u < CPT; ++u) {
+    const int kk = (tid + u * NT) / GRP_CHUNK;
+    cr[u] = kk < kg ? coef + ec_ptr[f0 + kk] + (tid + u * NT) % GRP_CHUNK : nullptr;
   }
-  for (int j = j0; j < j1; j += GRP_CHUNK) {
-    const int n = min(GRP_CHUNK, j1 - j);
-    __syncthreads();
-    const int64_t base = rowp[0];
-    if (threadIdx.x < n) nd[threadIdx.x] = ec_col[base + j + threadIdx.x];
+  double x[RPT];
+  float2 cv[CPT];
+  int nx[RPT];                       // node indexes of the chunk to fetch next
+  auto index = [&](int j) {
 #pragma unroll
-    for (int u = 0; u < GRP_KMAX * GRP_CHUNK / GRP_CT; ++u) {
-      const int t = threadIdx.x + u * GRP_CT;
-      const int k = t / GRP_CHUNK, jj = t % GRP_CHUNK;
-      if (k < kg) cf[k][jj] = jj < n ? coef[rowp[k] + j + jj] : make_float2(0.f, 0.f);
+    for (int u = 0; u < RPT; ++u) {
+      const int jj = j + k + u * GRP_KMAX;
+      nx[u] = jj < j1 ? cols[jj] : 0;
     }
-    __syncthreads();
-    if (c < N) {
-#pragma unroll 4
-      for (int jj = 0; jj < n; ++jj) {
-        float xh, xl;
-        df_split(Xc[nd[jj] * ldx + c], xh, xl);
+  };
+  auto fetch = [&](int j) {
 #pragma unroll
-        for (int k = 0; k < GRP_KMAX; ++k)
-          if (k < kg) df_fma(cf[k][jj].x, cf[k][jj].y, xh, xl, S[k], C[k]);
+    for (int u = 0; u < RPT; ++u)
+      x[u] = (j + k + u * GRP_KMAX < j1 && c < N) ? Xc[(int64_t)nx[u] * ldx + c] : 0.0;
+    index(j + GRP_CHUNK);
+#pragma unroll
+    for (int u = 0; u < CPT; ++u)
+      cv[u] = (cr[u] && j + (tid + u * NT) % GRP_CHUNK < j1) ? cr[u][j] : make_float2(0.f, 0.f);
+  };
+  auto stage = [&](int b) {
+#pragma unroll
+    for (int u = 0; u < RPT; ++u) {
+      float xh, xl;
+      df_split(x[u], xh, xl);
+      xs[b][k + u * GRP_KMAX][tx] = make_float2(xh, xl);
+    }
+#pragma unroll
+    for (int u = 0; u < CPT; ++u) (&cf[b][0][0])[tid + u * NT] = cv[u];
+  };
+  float S = 0.f, C = 0.f;
+  index(j0);
+  fetch(j0);
+  stage(0);
+  __syncthreads();
+  int b = 0;
+  for (int j = j0; j < j1; j += GRP_CHUNK, b ^= 1) {
+    const bool more = j + GRP_CHUNK < j1;
+    if (more) fetch(j + GRP_CHUNK);
+    if (k < kg && c < N) {
+      const int n = min(GRP_CHUNK, j1 - j);
+#pragma unroll 8
+      for (int jj = 0; jj < n; ++jj) {
+        const float2 a = cf[b][k][jj], v = xs[b][jj][tx];
+        df_fma(a.x, a.y, v.x, v.y, S, C);
       }
     }
+    if (more) stage(b ^ 1);
+    __syncthreads();
   }
-  if (c < N) {
-    double* o = part + (int64_t)blockIdx.x * GRP_KMAX * N + c;
-#pragma unroll
-    for (int k = 0; k < GRP_KMAX; ++k)
-      if (k < kg) o[(int64_t)k * N] = df_f2d(S[k]) + df_f2d(C[k]);
-  }
+  if (k < kg && c < N) part[((int64_t)blockIdx.x * GRP_KMAX + k) * N + c] = df_f2d(S) + df_f2d(C);
 }
 
 // Columns product: W[g_u][c] += sgn * sum_slot tile[slot][u] * Xe[f(slot)][c]
@@ -1500,6 +1575,13 @@ void launch_gather_sum(int64_t n_out, const double* base, const int64_t* cptr, c
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
+void launch_col_scale(int64_t n, const double* v, const double* scale, const int32_t* col, double* out,
+                      cudaStream_t st) {
+  if (n <= 0) return;
+  k_col_scale<<<grid1(n, 256), 256, 0, st>>>(n, v, scale, col, out);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+}
+
 void launch_permute(int64_t n, const double* src, const int64_t* perm, double* dst, cudaStream_t st) {
   if (n <= 0) return;
   k_permute<<<grid1(n, 256), 256, 0, st>>>(n, src, perm, dst);
@@ -1549,23 +1631,51 @@ template void launch_spmm_nodes<double>(int64_t, const int32_t*, const int64_t*,
 template void launch_spmm_nodes<float>(int64_t, const int32_t*, const int64_t*, const int32_t*, const double*,
                                        double, const double*, int64_t, float*, int64_t, int, cudaStream_t);
 
+namespace {
+template <typename T, int CX>
+void spmm_segments_cx(int64_t nseg, const int64_t* seg_start, const int64_t* seg_end, const int32_t* col,
+                      const double* val, const T* Xc, int64_t ldx, double* part, int N, cudaStream_t st) {
+  const unsigned ny = (unsigned)((N + CX - 1) / CX);
+  // fewer than two CTAs per SM: a cluster of four CTAs to a segment
+  if (nseg * ny < 2 * (int64_t)current_sm_count()) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nseg * SEG_CL, ny);
+    cfg.blockDim = dim3(SEG_T);
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = SEG_CL;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_spmm_segments<T, CX, SEG_CL>, seg_start, seg_end, col, val, Xc, ldx, part, N);
+  } else {
+    k_spmm_segments<T, CX, 1><<<dim3((unsigned)nseg, ny), SEG_T, 0, st>>>(seg_start, seg_end, col, val, Xc, ldx, part, N);
+  }
+}
+}  // namespace
+
 template <typename T>
 void launch_spmm_segments(int64_t nseg, const int64_t* seg_start, const int64_t* seg_end, const int32_t* col,
-                          const double* val, const double* scale, const T* Xc, int64_t ldx, double* part, int N,
-                          cudaStream_t st) {
+                          const double* val, const T* Xc, int64_t ldx, double* part, int N, cudaStream_t st) {
   if (nseg <= 0 || N <= 0) return;
-  if (N <= SPMM_NARROW) {
-    k_spmm_segments_narrow<T><<<(unsigned)nseg, 256, 0, st>>>(seg_start, seg_end, col, val, scale, Xc, ldx, part, N);
-  } else {
-    const int t = N >= 128 ? 128 : ((N + 31) / 32) * 32;
-    k_spmm_segments<T><<<(unsigned)nseg, t, 0, st>>>(seg_start, seg_end, col, val, scale, Xc, ldx, part, N);
-  }
+  // columns per CTA: the smallest power of two that holds N, 32 above 16 (a wider
+  // CTA would leave fewer threads to share a segment's entries)
+  if (N <= SPMM_NARROW)
+    k_spmm_segments_narrow<T><<<(unsigned)nseg, 256, 0, st>>>(seg_start, seg_end, col, val, Xc, ldx, part, N);
+  else if (N <= 8)
+    spmm_segments_cx<T, 8>(nseg, seg_start, seg_end, col, val, Xc, ldx, part, N, st);
+  else if (N <= 16)
+    spmm_segments_cx<T, 16>(nseg, seg_start, seg_end, col, val, Xc, ldx, part, N, st);
+  else
+    spmm_segments_cx<T, 32>(nseg, seg_start, seg_end, col, val, Xc, ldx, part, N, st);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 template void launch_spmm_segments<double>(int64_t, const int64_t*, const int64_t*, const int32_t*, const double*,
-                                           const double*, const double*, int64_t, double*, int, cudaStream_t);
+                                           const double*, int64_t, double*, int, cudaStream_t);
 template void launch_spmm_segments<float>(int64_t, const int64_t*, const int64_t*, const int32_t*, const double*,
-                                          const double*, const float*, int64_t, double*, int, cudaStream_t);
+                                          const float*, int64_t, double*, int, cudaStream_t);
 
 void launch_seg_reduce(int nrows, const int64_t* row_seg_ptr, const double* part, double sgn, const double* base,
                        int64_t ldb, double alpha_base, double* out, int64_t ldo, int N, cudaStream_t st) {
@@ -1932,8 +2042,12 @@ void launch_spmm_nodes_df(int64_t nrows, const int32_t* rnode, const int64_t* pt
 void launch_grp_rows_df(int n_items, const int4* items, const int64_t* ec_ptr, const int32_t* ec_col,
                         const float2* coef, const double* Xc, int64_t ldx, double* part, int N, cudaStream_t st) {
   if (n_items <= 0 || N <= 0) return;
-  dim3 g((unsigned)n_items, (unsigned)((N + GRP_CT - 1) / GRP_CT));
-  k_grp_rows_df<<<g, GRP_CT, 0, st>>>(items, ec_ptr, ec_col, coef, Xc, ldx, part, N);
+  // 16 columns a CTA while one tile of 16 holds the block, else 32
+  if (N <= 16)
+    k_grp_rows_df<16><<<(unsigned)n_items, 16 * GRP_KMAX, 0, st>>>(items, ec_ptr, ec_col, coef, Xc, ldx, part, N);
+  else
+    k_grp_rows_df<32><<<dim3((unsigned)n_items, (unsigned)((N + 31) / 32)), 32 * GRP_KMAX, 0, st>>>(
+        items, ec_ptr, ec_col, coef, Xc, ldx, part, N);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 

@@ -36,6 +36,9 @@ void launch_potential_analytic(const double* qpts, int64_t nq, const double* axy
 void launch_check_finite(const double* x, int64_t n, int* flag, cudaStream_t st);
 void launch_gather_sum(int64_t n_out, const double* base, const int64_t* cptr, const int64_t* cidx,
                        const double* blk, double* out, cudaStream_t st);
+// out[q] = v[q] * scale[col[q]]
+void launch_col_scale(int64_t n, const double* v, const double* scale, const int32_t* col, double* out,
+                      cudaStream_t st);
 void launch_permute(int64_t n, const double* src, const int64_t* perm, double* dst, cudaStream_t st);
 void launch_to_f32(const double* src, float* dst, int64_t n, cudaStream_t st);
 
@@ -110,11 +113,10 @@ template <typename T>
 void launch_spmm_nodes(int64_t nrows, const int32_t* rnode, const int64_t* ptr, const int32_t* col,
                        const double* val, double sgn, const double* Xe, int64_t ldxe, T* out, int64_t ldo,
                        int N, cudaStream_t st);
-// part[seg] = sum_{q in seg} val[q] * scale[col[q]] * Xc[col[q]]  (scale may be NULL)
+// part[seg] = sum_{q in seg} val[q] * Xc[col[q]]
 template <typename T>
 void launch_spmm_segments(int64_t nseg, const int64_t* seg_start, const int64_t* seg_end, const int32_t* col,
-                          const double* val, const double* scale, const T* Xc, int64_t ldx, double* part,
-                          int N, cudaStream_t st);
+                          const double* val, const T* Xc, int64_t ldx, double* part, int N, cudaStream_t st);
 // out[r] = alpha_base * base[r] + sgn * sum_{segs of r} part[seg]
 void launch_seg_reduce(int nrows, const int64_t* row_seg_ptr, const double* part, double sgn,
                        const double* base, int64_t ldb, double alpha_base, double* out, int64_t ldo, int N,

@@ -1,0 +1,36 @@
+"""Sizes at the edges of the kernels' column tiles, thread splits and dispatch rules,
+against the FP64 CPU oracle (products) or the general path (whole calls)."""
+import numpy as np
+import pytest
+
+import workloads as W
+from tests.gpu_util import cuda_available, gpu_system, rel_err, to_dev, torch
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")]
+
+
+@pytest.fixture(scope="module")
+def tiny_pair():
+    from oracle.operators import Discretisation
+    s = W.tiny(seed=11)
+    return Discretisation(s), gpu_system(s)
+
+
+# FP64 products: sums of up to a few thousand terms whose magnitudes exceed the result by
+# at most ~1e3 here, at 2^-53 (DFMA) or a few 2^-48 (the tensor engine) a term: 1e-10 of
+# the largest entry for H, 1e-11 for M (smaller terms), 1e-10 after the Schur solve
+@pytest.mark.parametrize("engine", ["dfma", "tensor"])
+@pytest.mark.parametrize("N", [5, 8, 9, 15, 16, 17, 31, 32, 65])
+def test_products_at_tile_edges(tiny_pair, engine, N):
+    d, G = tiny_pair
+    X = W.random_block(d.system, N, seed=300 + N)
+    wide = torch.zeros((X.shape[0], N + 3), dtype=torch.float64, device="cuda")
+    wide[:, :N] = to_dev(X)
+    G.set_fp64_engine(engine)
+    try:
+        for Xd in (to_dev(X), wide[:, :N]):
+            assert rel_err(G.apply_H(Xd, torch.empty_like(wide)[:, :N]), d.apply_H_assembled(X)) < 1e-10
+            assert rel_err(G.apply_M(Xd), d.apply_M_assembled(X)) < 1e-11
+            assert rel_err(G.apply_Minv(Xd), d.apply_Minv_block(X)) < 1e-10
+    finally:
+        G.set_fp64_engine("dfma")
