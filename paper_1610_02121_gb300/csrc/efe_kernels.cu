@@ -1118,42 +1118,48 @@ __global__ void k_cheb_combine_f4(int64_t nrows, int ld4, const double* __restri
 // ---------------------------------------------------------------------------
 // dense FP64
 // ---------------------------------------------------------------------------
-constexpr int GT = 48;  // output tile (16 x 16 threads, 3 x 3 each)
+constexpr int GT = 48;  // output tile rows (and widest tile): 16 x 16 threads, 3 x TN outputs each
 
+// TN: outputs per thread along the columns (tile 48 x 16 TN); the launcher takes
+// the tile that pads the columns least
+template <int TN>
 __global__ void __launch_bounds__(256) k_gemm_nn(int64_t M, int Nc, int K, double alpha,
                                                  const double* __restrict__ A, int64_t lda,
                                                  const double* __restrict__ B, int64_t ldb, double beta,
                                                  double* __restrict__ C, int64_t ldc, int64_t sA, int64_t sB,
                                                  int64_t sC) {
+  constexpr int TC = 16 * TN;
   __shared__ double As[16][GT + 1];
-  __shared__ double Bs[16][GT + 1];
+  __shared__ double Bs[16][TC + 1];
   // batch member blockIdx.z (strides 0 for a single product)
   A += blockIdx.z * sA;
   B += blockIdx.z * sB;
   C += blockIdx.z * sC;
   const int64_t row0 = (int64_t)blockIdx.x * GT;
-  const int col0 = blockIdx.y * GT;
+  const int col0 = blockIdx.y * TC;
   const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-  double acc[3][3] = {};
+  double acc[3][TN] = {};
   for (int k0 = 0; k0 < K; k0 += 16) {
     for (int idx = tid; idx < 16 * GT; idx += 256) {
       const int r = idx / 16, kk = idx % 16;
       As[kk][r] = (row0 + r < M && k0 + kk < K) ? A[(row0 + r) * lda + k0 + kk] : 0.0;
-      const int kb = idx / GT, cc = idx % GT;
+    }
+    for (int idx = tid; idx < 16 * TC; idx += 256) {
+      const int kb = idx / TC, cc = idx % TC;
       Bs[kb][cc] = (k0 + kb < K && col0 + cc < Nc) ? B[(int64_t)(k0 + kb) * ldb + col0 + cc] : 0.0;
     }
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < 16; ++kk) {
-      double av[3], bv[3];
+      double av[3], bv[TN];
 #pragma unroll
       for (int a = 0; a < 3; ++a) av[a] = As[kk][ty * 3 + a];
 #pragma unroll
-      for (int b = 0; b < 3; ++b) bv[b] = Bs[kk][tx * 3 + b];
+      for (int b = 0; b < TN; ++b) bv[b] = Bs[kk][tx * TN + b];
 #pragma unroll
       for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+        for (int b = 0; b < TN; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
     }
     __syncthreads();
   }
@@ -1162,8 +1168,8 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int64_t M, int Nc, int K, doubl
     const int64_t r = row0 + ty * 3 + a;
     if (r >= M) continue;
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int c = col0 + tx * 3 + b;
+    for (int b = 0; b < TN; ++b) {
+      const int c = col0 + tx * TN + b;
       if (c >= Nc) continue;
       double v = alpha * acc[a][b];
       if (beta != 0.0) v += beta * C[r * ldc + c];
@@ -1201,24 +1207,32 @@ __global__ void __launch_bounds__(256) k_gemm_nn_small(int64_t M, int Nc, int K,
   }
 }
 
-constexpr int64_t TN_KC = 8192;
+// A^T B (split K): each CTA forms one (16 TM) x (16 TM) output tile over a range of
+// rows, TM x TM outputs a thread.  The FP64 pipe bounds it (about two FMAs a clock
+// and SM), so the tile is the one that pads the block least (gemm_tn_tile) and K is
+// split until every SM has work.  49,005 rows: 12 vectors in one 48 x 48 tile over
+// six 8192-row splits took 3.1 ms, in 16 x 16 tiles over 294 splits 29 us.
+constexpr int64_t TN_KC = 64;    // fewest rows of a split
 
+template <int TM>
 __global__ void __launch_bounds__(256) k_gemm_tn_part(int64_t K, int64_t kc, int Na, int Nb,
                                                       const double* __restrict__ A, int64_t lda,
                                                       const double* __restrict__ B, int64_t ldb,
                                                       double* __restrict__ part, int sym) {
+  constexpr int T = 16 * TM;
   // symmetric products: only tiles on or above the diagonal are formed
   if (sym && blockIdx.x > blockIdx.y) return;
-  __shared__ double As[16][GT + 1];
-  __shared__ double Bs[16][GT + 1];
-  const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+  __shared__ double As[16][T + 1];
+  __shared__ double Bs[16][T + 1];
+  const int i0 = blockIdx.x * T, j0 = blockIdx.y * T;
   const int64_t kb = (int64_t)blockIdx.z * kc;
   const int64_t ke = min(K, kb + kc);
   const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-  double acc[3][3] = {};
+  double acc[TM][TM] = {};
   for (int64_t k0 = kb; k0 < ke; k0 += 16) {
-    for (int idx = tid; idx < 16 * GT; idx += 256) {
-      const int kk = idx / GT, c = idx % GT;
+#pragma unroll
+    for (int idx = tid; idx < 16 * T; idx += 256) {
+      const int kk = idx / T, c = idx % T;
       const bool okk = k0 + kk < ke;
       As[kk][c] = (okk && i0 + c < Na) ? A[(k0 + kk) * lda + i0 + c] : 0.0;
       Bs[kk][c] = (okk && j0 + c < Nb) ? B[(k0 + kk) * ldb + j0 + c] : 0.0;
@@ -1226,44 +1240,57 @@ __global__ void __launch_bounds__(256) k_gemm_tn_part(int64_t K, int64_t kc, int
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < 16; ++kk) {
-      double av[3], bv[3];
+      double av[TM], bv[TM];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) av[a] = As[kk][ty * 3 + a];
+      for (int a = 0; a < TM; ++a) av[a] = As[kk][ty * TM + a];
 #pragma unroll
-      for (int b = 0; b < 3; ++b) bv[b] = Bs[kk][tx * 3 + b];
+      for (int b = 0; b < TM; ++b) bv[b] = Bs[kk][tx * TM + b];
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+      for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+        for (int b = 0; b < TM; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
     }
     __syncthreads();
   }
   double* Pp = part + (int64_t)blockIdx.z * Na * Nb;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int r = i0 + ty * 3 + a;
+  for (int a = 0; a < TM; ++a) {
+    const int r = i0 + ty * TM + a;
     if (r >= Na) continue;
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int c = j0 + tx * 3 + b;
+    for (int b = 0; b < TM; ++b) {
+      const int c = j0 + tx * TM + b;
       if (c < Nb) Pp[(int64_t)r * Nb + c] = acc[a][b];
     }
   }
 }
 
-__global__ void k_gemm_tn_reduce(int nsplit, int Na, int Nb, const double* __restrict__ part, double* __restrict__ C,
-                                 int64_t ldc, int sym) {
-  const int64_t idx0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx0 >= (int64_t)Na * Nb) return;
-  const int64_t idx = idx0;
-  int64_t src = idx;
-  if (sym) {
-    const int i = (int)(idx / Nb), j = (int)(idx % Nb);
-    if (i / GT > j / GT) src = (int64_t)j * Nb + i;  // mirrored from the tile above the diagonal
-  }
+// C = sum of the split-K partials in fixed order: 32 outputs a block, eight thread
+// rows take every eighth partial and the row sums are added in order.  tile: the
+// products' tile size (the mirrored tiles of a symmetric product were not formed)
+__global__ void __launch_bounds__(256) k_gemm_tn_reduce(int nsplit, int Na, int Nb, int tile,
+                                                        const double* __restrict__ part, double* __restrict__ C,
+                                                        int64_t ldc, int sym) {
+  __shared__ double rs[8][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int64_t idx = blockIdx.x * 32LL + x, tot = (int64_t)Na * Nb;
   double s = 0.0;
-  for (int sp = 0; sp < nsplit; ++sp) s += part[(int64_t)sp * Na * Nb + src];
-  C[(idx / Nb) * ldc + idx % Nb] = s;
+  if (idx < tot) {
+    int64_t src = idx;
+    if (sym) {
+      const int i = (int)(idx / Nb), j = (int)(idx % Nb);
+      if (i / tile > j / tile) src = (int64_t)j * Nb + i;
+    }
+    for (int sp = y; sp < nsplit; sp += 8) s += part[(int64_t)sp * tot + src];
+  }
+  rs[y][x] = s;
+  __syncthreads();
+  if (y == 0 && idx < tot) {
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v += rs[k][x];
+    C[(idx / Nb) * ldc + idx % Nb] = v;
+  }
 }
 
 // Right-looking Cholesky A = L L^T in one CTA (lower triangle; upper zeroed),
@@ -1491,18 +1518,32 @@ __global__ void k_sort_eig(const double* __restrict__ w, const double* __restric
 
 constexpr int RN_ROWS = 2048;
 
-__global__ void k_resid_part(int64_t nrows, const double* __restrict__ HX, int64_t ldh, const double* __restrict__ MX,
-                             int64_t ldm, const double* __restrict__ eps, int N, double* __restrict__ part) {
+// a CTA: 32 columns x 8 thread rows over RN_ROWS rows, row sums added in order (one
+// thread per column left a single load in flight: 1.6 ms for 559,625 x 135, now 0.31)
+__global__ void __launch_bounds__(256) k_resid_part(int64_t nrows, const double* __restrict__ HX, int64_t ldh,
+                                                    const double* __restrict__ MX, int64_t ldm,
+                                                    const double* __restrict__ eps, int N, double* __restrict__ part) {
+  __shared__ double red[8][32];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t r0 = (int64_t)blockIdx.x * RN_ROWS;
   const int64_t r1 = min(nrows, r0 + RN_ROWS);
-  for (int c = threadIdx.x; c < N; c += blockDim.x) {
+  const int c = blockIdx.y * 32 + tx;
+  double s = 0.0;
+  if (c < N) {
     const double ec = eps[c];
-    double s = 0.0;
-    for (int64_t r = r0; r < r1; ++r) {
+#pragma unroll 8
+    for (int64_t r = r0 + ty; r < r1; r += 8) {
       const double d = HX[r * ldh + c] - ec * MX[r * ldm + c];
       s = fma(d, d, s);
     }
-    part[(int64_t)blockIdx.x * N + c] = s;
+  }
+  red[ty][tx] = s;
+  __syncthreads();
+  if (ty == 0 && c < N) {
+    double t = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t += red[k][tx];
+    part[(int64_t)blockIdx.x * N + c] = t;
   }
 }
 
@@ -1530,11 +1571,20 @@ __global__ void k_dot_part(int64_t n, const double* __restrict__ x, const double
   }
 }
 
-__global__ void k_dot_final(int nb, const double* __restrict__ part, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[b];
-    *out = s;
+// fixed-order tree over the block partials (one thread adding 256 of them in turn
+// took 16.6 us of every Lanczos dot; the tree takes 2.5)
+__global__ void __launch_bounds__(256) k_dot_final(int nb, const double* __restrict__ part, double* __restrict__ out) {
+  __shared__ double red[8];
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nb; b += 256) s += part[b];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t += red[i];
+    *out = t;
   }
 }
 
@@ -1743,34 +1793,65 @@ void launch_zero_rows_f32(int64_t nrows, float* X, int64_t ldx, int N, cudaStrea
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
+namespace {
+void gemm_nn_tiles(int64_t M, int Nc, int K, double alpha, const double* A, int64_t lda, int64_t sA, const double* B,
+                   int64_t ldb, int64_t sB, double beta, double* C, int64_t ldc, int64_t sC, int batch,
+                   cudaStream_t st) {
+  // columns per tile: 48, 32 or 16, whichever pads Nc least (the FP64 pipe spends
+  // the same time on a padded column as on a real one)
+  int tn = 3, pad = (Nc + 47) / 48 * 48;
+  for (int t = 2; t >= 1; --t)
+    if ((Nc + 16 * t - 1) / (16 * t) * (16 * t) < pad) { tn = t; pad = (Nc + 16 * t - 1) / (16 * t) * (16 * t); }
+  dim3 g((unsigned)((M + GT - 1) / GT), (unsigned)(pad / (16 * tn)), (unsigned)batch);
+  if (tn == 3) k_gemm_nn<3><<<g, 256, 0, st>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc, sA, sB, sC);
+  else if (tn == 2) k_gemm_nn<2><<<g, 256, 0, st>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc, sA, sB, sC);
+  else k_gemm_nn<1><<<g, 256, 0, st>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc, sA, sB, sC);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+}
+}  // namespace
+
 void launch_gemm_nn(int64_t M, int Nc, int K, double alpha, const double* A, int64_t lda, const double* B,
                     int64_t ldb, double beta, double* C, int64_t ldc, cudaStream_t st) {
   if (M <= 0 || Nc <= 0) return;
-  dim3 g((unsigned)((M + GT - 1) / GT), (unsigned)((Nc + GT - 1) / GT));
   // fewer 48 x 48 output tiles than SMs: one output per thread in 16 x 16 tiles
-  if ((int64_t)g.x * g.y < current_sm_count()) {
+  if (((M + GT - 1) / GT) * ((Nc + GT - 1) / GT) < current_sm_count()) {
     dim3 gs((unsigned)((M + 15) / 16), (unsigned)((Nc + 15) / 16));
     k_gemm_nn_small<<<gs, 256, 0, st>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
   } else {
-    k_gemm_nn<<<g, 256, 0, st>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc, 0, 0, 0);
+    gemm_nn_tiles(M, Nc, K, alpha, A, lda, 0, B, ldb, 0, beta, C, ldc, 0, 1, st);
   }
-  g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
 void launch_gemm_nn_batched(int64_t M, int Nc, int K, const double* A, int64_t lda, int64_t sA, const double* B,
                             int64_t ldb, int64_t sB, double* C, int64_t ldc, int64_t sC, int batch,
                             cudaStream_t st) {
   if (M <= 0 || Nc <= 0 || batch <= 0) return;
-  dim3 g((unsigned)((M + GT - 1) / GT), (unsigned)((Nc + GT - 1) / GT), (unsigned)batch);
-  k_gemm_nn<<<g, 256, 0, st>>>(M, Nc, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, sA, sB, sC);
-  g_launches.fetch_add(1, std::memory_order_relaxed);
+  gemm_nn_tiles(M, Nc, K, 1.0, A, lda, sA, B, ldb, sB, 0.0, C, ldc, sC, batch, st);
 }
 
-// K splits of an A^T B product: enough for about four CTAs per SM over the
-// output tiles, none shorter than TN_KC rows
+namespace {
+// outputs per thread and axis (tile 16 TM) that pad an (Na x Nb) product least; the
+// larger tile on a tie
+int gemm_tn_tm(int Na, int Nb) {
+  int best = 3;
+  int64_t area = -1;
+  for (int tm = 3; tm >= 1; --tm) {
+    const int64_t t = 16 * tm;
+    const int64_t ar = ((Na + t - 1) / t) * ((Nb + t - 1) / t) * t * t;
+    if (area < 0 || ar < area) { area = ar; best = tm; }
+  }
+  return best;
+}
+}  // namespace
+
+// K splits of an A^T B product: about two CTAs per SM over the output tiles (four
+// for 48 x 48 tiles), none shorter than TN_KC rows
 int64_t gemm_tn_splits(int64_t K, int Na, int Nb) {
-  const int64_t tiles = (int64_t)((Na + GT - 1) / GT) * ((Nb + GT - 1) / GT);
-  const int64_t want = (4 * (int64_t)current_sm_count() + tiles - 1) / tiles;
+  const int tm = gemm_tn_tm(Na, Nb);
+  const int64_t t = 16 * tm;
+  const int64_t tiles = (int64_t)((Na + t - 1) / t) * ((Nb + t - 1) / t);
+  const int64_t want = ((tm == 3 ? 4 : 2) * (int64_t)current_sm_count() + tiles - 1) / tiles;
   const int64_t most = (K + TN_KC - 1) / TN_KC;
   return std::max<int64_t>(1, std::min(want, most));
 }
@@ -1784,11 +1865,14 @@ void launch_gemm_tn(int64_t K, int Na, int Nb, const double* A, int64_t lda, con
   nsplit = std::max<int64_t>(1, std::min(nsplit, work_elems / ((int64_t)Na * Nb)));
   const int64_t kc = ((K + nsplit - 1) / nsplit + 15) / 16 * 16;
   nsplit = std::max<int64_t>(1, (K + kc - 1) / kc);
-  dim3 g((unsigned)((Na + GT - 1) / GT), (unsigned)((Nb + GT - 1) / GT), (unsigned)nsplit);
+  const int tm = gemm_tn_tm(Na, Nb), t = 16 * tm;
+  dim3 g((unsigned)((Na + t - 1) / t), (unsigned)((Nb + t - 1) / t), (unsigned)nsplit);
   const int sy = (sym && Na == Nb) ? 1 : 0;
-  k_gemm_tn_part<<<g, 256, 0, st>>>(K, kc, Na, Nb, A, lda, B, ldb, work, sy);
+  if (tm == 1) k_gemm_tn_part<1><<<g, 256, 0, st>>>(K, kc, Na, Nb, A, lda, B, ldb, work, sy);
+  else if (tm == 2) k_gemm_tn_part<2><<<g, 256, 0, st>>>(K, kc, Na, Nb, A, lda, B, ldb, work, sy);
+  else k_gemm_tn_part<3><<<g, 256, 0, st>>>(K, kc, Na, Nb, A, lda, B, ldb, work, sy);
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  k_gemm_tn_reduce<<<grid1((int64_t)Na * Nb, 256), 256, 0, st>>>((int)nsplit, Na, Nb, work, C, ldc, sy);
+  k_gemm_tn_reduce<<<grid1((int64_t)Na * Nb, 32), 256, 0, st>>>((int)nsplit, Na, Nb, t, work, C, ldc, sy);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
@@ -1854,7 +1938,7 @@ void launch_sort_eig(const double* w, const double* V, int n, int ldv, double* w
 void launch_resid_norms(int64_t nrows, const double* HX, int64_t ldh, const double* MX, int64_t ldm,
                         const double* eps, int N, double* part, double* out, cudaStream_t st) {
   const int nb = (int)((nrows + RN_ROWS - 1) / RN_ROWS);
-  k_resid_part<<<nb, 128, 0, st>>>(nrows, HX, ldh, MX, ldm, eps, N, part);
+  k_resid_part<<<dim3((unsigned)nb, (unsigned)((N + 31) / 32)), 256, 0, st>>>(nrows, HX, ldh, MX, ldm, eps, N, part);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   k_resid_final<<<grid1(N, 128), 128, 0, st>>>(nb, N, part, out);
   g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -1863,7 +1947,7 @@ void launch_resid_norms(int64_t nrows, const double* HX, int64_t ldh, const doub
 void launch_dot(int64_t n, const double* x, const double* y, double* part, double* out, cudaStream_t st) {
   k_dot_part<<<256, 256, 0, st>>>(n, x, y, part);
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  k_dot_final<<<1, 32, 0, st>>>(256, part, out);
+  k_dot_final<<<1, 256, 0, st>>>(256, part, out);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 

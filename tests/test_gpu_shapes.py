@@ -34,3 +34,19 @@ def test_products_at_tile_edges(tiny_pair, engine, N):
             assert rel_err(G.apply_Minv(Xd), d.apply_Minv_block(X)) < 1e-10
     finally:
         G.set_fp64_engine("dfma")
+
+
+# Cholesky-QR and Rayleigh-Ritz at the edges of the A^T B and A B tiles (16, 32, 48), against the
+# oracle; the figures of the ordinary case (1e-9 on the Ritz values, 1e-8 on the residuals)
+@pytest.mark.parametrize("N", [1, 2, 15, 16, 17, 32, 33, 48, 49])
+def test_rayleigh_ritz_at_tile_edges(tiny_pair, N):
+    from oracle.chfsi import cholqr, rayleigh_ritz
+    d, G = tiny_pair
+    X = W.random_block(d.system, N, seed=400 + N)
+    eps_ref, _, res_ref = rayleigh_ritz(d.apply_H_assembled, d.apply_M_assembled, cholqr(X)[0])
+    Xd = to_dev(X)
+    eps, res = G.rayleigh_ritz(Xd)
+    np.testing.assert_allclose(eps, eps_ref, atol=1e-9, rtol=1e-10)
+    np.testing.assert_allclose(res, res_ref, atol=1e-8, rtol=1e-6)
+    gram = (Xd.T @ G.apply_M(Xd)).cpu().numpy()
+    np.testing.assert_allclose(gram, np.eye(N), atol=1e-10)
