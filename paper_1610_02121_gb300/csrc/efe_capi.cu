@@ -99,6 +99,8 @@ struct efe_handle {
   double* tnwork = nullptr;
   int64_t tnwork_elems = 0;
   double* rpart = nullptr;
+  double* cellP = nullptr;    // FP64 cell products of up to cellP_cols columns, all cells
+  int cellP_cols = 0;
   double* lz = nullptr;       // Lanczos vectors (6 * rows) + scalars
   int Nres32 = 0, ld32 = 0, ncb = 0;
   // FP32 classical blocks of the mixed degrees: two recurrence slots (each
@@ -262,6 +264,11 @@ inline bool coup_tiles_fit(const efe_handle* h, int N) {
 // blocks (a third FP64 block) but forms them in two column panels inside W.
 constexpr int64_t WHOLE_RR_MAX_BYTES = 16ll << 30;
 
+// Largest scratch array of the FP64 cell products (reserve): 256 MB hold 32 columns
+// on 8,388 cells or 11 on the 23,125 of the 16-atom silicon mesh.  Beyond it the
+// cells of one colour are enough to fill the chip.
+constexpr int64_t CELLP_MAX_BYTES = 256ll << 20;
+
 // FP32 blocks of the mixed degrees (see efe_handle): dropped before the FP64
 // workspace they may live in is reallocated
 void free32(efe_handle* h) {
@@ -312,6 +319,17 @@ int reserve(efe_handle* h, int N) {
   h->tnwork_elems = std::max<int64_t>(gemm_tn_work_elems(R, N, N), 4 * (int64_t)N * N);
   TRY(dalloc(h, &h->tnwork, h->tnwork_elems));
   TRY(dalloc(h, &h->rpart, ((R + 2047) / 2048 + 1) * (int64_t)N));
+  // scratch of the FP64 cell products: as many columns as the kernel takes at once
+  // and CELLP_MAX_BYTES hold (narrow blocks on large meshes, wider ones on small)
+  dfree(h, h->cellP);
+  h->cellP = nullptr;
+  h->cellP_cols = 0;
+  {
+    const int64_t per = (int64_t)sizeof(double) * cell_f64_scratch_elems(h->n_cell, 1);
+    const int nc = (int)std::min<int64_t>({N, cell_f64_max_cols(), CELLP_MAX_BYTES / std::max<int64_t>(1, per)});
+    if (nc > 0) TRY(dalloc(h, &h->cellP, cell_f64_scratch_elems(h->n_cell, nc)));
+    h->cellP_cols = nc;
+  }
   dfree(h, h->oz_fexp);
   dfree(h, h->oz_bexp);
   dfree(h, h->oz_pairs);
@@ -472,10 +490,7 @@ int cell_apply_all(efe_handle* h, const T* Hc, const T* Y, int64_t ldy, T* Wc, i
     TRY(timed_begin(h, st, &slot));
     const int32_t* cl = h->colour_cells + h->colour_off[c];
     if constexpr (sizeof(T) == 8) {
-      if (N <= 8)
-        launch_cell_apply_narrow_f64((const double*)Hc, cl, nc, h->mesh, (const double*)Y, ldy, (double*)Wc, ldw, N, st);
-      else
-        launch_cell_apply_f64((const double*)Hc, cl, nc, h->mesh, (const double*)Y, ldy, (double*)Wc, ldw, N, st);
+      launch_cell_apply_f64((const double*)Hc, cl, nc, h->mesh, (const double*)Y, ldy, (double*)Wc, ldw, N, st);
     } else {
       if (tc) {
         if (launch_cell_tc3(h->Aimg32, cl, nc, h->mesh, (const float*)Y, ldy, (float*)Wc, ldw, N,
@@ -501,11 +516,28 @@ int cell_apply_all(efe_handle* h, const T* Hc, const T* Y, int64_t ldy, T* Wc, i
 // vectors; the plain FP64 kernels otherwise.
 bool use_df(const efe_handle* h, int N) { return h->fp64_engine == 1 && h->nE > 0 && N > 8; }
 
+// The FP64 cell products run over all cells at once, through a scratch array, where
+// that array was reserved for this many columns (reserve()) and the DFMA kernel is
+// the one that runs.
+bool cells_at_once(const efe_handle* h, int N) {
+  return N <= h->cellP_cols && (h->fp64_engine == 0 || N <= 8);
+}
+
+template <typename T>
+int couple_H(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, int64_t ldxe, T* Wc, int64_t ldw, double* We,
+             int64_t ldwe, int N, cudaStream_t st);
+
 // --- H^E X: classical cell products + enrichment coupling (Eq. H2x2) ---
 //   Wc = H^cc Xc + (H^ec)^T Xe ;  We = H^ec Xc + H^ee Xe
 template <typename T>
 int apply_H_generic(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, int64_t ldxe, T* Wc, int64_t ldw,
                     double* We, int64_t ldwe, int N, cudaStream_t st, const T* Hc) {
+  if (sizeof(T) == 8 && cells_at_once(h, N)) {
+    launch_cell_apply_f64_all((const double*)Hc, h->n_cell, h->mesh, (const double*)Xc, ldx, h->cellP, (double*)Wc, ldw,
+                              N, st);
+    CKL();
+    return couple_H<T>(h, Xc, ldx, Xe, ldxe, Wc, ldw, We, ldwe, N, st);
+  }
   if (ldw == N) {
     CK(cudaMemsetAsync(Wc, 0, sizeof(T) * h->n_nodes * N, st));
   } else {
@@ -514,6 +546,13 @@ int apply_H_generic(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, i
     CKL();
   }
   TRY(cell_apply_all<T>(h, Hc, Xc, ldx, Wc, ldw, N, st));
+  return couple_H<T>(h, Xc, ldx, Xe, ldxe, Wc, ldw, We, ldwe, N, st);
+}
+
+// the enrichment coupling of H^E X: Wc += (H^ec)^T Xe, We = H^ec Xc + H^ee Xe
+template <typename T>
+int couple_H(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, int64_t ldxe, T* Wc, int64_t ldw, double* We,
+             int64_t ldwe, int N, cudaStream_t st) {
   if constexpr (sizeof(T) == 8) {
     if (use_df(h, N)) {
       launch_df_rows(h->nE, N, Xe, ldxe, h->xe2, st);

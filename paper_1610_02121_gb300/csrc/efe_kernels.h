@@ -48,9 +48,13 @@ void launch_cell_apply_f64(const double* Hcc, const int32_t* cells, int64_t ncel
                            const double* Y, int64_t ldy, double* W, int64_t ldw, int N, cudaStream_t st);
 void launch_cell_apply_f32(const float* Hcc, const int32_t* cells, int64_t ncells, const MeshDev& m,
                            const float* Y, int64_t ldy, float* W, int64_t ldw, int N, cudaStream_t st);
+// W = sum over all cells of H_e Y_e (every row of W written) in two launches through
+// the scratch array Pc of cell_f64_scratch_elems(n_cell, N) doubles; N <= cell_f64_max_cols()
+int cell_f64_max_cols();
+int64_t cell_f64_scratch_elems(int64_t n_cell, int N);
+void launch_cell_apply_f64_all(const double* Hcc, int64_t n_cell, const MeshDev& m, const double* Y, int64_t ldy,
+                               double* Pc, double* W, int64_t ldw, int N, cudaStream_t st);
 // narrow blocks (N <= 8): one warp per row of H_e
-void launch_cell_apply_narrow_f64(const double* Hcc, const int32_t* cells, int64_t ncells, const MeshDev& m,
-                                  const double* Y, int64_t ldy, double* W, int64_t ldw, int N, cudaStream_t st);
 void launch_cell_apply_narrow_f32(const float* Hcc, const int32_t* cells, int64_t ncells, const MeshDev& m,
                                   const float* Y, int64_t ldy, float* W, int64_t ldw, int N, cudaStream_t st);
 // node-major enrichment products with FP32 arithmetic (mixed-precision filter) over
