@@ -1852,8 +1852,14 @@ int dense_scratch(efe_handle* h, int64_t bytes) {
   return EFE_OK;
 }
 
-// the one-CTA dense kernels up to these sizes, the blocked multi-CTA ones above
-constexpr int CHOL_ONE_CTA_MAX = 2048;
+// the one-CTA dense kernels up to these sizes, the blocked multi-CTA ones above:
+// the one-CTA Cholesky took 410 us at n = 135 and 28 ms at 640 (blocked: 0.25 and 2.4
+// ms), the one-CTA Jacobi eigensolver 16 ms at 135 (blocked: 3.4); a whole
+// Rayleigh-Ritz call of 33 vectors takes 3.2 ms with the one-CTA kernels and 3.6 with
+// the blocked ones, of 48 the same, of 12 2.36 and 2.39.  DENSE_SMALL_MAX: the N x N
+// products go to the tensor-core FP64 engine above it.
+constexpr int CHOL_ONE_CTA_MAX = 64;
+constexpr int EIG_ONE_CTA_MAX = 48;
 constexpr int DENSE_SMALL_MAX = 512;
 
 // A = L L^T in place (lower, n x n, ld n); *info: 0 or j + 1 of the first breakdown
@@ -1871,12 +1877,8 @@ int chol_lower(efe_handle* h, double* A, int n, cudaStream_t st, double* min_rat
 
 // Li = L^-1 (lower, n x n, ld n)
 int trinv_lower(efe_handle* h, const double* L, int n, double* Li, cudaStream_t st) {
-  if (n <= DENSE_SMALL_MAX && !h->opt_dense_blocked) {
-    launch_trinv_lower(L, n, n, Li, n, st);
-  } else {
-    TRY(dense_scratch(h, (int64_t)sizeof(double) * ((int64_t)n * n / 4 + 64 * (int64_t)n)));
-    launch_trinv_blocked(L, n, n, Li, n, (double*)h->dsc, st);
-  }
+  TRY(dense_scratch(h, (int64_t)sizeof(double) * ((int64_t)n * n / 4 + 64 * (int64_t)n)));
+  launch_trinv_blocked(L, n, n, Li, n, (double*)h->dsc, st);
   CKL();
   return EFE_OK;
 }
@@ -1901,7 +1903,7 @@ int dense_nn(efe_handle* h, int N, const double* A, const double* B, double* C, 
 int sym_eig_blocked(efe_handle* h, const double* C, int N, double* V, double* w, double* E, cudaStream_t st);
 
 int sym_eig(efe_handle* h, const double* C, int N, double* V, double* w, double* E, cudaStream_t st) {
-  if (N > DENSE_SMALL_MAX || h->opt_dense_blocked) return sym_eig_blocked(h, C, N, V, w, E, st);
+  if (N > EIG_ONE_CTA_MAX || h->opt_dense_blocked) return sym_eig_blocked(h, C, N, V, w, E, st);
   const int64_t NN = (int64_t)N * N;
   float* C32 = reinterpret_cast<float*>(E);
   float* V32 = C32 + NN;
@@ -1931,7 +1933,7 @@ int sym_eig(efe_handle* h, const double* C, int N, double* V, double* w, double*
     CKL();
     return EFE_OK;
   }
-  launch_trinv_lower(G, N, N, Li, N, st);
+  TRY(trinv_lower(h, G, N, Li, st));
   launch_transpose(Li, N, N, LiT, N, st);
   launch_gemm_nn(N, N, N, 1.0, Q0, N, LiT, N, 0.0, Q, N, st);
   launch_gemm_tn(N, N, N, Q, N, C, N, T1, N, h->tnwork, h->tnwork_elems, st, false);
@@ -1961,6 +1963,8 @@ int sym_eig_blocked(efe_handle* h, const double* C, int N, double* V, double* w,
   double* V2 = C2 + NN;
   CK(cudaMemsetAsync(h->info + 1, 0, 2 * sizeof(int), st));
   TRY(dense_scratch(h, block_jacobi_scratch_bytes(N, (int)sizeof(double))));
+  // as dense_nn: below that size the DFMA products are the faster ones
+  const bool engine = h->fp64_engine == 1 && (N > DENSE_SMALL_MAX || h->opt_dense_blocked);
   double ratio = 0.0;
   const int r32 = block_jacobi<float>(C, N, N, V32, N, w32, 40, 1e-12, h->dsc, st, &ratio);
   if (r32 < 0) {
@@ -1970,7 +1974,7 @@ int sym_eig_blocked(efe_handle* h, const double* C, int N, double* V, double* w,
   bool refine = true;
   if (r32 == 0) {
     launch_f32_to_f64_rows(N, V32, N, Q0, N, N, st);
-    if (h->fp64_engine == 1) {
+    if (engine) {
       TRY(gemm_gram(h, N, N, N, Q0, N, Q0, N, G, N, true, st));
     } else {
       launch_gemm_tn(N, N, N, Q0, N, Q0, N, G, N, h->tnwork, h->tnwork_elems, st, true);
@@ -1988,7 +1992,7 @@ int sym_eig_blocked(efe_handle* h, const double* C, int N, double* V, double* w,
     TRY(trinv_lower(h, G, N, Li, st));
     launch_transpose(Li, N, N, LiT, N, st);
     TRY(mm(Q0, LiT, Q));
-    if (h->fp64_engine == 1) {
+    if (engine) {
       TRY(gemm_gram(h, N, N, N, Q, N, C, N, T1, N, false, st));
     } else {
       launch_gemm_tn(N, N, N, Q, N, C, N, T1, N, h->tnwork, h->tnwork_elems, st, false);

@@ -131,6 +131,39 @@ __global__ void k_chol_ratio(const double* L, int n, int lda, const double* d0, 
   if (threadIdx.x == 0) *out = *info ? 0.0 : red[0];
 }
 
+// Li = L^-1 for n <= 64 in one CTA: row k of the inverse is final after k steps (one
+// scaling by 1 / L_kk), then every row below takes its multiple of it.  A column per
+// thread by forward substitution is a serial chain of n^2 / 2 dependent FMAs (400 us
+// at n = 128, 517 us at 135); this takes 50 us at n = 64.  L keeps the lower triangle of the shared array, the
+// inverse (transposed) the upper one, a column to the right.
+__global__ void __launch_bounds__(512) k_trinv_leaf(const double* __restrict__ L, int n, int lda,
+                                                    double* __restrict__ Li, int ldi) {
+  __shared__ double S[CB][CB + 2];   // L[i][j] at (i, j), inverse[i][j] at (j, i + 1)
+  const int tid = threadIdx.x;
+  for (int t = tid; t < n * n; t += 512) {
+    const int i = t / n, j = t % n;
+    if (j <= i) {
+      S[i][j] = L[(int64_t)i * lda + j];
+      S[j][i + 1] = i == j ? 1.0 : 0.0;
+    }
+  }
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
+    if (tid <= k) S[tid][k + 1] /= S[k][k];
+    __syncthreads();
+    const int w = k + 1;
+    for (int t = tid; t < (n - 1 - k) * w; t += 512) {
+      const int i = k + 1 + t / w, j = t % w;
+      S[j][i + 1] = fma(-S[i][k], S[j][k + 1], S[j][i + 1]);
+    }
+    __syncthreads();
+  }
+  for (int t = tid; t < n * n; t += 512) {
+    const int i = t / n, j = t % n;
+    Li[(int64_t)i * ldi + j] = j <= i ? S[j][i + 1] : 0.0;
+  }
+}
+
 __global__ void k_zero_block(double* A, int rows, int cols, int lda) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= (int64_t)rows * cols) return;
@@ -160,20 +193,54 @@ __global__ void k_bj_pad(const double* __restrict__ C, int n, int ldc, T* __rest
   V[t] = i == j ? T(1) : T(0);
 }
 
-// One CTA per block pair of round r: diagonalise the BJ_S x BJ_S subproblem
-// [[A_pp, A_pq], [A_qp, A_qq]] in shared memory by cyclic Jacobi; write the
-// rotation J (BJ_S x BJ_S, row-major), the subproblem's eigenvalues, and whether
-// any rotation was applied.
+// Rotation of the pair (i, j) that (nearly) annihilates aij: FP32 in the float
+// stage; in the double stage the tangent comes from FP32 arithmetic and only
+// c = (1 + t^2)^-1/2 is refined to FP64 (an FP32 seed and two Newton steps), so the
+// rotation is orthogonal to FP64 rounding and leaves about 1e-7 of aij.  An exact
+// FP64 tangent costs two divisions and two square roots, about 100 instructions at
+// 64 clocks each in one warp: more than all the rotations of the round.
+__device__ __forceinline__ void bj_angle(float aii, float ajj, float aij, float& c, float& s) {
+  const float tau = (ajj - aii) / (2.f * aij);
+  const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
+  c = 1.f / sqrtf(1.f + t * t);
+  s = t * c;
+}
+__device__ __forceinline__ void bj_angle(double aii, double ajj, double aij, double& c, double& s) {
+  // both scaled by one power of two into the FP32 range
+  const double d = ajj - aii;
+  const int ex = (__double2hiint(fmax(fabs(d), fabs(aij))) >> 20) & 0x7FF;
+  const double sc = __hiloint2double((2046 - min(ex, 2045)) << 20, 0);
+  const float tau = (float)(d * sc) / (2.f * (float)(aij * sc));
+  const float tf = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
+  const double t = (double)tf;
+  const double x = fma(t, t, 1.0);
+  double y = (double)rsqrtf((float)x);
+  const double hx = 0.5 * x;
+  y = y * fma(-hx * y, y, 1.5);
+  y = y * fma(-hx * y, y, 1.5);
+  c = y;
+  s = t * y;
+}
+
+// One CTA per block pair of round r: one cyclic Jacobi sweep over the BJ_S x BJ_S
+// subproblem [[A_pp, A_pq], [A_qp, A_qq]] in shared memory; writes the rotation J
+// (BJ_S x BJ_S, row-major), the rotated subproblem and whether any rotation was
+// applied.  One sweep a visit: the outer sweeps come back to the pair anyway, and
+// diagonalising it on every visit took three to eight sweeps on one SM (640 rows:
+// 100 us a round in FP32 and 237 us in FP64; now 25 and 84, with as many outer
+// sweeps: 9 and 3).
+// The two-sided rotation of the pairs (e, f) acts on a 2 x 2 block of S: a thread
+// per block with e <= f (S is symmetric, the mirrored block is copied).
 template <typename T, int BJ_B>
 __global__ void __launch_bounds__(256) k_bj_solve(const T* __restrict__ A, int np, int nb, int r, T* __restrict__ Jb,
-                                                  T* __restrict__ lam, int* __restrict__ rotated, int max_sweeps) {
+                                                  T* __restrict__ Sb, int* __restrict__ rotated) {
   constexpr int BJ_S = 2 * BJ_B, BJ_LD = BJ_S + 1;
-  extern __shared__ double smraw[];
-  T* S = reinterpret_cast<T*>(smraw);
-  T* J = S + BJ_S * BJ_LD;
+  constexpr int NBLK = BJ_B * (BJ_B + 1) / 2;
+  __shared__ T S[BJ_S * BJ_LD];
+  __shared__ T J[BJ_S * BJ_LD];
   __shared__ T cs[BJ_B], sn[BJ_B];
   __shared__ int pp[BJ_B], qq[BJ_B];
-  __shared__ int any, any_sweep;
+  __shared__ int any;
   const int k = blockIdx.x, tid = threadIdx.x;
   int p, q;
   bj_pair(k, r, nb, p, q);
@@ -183,139 +250,170 @@ __global__ void __launch_bounds__(256) k_bj_solve(const T* __restrict__ A, int n
     J[i * BJ_LD + j] = i == j ? T(1) : T(0);
   }
   if (tid == 0) any = 0;
-  __syncthreads();
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    if (tid == 0) any_sweep = 0;
-    __syncthreads();
-    for (int rd = 0; rd < BJ_S - 1; ++rd) {
-      if (tid < BJ_B) {
-        const int a = tid == 0 ? 0 : ((tid - 1 + rd) % (BJ_S - 1)) + 1;
-        const int b2 = ((BJ_S - 1 - tid - 1 + rd) % (BJ_S - 1)) + 1;
-        const int i = min(a, b2), j = max(a, b2);
-        const T aij = S[i * BJ_LD + j], aii = S[i * BJ_LD + i], ajj = S[j * BJ_LD + j];
-        T c = T(1), s = T(0);
-        // negligible off-diagonal entry (below the rounding of both diagonal
-        // entries): no rotation
-        const T g = T(100) * fabs(aij);
-        if (aij != T(0) && !(fabs(aii) + g == fabs(aii) && fabs(ajj) + g == fabs(ajj))) {
-          const T tau = (ajj - aii) / (T(2) * aij);
-          const T t = (tau >= T(0) ? T(1) : T(-1)) / (fabs(tau) + sqrt(T(1) + tau * tau));
-          c = T(1) / sqrt(T(1) + t * t);
-          s = t * c;
-          any_sweep = 1;
-        }
-        pp[tid] = i;
-        qq[tid] = j;
-        cs[tid] = c;
-        sn[tid] = s;
-      }
-      __syncthreads();
-      // rows i, j of S
-      for (int t = tid; t < BJ_B * BJ_S; t += blockDim.x) {
-        const int e = t / BJ_S, col = t % BJ_S;
-        if (sn[e] == T(0)) continue;
-        const int i = pp[e], j = qq[e];
-        const T c = cs[e], s = sn[e];
-        const T x = S[i * BJ_LD + col], y = S[j * BJ_LD + col];
-        S[i * BJ_LD + col] = c * x - s * y;
-        S[j * BJ_LD + col] = s * x + c * y;
-      }
-      __syncthreads();
-      // columns i, j of S and of J
-      for (int t = tid; t < BJ_B * BJ_S; t += blockDim.x) {
-        const int e = t / BJ_S, row = t % BJ_S;
-        if (sn[e] == T(0)) continue;
-        const int i = pp[e], j = qq[e];
-        const T c = cs[e], s = sn[e];
-        const T x = S[row * BJ_LD + i], y = S[row * BJ_LD + j];
-        S[row * BJ_LD + i] = c * x - s * y;
-        S[row * BJ_LD + j] = s * x + c * y;
-        const T u = J[row * BJ_LD + i], v = J[row * BJ_LD + j];
-        J[row * BJ_LD + i] = c * u - s * v;
-        J[row * BJ_LD + j] = s * u + c * v;
-      }
-      __syncthreads();
-      if (tid < BJ_B && sn[tid] != T(0)) {
-        S[pp[tid] * BJ_LD + qq[tid]] = T(0);
-        S[qq[tid] * BJ_LD + pp[tid]] = T(0);
-      }
-      __syncthreads();
+  // this thread's 2 x 2 block of pairs (e, f), e <= f
+  int be = 0, bf = 0;
+  if (tid < NBLK) {
+    int t = tid;
+    while (t >= BJ_B - be) {
+      t -= BJ_B - be;
+      ++be;
     }
-    if (tid == 0 && any_sweep) any = 1;
+    bf = be + t;
+  }
+  __syncthreads();
+  for (int rd = 0; rd < BJ_S - 1; ++rd) {
+    if (tid < BJ_B) {
+      const int a = tid == 0 ? 0 : ((tid - 1 + rd) % (BJ_S - 1)) + 1;
+      const int b2 = ((BJ_S - 1 - tid - 1 + rd) % (BJ_S - 1)) + 1;
+      const int i = min(a, b2), j = max(a, b2);
+      const T aij = S[i * BJ_LD + j], aii = S[i * BJ_LD + i], ajj = S[j * BJ_LD + j];
+      T c = T(1), s = T(0);
+      // negligible off-diagonal entry (below the rounding of both diagonal
+      // entries): no rotation
+      const T g = T(100) * fabs(aij);
+      if (aij != T(0) && !(fabs(aii) + g == fabs(aii) && fabs(ajj) + g == fabs(ajj))) {
+        bj_angle(aii, ajj, aij, c, s);
+        any = 1;
+      }
+      pp[tid] = i;
+      qq[tid] = j;
+      cs[tid] = c;
+      sn[tid] = s;
+    }
     __syncthreads();
-    if (!any_sweep) break;
+    if (tid < NBLK) {
+      const T ce = cs[be], se = sn[be], cf = cs[bf], sf = sn[bf];
+      if (se != T(0) || sf != T(0)) {
+        const int i = pp[be], j = qq[be], u = pp[bf], v = qq[bf];
+        const T x00 = S[i * BJ_LD + u], x01 = S[i * BJ_LD + v], x10 = S[j * BJ_LD + u], x11 = S[j * BJ_LD + v];
+        // rows by (ce, se), then columns by (cf, sf)
+        const T y00 = ce * x00 - se * x10, y01 = ce * x01 - se * x11;
+        const T y10 = se * x00 + ce * x10, y11 = se * x01 + ce * x11;
+        const T z00 = cf * y00 - sf * y01, z01 = sf * y00 + cf * y01;
+        const T z10 = cf * y10 - sf * y11, z11 = sf * y10 + cf * y11;
+        S[i * BJ_LD + u] = z00;
+        S[i * BJ_LD + v] = z01;
+        S[j * BJ_LD + v] = z11;
+        S[u * BJ_LD + i] = z00;
+        S[v * BJ_LD + i] = z01;
+        S[v * BJ_LD + j] = z11;
+        if (be != bf) {
+          S[j * BJ_LD + u] = z10;
+          S[u * BJ_LD + j] = z10;
+        } else {
+          S[j * BJ_LD + u] = z01;   // the pair's own block stays symmetric
+        }
+      }
+    }
+    for (int t = tid; t < BJ_B * BJ_S; t += blockDim.x) {
+      const int e = t / BJ_S, row = t % BJ_S;
+      if (sn[e] == T(0)) continue;
+      const int i = pp[e], j = qq[e];
+      const T c = cs[e], s = sn[e];
+      const T u = J[row * BJ_LD + i], v = J[row * BJ_LD + j];
+      J[row * BJ_LD + i] = c * u - s * v;
+      J[row * BJ_LD + j] = s * u + c * v;
+    }
+    __syncthreads();
   }
   T* Jo = Jb + (int64_t)k * BJ_S * BJ_S;
-  for (int t = tid; t < BJ_S * BJ_S; t += blockDim.x) Jo[t] = J[(t / BJ_S) * BJ_LD + t % BJ_S];
-  for (int t = tid; t < BJ_S; t += blockDim.x) lam[(int64_t)k * BJ_S + t] = S[t * BJ_LD + t];
+  T* So = Sb + (int64_t)k * BJ_S * BJ_S;
+  for (int t = tid; t < BJ_S * BJ_S; t += blockDim.x) {
+    Jo[t] = J[(t / BJ_S) * BJ_LD + t % BJ_S];
+    So[t] = S[(t / BJ_S) * BJ_LD + t % BJ_S];
+  }
   if (tid == 0) rotated[k] = any;
 }
 
-// M[:, idx(p,q)] <- M[:, idx(p,q)] J_k for every pair k (rows in chunks of 32).
+// One round's updates in one launch.  blockIdx.x < pairs: the block (k, l) of A,
+// k <= l, of the pairs' 2B rows and columns becomes J_k^T A_kl J_l (the diagonal
+// one is the solved subproblem), its mirror image the transpose.  blockIdx.x >=
+// pairs: 32 rows of V, V[:, idx(k)] <- V[:, idx(k)] J_k.  Blocks are independent,
+// so A needs no separate row and column pass (three launches a round and twice the
+// products before: 640 rows 82 us in FP64 and 24 in FP32, now 69 and 12).
 template <typename T, int BJ_B>
-__global__ void __launch_bounds__(256) k_bj_cols(T* __restrict__ M, int np, int nb, int r, const T* __restrict__ Jb,
-                                                 const int* __restrict__ rotated) {
-  constexpr int BJ_S = 2 * BJ_B;
-  const int k = blockIdx.y;
-  if (!rotated[k]) return;
-  __shared__ T Js[BJ_S][BJ_S + 1];
-  __shared__ T Xs[32][BJ_S + 1];
+__global__ void __launch_bounds__(256) k_bj_update(T* __restrict__ A, T* __restrict__ V, int np, int nb, int r,
+                                                   const T* __restrict__ Jb, const T* __restrict__ Sb,
+                                                   const int* __restrict__ rotated) {
+  constexpr int BJ_S = 2 * BJ_B, LD = BJ_S + 1;
+  __shared__ T Js[BJ_S * LD];
+  __shared__ T Xs[BJ_S * LD];
+  __shared__ T Ys[BJ_S * LD];
+  const int pairs = nb / 2, k = blockIdx.y, tid = threadIdx.x;
   int p, q;
   bj_pair(k, r, nb, p, q);
-  const T* Jk = Jb + (int64_t)k * BJ_S * BJ_S;
-  for (int t = threadIdx.x; t < BJ_S * BJ_S; t += blockDim.x) Js[t / BJ_S][t % BJ_S] = Jk[t];
-  const int r0 = blockIdx.x * 32;
-  for (int t = threadIdx.x; t < 32 * BJ_S; t += blockDim.x) {
-    const int rr = t / BJ_S, c = t % BJ_S;
-    Xs[rr][c] = (r0 + rr < np) ? M[(int64_t)(r0 + rr) * np + bj_index<BJ_B>(c, p, q)] : T(0);
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < 32 * BJ_S; t += blockDim.x) {
-    const int rr = t / BJ_S, c = t % BJ_S;
-    if (r0 + rr >= np) continue;
-    T acc = T(0);
-#pragma unroll 8
-    for (int l = 0; l < BJ_S; ++l) acc = fma(Xs[rr][l], Js[l][c], acc);
-    M[(int64_t)(r0 + rr) * np + bj_index<BJ_B>(c, p, q)] = acc;
-  }
-}
-
-// A[idx(p,q), :] <- J_k^T A[idx(p,q), :] for every pair k (columns in chunks
-// of one block); the pair's own BJ_S x BJ_S block becomes diag(lambda_k).
-template <typename T, int BJ_B>
-__global__ void __launch_bounds__(256) k_bj_rows(T* __restrict__ A, int np, int nb, int r, const T* __restrict__ Jb,
-                                                 const T* __restrict__ lam, const int* __restrict__ rotated) {
-  constexpr int BJ_S = 2 * BJ_B;
-  const int k = blockIdx.y;
-  if (!rotated[k]) return;
-  __shared__ T Js[BJ_S][BJ_S + 1];
-  __shared__ T Xs[BJ_S][BJ_B + 1];
-  int p, q;
-  bj_pair(k, r, nb, p, q);
-  const int cblk = blockIdx.x, c0 = cblk * BJ_B;
-  if (cblk == p || cblk == q) {
-    // own block columns: diag(lambda) in rows idx(p,q), columns of this block
-    const int off = cblk == p ? 0 : BJ_B;
-    for (int t = threadIdx.x; t < BJ_S * BJ_B; t += blockDim.x) {
-      const int i = t / BJ_B, c = t % BJ_B;
-      A[(int64_t)bj_index<BJ_B>(i, p, q) * np + c0 + c] = (i == off + c) ? lam[(int64_t)k * BJ_S + i] : T(0);
+  // a thread forms four outputs of one row of a BJ_S x BJ_S product
+  const int row = tid / (BJ_S / 4), cq = (tid % (BJ_S / 4)) * 4;
+  static_assert(BJ_S * (BJ_S / 4) == 256, "256 threads x 4 outputs");
+  if ((int)blockIdx.x >= pairs) {
+    if (!rotated[k]) return;
+    const int r0 = ((int)blockIdx.x - pairs) * BJ_S;
+    const T* Jk = Jb + (int64_t)k * BJ_S * BJ_S;
+    for (int t = tid; t < BJ_S * BJ_S; t += 256) {
+      const int i = t / BJ_S, j = t % BJ_S;
+      Js[i * LD + j] = Jk[t];
+      Xs[i * LD + j] = r0 + i < np ? V[(int64_t)(r0 + i) * np + bj_index<BJ_B>(j, p, q)] : T(0);
     }
+    __syncthreads();
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll 8
+    for (int l = 0; l < BJ_S; ++l) {
+      const T x = Xs[row * LD + l];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[c] = fma(x, Js[l * LD + cq + c], acc[c]);
+    }
+    if (r0 + row < np)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) V[(int64_t)(r0 + row) * np + bj_index<BJ_B>(cq + c, p, q)] = acc[c];
     return;
   }
+  const int l2 = blockIdx.x;
+  if (l2 < k || !(rotated[k] | rotated[l2])) return;
+  if (l2 == k) {
+    const T* So = Sb + (int64_t)k * BJ_S * BJ_S;
+    for (int t = tid; t < BJ_S * BJ_S; t += 256)
+      A[(int64_t)bj_index<BJ_B>(t / BJ_S, p, q) * np + bj_index<BJ_B>(t % BJ_S, p, q)] = So[t];
+    return;
+  }
+  int u, v;
+  bj_pair(l2, r, nb, u, v);
   const T* Jk = Jb + (int64_t)k * BJ_S * BJ_S;
-  for (int t = threadIdx.x; t < BJ_S * BJ_S; t += blockDim.x) Js[t / BJ_S][t % BJ_S] = Jk[t];
-  for (int t = threadIdx.x; t < BJ_S * BJ_B; t += blockDim.x) {
-    const int i = t / BJ_B, c = t % BJ_B;
-    Xs[i][c] = A[(int64_t)bj_index<BJ_B>(i, p, q) * np + c0 + c];
+  const T* Jl = Jb + (int64_t)l2 * BJ_S * BJ_S;
+  for (int t = tid; t < BJ_S * BJ_S; t += 256) {
+    const int i = t / BJ_S, j = t % BJ_S;
+    Js[i * LD + j] = Jl[t];
+    Xs[i * LD + j] = A[(int64_t)bj_index<BJ_B>(i, p, q) * np + bj_index<BJ_B>(j, u, v)];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < BJ_S * BJ_B; t += blockDim.x) {
-    const int i = t / BJ_B, c = t % BJ_B;
-    T acc = T(0);
+  T acc[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll 8
-    for (int l = 0; l < BJ_S; ++l) acc = fma(Js[l][i], Xs[l][c], acc);
-    A[(int64_t)bj_index<BJ_B>(i, p, q) * np + c0 + c] = acc;
+  for (int l = 0; l < BJ_S; ++l) {   // Y = A_kl J_l
+    const T x = Xs[row * LD + l];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] = fma(x, Js[l * LD + cq + c], acc[c]);
   }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) Ys[row * LD + cq + c] = acc[c];
+  __syncthreads();
+  for (int t = tid; t < BJ_S * BJ_S; t += 256) Js[(t / BJ_S) * LD + t % BJ_S] = Jk[t];
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 4; ++c) acc[c] = T(0);
+#pragma unroll 8
+  for (int l = 0; l < BJ_S; ++l) {   // Z = J_k^T Y
+    const T x = Js[l * LD + row];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] = fma(x, Ys[l * LD + cq + c], acc[c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    A[(int64_t)bj_index<BJ_B>(row, p, q) * np + bj_index<BJ_B>(cq + c, u, v)] = acc[c];
+    Xs[(cq + c) * LD + row] = acc[c];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    A[(int64_t)bj_index<BJ_B>(row, u, v) * np + bj_index<BJ_B>(cq + c, p, q)] = Xs[row * LD + cq + c];
 }
 
 // partial sums of the squared off-diagonal and total entries of the leading n x n part
@@ -394,12 +492,13 @@ void launch_chol_blocked(double* A, int n, int lda, int* info, double* min_ratio
 
 int64_t chol_blocked_scratch(int n) { return (int64_t)n + (int64_t)CB * n; }
 
-// Li = L^-1 (lower, n x n, ld ldi), 2 x 2 block recursion down to 128-wide
-// diagonal blocks, which the column-per-thread kernel inverts.
+// Li = L^-1 (lower, n x n, ld ldi), 2 x 2 block recursion down to 64-wide
+// diagonal blocks, which one CTA inverts in shared memory.
 // scratch: n * n / 4 doubles (the largest off-diagonal block).
 void launch_trinv_blocked(const double* L, int n, int lda, double* Li, int ldi, double* scratch, cudaStream_t st) {
-  if (n <= 128) {
-    launch_trinv_lower(L, n, lda, Li, ldi, st);
+  if (n <= CB) {
+    k_trinv_leaf<<<1, 512, 0, st>>>(L, n, lda, Li, ldi);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
     return;
   }
   const int n1 = (n / 2 + 63) / 64 * 64, n2 = n - n1;
@@ -421,7 +520,7 @@ static int64_t bj_scratch_bytes(int n, int elem, int B) {
   const int nb = std::max(2, nb0 + (nb0 & 1));
   const int64_t np = (int64_t)nb * B;
   const int64_t pairs = nb / 2;
-  return elem * (2 * np * np + pairs * S * S + pairs * S) + (int64_t)sizeof(int) * pairs +
+  return elem * (2 * np * np + 2 * pairs * S * S) + (int64_t)sizeof(int) * pairs +
          (int64_t)sizeof(double) * 2 * BJ_NORM_BLOCKS + 1024;
 }
 
@@ -435,7 +534,7 @@ namespace {
 template <typename T, int BJ_B>
 int block_jacobi_b(const double* C, int n, int ldc, T* V, int ldv, T* w, int max_sweeps, double tol2, void* scratch,
                    cudaStream_t st, double* ratio_out) {
-  constexpr int BJ_S = 2 * BJ_B, BJ_LD = BJ_S + 1;
+  constexpr int BJ_S = 2 * BJ_B;
   const int nb0 = (n + BJ_B - 1) / BJ_B;
   const int nb = std::max(2, nb0 + (nb0 & 1));
   const int np = nb * BJ_B;
@@ -443,14 +542,11 @@ int block_jacobi_b(const double* C, int n, int ldc, T* V, int ldv, T* w, int max
   T* A = reinterpret_cast<T*>(scratch);
   T* Vp = A + (int64_t)np * np;
   T* Jb = Vp + (int64_t)np * np;
-  T* lam = Jb + (int64_t)pairs * BJ_S * BJ_S;
-  int* rot = reinterpret_cast<int*>(lam + (int64_t)pairs * BJ_S);
+  T* Sb = Jb + (int64_t)pairs * BJ_S * BJ_S;
+  int* rot = reinterpret_cast<int*>(Sb + (int64_t)pairs * BJ_S * BJ_S);
   double* part = reinterpret_cast<double*>(((uintptr_t)(rot + pairs) + 255) & ~(uintptr_t)255);
   k_bj_pad<T><<<nblk((int64_t)np * np, 256), 256, 0, st>>>(C, n, ldc, A, Vp, np);
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  const size_t smem = sizeof(T) * 2 * BJ_S * BJ_LD;
-  if (cudaFuncSetAttribute(k_bj_solve<T, BJ_B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return -1;
   std::vector<double> hp(2 * BJ_NORM_BLOCKS);
   int rc = 1;
   for (int sweep = 0; sweep <= max_sweeps; ++sweep) {
@@ -471,11 +567,9 @@ int block_jacobi_b(const double* C, int n, int ldc, T* V, int ldv, T* w, int max
     }
     if (sweep == max_sweeps) break;
     for (int r = 0; r < nb - 1; ++r) {
-      k_bj_solve<T, BJ_B><<<pairs, 256, smem, st>>>(A, np, nb, r, Jb, lam, rot, 30);
-      k_bj_cols<T, BJ_B><<<dim3(nblk(np, 32), pairs), 256, 0, st>>>(A, np, nb, r, Jb, rot);
-      k_bj_rows<T, BJ_B><<<dim3(nb, pairs), 256, 0, st>>>(A, np, nb, r, Jb, lam, rot);
-      k_bj_cols<T, BJ_B><<<dim3(nblk(np, 32), pairs), 256, 0, st>>>(Vp, np, nb, r, Jb, rot);
-      g_launches.fetch_add(4, std::memory_order_relaxed);
+      k_bj_solve<T, BJ_B><<<pairs, 256, 0, st>>>(A, np, nb, r, Jb, Sb, rot);
+      k_bj_update<T, BJ_B><<<dim3((unsigned)pairs + nblk(np, BJ_S), pairs), 256, 0, st>>>(A, Vp, np, nb, r, Jb, Sb, rot);
+      g_launches.fetch_add(2, std::memory_order_relaxed);
     }
   }
   k_bj_out<T><<<nblk((int64_t)n * n, 256), 256, 0, st>>>(A, Vp, np, n, V, ldv, w);

@@ -1462,18 +1462,6 @@ __global__ void k_shift_diag(double* A, int n, int lda, double coef) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) A[(int64_t)i * lda + i] += shift;
 }
 
-// Li = L^-1 (lower), one column per thread by forward substitution.
-__global__ void k_trinv_lower(const double* __restrict__ L, int n, int lda, double* __restrict__ Li, int ldi) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    for (int i = 0; i < j; ++i) Li[(int64_t)i * ldi + j] = 0.0;
-    for (int i = j; i < n; ++i) {
-      double v = (i == j) ? 1.0 : 0.0;
-      for (int k = j; k < i; ++k) v -= L[(int64_t)i * lda + k] * Li[(int64_t)k * ldi + j];
-      Li[(int64_t)i * ldi + j] = v / L[(int64_t)i * lda + i];
-    }
-  }
-}
-
 __global__ void k_transpose(const double* __restrict__ A, int n, int lda, double* __restrict__ B, int ldb) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * n) return;
@@ -1499,26 +1487,24 @@ __global__ void k_mirror_upper(double* A, int n, int lda) {
 }
 
 // Parallel cyclic Jacobi (round-robin pairing) for a symmetric n x n matrix in
-// one CTA: A <- J^T A J with disjoint rotations per round, V <- V J.
+// one CTA, n <= 64: A <- J^T A J with disjoint rotations per round, V <- V J.
 // T = double, or float for the pre-diagonalisation of the mixed eigensolver;
 // stops when the off-diagonal square sum is <= tol2 times the total.
-template <typename T, bool SMEM>
+template <typename T>
 __global__ void __launch_bounds__(1024) k_jacobi(T* Ag, int n, int ldag, T* V, int ldv, T* w, int max_sweeps,
                                                  double tol2, int* info) {
-  __shared__ T cs[1024], sn[1024];
-  __shared__ int pp[1024], qq[1024];
+  __shared__ T cs[32], sn[32];
+  __shared__ int pp[32], qq[32];
   __shared__ double red[2][32];
   __shared__ int done;
   extern __shared__ double As_raw[];
   T* As_dyn = reinterpret_cast<T*>(As_raw);
   const int tid = threadIdx.x, bd = blockDim.x;
-  // the working matrix lives in shared memory when it fits (n <= 150), else in global memory
-  T* A = SMEM ? As_dyn : Ag;
-  const int lda = SMEM ? n : ldag;
-  if (SMEM) {
-    for (int64_t t = tid; t < (int64_t)n * n; t += bd) As_dyn[t] = Ag[(t / n) * (int64_t)ldag + t % n];
-    __syncthreads();
-  }
+  // the working matrix lives in shared memory (n <= 64)
+  T* A = As_dyn;
+  const int lda = n;
+  for (int64_t t = tid; t < (int64_t)n * n; t += bd) As_dyn[t] = Ag[(t / n) * (int64_t)ldag + t % n];
+  __syncthreads();
   const int n2 = n + (n & 1);
   const int np = n2 / 2;
   for (int64_t t = tid; t < (int64_t)n * n; t += bd) V[(t / n) * ldv + t % n] = (t / n == t % n) ? T(1) : T(0);
@@ -2025,11 +2011,6 @@ void launch_chol(double* A, int n, int lda, int* info, cudaStream_t st, double* 
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
-void launch_trinv_lower(const double* L, int n, int lda, double* Li, int ldi, cudaStream_t st) {
-  k_trinv_lower<<<grid1(n, 128), 128, 0, st>>>(L, n, lda, Li, ldi);
-  g_launches.fetch_add(1, std::memory_order_relaxed);
-}
-
 void launch_transpose(const double* A, int n, int lda, double* B, int ldb, cudaStream_t st) {
   k_transpose<<<grid1((int64_t)n * n, 256), 256, 0, st>>>(A, n, lda, B, ldb);
   g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -2049,12 +2030,7 @@ template <typename T>
 void launch_jacobi_t(T* A, int n, int lda, T* V, int ldv, T* w, int max_sweeps, double tol2, int* info,
                      cudaStream_t st) {
   const size_t smem = sizeof(T) * (size_t)n * n;
-  if (smem <= 180 * 1024) {
-    cudaFuncSetAttribute(k_jacobi<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_jacobi<T, true><<<1, 1024, smem, st>>>(A, n, lda, V, ldv, w, max_sweeps, tol2, info);
-  } else {
-    k_jacobi<T, false><<<1, 1024, 0, st>>>(A, n, lda, V, ldv, w, max_sweeps, tol2, info);
-  }
+  k_jacobi<T><<<1, 1024, smem, st>>>(A, n, lda, V, ldv, w, max_sweeps, tol2, info);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 

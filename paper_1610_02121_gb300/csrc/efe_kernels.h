@@ -205,7 +205,6 @@ void launch_gemm_tn(int64_t K, int Na, int Nb, const double* A, int64_t lda, con
 int64_t gemm_tn_work_elems(int64_t K, int Na, int Nb);
 void launch_chol(double* A, int n, int lda, int* info, cudaStream_t st, double* min_ratio = nullptr);
 void launch_shift_diag(double* A, int n, int lda, double coef, cudaStream_t st);
-void launch_trinv_lower(const double* L, int n, int lda, double* Li, int ldi, cudaStream_t st);
 void launch_transpose(const double* A, int n, int lda, double* B, int ldb, cudaStream_t st);
 void launch_symmetrize(double* A, int n, int lda, cudaStream_t st);
 // A[i][j] = A[j][i] for i > j (the strict lower triangle from the upper one)

@@ -50,3 +50,24 @@ def test_rayleigh_ritz_at_tile_edges(tiny_pair, N):
     np.testing.assert_allclose(res, res_ref, atol=1e-8, rtol=1e-6)
     gram = (Xd.T @ G.apply_M(Xd)).cpu().numpy()
     np.testing.assert_allclose(gram, np.eye(N), atol=1e-10)
+
+
+# the blocked eigensolver, Cholesky and triangular inverse at their block edges (16, 64) and
+# at the size where they take over, on a problem whose Ritz values are the oracle's; the FP64
+# engine's 2^-48 a term for the tall products gives the wider figure
+@pytest.mark.parametrize("engine,tol", [("dfma", 1e-9), ("tensor", 1e-8)])
+@pytest.mark.parametrize("N", [47, 50, 63, 64, 65, 97, 129, 150])
+def test_blocked_dense_edges(tiny_pair, engine, tol, N):
+    from oracle.chfsi import cholqr, rayleigh_ritz
+    d, G = tiny_pair
+    X = W.random_block(d.system, N, seed=500 + N)
+    eps_ref, _, _ = rayleigh_ritz(d.apply_H_assembled, d.apply_M_assembled, cholqr(X)[0])
+    G.set_fp64_engine(engine)
+    try:
+        Xd = to_dev(X)
+        eps, _ = G.rayleigh_ritz(Xd)
+    finally:
+        G.set_fp64_engine("dfma")
+    np.testing.assert_allclose(eps, eps_ref, atol=tol, rtol=tol)
+    gram = (Xd.T @ G.apply_M(Xd)).cpu().numpy()
+    np.testing.assert_allclose(gram, np.eye(N), atol=1e-8)
