@@ -10,6 +10,8 @@
 // reductions use fixed-order partials (bitwise reproducible).
 #include <math.h>
 
+#include <type_traits>
+
 #include "efe_kernels.h"
 
 namespace efe {
@@ -156,6 +158,213 @@ __global__ void __launch_bounds__(256) k_gemm_g(int64_t M, int64_t Nn, int64_t K
   }
 }
 
+// FP32 GEMM of the network's layers: C[m][n] = sum_k A(m, k) B(k, n), FP32 FMAs in k
+// order (split K: blockIdx.z takes kch of them, partial products at C + z M ldc).  A
+// CTA forms a 128 x 128 tile, a thread 8 x 8 of it (two 4-wide groups per axis, so the
+// shared rows are read as 16-byte vectors), K in steps of 16 through two buffers: the
+// next step's global loads are in registers while this one is multiplied.  The FP32
+// pipe bounds it: 64 FMAs, as 32 two-wide instructions, for four 16-byte shared loads
+// a thread and k.  3.84M rows through 64 -> 256 -> 256 -> 256: 63 ms in 64 x 64 tiles
+// of 4 x 4 outputs with scalar loads and separate bias/SiLU passes, 27.8 with this tile
+// and one-wide FMAs, 23.0 (49 TFLOP/s) with two-wide ones; same bits.
+// AK: element (m, k) of A is A[m lda + k], else A[k lda + m]; BK: (k, n) of B is
+// B[n ldb + k], else B[k ldb + n].  VEC: rows and pointers allow 16-byte loads.
+// EPI 0: C = product; 1: C = Z = product + bias[n], act = silu(Z) or Z; 2: C = product *
+// silu'(Zp[m][n]).
+constexpr int FT = 128, FK = 16;
+
+// two FP32 FMAs (each rounded once) in one instruction: acc += (a, a) * (b0, b1)
+__device__ __forceinline__ unsigned long long pack2(float a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+template <bool AK, bool BK, bool VEC, int EPI>
+__global__ void __launch_bounds__(256, 2) k_gemm_f32(int64_t M, int64_t Nn, int64_t K, int64_t kch,
+                                                     const float* __restrict__ A, int64_t lda,
+                                                     const float* __restrict__ B, int64_t ldb, float* __restrict__ C,
+                                                     int64_t ldc, const float* __restrict__ bias,
+                                                     float* __restrict__ act, const float* __restrict__ Zp, int silu) {
+  __shared__ __align__(16) float As[2][FK][FT + 4];
+  __shared__ __align__(16) float Bs[2][FK][FT + 4];
+  const int64_t m0 = (int64_t)blockIdx.x * FT, n0 = (int64_t)blockIdx.y * FT;
+  const int64_t kb = (int64_t)blockIdx.z * kch, ke = min(K, kb + kch);
+  C += (int64_t)blockIdx.z * M * ldc;
+  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
+  float4 ra[2], rb[2];
+  // operand tile 128 (rows of the operand's own index) x 16 k: 512 quads, two a thread.
+  // KF (k fastest): quad = (row, 4 k); else quad = (k, 4 rows)
+  auto load = [&](auto kf, const float* P, int64_t ld, int64_t r0, int64_t R, int64_t k0, float4 (&v)[2]) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int t = tid + 256 * u;
+      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      float* e = reinterpret_cast<float*>(&v[u]);
+      if constexpr (decltype(kf)::value) {
+        const int64_t r = r0 + t / 4, k = k0 + (t % 4) * 4;
+        if (r < R) {
+          if (VEC && k + 4 <= ke) {
+            v[u] = *reinterpret_cast<const float4*>(P + r * ld + k);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (k + i < ke) e[i] = P[r * ld + k + i];
+          }
+        }
+      } else {
+        const int64_t k = k0 + t / 32, r = r0 + (t % 32) * 4;
+        if (k < ke) {
+          if (VEC && r + 4 <= R) {
+            v[u] = *reinterpret_cast<const float4*>(P + k * ld + r);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (r + i < R) e[i] = P[k * ld + r + i];
+          }
+        }
+      }
+    }
+  };
+  auto store = [&](auto kf, float (*S)[FT + 4], const float4 (&v)[2]) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int t = tid + 256 * u;
+      const float* e = reinterpret_cast<const float*>(&v[u]);
+      if constexpr (decltype(kf)::value) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) S[(t % 4) * 4 + i][t / 4] = e[i];
+      } else {
+        *reinterpret_cast<float4*>(&S[t / 32][(t % 32) * 4]) = v[u];
+      }
+    }
+  };
+  const std::integral_constant<bool, AK> akf{};
+  const std::integral_constant<bool, BK> bkf{};
+  unsigned long long acc[8][4];   // column pairs (c, c + 1) of a row
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  load(akf, A, lda, m0, M, kb, ra);
+  load(bkf, B, ldb, n0, Nn, kb, rb);
+  store(akf, As[0], ra);
+  store(bkf, Bs[0], rb);
+  __syncthreads();
+  int b = 0;
+  for (int64_t k0 = kb; k0 < ke; k0 += FK, b ^= 1) {
+    const bool more = k0 + FK < ke;
+    if (more) {
+      load(akf, A, lda, m0, M, k0 + FK, ra);
+      load(bkf, B, ldb, n0, Nn, k0 + FK, rb);
+    }
+#pragma unroll
+    for (int kk = 0; kk < FK; ++kk) {
+      float av[8];
+      ulonglong2 b0, b1;
+      *reinterpret_cast<float4*>(av) = *reinterpret_cast<const float4*>(&As[b][kk][ty * 4]);
+      *reinterpret_cast<float4*>(av + 4) = *reinterpret_cast<const float4*>(&As[b][kk][64 + ty * 4]);
+      b0 = *reinterpret_cast<const ulonglong2*>(&Bs[b][kk][tx * 4]);
+      b1 = *reinterpret_cast<const ulonglong2*>(&Bs[b][kk][64 + tx * 4]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const unsigned long long a2 = pack2(av[i]);
+        fma2(acc[i][0], a2, b0.x);
+        fma2(acc[i][1], a2, b0.y);
+        fma2(acc[i][2], a2, b1.x);
+        fma2(acc[i][3], a2, b1.y);
+      }
+    }
+    if (more) {
+      store(akf, As[b ^ 1], ra);
+      store(bkf, Bs[b ^ 1], rb);
+    }
+    __syncthreads();
+  }
+  // 16-byte stores where the row is aligned and the four columns exist
+  const bool vst = (ldc & 3) == 0 && ((uintptr_t)C & 15) == 0 && (EPI != 1 || ((uintptr_t)act & 15) == 0) &&
+                   (EPI != 2 || ((uintptr_t)Zp & 15) == 0);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int64_t m = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4);
+    if (m >= M) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t n = n0 + h * 64 + tx * 4;
+      if (n >= Nn) continue;
+      float z[4], a4[4];
+      const bool v4 = vst && n + 4 <= Nn;
+      if (EPI == 2 && v4) *reinterpret_cast<float4*>(a4) = *reinterpret_cast<const float4*>(Zp + m * ldc + n);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        z[j] = __uint_as_float((unsigned)(acc[i][h * 2 + j / 2] >> (32 * (j & 1))));
+        if (n + j >= Nn) continue;
+        if (EPI == 1) {
+          z[j] += bias[n + j];
+          a4[j] = silu ? silu_d(z[j]) : z[j];
+        }
+        if (EPI == 2) z[j] *= silu_grad_d(v4 ? a4[j] : Zp[m * ldc + n + j]);
+      }
+      if (v4) {
+        *reinterpret_cast<float4*>(C + m * ldc + n) = *reinterpret_cast<float4*>(z);
+        if (EPI == 1) *reinterpret_cast<float4*>(act + m * ldc + n) = *reinterpret_cast<float4*>(a4);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (n + j >= Nn) continue;
+          C[m * ldc + n + j] = z[j];
+          if (EPI == 1) act[m * ldc + n + j] = a4[j];
+        }
+      }
+    }
+  }
+}
+
+// the scalar output layer (one column): z = sum_k a[k] w[k] + b with the sum in k order,
+// one thread a row; 256 columns of 32 rows at a time go through shared memory so that
+// the loads are coalesced and many.  z goes to the pre-activation, the activation and
+// y.  Read-bound (3.9 GB on 3.8M rows of 256); as a 64-column GEMM tile for the one
+// column it took a quarter of the network's time.
+constexpr int RD_R = 32, RD_C = 256;
+__global__ void __launch_bounds__(256) k_row_dot(int64_t n, int d, const float* __restrict__ a,
+                                                const float* __restrict__ w, const float* __restrict__ b,
+                                                float* __restrict__ Z, float* __restrict__ A, float* __restrict__ y) {
+  __shared__ float S[RD_R][RD_C + 1];
+  __shared__ float ws[RD_C];
+  const int tid = threadIdx.x;
+  const int64_t r0 = blockIdx.x * (int64_t)RD_R;
+  const int nr = (int)min((int64_t)RD_R, n - r0);
+  float s = 0.f;
+  for (int k0 = 0; k0 < d; k0 += RD_C) {
+    const int nk = min(RD_C, d - k0);
+    __syncthreads();
+    if (tid < nk) {
+      ws[tid] = w[k0 + tid];
+      const float* ar = a + r0 * d + k0 + tid;
+      if (nr == RD_R) {
+#pragma unroll
+        for (int r = 0; r < RD_R; ++r) S[r][tid] = ar[(int64_t)r * d];
+      } else {
+        for (int r = 0; r < nr; ++r) S[r][tid] = ar[(int64_t)r * d];
+      }
+    }
+    __syncthreads();
+    if (tid < nr) {
+#pragma unroll 8
+      for (int k = 0; k < nk; ++k) s = fmaf(S[tid][k], ws[k], s);
+    }
+  }
+  if (tid < nr) {
+    const float z = s + b[0];
+    Z[r0 + tid] = z;
+    A[r0 + tid] = z;
+    y[r0 + tid] = z;
+  }
+}
+
 // Z = C + b (bias per column), A = act(Z) (SiLU or identity); Z, A row-major n x d
 template <typename T>
 __global__ void k_bias_act(int64_t n, int d, const T* __restrict__ b, T* __restrict__ Z, T* __restrict__ A, int act) {
@@ -173,14 +382,24 @@ __global__ void k_act_back(int64_t n, const T* __restrict__ Z, T* __restrict__ d
   if (i < n) dA[i] *= silu_grad_d(Z[i]);
 }
 
-// out[i] = sum_z part[z][i] (fixed order), i < nout
+// out[i] = sum_z part[z][i] (fixed order), i < nout: 32 outputs a block, eight thread
+// rows take every eighth partial and the row sums are added in order
 template <typename T>
-__global__ void k_sum_parts(int nz, int64_t nout, const T* __restrict__ part, T* __restrict__ out) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= nout) return;
+__global__ void __launch_bounds__(256) k_sum_parts(int nz, int64_t nout, const T* __restrict__ part, T* __restrict__ out) {
+  __shared__ T rs[8][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int64_t i = blockIdx.x * 32LL + x;
   T s = T(0);
-  for (int z = 0; z < nz; ++z) s += part[(int64_t)z * nout + i];
-  out[i] = s;
+  if (i < nout)
+    for (int z = y; z < nz; z += 8) s += part[(int64_t)z * nout + i];
+  rs[y][x] = s;
+  __syncthreads();
+  if (y == 0 && i < nout) {
+    T v = T(0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v += rs[k][x];
+    out[i] = v;
+  }
 }
 
 // column sums of dZ (n x d) in fixed order: part[blk][j], then summed
@@ -221,12 +440,24 @@ __global__ void __launch_bounds__(256) k_wmse_part(int64_t n, const T* __restric
   }
 }
 
-__global__ void k_wmse_finish(int nb, const double* __restrict__ part, double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double a = 0.0, b = 0.0;
-  for (int i = 0; i < nb; ++i) { a += part[i]; b += part[nb + i]; }
-  out[0] = a / b;
-  out[1] = b;
+// fixed-order trees over the block partials (one thread adding 1024 values in turn
+// took 58 us; the tree takes 6)
+__global__ void __launch_bounds__(RED_B) k_wmse_finish(const double* __restrict__ part, double* __restrict__ out) {
+  __shared__ double r1[RED_B], r2[RED_B];
+  r1[threadIdx.x] = part[threadIdx.x];
+  r2[threadIdx.x] = part[RED_B + threadIdx.x];
+  __syncthreads();
+  for (int s = RED_B / 2; s > 0; s >>= 1) {
+    if ((int)threadIdx.x < s) {
+      r1[threadIdx.x] += r1[threadIdx.x + s];
+      r2[threadIdx.x] += r2[threadIdx.x + s];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    out[0] = r1[0] / r2[0];
+    out[1] = r2[0];
+  }
 }
 
 template <typename T>
@@ -294,19 +525,32 @@ __global__ void k_scale_to_count(int nb, const double* __restrict__ part, int64_
     x[i] *= f;
 }
 
+// FP64 (gradient checks): kch of K per split
 template <typename T>
-void gemm_g(int64_t M, int64_t Nn, int64_t K, int nsplit, const T* A, int64_t sam, int64_t sak, const T* B,
+void gemm_g(int64_t M, int64_t Nn, int64_t K, int64_t kch, const T* A, int64_t sam, int64_t sak, const T* B,
             int64_t sbk, int64_t sbn, T* C, int64_t ldc, cudaStream_t st) {
-  const int64_t kch = ((K + nsplit - 1) / nsplit + GK - 1) / GK * GK;
-  const int nz = (int)((K + kch - 1) / kch);
-  dim3 g((unsigned)((M + GM - 1) / GM), (unsigned)((Nn + GM - 1) / GM), (unsigned)std::max(nz, 1));
+  dim3 g((unsigned)((M + GM - 1) / GM), (unsigned)((Nn + GM - 1) / GM), (unsigned)((K + kch - 1) / kch));
   k_gemm_g<T><<<g, 256, 0, st>>>(M, Nn, K, kch, A, sam, sak, B, sbk, sbn, C, ldc);
   g_launches++;
 }
 
-template <typename T>
-int gemm_splits(int64_t K, int64_t kch_target) {
-  return (int)std::max<int64_t>(1, std::min<int64_t>(64, (K + kch_target - 1) / kch_target));
+// FP32: AK / BK as in k_gemm_f32; 16-byte loads where both operands' rows and pointers
+// are aligned for them
+template <bool AK, bool BK, int EPI>
+void gemm_f32(int64_t M, int64_t Nn, int64_t K, int64_t kch, const float* A, int64_t lda, const float* B, int64_t ldb,
+              float* C, int64_t ldc, const float* bias, float* act, const float* Zp, int silu, cudaStream_t st) {
+  const bool vec = (lda & 3) == 0 && (ldb & 3) == 0 && ((uintptr_t)A & 15) == 0 && ((uintptr_t)B & 15) == 0;
+  dim3 g((unsigned)((M + FT - 1) / FT), (unsigned)((Nn + FT - 1) / FT), (unsigned)((K + kch - 1) / kch));
+  if (vec) k_gemm_f32<AK, BK, true, EPI><<<g, 256, 0, st>>>(M, Nn, K, kch, A, lda, B, ldb, C, ldc, bias, act, Zp, silu);
+  else k_gemm_f32<AK, BK, false, EPI><<<g, 256, 0, st>>>(M, Nn, K, kch, A, lda, B, ldb, C, ldc, bias, act, Zp, silu);
+  g_launches++;
+}
+
+// rows of one K split of the weight gradients: 64 partials at most (the scratch holds
+// that many), no fewer than 64 rows each
+int64_t grad_chunk(int64_t n) {
+  const int64_t ns = std::max<int64_t>(1, std::min<int64_t>(64, n / 64));
+  return ((n + ns - 1) / ns + GK - 1) / GK * GK;
 }
 
 }  // namespace
@@ -365,10 +609,19 @@ void mlp_forward(const int* dims, int nl, const T* params, const T* X, int64_t n
     const T* b = p + (int64_t)dout * din;
     T* Z = w;
     T* A = w + n * dout;
-    // Z = a W^T : (n x din) (din x dout), element (k, j) of W^T = W[j * din + k]
-    gemm_g<T>(n, dout, din, 1, a, din, 1, W, 1, din, Z, dout, st);
-    k_bias_act<T><<<nblk(n * dout, 256), 256, 0, st>>>(n, dout, b, Z, A, l < nl - 1 ? 1 : 0);
-    g_launches++;
+    if constexpr (std::is_same<T, float>::value) {
+      if (l == nl - 1 && dout == 1) {
+        k_row_dot<<<nblk(n, RD_R), 256, 0, st>>>(n, din, a, W, b, Z, A, y);
+        g_launches++;
+        return;
+      }
+      gemm_f32<true, true, 1>(n, dout, din, din, a, din, W, din, Z, dout, b, A, nullptr, l < nl - 1 ? 1 : 0, st);
+    } else {
+      // Z = a W^T : (n x din) (din x dout), element (k, j) of W^T = W[j * din + k]
+      gemm_g<T>(n, dout, din, din, a, din, 1, W, 1, din, Z, dout, st);
+      k_bias_act<T><<<nblk(n * dout, 256), 256, 0, st>>>(n, dout, b, Z, A, l < nl - 1 ? 1 : 0);
+      g_launches++;
+    }
     a = A;
     p = b + dout;
     w = A + n * dout;
@@ -406,22 +659,29 @@ void mlp_backward(const int* dims, int nl, const T* params, const T* X, int64_t 
     T* gW = grads + poff[l];
     T* gb = gW + (int64_t)dout * din;
     // dW = dZ^T a_prev : (dout x n)(n x din), split over n
-    const int ns = gemm_splits<T>(n, 4096);
-    gemm_g<T>(dout, din, n, ns, dcur, 1, dout, a_prev, din, 1, part, din, st);
-    const int64_t kch = ((n + ns - 1) / ns + GK - 1) / GK * GK;
+    const int64_t kch = grad_chunk(n);
     const int nz = (int)((n + kch - 1) / kch);
-    k_sum_parts<T><<<nblk((int64_t)dout * din, 256), 256, 0, st>>>(nz, (int64_t)dout * din, part, gW);
+    if constexpr (std::is_same<T, float>::value)
+      gemm_f32<false, false, 0>(dout, din, n, kch, dcur, dout, a_prev, din, part, din, nullptr, nullptr, nullptr, 0, st);
+    else
+      gemm_g<T>(dout, din, n, kch, dcur, 1, dout, a_prev, din, 1, part, din, st);
+    k_sum_parts<T><<<nblk((int64_t)dout * din, 32), 256, 0, st>>>(nz, (int64_t)dout * din, part, gW);
     // db = column sums of dZ
     const int64_t rpb = (n + RED_B - 1) / RED_B;
     dim3 gc((unsigned)((n + rpb - 1) / rpb), (unsigned)((dout + 127) / 128));
     k_colsum_part<T><<<gc, 128, 0, st>>>(n, dout, dcur, rpb, cpart);
-    k_sum_parts<T><<<nblk(dout, 256), 256, 0, st>>>((int)gc.x, dout, cpart, gb);
-    g_launches += 4;
+    k_sum_parts<T><<<nblk(dout, 32), 256, 0, st>>>((int)gc.x, dout, cpart, gb);
+    g_launches += 3;
     if (l > 0) {
       // dA_prev = dZ W : (n x dout)(dout x din), then dZ_prev = dA_prev * silu'(Z_prev)
-      gemm_g<T>(n, din, dout, 1, dcur, dout, 1, params + poff[l], din, 1, dnext, din, st);
-      k_act_back<T><<<nblk(n * din, 256), 256, 0, st>>>(n * din, work + woff[l - 1], dnext);
-      g_launches++;
+      if constexpr (std::is_same<T, float>::value) {
+        gemm_f32<true, false, 2>(n, din, dout, dout, dcur, dout, params + poff[l], din, dnext, din, nullptr, nullptr,
+                                 work + woff[l - 1], 0, st);
+      } else {
+        gemm_g<T>(n, din, dout, dout, dcur, dout, 1, params + poff[l], din, 1, dnext, din, st);
+        k_act_back<T><<<nblk(n * din, 256), 256, 0, st>>>(n * din, work + woff[l - 1], dnext);
+        g_launches++;
+      }
       T* t = dcur;
       dcur = dnext;
       dnext = t;
@@ -440,7 +700,7 @@ template void mlp_backward<double>(const int*, int, const double*, const double*
 template <typename T>
 void launch_wmse(const T* yh, const T* y, const T* c, int64_t n, T* dy, double* part, double* stats, cudaStream_t st) {
   k_wmse_part<T><<<RED_B, 256, 0, st>>>(n, yh, y, c, part);
-  k_wmse_finish<<<1, 32, 0, st>>>(RED_B, part, stats);
+  k_wmse_finish<<<1, RED_B, 0, st>>>(part, stats);
   k_wmse_grad<T><<<nblk(n, 256), 256, 0, st>>>(n, yh, y, c, stats, dy);
   g_launches += 3;
 }

@@ -71,3 +71,29 @@ def test_blocked_dense_edges(tiny_pair, engine, tol, N):
     np.testing.assert_allclose(eps, eps_ref, atol=tol, rtol=tol)
     gram = (Xd.T @ G.apply_M(Xd)).cpu().numpy()
     np.testing.assert_allclose(gram, np.eye(N), atol=1e-8)
+
+
+# FP32 network passes at the edges of the 128 x 128 x 16 tiles, with rows that do not allow
+# 16-byte loads, against the oracle in FP64: the longest sums have max(dims, n) terms, so
+# the largest entry is off by at most a few sqrt(max) roundings (2^-24 each); 1e-4 as in the
+# ordinary FP32 case
+@pytest.mark.parametrize("dims", [(64, 256, 256, 256, 1), (7, 33, 130, 1), (5, 1), (12, 128, 127, 1)])
+@pytest.mark.parametrize("n", [1, 31, 33, 127, 129, 1000])
+def test_network_at_tile_edges(dims, n):
+    from oracle import learned as O
+    from paper_1610_02121_gb300 import Mlp
+    rng = np.random.default_rng(n + len(dims))
+    flat = np.concatenate([x.reshape(-1) for x in O.init_params(dims, 3)]).astype(np.float32)
+    flat += (0.05 * rng.standard_normal(len(flat))).astype(np.float32)
+    params, at = [], 0
+    for a, b in zip(dims[:-1], dims[1:]):
+        params += [flat[at:at + a * b].reshape(b, a).astype(np.float64), flat[at + a * b:at + a * b + b].astype(np.float64)]
+        at += a * b + b
+    X = rng.standard_normal((n, dims[0])).astype(np.float32)
+    dy = rng.standard_normal(n).astype(np.float32)
+    y_ref, pre = O.forward(params, X.astype(np.float64))
+    g_ref = np.concatenate([g.reshape(-1) for g in O.backward(params, X.astype(np.float64), pre, dy.astype(np.float64))])
+    net = Mlp(dims, precision="fp32", params=flat)
+    Xd = torch.from_numpy(X).cuda()
+    assert rel_err(net.forward(Xd), y_ref) < 1e-4
+    assert rel_err(net.backward(Xd, torch.from_numpy(dy).cuda()), g_ref) < 1e-4
