@@ -62,7 +62,11 @@ struct efe_handle {
   int* hexp = nullptr;      // per-cell row exponents of H^cc_e (tensor-core FP64 products)
   unsigned char* oz_aimg = nullptr;  // pre-sliced BF16 digit images of H^cc_e (made on first use)
   bool oz_aimg_valid = false;
-  int* oz_fexp = nullptr;   // per-column exponents (N)
+  unsigned char* ozc_digits = nullptr;   // FP64 engine's cell products: digit planes of a column panel,
+  double* ozc_products = nullptr;        // its products (grow-only)
+  int64_t ozc_digits_bytes = 0, ozc_products_bytes = 0;
+  int64_t ws_gen = 0;       // counts reallocations of workspace that a recorded graph may point to
+  int* oz_fexp = nullptr;   // per-column exponents (N, readable up to a multiple of 16)
   int* oz_bexp = nullptr;   // per-column exponents of small right-hand matrices (N)
   int* oz_aexp = nullptr;   // per-row exponents of tall left-hand matrices (rows)
   int2* oz_pairs = nullptr; // tile pairs of the tensor-core A^T B products
@@ -296,6 +300,7 @@ void free32(efe_handle* h) {
 
 int reserve(efe_handle* h, int N) {
   if (N <= h->Nres) return EFE_OK;
+  h->ws_gen++;
   free32(h);
   for (void* p : {(void*)h->B1, (void*)h->B2, (void*)h->W, (void*)h->xe, (void*)h->rb, (void*)h->part,
                   (void*)h->small, (void*)h->tnwork, (void*)h->rpart})
@@ -333,7 +338,7 @@ int reserve(efe_handle* h, int N) {
   dfree(h, h->oz_fexp);
   dfree(h, h->oz_bexp);
   dfree(h, h->oz_pairs);
-  TRY(dalloc(h, &h->oz_fexp, N));
+  TRY(dalloc(h, &h->oz_fexp, N + 16));
   TRY(dalloc(h, &h->oz_bexp, N));
   TRY(dalloc(h, &h->oz_pairs, oz_gram_max_pairs(N, N)));
   h->Nres = N;
@@ -343,6 +348,7 @@ int reserve(efe_handle* h, int N) {
 int reserve32(efe_handle* h, int N) {
   if (N <= h->Nres32) return EFE_OK;
   TRY(reserve(h, std::max(N, h->Nres)));
+  h->ws_gen++;
   free32(h);
   // classical rows padded to a multiple of 8 elements: 16-byte aligned rows for
   // vector loads and bulk copies; the padding columns are zero and stay zero
@@ -458,31 +464,70 @@ int timed_end(efe_handle* h, cudaStream_t st, int slot, double units, int ch = 0
   return EFE_OK;
 }
 
+// digit images of H^cc_e for the FP64 engine, made on the first use after a new potential
+int ensure_oz_aimg(efe_handle* h, cudaStream_t st) {
+  if (h->oz_aimg_valid) return EFE_OK;
+  if (!h->oz_aimg) TRY(dalloc(h, &h->oz_aimg, h->n_cell * oz_cell_image_bytes()));
+  launch_oz_preslice(h->Hcc, h->hexp, h->n_cell, h->oz_aimg, st);
+  CKL();
+  h->oz_aimg_valid = true;
+  return EFE_OK;
+}
+
+// Device bytes of the digit planes and of the products of one column panel of the FP64
+// engine's cell products (each): the 16-atom silicon mesh takes its 135 columns in one
+// panel (2.9 and 3.3 GB), the 280-atom mesh 144 columns at a time (6.1 and 6.7 GB).
+constexpr int64_t OZ_CELL_BUDGET = 8ll << 30;
+
+// scratch of the FP64 engine's cell products for blocks of N columns (grow-only)
+int oz_cell_scratch(efe_handle* h, int N, int* panel) {
+  const int w = ozc_panel_cols(h->n_nodes, h->n_cell, N, OZ_CELL_BUDGET, OZ_CELL_BUDGET);
+  *panel = w;
+  const int64_t db = ozc_digit_bytes(h->n_nodes, w), pb = ozc_product_bytes(h->n_cell, w);
+  if (db > h->ozc_digits_bytes) {
+    dfree(h, h->ozc_digits);
+    h->ozc_digits = nullptr;
+    h->ozc_digits_bytes = 0;
+    h->ws_gen++;
+    TRY(dalloc(h, &h->ozc_digits, db));
+    h->ozc_digits_bytes = db;
+  }
+  if (pb > h->ozc_products_bytes) {
+    dfree(h, h->ozc_products);
+    h->ozc_products = nullptr;
+    h->ozc_products_bytes = 0;
+    h->ws_gen++;
+    TRY(dalloc(h, &h->ozc_products, pb / (int64_t)sizeof(double)));
+    h->ozc_products_bytes = pb;
+  }
+  return EFE_OK;
+}
+
+// --- FP64 engine: W_c = H^cc Y_c over all cells, in column panels ---
+int cell_apply_engine(efe_handle* h, const double* Y, int64_t ldy, double* Wc, int64_t ldw, int N, cudaStream_t st) {
+  TRY(ensure_oz_aimg(h, st));
+  int w;
+  TRY(oz_cell_scratch(h, N, &w));
+  launch_oz_colexp(Y, ldy, h->n_nodes, N, h->oz_fexp, st);
+  for (int c0 = 0; c0 < N; c0 += w) {
+    const int nc = std::min(w, N - c0);
+    int slot;
+    TRY(timed_begin(h, st, &slot, 1));
+    if (launch_ozc_cells(h->oz_aimg, h->hexp, h->n_cell, h->mesh, Y + c0, ldy, h->oz_fexp + c0, h->ozc_digits,
+                         h->ozc_products, Wc + c0, ldw, nc, tc_grid(h), h->info + 4, st, h->opt_test_stall)) {
+      h->err = "FP64 engine: tensor map or launch configuration of the cell products refused";
+      return EFE_ERR_CUDA;
+    }
+    TRY(timed_end(h, st, slot, 2.0 * NL * NL * (double)nc * (double)h->n_cell, 1));
+  }
+  CKL();
+  return EFE_OK;
+}
+
 // --- classical cell products, all 8 parity colours: W_c += H^cc Y_c ---
 template <typename T>
 int cell_apply_all(efe_handle* h, const T* Hc, const T* Y, int64_t ldy, T* Wc, int64_t ldw, int N, cudaStream_t st,
                    bool tc = false) {
-  if constexpr (sizeof(T) == 8) {
-    if (h->fp64_engine == 1 && N > 8) {
-      if (!h->oz_aimg_valid) {
-        if (!h->oz_aimg) TRY(dalloc(h, &h->oz_aimg, h->n_cell * oz_cell_image_bytes()));
-        launch_oz_preslice(h->Hcc, h->hexp, h->n_cell, h->oz_aimg, st);
-        h->oz_aimg_valid = true;
-      }
-      launch_oz_colexp((const double*)Y, ldy, h->n_nodes, N, h->oz_fexp, st);
-      for (int c = 0; c < 8; ++c) {
-        const int64_t nc = h->colour_off[c + 1] - h->colour_off[c];
-        if (nc == 0) continue;
-        int slot;
-        TRY(timed_begin(h, st, &slot, 1));
-        launch_oz_cell(h->Hcc, h->hexp, h->colour_cells + h->colour_off[c], nc, h->mesh, (const double*)Y, ldy,
-                       h->oz_fexp, (double*)Wc, ldw, N, tc_grid(h), h->info + 4, st, h->oz_aimg, h->opt_test_stall);
-        TRY(timed_end(h, st, slot, 2.0 * NL * NL * (double)N * (double)nc, 1));
-      }
-      CKL();
-      return EFE_OK;
-    }
-  }
   for (int c = 0; c < 8; ++c) {
     const int64_t nc = h->colour_off[c + 1] - h->colour_off[c];
     if (nc == 0) continue;
@@ -532,6 +577,10 @@ int couple_H(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, int64_t 
 template <typename T>
 int apply_H_generic(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, int64_t ldxe, T* Wc, int64_t ldw,
                     double* We, int64_t ldwe, int N, cudaStream_t st, const T* Hc) {
+  if (sizeof(T) == 8 && h->fp64_engine == 1 && N > 8) {
+    TRY(cell_apply_engine(h, (const double*)Xc, ldx, (double*)Wc, ldw, N, st));
+    return couple_H<T>(h, Xc, ldx, Xe, ldxe, Wc, ldw, We, ldwe, N, st);
+  }
   if (sizeof(T) == 8 && cells_at_once(h, N)) {
     launch_cell_apply_f64_all((const double*)Hc, h->n_cell, h->mesh, (const double*)Xc, ldx, h->cellP, (double*)Wc, ldw,
                               N, st);
@@ -1199,6 +1248,7 @@ int efe_create(const efe_mesh_desc* mesh, const efe_atoms_desc* atoms, const efe
   TRY(dalloc(h, &h->oz_aexp, h->rows));
   TRY(dalloc(h, &h->Aimg32, tc3_image_elems(h->n_cell)));
   TRY(dalloc(h, &h->info, 8));
+  CK(cudaMemset(h->info, 0, 8 * sizeof(int)));
   TRY(dalloc(h, &h->chol_ratio, 1));
   if (h->nE > 0) {
     TRY(upload(h, &h->funcs, s.funcs));
@@ -1786,8 +1836,8 @@ int gemm_tall_ld(efe_handle* h, int64_t rows, int K, int Nc, const double* A, in
       launch_oz_img_rows(A + r0 * lda, lda, n, K, h->oz_aexp + r0, h->oz_img[0], st);
       int slot;
       TRY(timed_begin(h, st, &slot, 1));
-      launch_oz_rows(A + r0 * lda, lda, n, K, h->oz_aexp + r0, B, ldb, h->oz_bexp, C + r0 * ldc, ldc, Nc, tc_grid(h),
-                     h->info + 4, st, h->oz_img[0], h->oz_img[1], h->opt_test_stall);
+      launch_oz_rows(n, K, h->oz_aexp + r0, h->oz_bexp, C + r0 * ldc, ldc, Nc, tc_grid(h), h->info + 4, st, h->oz_img[0],
+                     h->oz_img[1], h->opt_test_stall);
       TRY(timed_end(h, st, slot, 2.0 * (double)n * K * Nc, 1));
     }
   } else {
@@ -2873,6 +2923,7 @@ struct efe_batch {
   std::vector<double*> X;
   std::vector<int64_t> ldx;
   std::vector<int32_t> N;
+  std::vector<int64_t> gen;   // workspace generation of every handle (efe_handle::ws_gen)
   int m = 0, precision = -1, fp64_tail = -1, engine = -1;
   std::string err;
 };
@@ -2965,6 +3016,12 @@ int efe_batch_chfsi_step(efe_batch* b, double* const* X, const int64_t* ldx, con
     efe_handle* h = b->hs[i];
     int rc = reserve(h, N[i]);
     if (rc == EFE_OK && n_low > 0) rc = reserve32(h, N[i]);
+    // the digit images follow the potential, not the recorded graph
+    if (rc == EFE_OK && n_low < m && h->fp64_engine == 1 && N[i] > 8) {
+      int w;
+      rc = oz_cell_scratch(h, N[i], &w);
+      if (rc == EFE_OK) rc = ensure_oz_aimg(h, caller);
+    }
     if (rc != EFE_OK) return fail(i, rc);
     if (h->coef_cap < m) {
       rc = stage_coefs(h, m, a[i], bnd[i], a0[i], caller, false);
@@ -2975,7 +3032,8 @@ int efe_batch_chfsi_step(efe_batch* b, double* const* X, const int64_t* ldx, con
   }
   bool same = b->exec && b->m == m && b->precision == precision && b->fp64_tail == fp64_tail &&
               (int)b->X.size() == n && b->engine == b->hs[0]->fp64_engine;
-  for (int i = 0; same && i < n; ++i) same = b->X[i] == X[i] && b->ldx[i] == ldx[i] && b->N[i] == N[i];
+  for (int i = 0; same && i < n; ++i)
+    same = b->X[i] == X[i] && b->ldx[i] == ldx[i] && b->N[i] == N[i] && b->gen[i] == b->hs[i]->ws_gen;
   if (!same) {
     batch_clear_graph(b);
     const int64_t l0 = g_launches.load();
@@ -3032,6 +3090,8 @@ int efe_batch_chfsi_step(efe_batch* b, double* const* X, const int64_t* ldx, con
     b->X.assign(X, X + n);
     b->ldx.assign(ldx, ldx + n);
     b->N.assign(N, N + n);
+    b->gen.resize(n);
+    for (int i = 0; i < n; ++i) b->gen[i] = b->hs[i]->ws_gen;
     b->m = m;
     b->precision = precision;
     b->fp64_tail = fp64_tail;

@@ -164,15 +164,21 @@ int64_t oz_hexp_elems(int64_t n_cell);
 void launch_oz_hexp(const double* Hcc, int64_t n_cell, int* hexp, cudaStream_t st);
 void launch_oz_colexp(const double* Y, int64_t ldy, int64_t rows, int N, int* fexp, cudaStream_t st);
 void launch_oz_rowexp(const double* A, int64_t lda, int64_t rows, int K, int* aexp, cudaStream_t st);
-// Aimg: pre-sliced digit images of H^cc_e (launch_oz_preslice), or NULL to slice on the fly
-int launch_oz_cell(const double* Hcc, const int* hexp, const int32_t* cells, int64_t ncells, const MeshDev& m,
-                   const double* Y, int64_t ldy, const int* fexp, double* W, int64_t ldw, int N, int n_sm, int* err,
-                   cudaStream_t st, const unsigned char* Aimg = nullptr, int stall = 0);
+// cell products of all cells (efe_oz_cell.cu), W = sum_e H^cc_e Y_e with every row of W
+// written: Aimg from launch_oz_preslice, fexp: column exponents of Y
+// (launch_oz_colexp; readable up to N rounded up to 16), digits / products: scratch of
+// ozc_digit_bytes / ozc_product_bytes; nonzero when the tensor map or the launch
+// configuration is refused
+int64_t ozc_digit_bytes(int64_t nn, int nc);
+int64_t ozc_product_bytes(int64_t n_cell, int nc);
+int ozc_panel_cols(int64_t nn, int64_t n_cell, int N, int64_t digit_budget, int64_t product_budget);
+int launch_ozc_cells(const unsigned char* Aimg, const int* hexp, int64_t n_cell, const MeshDev& m, const double* Y,
+                     int64_t ldy, const int* fexp, unsigned char* digits, double* products, double* W, int64_t ldw, int N,
+                     int n_sm, int* err, cudaStream_t st, int stall);
 int64_t oz_cell_image_bytes();
 void launch_oz_preslice(const double* Hcc, const int* hexp, int64_t n_cell, unsigned char* img, cudaStream_t st);
-int launch_oz_rows(const double* A, int64_t lda, int64_t rows, int K, const int* aexp, const double* B, int64_t ldb,
-                   const int* bexp, double* C, int64_t ldc, int N, int n_sm, int* err, cudaStream_t st,
-                   const unsigned char* Aimg = nullptr, const unsigned char* Bimg = nullptr, int stall = 0);
+int launch_oz_rows(int64_t rows, int K, const int* aexp, const int* bexp, double* C, int64_t ldc, int N, int n_sm,
+                   int* err, cudaStream_t st, const unsigned char* Aimg, const unsigned char* Bimg, int stall);
 // pre-sliced operand images for the ROWS / GRAM products (bytes, builders)
 int64_t oz_img_rows_bytes(int64_t rows, int K);
 int64_t oz_img_cols_bytes(int64_t nch, int ncols);
@@ -181,7 +187,7 @@ void launch_oz_img_rows(const double* A, int64_t lda, int64_t rows, int K, const
 void launch_oz_img_cols(const double* A, int64_t lda, int64_t Krows, int ncols, const int* cexp, int64_t nch,
                         unsigned char* img, cudaStream_t st);
 // C (Na x N) = A^T B (+ C when accumulate), A: K x Na, B: K x N (K large); aexp / bexp per
-// column (launch_oz_colexp)
+// column (launch_oz_colexp); nonzero when the images or the work array are too small
 int launch_oz_gram(int64_t K, int Na, int N, const double* A, int64_t lda, const int* aexp, const double* B,
                    int64_t ldb, const int* bexp, double* C, int64_t ldc, bool sym, double* work, int64_t work_elems,
                    int2* pairs_dev, int n_sm, int* err, cudaStream_t st, unsigned char* img_a = nullptr,

@@ -36,6 +36,26 @@ def test_products_at_tile_edges(tiny_pair, engine, N):
         G.set_fp64_engine("dfma")
 
 
+# FP64 engine's cell products: column tiles of 48 in groups of 16, few and many items per
+# CTA (1 and 3 CTAs), column panels narrower than the block through the filter
+@pytest.mark.parametrize("cap", [0, 1, 3])
+@pytest.mark.parametrize("N", [9, 16, 17, 33, 47, 48, 49, 96, 97, 145])
+def test_engine_cell_tiles(tiny_pair, cap, N):
+    d, G = tiny_pair
+    X = W.random_block(d.system, N, seed=700 + N)
+    G.set_fp64_engine("tensor")
+    G.set_grid_cap(cap)
+    try:
+        Y = G.apply_H(to_dev(X))
+        assert rel_err(Y, d.apply_H_assembled(X)) < 1e-10
+        assert torch.equal(Y, G.apply_H(to_dev(X)))          # reproducible, whatever the grid
+        G.set_grid_cap(0)
+        assert torch.equal(Y, G.apply_H(to_dev(X)))
+    finally:
+        G.set_grid_cap(0)
+        G.set_fp64_engine("dfma")
+
+
 # Cholesky-QR and Rayleigh-Ritz at the edges of the A^T B and A B tiles (16, 32, 48), against the
 # oracle; the figures of the ordinary case (1e-9 on the Ritz values, 1e-8 on the residuals)
 @pytest.mark.parametrize("N", [1, 2, 15, 16, 17, 32, 33, 48, 49])
