@@ -515,7 +515,7 @@ int cell_apply_engine(efe_handle* h, const double* Y, int64_t ldy, double* Wc, i
     TRY(timed_begin(h, st, &slot, 1));
     if (launch_ozc_cells(h->oz_aimg, h->hexp, h->n_cell, h->mesh, Y + c0, ldy, h->oz_fexp + c0, h->ozc_digits,
                          h->ozc_products, Wc + c0, ldw, nc, tc_grid(h), h->info + 4, st, h->opt_test_stall)) {
-      h->err = "FP64 engine: tensor map or launch configuration of the cell products refused";
+      h->err = "FP64 engine: launch configuration of the cell products refused";
       return EFE_ERR_CUDA;
     }
     TRY(timed_end(h, st, slot, 2.0 * NL * NL * (double)nc * (double)h->n_cell, 1));

@@ -167,8 +167,7 @@ void launch_oz_rowexp(const double* A, int64_t lda, int64_t rows, int K, int* ae
 // cell products of all cells (efe_oz_cell.cu), W = sum_e H^cc_e Y_e with every row of W
 // written: Aimg from launch_oz_preslice, fexp: column exponents of Y
 // (launch_oz_colexp; readable up to N rounded up to 16), digits / products: scratch of
-// ozc_digit_bytes / ozc_product_bytes; nonzero when the tensor map or the launch
-// configuration is refused
+// ozc_digit_bytes / ozc_product_bytes; nonzero when the launch configuration is refused
 int64_t ozc_digit_bytes(int64_t nn, int nc);
 int64_t ozc_product_bytes(int64_t n_cell, int nc);
 int ozc_panel_cols(int64_t nn, int64_t n_cell, int N, int64_t digit_budget, int64_t product_budget);

@@ -1,15 +1,14 @@
 // FP64-grade cell products H^cc_e Y_e of all cells on the BF16 tensor cores (the
 // CELL products of the FP64 engine; the slicing and its error bound are described in
-// efe_oz.cu), sm_103a tcgen05 and TMA.
+// efe_oz.cu), sm_103a tcgen05.
 //
 // Three kernels per panel of columns:
 //   k_ozc_slice   cuts the panel of Y into seven BF16 digit planes, one row per node
 //                 (14 bytes a value, columns padded to 16);
-//   k_ozc_cell    persistent, one (cell, 48-column tile) at a time: the cell's 125 node
-//                 rows of every digit plane come in as 5 x 5 x 5-node TMA boxes (the
-//                 nodes of a cell are a box of the node grid) in the MN-major layout
-//                 the MMA reads, H^cc_e's digits as 28 KB bulk copies per 16-wide K
-//                 chunk, and the products leave as FP64 rows of a scratch array;
+//   k_ozc_cell    persistent, one (cell, 48-column tile) at a time: per 16-wide K chunk
+//                 H^cc_e's digits arrive as one 28 KB bulk copy and 16 node rows of every
+//                 digit plane as 16-byte asynchronous copies in the MN-major layout the
+//                 MMA reads; the products leave as FP64 rows of a scratch array;
 //   k_ozc_gather  adds the products of the cells around every node in the order of
 //                 their parity colours, so the sums do not depend on the launch.
 //
@@ -17,17 +16,18 @@
 // gathered and cut once per cell that holds it (about twice) by seven warps, at
 // 64 us for a 96-column tile whose MMAs take 6; and one accumulator set made the
 // epilogue wait for the MMAs and the MMAs for it.  48 columns leave TMEM for two
-// sets (2 x 5 x 48 of 512 columns), and shared memory for two column tiles of Y
-// (2 x 84 KB) beside two chunks of H (2 x 28 KB).  Per apply, 8,424 cells x 135 columns:
-// 7.2 ms before; now 0.25 (slice) + 1.94 (cells: 11.6 us a tile) + 0.63 (gather); x 640
-// columns 23.6 -> 12.3 ms.  What is left: operand traffic from L2 (310 KB a tile) and
-// the shared-memory reads of the MMAs (128 x 48 x 16: 44 clocks for 24 of math).
+// sets (2 x 5 x 48 of 512 columns) and shared memory for five chunks of both operands
+// in flight.  Taking the rows as 5 x 5 x 5-node TMA boxes of 32-byte rows (21 boxes
+// and so whole column tiles a cell) ran at 11.6 us a tile: it left room for two chunks
+// of H only.  What bounds it now: the MMAs' shared-memory reads (128 x 48 x 16: 4 KB of
+// H and 1.5 KB of Y, 44 clocks for 24 of math; measured 44.4 back to back).  Per apply,
+// 8,424 cells x 135 columns: 7.2 ms in the old form; now 0.25 (slice) + 1.42 (cells, 8.5
+// us a tile) + 0.50 (gather); x 640 columns 23.6 -> 9.3 ms.
 //
-// Warp roles (512 threads): warp 0 issues the MMAs (one elected lane), one lane of
-// warp 1 the copies, warps 4-15 share the epilogue (three per TMEM lane quarter).
-// All waits are bounded; on timeout the CTA records an error, stops issuing, drains
-// its copies and MMAs and frees its TMEM.
-#include <cuda.h>
+// Warp roles (512 threads): warp 0 issues the MMAs (one elected lane), warps 1-3 the
+// copies (a thread takes one (K row, 8 columns) of all digits), warps 4-15 share the
+// epilogue (three per TMEM lane quarter).  All waits are bounded; on timeout the CTA
+// records an error, stops issuing, drains its copies and MMAs and frees its TMEM.
 #include <stdint.h>
 
 #include <algorithm>
@@ -40,17 +40,22 @@ namespace efe {
 namespace {
 
 constexpr int OC_TW = 48;                                // column tile
-constexpr int OC_G = OC_TW / 16;                         // 16-column groups (one TMA box each)
+constexpr int OC_NO = OC_TW / 8;                         // 8-column octets
 constexpr int OC_NCH = (NL + OZ_KC - 1) / OZ_KC;         // K chunks of a cell
-constexpr uint32_t OC_BOX = 4096;                        // a box: 125 rows of 32 B, padded to 128 rows
-constexpr uint32_t OC_BOX_BYTES = NL * 32;               // bytes the TMA writes of it
-constexpr uint32_t OC_B = OZ_S * OC_G * OC_BOX;          // one column tile of Y, 84 KB
-constexpr uint32_t OC_A = OZ_S * OZ_ASL;                 // one chunk of H, 28 KB
-constexpr uint32_t OC_A0 = 2 * OC_B;
-constexpr uint32_t OC_BARS = OC_A0 + 2 * OC_A;
+// B of a chunk: per digit and octet two 8 x 16 B core matrices (K rows 0-7, 8-15); octets
+// 272 B apart, so that the 16-byte copies of a row fall into different banks
+constexpr uint32_t OC_OCT = 272;
+constexpr uint32_t OC_BSL = OC_NO * OC_OCT;
+constexpr uint32_t OC_A = OZ_S * OZ_ASL;                 // H, 28 KB
+constexpr uint32_t OC_STAGE = (OC_A + OZ_S * OC_BSL + 127) / 128 * 128;
+constexpr int OC_STAGES = 5;
+constexpr uint32_t OC_BARS = OC_STAGES * OC_STAGE;
 constexpr size_t OC_SMEM = (size_t)OC_BARS + 256;
 constexpr int OC_THREADS = 512;
+constexpr int OC_CPY_W0 = 1, OC_CPY_T = OZ_KC * OC_NO;   // copy threads: 16 rows x 6 octets = warps 1-3
+constexpr int OC_DEPTH = 3;                              // chunks of 16-byte copies in flight per thread
 constexpr int OC_EPI_W0 = 4, OC_EPI_WN = 12;
+static_assert(OC_CPY_T == 96, "warps 1-3");
 
 // A: K-major, no swizzle (core matrix 8 rows x 16 B; LBO 128 B to the next 8 K, SBO 256 B
 // to the next 8 rows)
@@ -58,22 +63,24 @@ __device__ __forceinline__ uint64_t desc_a(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(256u >> 4) << 32) |
          ((uint64_t)1 << 46);
 }
-// B: MN-major, 32-byte swizzle (16 columns of 8 K rows a pattern; LBO to the next 16
-// columns, SBO to the next 8 K)
+// B: MN-major, no swizzle (core matrix 8 K x 8 columns; LBO 128 B to the next 8 K, SBO to
+// the next 8 columns)
 __device__ __forceinline__ uint64_t desc_b(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(OC_BOX >> 4) << 16) | ((uint64_t)(256u >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(OC_OCT >> 4) << 32) |
+         ((uint64_t)1 << 46);
 }
 // FP32 accumulate, BF16 operands, B MN-major (bit 16)
 __device__ __forceinline__ uint32_t idesc_cell(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
 }
-__device__ __forceinline__ void tma_box(void* dst, const CUtensorMap* tm, int c, int x, int y, int z, int s, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
-      "[%7];" ::"r"(su32(dst)),
-      "l"(tm), "r"(c), "r"(x), "r"(y), "r"(z), "r"(s), "r"(su32(bar))
-      : "memory");
+// 16 bytes to shared memory (zeros when valid is false)
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16u : 0u) : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
 }
 
 // digit planes of Y[:, c0 .. c0 + nc): D[s][node][ldn] (BF16 digit s times 2^-7s, columns
@@ -121,31 +128,36 @@ struct OzCellArgs {
   const unsigned char* Aimg;   // digit images of H^cc_e (launch_oz_preslice)
   const int* hexp;             // n_cell x 128 row exponents
   const int* fexp;             // column exponents of the panel
-  int64_t n_cell;
-  int nc[3];
+  const uint16_t* D;           // digit planes (k_ozc_slice)
+  int64_t n_cell, nn;
+  MeshDev m;
   double* P;                   // products, [cell][125][ldn]
   int ldn, ntiles;
   int* err;
   int stall;
 };
 
-__global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(const __grid_constant__ CUtensorMap tmap, OzCellArgs g) {
+__global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
   extern __shared__ __align__(1024) unsigned char sm[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   // an earlier launch already failed: leave at once (CTA-uniform decision)
   __shared__ int s_skip;
+  __shared__ int koff[OC_NCH * OZ_KC];   // node offset of K row k from the cell's first node; -1: padding
   if (tid == 0) s_skip = *(volatile int*)g.err;
+  if (tid < OC_NCH * OZ_KC) {
+    const int a = tid % NP1, b = (tid / NP1) % NP1, c = tid / (NP1 * NP1);
+    koff[tid] = tid < NL ? a + g.m.nn[0] * (b + g.m.nn[1] * c) : -1;
+  }
   __syncthreads();
   if (s_skip) return;
-  uint64_t* afull = reinterpret_cast<uint64_t*>(sm + OC_BARS);   // [2] chunk of H landed
-  uint64_t* aempty = afull + 2;                                  // [2] its MMAs are done
-  uint64_t* bfull = afull + 4;                                   // [2] column tile of Y landed
-  uint64_t* bempty = afull + 6;                                  // [2] its MMAs are done
-  uint64_t* accf = afull + 8;                                    // [2] accumulator set complete
-  uint64_t* acce = afull + 10;                                   // [2] accumulator set read
-  uint64_t* never = afull + 12;                                  // no thread ever arrives here (test stall)
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(afull + 13);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(afull + 14);
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + OC_BARS);   // [stages] both operands of a chunk landed
+  uint64_t* empty = full + OC_STAGES;                           // [stages] its MMAs are done
+  uint64_t* accf = full + 2 * OC_STAGES;                        // [2] accumulator set complete
+  uint64_t* acce = accf + 2;                                    // [2] accumulator set read
+  uint64_t* never = accf + 4;                                   // no thread ever arrives here (test stall)
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(accf + 5);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(accf + 6);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)),
                  "r"(OZ_TMEM_COLS)
@@ -153,11 +165,11 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(const __grid_constan
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 32) {
+    for (int i = 0; i < OC_STAGES; ++i) {
+      bar_init(full + i, OC_CPY_T + 1);
+      bar_init(empty + i, 1);
+    }
     for (int i = 0; i < 2; ++i) {
-      bar_init(afull + i, 1);
-      bar_init(aempty + i, 1);
-      bar_init(bfull + i, 1);
-      bar_init(bempty + i, 1);
       bar_init(accf + i, 1);
       bar_init(acce + i, OC_EPI_WN * 32);
     }
@@ -165,18 +177,15 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(const __grid_constan
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // K rows 125 .. 127 of every box stay zero (the TMA writes 125 rows)
-  for (int t = tid; t < 2 * OZ_S * OC_G * 6; t += OC_THREADS)
-    *reinterpret_cast<uint4*>(sm + (t / 6) * OC_BOX + OC_BOX_BYTES + (t % 6) * 16) = make_uint4(0, 0, 0, 0);
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
   const int64_t nitems = g.n_cell * g.ntiles;
   const int64_t my = nitems > blockIdx.x ? (nitems - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  // what this thread issued last (drained after an abort)
-  int64_t last_mma = -1, last_a = -1, last_b = -1;
+  // the last chunk whose MMAs were committed / whose bulk copy was issued (drained
+  // after an abort)
+  int64_t last_mma = -1, last_copy = -1;
 
   if (warp == 0) {
     // ---------------------------------------------------------------- MMA issuer
@@ -184,6 +193,8 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(const __grid_constan
       // test stall: a wait that nothing completes runs out like a real one
       if (lane == 0) { *abort_flag = 1; atomicExch(g.err, 1); }
     }
+    int s = 0;
+    uint32_t ph = 0;
     for (int64_t t = 0; t < my && !*abort_flag; ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % g.ntiles) * OC_TW;
@@ -191,18 +202,15 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(const __grid_constan
       const int b = (int)(t & 1);
       bool ok = true;
       if (t >= 2) ok = bar_wait(acce + b, (uint32_t)((t / 2 - 1) & 1));
-      if (ok) ok = bar_wait(bfull + b, (uint32_t)((t / 2) & 1));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d = tmem + (uint32_t)(b * OZ_NACC * OC_TW);
       for (int kc = 0; kc < OC_NCH && ok; ++kc) {
-        const int64_t ch = t * OC_NCH + kc;
-        const int s = (int)(ch & 1);
-        ok = bar_wait(afull + s, (uint32_t)((ch / 2) & 1));
+        ok = bar_wait(full + s, ph);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!ok) break;
-        if (lane == 0) {
-          const uint32_t sA = su32(sm + OC_A0 + s * OC_A);
-          const uint32_t sB = su32(sm + b * OC_B) + (uint32_t)kc * 512u;
-          const uint32_t d = tmem + (uint32_t)(b * OZ_NACC * OC_TW);
+        const uint32_t sA = su32(sm) + (uint32_t)s * OC_STAGE;
+        const uint64_t da = desc_a(sA), db = desc_b(sA + OC_A);
+        if (elect_one()) {
           bool first[OZ_NACC] = {true, true, true, true, true};
 #pragma unroll
           for (int tt = 2; tt <= 8; ++tt) {
@@ -213,58 +221,77 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(const __grid_constan
               if (i > OZ_S || j > OZ_S) continue;
               const uint32_t acc = (kc > 0 || !first[a]) ? 1u : 0u;
               first[a] = false;
-              mma_bf16(d + (uint32_t)(a * OC_TW), desc_a(sA + (uint32_t)(i - 1) * OZ_ASL),
-                       desc_b(sB + (uint32_t)(j - 1) * (OC_G * OC_BOX)), id, acc);
+              mma_bf16(d + (uint32_t)(a * OC_TW), da + (uint64_t)((i - 1) * (OZ_ASL >> 4)),
+                       db + (uint64_t)((j - 1) * (OC_BSL >> 4)), id, acc);
             }
           }
-          mma_commit(aempty + s);
-          if (kc == OC_NCH - 1) {
-            mma_commit(bempty + b);
-            mma_commit(accf + b);
-          }
+          mma_commit(empty + s);
+          if (kc == OC_NCH - 1) mma_commit(accf + b);
         }
-        last_mma = ch;
         __syncwarp();
+        last_mma = t * OC_NCH + kc;
+        if (++s == OC_STAGES) { s = 0; ph ^= 1; }
       }
       if (!ok) {
         if (lane == 0) { *abort_flag = 1; atomicExch(g.err, 1); }
         break;
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp < OC_EPI_W0) {
     // ---------------------------------------------------------------- copies
-    auto load_b = [&](int64_t t) -> bool {
+    const int ct = tid - OC_CPY_W0 * 32;
+    const int k = ct / OC_NO, oct = ct % OC_NO;
+    const uint32_t dst0 = su32(sm) + OC_A + (uint32_t)oct * OC_OCT + (uint32_t)(k >> 3) * 128u + (uint32_t)(k & 7) * 16u;
+    const int64_t plane = g.nn * g.ldn;   // elements of a digit plane
+    int s = 0, sd = 0;                    // stage to fill, stage whose copies are waited for next
+    uint32_t ph = 0;
+    int64_t ch = 0, done = 0;             // chunks issued / announced
+    bool ok = true;
+    auto announce = [&]() {
+      // this thread's copies of the oldest chunk have landed: make them visible to the
+      // MMAs' reads and arrive
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      bar_arrive(full + sd);
+      if (++sd == OC_STAGES) sd = 0;
+      ++done;
+    };
+    for (int64_t t = 0; t < my && ok && !*abort_flag; ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int64_t e = item / g.ntiles;
       const int c0 = (int)(item % g.ntiles) * OC_TW;
-      const int ng = (min(OC_TW, g.ldn - c0) + 15) / 16;
-      const int b = (int)(t & 1);
-      if (t >= 2 && !bar_wait(bempty + b, (uint32_t)((t / 2 - 1) & 1))) return false;
-      const int x = P * (int)(e % g.nc[0]), y = P * (int)((e / g.nc[0]) % g.nc[1]),
-                z = P * (int)(e / ((int64_t)g.nc[0] * g.nc[1]));
-      bar_expect_tx(bfull + b, (uint32_t)(OZ_S * ng) * OC_BOX_BYTES);
-      for (int s = 0; s < OZ_S; ++s)
-        for (int q = 0; q < ng; ++q)
-          tma_box(sm + b * OC_B + (s * OC_G + q) * OC_BOX, &tmap, c0 + 16 * q, x, y, z, s, bfull + b);
-      last_b = t;
-      return true;
-    };
-    bool ok = my > 0 ? load_b(0) : true;
-    for (int64_t t = 0; t < my && ok && !*abort_flag; ++t) {
-      const int64_t e = (blockIdx.x + t * gridDim.x) / g.ntiles;
-      for (int kc = 0; kc < OC_NCH && ok; ++kc) {
-        const int64_t ch = t * OC_NCH + kc;
-        const int s = (int)(ch & 1);
-        if (ch >= 2) ok = bar_wait(aempty + s, (uint32_t)((ch / 2 - 1) & 1));
-        if (!ok) break;
-        bar_expect_tx(afull + s, OC_A);
-        bulk_g2s(sm + OC_A0 + s * OC_A, g.Aimg + (e * OC_NCH + kc) * (int64_t)OC_A, OC_A, afull + s);
-        last_a = ch;
-        // the next item's columns, once this item's first chunks are on their way (the
-        // buffer was freed by the item before)
-        if (kc == 1 && t + 1 < my) ok = load_b(t + 1);
+      const int no = min(OC_TW, g.ldn - c0) / 8;
+      const int ci = (int)(e % g.m.nc[0]), cj = (int)((e / g.m.nc[0]) % g.m.nc[1]),
+                ck = (int)(e / ((int64_t)g.m.nc[0] * g.m.nc[1]));
+      const int64_t g0 = (int64_t)(P * ci) + (int64_t)g.m.nn[0] * ((int64_t)(P * cj) + (int64_t)g.m.nn[1] * (P * ck));
+      const uint16_t* src0 = g.D + g0 * g.ldn + c0 + 8 * oct;
+      for (int kc = 0; kc < OC_NCH; ++kc) {
+        if (ch >= OC_STAGES) {
+          ok = bar_wait(empty + s, ph ^ 1u);
+          if (!ok) break;
+        }
+        if (ct == 0) {
+          bar_expect_tx(full + s, OC_A);
+          bulk_g2s(sm + (uint32_t)s * OC_STAGE, g.Aimg + (e * OC_NCH + kc) * (int64_t)OC_A, OC_A, full + s);
+          last_copy = ch;
+        }
+        if (oct < no) {
+          const int ko = koff[kc * OZ_KC + k];
+          const uint16_t* src = src0 + (int64_t)max(ko, 0) * g.ldn;
+          const uint32_t dst = dst0 + (uint32_t)s * OC_STAGE;
+#pragma unroll
+          for (int i = 0; i < OZ_S; ++i) cp16(dst + (uint32_t)i * OC_BSL, src + i * plane, ko >= 0);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        ++ch;
+        if (++s == OC_STAGES) { s = 0; ph ^= 1; }
+        if (ch > OC_DEPTH) {
+          asm volatile("cp.async.wait_group %0;" ::"n"(OC_DEPTH) : "memory");
+          announce();
+        }
       }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    while (done < ch) announce();
     if (!ok) {
       *abort_flag = 1;
       atomicExch(g.err, 1);
@@ -326,17 +353,18 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(const __grid_constan
       bar_arrive(acce + b);
     }
   }
-  // all roles done.  After an abort every copy still in flight lands and the last MMA
-  // commit (it covers every MMA this CTA issued) arrives before the TMEM and the shared
-  // memory are released; each drain wait is bounded like the pipeline's own.
+  // all roles done.  After an abort every bulk copy still in flight lands (the copy
+  // threads announced all their own copies, and at most the last OC_STAGES chunks are
+  // outstanding) and the last MMA commit (it covers every MMA this CTA issued) arrives
+  // before the TMEM and the shared memory are released; each drain wait is bounded like
+  // the pipeline's own.
   __syncthreads();
   if (*abort_flag) {
-    for (int64_t ch = last_a - 1; ch <= last_a; ++ch)
-      if (ch >= 0) bar_wait(afull + (int)(ch & 1), (uint32_t)((ch / 2) & 1));
-    for (int64_t t = last_b - 1; t <= last_b; ++t)
-      if (t >= 0) bar_wait(bfull + (int)(t & 1), (uint32_t)((t / 2) & 1));
+    if (last_copy >= 0)
+      for (int64_t ch = max(last_copy - OC_STAGES + 1, (int64_t)0); ch <= last_copy; ++ch)
+        bar_wait(full + (int)(ch % OC_STAGES), (uint32_t)((ch / OC_STAGES) & 1));
     if (warp == 0 && lane == 0 && last_mma >= 0)
-      bar_wait(aempty + (int)(last_mma & 1), (uint32_t)((last_mma / 2) & 1));
+      bar_wait(empty + (int)(last_mma % OC_STAGES), (uint32_t)((last_mma / OC_STAGES) & 1));
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -347,12 +375,15 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(const __grid_constan
 }
 
 // W[node][c] = sum of the cell products around the node in the order of the parity
-// colours; a block of 16 nodes x 16 column pairs
+// colours; a block of 16 nodes x 16 threads of CPT column pairs 32 columns apart.  (A warp per
+// node with its eight row pointers found once took 2.5 times as long: seven of eight
+// are absent for most nodes, and their tests sat between the loads.)
+template <int CPT>
 __global__ void __launch_bounds__(256) k_ozc_gather(MeshDev m, int64_t nn, const double* __restrict__ Pc, int ldn, int nc,
                                                     double* __restrict__ W, int64_t ldw) {
   const int64_t gn = blockIdx.x * 16LL + threadIdx.y;
-  const int c = (blockIdx.y * 16 + threadIdx.x) * 2;
-  if (gn >= nn || c >= nc) return;
+  const int c0 = blockIdx.y * 32 * CPT + threadIdx.x * 2;
+  if (gn >= nn || c0 >= nc) return;
   const int G[3] = {(int)(gn % m.nn[0]), (int)((gn / m.nn[0]) % m.nn[1]), (int)(gn / ((int64_t)m.nn[0] * m.nn[1]))};
   int hi[3];
   bool two[3];
@@ -361,7 +392,9 @@ __global__ void __launch_bounds__(256) k_ozc_gather(MeshDev m, int64_t nn, const
     hi[d] = min(G[d] / P, m.nc[d] - 1);
     two[d] = G[d] % P == 0 && G[d] > 0 && G[d] / P < m.nc[d];
   }
-  double2 s = make_double2(0.0, 0.0);
+  double2 s[CPT];
+#pragma unroll
+  for (int u = 0; u < CPT; ++u) s[u] = make_double2(0.0, 0.0);
 #pragma unroll
   for (int col = 0; col < 8; ++col) {
     int cc[3], l[3];
@@ -374,30 +407,21 @@ __global__ void __launch_bounds__(256) k_ozc_gather(MeshDev m, int64_t nn, const
     }
     if (!ok) continue;
     const int64_t e = cc[0] + (int64_t)m.nc[0] * (cc[1] + (int64_t)m.nc[1] * cc[2]);
-    const double2 p = *reinterpret_cast<const double2*>(Pc + (e * NL + l[0] + NP1 * (l[1] + NP1 * l[2])) * (int64_t)ldn + c);
-    s.x += p.x;
-    s.y += p.y;
+    const double* row = Pc + (e * NL + l[0] + NP1 * (l[1] + NP1 * l[2])) * (int64_t)ldn + c0;
+#pragma unroll
+    for (int u = 0; u < CPT; ++u)
+      if (c0 + 32 * u < nc) {
+        const double2 p = *reinterpret_cast<const double2*>(row + 32 * u);
+        s[u].x += p.x;
+        s[u].y += p.y;
+      }
   }
-  W[gn * ldw + c] = s.x;
-  if (c + 1 < nc) W[gn * ldw + c + 1] = s.y;
-}
-
-typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiled encode_tiled() {
-  static const EncodeTiled fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      return (EncodeTiled) nullptr;
-    }
-    return (EncodeTiled)p;
-  }();
-  return fn;
+  double* w = W + gn * ldw + c0;
+#pragma unroll
+  for (int u = 0; u < CPT; ++u) {
+    if (c0 + 32 * u < nc) w[32 * u] = s[u].x;
+    if (c0 + 32 * u + 1 < nc) w[32 * u + 1] = s[u].y;
+  }
 }
 
 inline int pad16(int n) { return (n + 15) / 16 * 16; }
@@ -419,29 +443,18 @@ int launch_ozc_cells(const unsigned char* Aimg, const int* hexp, int64_t n_cell,
                      int64_t ldy, const int* fexp, unsigned char* digits, double* products, double* W, int64_t ldw, int N,
                      int n_sm, int* err, cudaStream_t st, int stall) {
   if (n_cell <= 0 || N <= 0) return 0;
-  const EncodeTiled enc = encode_tiled();
-  if (!enc) return 1;
   const int64_t nn = (int64_t)m.nn[0] * m.nn[1] * m.nn[2];
   const int ldn = pad16(N);
   const int64_t ns = nn * (ldn / 8);
   k_ozc_slice<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(Y, ldy, nn, N, ldn, fexp, reinterpret_cast<uint16_t*>(digits));
-  // digit planes as a 5-D tensor: column, x, y, z, digit; a box: 16 columns of the 125
-  // nodes of a cell
-  CUtensorMap tm;
-  const cuuint64_t row = (cuuint64_t)ldn * 2;
-  const cuuint64_t dims[5] = {(cuuint64_t)ldn, (cuuint64_t)m.nn[0], (cuuint64_t)m.nn[1], (cuuint64_t)m.nn[2], OZ_S};
-  const cuuint64_t strides[4] = {row, row * m.nn[0], row * m.nn[0] * m.nn[1], row * (cuuint64_t)nn};
-  const cuuint32_t box[5] = {16, NP1, NP1, NP1, 1};
-  const cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  if (enc(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, digits, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-          CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return 1;
   OzCellArgs a{};
   a.Aimg = Aimg;
   a.hexp = hexp;
   a.fexp = fexp;
+  a.D = reinterpret_cast<const uint16_t*>(digits);
   a.n_cell = n_cell;
-  for (int d = 0; d < 3; ++d) a.nc[d] = m.nc[d];
+  a.nn = nn;
+  a.m = m;
   a.P = products;
   a.ldn = ldn;
   a.ntiles = (ldn + OC_TW - 1) / OC_TW;
@@ -449,9 +462,12 @@ int launch_ozc_cells(const unsigned char* Aimg, const int* hexp, int64_t n_cell,
   a.stall = stall;
   const int64_t items = n_cell * a.ntiles;
   if (cudaFuncSetAttribute(k_ozc_cell, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OC_SMEM) != cudaSuccess) return 1;
-  k_ozc_cell<<<(unsigned)std::min<int64_t>(items, n_sm), OC_THREADS, OC_SMEM, st>>>(tm, a);
-  k_ozc_gather<<<dim3((unsigned)((nn + 15) / 16), (unsigned)((N + 31) / 32)), dim3(16, 16), 0, st>>>(m, nn, products, ldn, N, W,
-                                                                                                  ldw);
+  k_ozc_cell<<<(unsigned)std::min<int64_t>(items, n_sm), OC_THREADS, OC_SMEM, st>>>(a);
+  if (N > 32)
+    k_ozc_gather<2><<<dim3((unsigned)((nn + 15) / 16), (unsigned)((N + 63) / 64)), dim3(16, 16), 0, st>>>(m, nn, products,
+                                                                                                       ldn, N, W, ldw);
+  else
+    k_ozc_gather<1><<<(unsigned)((nn + 15) / 16), dim3(16, 16), 0, st>>>(m, nn, products, ldn, N, W, ldw);
   g_launches.fetch_add(3, std::memory_order_relaxed);
   return 0;
 }
