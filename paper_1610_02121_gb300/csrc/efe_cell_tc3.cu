@@ -2,26 +2,30 @@
 //
 // Paper, Sec. V (last paragraph): W_c(e) += H^cc_e Y_c(e) for every cell of
 // one parity colour (cells of a colour share no node, so the scatter needs no
-// atomics), one M = 128, K = 128 (four 32-wide chunks), N <= 160 TF32 product
+// atomics), one M = 128, K = 128 (eight 16-wide chunks), N <= 160 TF32 product
 // per cell and column tile, FP32 accumulation in tensor memory.
 //
-// Roles of the 16 warps of a persistent CTA:
-//   warp 0      producer: per chunk one bulk copy of the cell's FP32 image
-//               (H^cc_e, 16 KB, already in the core-matrix layout) and one
-//               bulk copy per node row of Y into a raw staging buffer, all
-//               completing on mbarrier `full`;
-//   warp 1      MMA issuer: 4 (one pass) or 12 (3-term split: A1 B1 + A1 B2 +
-//               A2 B1) tcgen05.mma per chunk into one of two TMEM
-//               accumulators, commits to `empty` (stage reusable) and, after
-//               the last chunk, to `acc_full`;
-//   warps 2-7   converters: the A chunk in place -> A1 = TF32(A) (and A2 =
-//               the TF32 remainder), raw rows -> K-major core-matrix B1 (and
-//               B2), arrive on `conv`;
-//   warps 8-15  epilogue: tcgen05.ld of the accumulator rows, scatter-add into
-//               W as vector reductions performed in L2 (no read-back), arrive
-//               on `acc_empty`.
-// Two stages ring the chunks.  Every wait is bounded (about one second); on
-// timeout the CTA records an error, stops issuing, drains and frees its TMEM.
+// Roles of the warps of a persistent CTA (25 at a column tile of 160):
+//   warp 0       MMA issuer (one elected lane): per 8 K one (one pass) or three
+//                (3-term split: A1 B1 + A1 B2 + A2 B1) tcgen05.mma into one of two TMEM
+//                accumulators, commits to `empty` (stage reusable) and, after
+//                the last chunk, to `acc_full`;
+//   then two groups of TW / 16 converter warps, one for the even and one for the odd
+//                chunks: each warp copies its own 8 node rows x 32 columns of Y and its
+//                share of the H^cc_e image (FP32, already in the core-matrix layout) by
+//                16-byte asynchronous copies into a ring of its own, splits them into
+//                A1 = TF32(A), A2 the TF32 remainder, K-major B1 = TF32(Y) and B2 (or the
+//                BF16 forms) in the stage and arrives on `conv`;
+//   last 4 warps epilogue: tcgen05.ld of the accumulator rows, scatter-add into
+//                W as vector reductions performed in L2 (no read-back; four lanes add 64
+//                contiguous bytes of a row), arrive on `acc_empty`.
+// The chunks in flight come from warp-private rings because one bulk copy per node row
+// bounds the whole kernel: its issue took 2,100 cycles per 16 rows, whatever the stages
+// behind it (2 to 7) or the converter warps (6 to 16).  A launch over 3,670 cells x 135
+// columns: 250 -> 163 us (64 KB of H, 68 KB of Y and twice 68 KB of W a cell, 6.0 TB/s: DRAM
+// bounds it now); over 150 cells x 12 columns: 15 -> 11.5 us (one cell a CTA: latency).
+// Every wait is bounded (about one second); on timeout the CTA records an error, stops
+// issuing, drains and frees its TMEM.
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -31,34 +35,42 @@ namespace efe {
 
 namespace {
 
-constexpr int T3_M = 128, T3_K = 128, T3_KC = 32, T3_NCH = 4;
-constexpr int T3_STAGES = 2;
+constexpr int T3_M = 128, T3_K = 128, T3_KC = 16, T3_NCH = 8;
 // column tile (template parameter TW of the kernel): 64, 96 or 160, picked per
 // system and N by the autotuner (efe_autotune); 160 by default
-constexpr int T3_THREADS = 512;
-constexpr int T3_CONV_WARP0 = 2, T3_CONV_WARPS = 6;
-constexpr int T3_EPI_WARP0 = 8, T3_EPI_WARPS = 8;
+constexpr int T3_EPI_WARPS = 4;
 constexpr uint32_t T3_TMEM_COLS = 512;     // accumulators at columns 0 and 256
 constexpr long long T3_WAIT = 2000000000LL;
+constexpr uint32_t T3_AP = T3_M * T3_KC * 4;    // a chunk of H, or one of its TF32 parts: 8 KB
 
 template <int TW>
 struct T3Layout {
-  // stage: A1 | A2 | B1 | B2 | Braw      (bytes)
-  static constexpr uint32_t A = T3_M * T3_KC * 4;           // 16 KB
-  static constexpr uint32_t B = TW * T3_KC * 4;             // 20 KB at TW = 160
-  static constexpr uint32_t RAW = T3_KC * TW * 4;           // 20 KB at TW = 160
-  static constexpr uint32_t STAGE = 2 * A + 2 * B + RAW;    // 92 KB at TW = 160
-  static constexpr uint32_t BARS = T3_STAGES * STAGE;       // barrier area offset
+  // stage: A1 | A2 (or BF16 A) | B1 | B2; ring slot: A | 1 KB of Y for each warp of the group
+  static constexpr uint32_t A = 2 * T3_AP;                  // 16 KB
+  static constexpr uint32_t B = TW * T3_KC * 4;             // 10 KB at TW = 160
+  static constexpr uint32_t STAGE = A + 2 * B;              // 36 KB
+  static constexpr int STAGES = TW == 160 ? 3 : 4;
+  static constexpr int GW = TW / 16;                        // warps of a converter group
+  static constexpr uint32_t SLOT = T3_AP + GW * 1024;       // 18 KB
+  static constexpr int DEPTH = TW == 160 ? 3 : (TW == 96 ? 4 : 5);   // slots of a group
+  static constexpr uint32_t RING = STAGES * STAGE;
+  static constexpr uint32_t LUT = RING + 2 * DEPTH * SLOT;  // node offsets of the 128 rows
+  static constexpr uint32_t BARS = LUT + T3_M * 4;
   static constexpr size_t TOTAL = (size_t)BARS + 256;
+  static constexpr int THREADS = (1 + 2 * GW + T3_EPI_WARPS) * 32;
+  static_assert(TOTAL <= 227 * 1024, "shared memory of one CTA");
 };
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// K-major, no swizzle: core matrix 8 rows x 16 B; LBO = 128 B (next K core matrix), SBO to
+// the next 8 rows, version 1
+template <uint32_t SBO>
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  // K-major, no swizzle: LBO = 128 B (next K core matrix), SBO = 1024 B (next 8 rows), version 1
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) |
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(SBO >> 4) << 32) |
          ((uint64_t)1 << 46);
 }
+constexpr uint32_t T3_SBO = 512, T3_SBO_BF = 256;   // 16 K of 4 and of 2 bytes
 
 __device__ __forceinline__ uint32_t idesc_tf32(int n) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(T3_M >> 4) << 24);
@@ -69,14 +81,8 @@ __device__ __forceinline__ uint32_t idesc_bf16(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(T3_M >> 4) << 24);
 }
 
-// K-major BF16 chunk of 32 K: core matrix 8 rows x 16 B (8 K); LBO = 128 B (next 8 K),
-// SBO = 512 B (next 8 rows)
-__device__ __forceinline__ uint64_t sdesc_bf16(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(512u >> 4) << 32) |
-         ((uint64_t)1 << 46);
-}
 __device__ __forceinline__ uint32_t bmo(int row, int k) {
-  return (uint32_t)(row >> 3) * 512u + (uint32_t)(k >> 3) * 128u + (uint32_t)(row & 7) * 16u + (uint32_t)(k & 7) * 2u;
+  return (uint32_t)(row >> 3) * T3_SBO_BF + (uint32_t)(k >> 3) * 128u + (uint32_t)(row & 7) * 16u + (uint32_t)(k & 7) * 2u;
 }
 __device__ __forceinline__ uint16_t bf16r(float x) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(x));
@@ -94,11 +100,7 @@ __device__ __forceinline__ void bar_init(uint64_t* b, uint32_t n) {
 __device__ __forceinline__ void bar_arrive(uint64_t* b) {
   asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(su32(b)) : "memory");
 }
-__device__ __forceinline__ void bar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(su32(b)),
-               "r"(bytes)
-               : "memory");
-}
+
 __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
   uint32_t done = 0;
   const long long t0 = clock64();
@@ -113,12 +115,7 @@ __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
   } while (clock64() - t0 < T3_WAIT);
   return false;
 }
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(su32(dst)),
-      "l"(src), "r"(bytes), "r"(su32(bar))
-      : "memory");
-}
+
 __device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -138,40 +135,51 @@ __device__ __forceinline__ void mma_commit(uint64_t* b) {
                : "memory");
 }
 
-// node id of local row k (0..124) of cell e
-__device__ __forceinline__ int64_t cell_node(const MeshDev& m, int64_t e, int k) {
+// node id of the corner of cell e (its local row 0)
+__device__ __forceinline__ int64_t cell_corner(const MeshDev& m, int64_t e) {
   const int i = (int)(e % m.nc[0]), j = (int)((e / m.nc[0]) % m.nc[1]), kk = (int)(e / ((int64_t)m.nc[0] * m.nc[1]));
-  const int a = k % NP1, b = (k / NP1) % NP1, c = k / (NP1 * NP1);
-  return (int64_t)(P * i + a) + (int64_t)m.nn[0] * ((int64_t)(P * j + b) + (int64_t)m.nn[1] * (int64_t)(P * kk + c));
+  return (int64_t)(P * i) + (int64_t)m.nn[0] * ((int64_t)(P * j) + (int64_t)m.nn[1] * (int64_t)(P * kk));
 }
 
-// K-major core-matrix offset (bytes) within a 32-wide chunk
-__device__ __forceinline__ uint32_t cmo(int row, int k) {
-  return (uint32_t)(row >> 3) * 1024u + (uint32_t)(k >> 2) * 128u + (uint32_t)(row & 7) * 16u;
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool real) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(real ? 16 : 0) : "memory");
+}
+
+// K-major core-matrix offset (bytes) within a 16-wide chunk of 4-byte values
+__host__ __device__ __forceinline__ uint32_t cmo(int row, int k) {
+  return (uint32_t)(row >> 3) * T3_SBO + (uint32_t)(k >> 2) * 128u + (uint32_t)(row & 7) * 16u;
+}
+
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
 }
 
 // MODE 0: one TF32 pass; 1: 3-term TF32 split (a1 b1 + a1 b2 + a2 b1); 2: BF16 operands
 template <int MODE, int TW>
-__global__ void __launch_bounds__(T3_THREADS, 1) k_cell_tc3(const float* __restrict__ Ag,
-                                                            const int32_t* __restrict__ cells, int64_t ncells,
-                                                            MeshDev m, const float* __restrict__ Y, int64_t ldy,
-                                                            float* __restrict__ W, int64_t ldw, int N, int ntiles,
-                                                            int* __restrict__ err, int stall) {
+__global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
+    k_cell_tc3(const float* __restrict__ Ag, const int32_t* __restrict__ cells, int64_t ncells, MeshDev m,
+               const float* __restrict__ Y, int64_t ldy, float* __restrict__ W, int64_t ldw, int N, int ntiles,
+               int* __restrict__ err, int stall) {
+  using L = T3Layout<TW>;
+  constexpr int ST = L::STAGES;
   extern __shared__ __align__(1024) unsigned char sm[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  uint64_t* conv = reinterpret_cast<uint64_t*>(sm + L::BARS);   // [ST]
+  uint64_t* empty = conv + ST;                                  // [ST]
+  uint64_t* accf = conv + 2 * ST;                               // [2]
+  uint64_t* acce = accf + 2;                                    // [2]
+  uint64_t* never = accf + 4;   // no thread ever arrives here (the test stall waits on it)
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(accf + 5);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(accf + 6);
+  int32_t* lut = reinterpret_cast<int32_t*>(sm + L::LUT);
   // an earlier launch already failed: leave at once (CTA-uniform decision)
-  __shared__ int s_skip;
-  if (tid == 0) s_skip = *(volatile int*)err;
+  if (tid == 0) *abort_flag = *(volatile int*)err;
   __syncthreads();
-  if (s_skip) return;
-  uint64_t* full = reinterpret_cast<uint64_t*>(sm + T3Layout<TW>::BARS);  // [2]
-  uint64_t* conv = full + 2;                                          // [2]
-  uint64_t* empty = full + 4;                                         // [2]
-  uint64_t* accf = full + 6;                                          // [2]
-  uint64_t* acce = full + 8;                                          // [2]
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(full + 10);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(full + 11);
-  uint64_t* never = full + 12;   // no thread ever arrives here (the test stall waits on it)
+  if (*abort_flag) return;
+  __syncthreads();
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)),
@@ -180,18 +188,20 @@ __global__ void __launch_bounds__(T3_THREADS, 1) k_cell_tc3(const float* __restr
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 32) {
-    for (int s = 0; s < T3_STAGES; ++s) {
-      bar_init(full + s, 1);
-      bar_init(conv + s, T3_CONV_WARPS * 32);
+    for (int s = 0; s < ST; ++s) {
+      bar_init(conv + s, L::GW);
       bar_init(empty + s, 1);
     }
     for (int b = 0; b < 2; ++b) {
       bar_init(accf + b, 1);
-      bar_init(acce + b, T3_EPI_WARPS * 32);
+      bar_init(acce + b, T3_EPI_WARPS);
     }
     bar_init(never, 1);
-    *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (tid >= 64 && tid < 64 + T3_M) {
+    const int k = min(tid - 64, NL - 1);
+    lut[tid - 64] = k % NP1 + m.nn[0] * (k / NP1 % NP1 + m.nn[1] * (k / (NP1 * NP1)));
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -199,177 +209,187 @@ __global__ void __launch_bounds__(T3_THREADS, 1) k_cell_tc3(const float* __restr
   const uint32_t tmem = *tslot;
   const int64_t nitems = ncells * ntiles;
   const int64_t my_items = nitems > blockIdx.x ? (nitems - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  // the last chunk whose bulk copies this thread issued / whose MMAs it committed
-  // (drained before the TMEM is released if the CTA aborts)
-  int64_t last_copy = -1, last_mma = -1;
+  // the last chunk whose MMAs this thread committed (drained before the TMEM is
+  // released if the CTA aborts)
+  int64_t last_mma = -1;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ producer
-    for (int64_t t = 0; t < my_items && !*abort_flag; ++t) {
-      const int64_t item = blockIdx.x + t * gridDim.x;
-      const int64_t e = cells[item / ntiles];
-      const int c0 = (int)(item % ntiles) * TW;
-      const int ncol = min(TW, N - c0);
-      const uint32_t row_bytes = (uint32_t)((ncol + 3) / 4) * 16u;
-      for (int kc = 0; kc < T3_NCH; ++kc) {
-        const int64_t ch = t * T3_NCH + kc;
-        const int s = (int)(ch % T3_STAGES);
-        if (ch >= T3_STAGES && !bar_wait(empty + s, (uint32_t)((ch / T3_STAGES - 1) & 1))) {
-          if (lane == 0) { *abort_flag = 1; atomicExch(err, 1); }
-          break;
-        }
-        unsigned char* S = sm + s * T3Layout<TW>::STAGE;
-        const int nrows = min(T3_KC, NL - kc * T3_KC);
-        if (lane == 0) bar_expect_tx(full + s, T3Layout<TW>::A + (uint32_t)nrows * row_bytes);
-        __syncwarp();
-        if (lane == 0) bulk_g2s(S, Ag + (e * T3_NCH + kc) * (T3_M * T3_KC), T3Layout<TW>::A, full + s);
-        if (lane < nrows) {
-          const int64_t g = cell_node(m, e, kc * T3_KC + lane);
-          bulk_g2s(S + 2 * T3Layout<TW>::A + 2 * T3Layout<TW>::B + (uint32_t)lane * (TW * 4), Y + g * ldy + c0, row_bytes,
-                   full + s);
-        }
-        last_copy = ch;
-        __syncwarp();
-      }
-    }
-  } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     if (stall && my_items > 0 && !bar_wait(never, 0u)) {
       // test stall: a wait that nothing completes runs out like a real one
       if (lane == 0) { *abort_flag = 1; atomicExch(err, 1); }
     }
+    int s = 0;
+    uint32_t ph = 0;
     for (int64_t t = 0; t < my_items && !*abort_flag; ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % ntiles) * TW;
       const int ncol = min(TW, N - c0);
       const int nmma = ((ncol + 15) / 16) * 16;
+      const uint32_t id = MODE == 2 ? idesc_bf16(nmma) : idesc_tf32(nmma);
       const int b = (int)(t & 1);
       bool ok = true;
       if (t >= 2) ok = bar_wait(acce + b, (uint32_t)((t / 2 - 1) & 1));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d = tmem + (uint32_t)(b * 256);
       for (int kc = 0; kc < T3_NCH && ok; ++kc) {
-        const int64_t ch = t * T3_NCH + kc;
-        const int s = (int)(ch % T3_STAGES);
-        ok = bar_wait(conv + s, (uint32_t)((ch / T3_STAGES) & 1));
+        ok = bar_wait(conv + s, ph);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!ok) break;
-        if (lane == 0) {
-          unsigned char* S = sm + s * T3Layout<TW>::STAGE;
-          const uint32_t a1 = su32(S), a2 = a1 + T3Layout<TW>::A, b1 = a1 + 2 * T3Layout<TW>::A, b2 = b1 + T3Layout<TW>::B;
-          const uint32_t d = tmem + (uint32_t)(b * 256);
+        const uint32_t a1 = su32(sm) + (uint32_t)s * L::STAGE, b1 = a1 + L::A;
+        if (elect_one()) {
           if (MODE == 2) {
-            // BF16: the A chunk's BF16 copy in the A2 area, B in the B1 area; K = 16 per MMA
-            const uint32_t id = idesc_bf16(nmma);
-#pragma unroll
-            for (int ks = 0; ks < T3_KC / 16; ++ks) {
-              const uint32_t off = (uint32_t)ks * 256u;
-              mma_bf16(d, sdesc_bf16(a2 + off), sdesc_bf16(b1 + off), id, (kc > 0 || ks > 0) ? 1u : 0u);
-            }
+            mma_bf16(d, sdesc<T3_SBO_BF>(a1), sdesc<T3_SBO_BF>(b1), id, kc > 0 ? 1u : 0u);
           } else {
-            const uint32_t id = idesc_tf32(nmma);
+            const uint64_t da1 = sdesc<T3_SBO>(a1), da2 = sdesc<T3_SBO>(a1 + T3_AP);
+            const uint64_t db1 = sdesc<T3_SBO>(b1), db2 = sdesc<T3_SBO>(b1 + L::B);
 #pragma unroll
             for (int ks = 0; ks < T3_KC / 8; ++ks) {
-              const uint32_t off = (uint32_t)ks * 256u;
-              mma_tf32(d, sdesc(a1 + off), sdesc(b1 + off), id, (kc > 0 || ks > 0) ? 1u : 0u);
+              const uint64_t off = (uint64_t)ks * (256u >> 4);
+              mma_tf32(d, da1 + off, db1 + off, id, (kc > 0 || ks > 0) ? 1u : 0u);
               if (MODE == 1) {
-                mma_tf32(d, sdesc(a1 + off), sdesc(b2 + off), id, 1u);
-                mma_tf32(d, sdesc(a2 + off), sdesc(b1 + off), id, 1u);
+                mma_tf32(d, da1 + off, db2 + off, id, 1u);
+                mma_tf32(d, da2 + off, db1 + off, id, 1u);
               }
             }
           }
           mma_commit(empty + s);
           if (kc == T3_NCH - 1) mma_commit(accf + b);
         }
-        last_mma = ch;
         __syncwarp();
+        last_mma = t * T3_NCH + kc;
+        if (++s == ST) {
+          s = 0;
+          ph ^= 1;
+        }
       }
       if (!ok) {
         if (lane == 0) { *abort_flag = 1; atomicExch(err, 1); }
         break;
       }
     }
-  } else if (warp < T3_CONV_WARP0 + T3_CONV_WARPS) {
+  } else if (warp <= 2 * L::GW) {
     // ------------------------------------------------------------ converters
-    const int ct = tid - T3_CONV_WARP0 * 32;
+    const int g = (warp - 1) / L::GW, w = (warp - 1) % L::GW;   // chunks of parity g
+    const int cg = (w % (TW / 32)) * 32, k0 = (w / (TW / 32)) * 8;   // 32 columns, 8 rows of a chunk
+    const int gt = w * 32 + lane;
+    constexpr int UA = (int)(T3_AP / 16 + L::GW * 32 - 1) / (L::GW * 32);   // 16-byte units of H a thread
+    unsigned char* ring = sm + L::RING + (uint32_t)(g * L::DEPTH) * L::SLOT;
+    // the copies run DEPTH chunks of the group ahead, over the ends of items
+    int64_t ft = 0;
+    int fk = g, fs = 0, fcol = 0;
+    const float* fa = nullptr;
+    const float* fy = nullptr;
+    auto fetch = [&]() {
+      if (ft < my_items) {
+        if (fk < 2) {
+          const int64_t item = blockIdx.x + ft * gridDim.x;
+          const int64_t e = cells[item / ntiles];
+          const int c0 = (int)(item % ntiles) * TW, col = c0 + cg + (lane & 7) * 4;
+          fa = Ag + e * (int64_t)(T3_M * T3_K) + gt * 4;
+          fcol = col < min(N, c0 + TW);
+          fy = Y + cell_corner(m, e) * ldy + (fcol ? col : c0);
+        }
+        const uint32_t slot = su32(ring) + (uint32_t)fs * L::SLOT;
+#pragma unroll
+        for (int u = 0; u < UA; ++u)
+          if (gt + u * L::GW * 32 < (int)(T3_AP / 16))
+            cp16(slot + (uint32_t)(gt + u * L::GW * 32) * 16u, fa + fk * (T3_M * T3_KC) + u * L::GW * 128, true);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int k = fk * T3_KC + k0 + u * 4 + (lane >> 3);
+          cp16(slot + T3_AP + (uint32_t)w * 1024u + (uint32_t)(u * 32 + lane) * 16u, fy + (int64_t)lut[k] * ldy,
+               fcol && k < NL);
+        }
+        fk += 2;
+        if (fk >= T3_NCH) {
+          fk = g;
+          ++ft;
+        }
+        if (++fs == L::DEPTH) fs = 0;
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int i = 0; i < L::DEPTH; ++i) fetch();
+    int s = g, rs = 0;
+    uint32_t ph = 0;
     for (int64_t t = 0; t < my_items && !*abort_flag; ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % ntiles) * TW;
       const int ncol = min(TW, N - c0);
-      const int nmma = ((ncol + 15) / 16) * 16;
+      const int n = cg + lane;
+      const bool live = n < ((ncol + 15) / 16) * 16;
       bool ok = true;
-      for (int kc = 0; kc < T3_NCH; ++kc) {
-        const int64_t ch = t * T3_NCH + kc;
-        const int s = (int)(ch % T3_STAGES);
-        ok = bar_wait(full + s, (uint32_t)((ch / T3_STAGES) & 1));
-        if (!ok) break;
-        unsigned char* S = sm + s * T3Layout<TW>::STAGE;
-        const float* raw = reinterpret_cast<const float*>(S + 2 * T3Layout<TW>::A + 2 * T3Layout<TW>::B);
-        unsigned char* B1 = S + 2 * T3Layout<TW>::A;
-        unsigned char* B2 = B1 + T3Layout<TW>::B;
-        const int nrows = min(T3_KC, NL - kc * T3_KC);
-        if (MODE == 2) {
-          // BF16 copies: the A chunk (FP32 image, 4-wide K core matrices) into the A2
-          // area and the raw rows into the B1 area, both in the 8-wide K layout
-          unsigned char* A2 = S + T3Layout<TW>::A;
-          const float4* a1 = reinterpret_cast<const float4*>(S);
-          for (int v = ct; v < (int)(T3Layout<TW>::A / 16); v += T3_CONV_WARPS * 32) {
-            // 16-byte unit v of the FP32 image: row r, K quad kq (cmo layout)
-            const int rg = v >> 6, kq = (v >> 3) & 7, ri = v & 7;
-            const int r = rg * 8 + ri, k = kq * 4;
-            const float4 x = a1[v];
-            ushort4 h;
-            h.x = bf16r(x.x); h.y = bf16r(x.y); h.z = bf16r(x.z); h.w = bf16r(x.w);
-            *reinterpret_cast<ushort4*>(A2 + bmo(r, k)) = h;
-          }
-          for (int v = ct; v < nmma * 8; v += T3_CONV_WARPS * 32) {
-            const int n = v % nmma, kq = v / nmma;
-            ushort4 h;
-            uint16_t* hp = reinterpret_cast<uint16_t*>(&h);
+      for (int kc = g; kc < T3_NCH; kc += 2) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(L::DEPTH - 1) : "memory");
+        __syncwarp();
+        const unsigned char* slot = ring + (uint32_t)rs * L::SLOT;
+        const float* raw = reinterpret_cast<const float*>(slot + T3_AP + w * 1024) + lane;
+        float4 x[UA];
+        float y[2][4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int kr = kq * 4 + q;
-              hp[q] = bf16r((kr < nrows && n < ncol) ? raw[kr * TW + n] : 0.f);
-            }
-            *reinterpret_cast<ushort4*>(B1 + bmo(n, kq * 4)) = h;
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          bar_arrive(conv + s);
-          continue;
-        }
-        {
-          // the A chunk in place: A1 = TF32(A), A2 = TF32(A - A1) (elementwise, any layout)
-          float4* a1 = reinterpret_cast<float4*>(S);
-          float4* a2 = reinterpret_cast<float4*>(S + T3Layout<TW>::A);
-          for (int v = ct; v < (int)(T3Layout<TW>::A / 16); v += T3_CONV_WARPS * 32) {
-            const float4 x = a1[v];
+        for (int u = 0; u < UA; ++u)
+          if (gt + u * L::GW * 32 < (int)(T3_AP / 16)) x[u] = reinterpret_cast<const float4*>(slot)[gt + u * L::GW * 32];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) y[u][q] = n < ncol ? raw[(u * 4 + q) * 32] : 0.f;
+        __syncwarp();
+        fetch();   // into the slot just read
+        if (++rs == L::DEPTH) rs = 0;
+        if (t * T3_NCH + kc >= ST) ok = bar_wait(empty + s, ph ^ 1u);
+        if (!ok) break;
+        unsigned char* A1 = sm + (uint32_t)s * L::STAGE;
+        unsigned char* B1 = A1 + L::A;
+#pragma unroll
+        for (int u = 0; u < UA; ++u) {
+          const int v = gt + u * L::GW * 32;
+          if (v >= (int)(T3_AP / 16)) continue;
+          if (MODE == 2) {
+            // 16-byte unit v holds row 8 (v / 32) + v % 8, K quad (v / 8) % 4
+            ushort4 h;
+            h.x = bf16r(x[u].x); h.y = bf16r(x[u].y); h.z = bf16r(x[u].z); h.w = bf16r(x[u].w);
+            *reinterpret_cast<ushort4*>(A1 + bmo((v >> 5) * 8 + (v & 7), ((v >> 3) & 3) * 4)) = h;
+          } else {
             float4 h4;
-            h4.x = tf32r(x.x); h4.y = tf32r(x.y); h4.z = tf32r(x.z); h4.w = tf32r(x.w);
-            a1[v] = h4;
+            h4.x = tf32r(x[u].x); h4.y = tf32r(x[u].y); h4.z = tf32r(x[u].z); h4.w = tf32r(x[u].w);
+            reinterpret_cast<float4*>(A1)[v] = h4;
             if (MODE == 1) {
               float4 l4;
-              l4.x = tf32r(x.x - h4.x); l4.y = tf32r(x.y - h4.y); l4.z = tf32r(x.z - h4.z); l4.w = tf32r(x.w - h4.w);
-              a2[v] = l4;
+              l4.x = tf32r(x[u].x - h4.x); l4.y = tf32r(x[u].y - h4.y);
+              l4.z = tf32r(x[u].z - h4.z); l4.w = tf32r(x[u].w - h4.w);
+              reinterpret_cast<float4*>(A1 + T3_AP)[v] = l4;
             }
           }
         }
-        for (int v = ct; v < nmma * 8; v += T3_CONV_WARPS * 32) {
-          const int n = v % nmma, kq = v / nmma;
-          float y[4];
+        if (live) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int kr = kq * 4 + q;
-            y[q] = (kr < nrows && n < ncol) ? raw[kr * TW + n] : 0.f;
-          }
-          float4 h4, l4;
-          h4.x = tf32r(y[0]); h4.y = tf32r(y[1]); h4.z = tf32r(y[2]); h4.w = tf32r(y[3]);
-          *reinterpret_cast<float4*>(B1 + cmo(n, kq * 4)) = h4;
-          if (MODE == 1) {
-            l4.x = tf32r(y[0] - h4.x); l4.y = tf32r(y[1] - h4.y); l4.z = tf32r(y[2] - h4.z); l4.w = tf32r(y[3] - h4.w);
-            *reinterpret_cast<float4*>(B2 + cmo(n, kq * 4)) = l4;
+          for (int u = 0; u < 2; ++u) {
+            if (MODE == 2) {
+              ushort4 h;
+              h.x = bf16r(y[u][0]); h.y = bf16r(y[u][1]); h.z = bf16r(y[u][2]); h.w = bf16r(y[u][3]);
+              *reinterpret_cast<ushort4*>(B1 + bmo(n, k0 + u * 4)) = h;
+            } else {
+              float4 h4;
+              h4.x = tf32r(y[u][0]); h4.y = tf32r(y[u][1]); h4.z = tf32r(y[u][2]); h4.w = tf32r(y[u][3]);
+              *reinterpret_cast<float4*>(B1 + cmo(n, k0 + u * 4)) = h4;
+              if (MODE == 1) {
+                float4 l4;
+                l4.x = tf32r(y[u][0] - h4.x); l4.y = tf32r(y[u][1] - h4.y);
+                l4.z = tf32r(y[u][2] - h4.z); l4.w = tf32r(y[u][3] - h4.w);
+                *reinterpret_cast<float4*>(B1 + L::B + cmo(n, k0 + u * 4)) = l4;
+              }
+            }
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        bar_arrive(conv + s);
+        __syncwarp();
+        if (lane == 0) bar_arrive(conv + s);
+        s += 2;
+        if (s >= ST) {
+          s -= ST;
+          ph ^= 1;
+        }
       }
       if (!ok) {
         *abort_flag = 1;
@@ -377,28 +397,30 @@ __global__ void __launch_bounds__(T3_THREADS, 1) k_cell_tc3(const float* __restr
         break;
       }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   } else {
     // ------------------------------------------------------------ epilogue
-    const int ew = warp - T3_EPI_WARP0;  // 0..7
     const int quarter = warp & 3;         // TMEM lane quarter accessible to this warp
-    const int colgrp = ew >> 2;           // 0..1
-    const int r = quarter * 32 + lane;
+    const int sub = lane & 3;
     for (int64_t t = 0; t < my_items && !*abort_flag; ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int64_t e = cells[item / ntiles];
       const int c0 = (int)(item % ntiles) * TW;
       const int ncol = min(TW, N - c0);
       const int b = (int)(t & 1);
-      const int64_t g = (r < NL) ? cell_node(m, e, r) : 0;
-      float* wr = W + g * ldw + c0;
+      // after the exchange below this lane holds 16 bytes of each of the four rows of its lane quad
+      const int r0 = quarter * 32 + (lane & ~3);
+      float* wr = W + cell_corner(m, e) * ldw + c0;
+      int64_t ro[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) ro[i] = (int64_t)lut[r0 + i] * ldw;
       if (!bar_wait(accf + b, (uint32_t)((t / 2) & 1))) {
         *abort_flag = 1;
         atomicExch(err, 1);
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      for (int cb = colgrp * 16; cb < ncol; cb += 32) {
-        const bool full16 = (r < NL) && cb + 16 <= ncol;
+      for (int cb = 0; cb < ncol; cb += 16) {
         uint32_t v[16];
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -407,41 +429,50 @@ __global__ void __launch_bounds__(T3_THREADS, 1) k_cell_tc3(const float* __restr
             : "r"(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 256 + cb))
             : "memory");
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        // 4 x 4 exchange of 16-byte pieces between the lanes of a quad: v[4 i ..] becomes columns
+        // 4 sub .. of row r0 + i
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (i & o) continue;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t lo = v[4 * i + q], hi = v[4 * (i + o) + q];
+              const uint32_t got = __shfl_xor_sync(0xffffffffu, (sub & o) ? lo : hi, o);
+              v[4 * i + q] = (sub & o) ? got : lo;
+              v[4 * (i + o) + q] = (sub & o) ? hi : got;
+            }
+          }
         // the products are added in L2 (vector reductions, no read-back): a W value
         // receives one addition per launch (cells of a colour share no node)
-        if (r < NL) {
-          if (full16) {
+        const int c = cb + 4 * sub;
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-              asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(wr + cb + 4 * q),
-                           "f"(__uint_as_float(v[4 * q])), "f"(__uint_as_float(v[4 * q + 1])),
-                           "f"(__uint_as_float(v[4 * q + 2])), "f"(__uint_as_float(v[4 * q + 3]))
-                           : "memory");
+        for (int i = 0; i < 4; ++i) {
+          if (r0 + i >= NL) continue;
+          float* o = wr + ro[i] + c;
+          if (c + 4 <= ncol) {
+            asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(o),
+                         "f"(__uint_as_float(v[4 * i])), "f"(__uint_as_float(v[4 * i + 1])),
+                         "f"(__uint_as_float(v[4 * i + 2])), "f"(__uint_as_float(v[4 * i + 3]))
+                         : "memory");
           } else {
 #pragma unroll
-            for (int q = 0; q < 16; ++q)
-              if (cb + q < ncol) atomicAdd(wr + cb + q, __uint_as_float(v[q]));
+            for (int q = 0; q < 4; ++q)
+              if (c + q < ncol) atomicAdd(o + q, __uint_as_float(v[4 * i + q]));
           }
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      bar_arrive(acce + b);
+      __syncwarp();
+      if (lane == 0) bar_arrive(acce + b);
     }
   }
-  // all roles done.  After an abort, drain before the TMEM and the shared memory
-  // are released: every bulk copy issued into the stage ring lands (at most
-  // T3_STAGES chunks are in flight: the producer waits for a stage to empty
-  // before refilling it), and the last MMA commit (it covers every MMA this CTA
-  // issued) arrives; each drain wait is bounded like the pipeline's own.
+  // all roles done (the asynchronous copies have landed).  After an abort, drain before
+  // the TMEM is released: the last MMA commit (it covers every MMA this CTA issued)
+  // arrives; the drain wait is bounded like the pipeline's own.
   __syncthreads();
-  if (*abort_flag) {
-    if (warp == 0 && lane == 0 && last_copy >= 0) {
-      for (int64_t ch = last_copy - T3_STAGES + 1; ch <= last_copy; ++ch)
-        if (ch >= 0) bar_wait(full + (int)(ch % T3_STAGES), (uint32_t)((ch / T3_STAGES) & 1));
-    }
-    if (warp == 1 && lane == 0 && last_mma >= 0)
-      bar_wait(empty + (int)(last_mma % T3_STAGES), (uint32_t)((last_mma / T3_STAGES) & 1));
-  }
+  if (*abort_flag && warp == 0 && last_mma >= 0) bar_wait(empty + (int)(last_mma % ST), (uint32_t)((last_mma / ST) & 1));
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
@@ -450,34 +481,33 @@ __global__ void __launch_bounds__(T3_THREADS, 1) k_cell_tc3(const float* __restr
   }
 }
 
-// TF32 split images of H^cc_e, chunk-major: [cell][chunk][row group][1 KB], each
-// chunk a contiguous 16 KB image of the K-major core-matrix layout.
-// A1 = tf32(h), A2 = tf32(h - A1) (h in FP64).
+// FP32 images of H^cc_e, [cell][16-wide chunk], each in the K-major core-matrix layout
 __global__ void k_build_aimg(const double* __restrict__ Hcc, int64_t n_cell, float* __restrict__ A) {
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= n_cell * T3_M * T3_K) return;
-  const int64_t e = idx / (T3_M * T3_K);
-  const int rk = (int)(idx % (T3_M * T3_K));
-  const int r = rk / T3_K, k = rk % T3_K;
-  const double h = (r < NL && k < NL) ? Hcc[e * (int64_t)(NL * NL) + r * NL + k] : 0.0;
-  const int kc = k / T3_KC, kl = k % T3_KC;
-  const int64_t off = (e * T3_NCH + kc) * (T3_M * T3_KC) + (cmo(r, kl) + (uint32_t)(kl & 3) * 4u) / 4;
-  A[off] = (float)h;
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // (cell, row, K quad)
+  if (idx >= n_cell * T3_M * (T3_K / 4)) return;
+  const int64_t e = idx / (T3_M * (T3_K / 4));
+  const int r = (int)(idx / (T3_K / 4)) % T3_M, k = (int)(idx % (T3_K / 4)) * 4;
+  float h[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) h[q] = (r < NL && k + q < NL) ? (float)Hcc[e * (int64_t)(NL * NL) + r * NL + k + q] : 0.f;
+  unsigned char* o = reinterpret_cast<unsigned char*>(A) + (e * T3_NCH + k / T3_KC) * (int64_t)T3_AP + cmo(r, k % T3_KC);
+  *reinterpret_cast<float4*>(o) = make_float4(h[0], h[1], h[2], h[3]);
 }
 
 }  // namespace
 
-int64_t tc3_image_elems(int64_t n_cell) { return n_cell * T3_M * T3_K; }
+int64_t tc3_image_elems(int64_t n_cell) { return n_cell * T3_M * (int64_t)T3_K; }
 
 void launch_build_aimg(const double* Hcc, int64_t n_cell, float* A, cudaStream_t st) {
-  const int64_t n = n_cell * T3_M * T3_K;
-  if (n <= 0) return;
-  k_build_aimg<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(Hcc, n_cell, A);
-  g_launches.fetch_add(1, std::memory_order_relaxed);
+  const int64_t n = n_cell * T3_M * (T3_K / 4);
+  if (n > 0) {
+    k_build_aimg<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(Hcc, n_cell, A);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+  }
 }
 
 // W += H_e Y_e over the cells of one colour.  Y / W: FP32 rows, ld a multiple of 4
-// elements and rows 16-byte aligned (the bulk copies need 16-byte sizes and addresses).
+// elements and rows 16-byte aligned (the 16-byte copies and reductions).
 namespace {
 template <int TW>
 void tc3_launch(const float* A, const int32_t* cells, int64_t ncells, const MeshDev& m,
@@ -489,13 +519,13 @@ void tc3_launch(const float* A, const int32_t* cells, int64_t ncells, const Mesh
   const size_t smem = T3Layout<TW>::TOTAL;
   if (mode == 1) {
     cudaFuncSetAttribute(k_cell_tc3<1, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_cell_tc3<1, TW><<<grid, T3_THREADS, smem, st>>>(A, cells, ncells, m, Y, ldy, W, ldw, N, ntiles, err, stall);
+    k_cell_tc3<1, TW><<<grid, T3Layout<TW>::THREADS, smem, st>>>(A, cells, ncells, m, Y, ldy, W, ldw, N, ntiles, err, stall);
   } else if (mode == 2) {
     cudaFuncSetAttribute(k_cell_tc3<2, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_cell_tc3<2, TW><<<grid, T3_THREADS, smem, st>>>(A, cells, ncells, m, Y, ldy, W, ldw, N, ntiles, err, stall);
+    k_cell_tc3<2, TW><<<grid, T3Layout<TW>::THREADS, smem, st>>>(A, cells, ncells, m, Y, ldy, W, ldw, N, ntiles, err, stall);
   } else {
     cudaFuncSetAttribute(k_cell_tc3<0, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_cell_tc3<0, TW><<<grid, T3_THREADS, smem, st>>>(A, cells, ncells, m, Y, ldy, W, ldw, N, ntiles, err, stall);
+    k_cell_tc3<0, TW><<<grid, T3Layout<TW>::THREADS, smem, st>>>(A, cells, ncells, m, Y, ldy, W, ldw, N, ntiles, err, stall);
   }
 }
 }  // namespace

@@ -117,3 +117,28 @@ def test_network_at_tile_edges(dims, n):
     Xd = torch.from_numpy(X).cuda()
     assert rel_err(net.forward(Xd), y_ref) < 1e-4
     assert rel_err(net.backward(Xd, torch.from_numpy(dy).cuda()), g_ref) < 1e-4
+
+
+# tensor-core cell products of the FP32 filter at the edges of the 16-column groups, the
+# 160-column tile and the stage ring (one CTA walks every item; one item a CTA): one degree
+# against the oracle at the operand's round-off times the cancellation factor (as in the
+# ordinary case: 2^-11, 2^-24 and 2^-8 give 3e-3, 1e-5 and 3e-2)
+@pytest.mark.parametrize("prec,tol", [("tf32", 3e-3), ("tf32x3", 1e-5), ("bf16", 3e-2)])
+@pytest.mark.parametrize("N", [1, 5, 15, 16, 33, 64, 65, 96, 159, 160, 161])
+def test_split_cell_tiles(tiny_pair, prec, tol, N):
+    from oracle.chfsi import chebyshev_filter_scaled, lanczos_upper_bound
+    d, G = tiny_pair
+    X = W.random_block(d.system, N, seed=800 + N)
+    b = 1.05 * lanczos_upper_bound(d.apply_Htilde, d.apply_M_assembled, W.lanczos_start(d.system), 10)
+    ref = chebyshev_filter_scaled(d.apply_Htilde, X, 1, 0.2 * b, b, -1.0)
+    out = []
+    for cap in (0, 1):
+        G.set_grid_cap(cap)
+        try:
+            Xd = to_dev(X)
+            G.chfsi_step(Xd, 1, 0.2 * b, b, -1.0, precision=prec, fp64_tail=0)
+        finally:
+            G.set_grid_cap(0)
+        out.append(Xd)
+    assert rel_err(out[0], ref) < tol
+    assert torch.equal(out[0], out[1])
