@@ -89,6 +89,9 @@ struct efe_handle {
   int64_t *seg_start = nullptr, *seg_end = nullptr, *row_seg_ptr = nullptr;
   int64_t n_tn = 0;
   int32_t* t_nodes = nullptr;
+  float* tnD = nullptr;            // D^-1 of the pattern nodes
+  int32_t* rest_nodes = nullptr;   // the nodes outside the pattern
+  int64_t n_rest = 0;
   int64_t* t_ptr = nullptr;
   int32_t* t_col = nullptr;
   int64_t* t_perm = nullptr;
@@ -729,22 +732,24 @@ int degree_f32(efe_handle* h, const float* Yc, const double* Yce, const float* Y
   h->time_this = true;
   TRY(cell_apply_all<float>(h, h->Hcc32, Yc, ld, h->Wf, ld, N, st, h->tc_mode != 0));
   h->time_this = false;
+  const bool tiles = h->nE > 0 && coup_tiles_fit(h, N);
   if (h->nE > 0) {
     const int nE = (int)h->nE;
-    if (coup_tiles_fit(h, N)) {
-      launch_coup_cols<float>(h->n_tn, h->ncb_cols, h->cb_cta_cols, h->t_nodes, h->cb_slot_off, h->cb_slots, h->tileH, 1.f, Yce, N, nE,
-                              N, h->Wf, ld, st);
-      launch_coup_rows<float>(h->n_tn, h->ncb, h->cb_cta, h->t_nodes, h->cb_slot_off, h->cb_slots, h->tileH, nullptr, Yc, ld,
-                              nE, N, h->cpart, st);
+    if (tiles) {
+      const CombArgs comb{h->tnD, Yc, Yp, Yn, coef};
+      launch_coup_cols(h->n_tn, h->ncb_cols, h->cb_cta_cols, h->t_nodes, h->cb_slot_off, h->cb_slots, h->tileH, 1.f, Yce, N, nE,
+                       N, h->Wf, ld, st);
+      launch_coup_rows(h->n_tn, h->ncb, h->cb_cta, h->t_nodes, h->cb_slot_off, h->cb_slots, h->tileH, nullptr, Yc, ld,
+                       nE, N, h->cpart, st);
       launch_coup_reduce(h->ncb, nE, N, h->cpart, 1.0, nullptr, 0, 0.0, We, N, st);
       launch_gemm_nn(nE, N, nE, 1.0, h->Hee, nE, Yce, N, 1.0, We, N, st);
       // block-wise inverse: r = We - M^ec D^-1 Wc, x_e = S^-1 r, Wc -= M^ec^T x_e
-      launch_coup_rows<float>(h->n_tn, h->ncb, h->cb_cta, h->t_nodes, h->cb_slot_off, h->cb_slots, h->tileM, h->Dinv, h->Wf,
-                              ld, nE, N, h->cpart, st);
+      launch_coup_rows(h->n_tn, h->ncb, h->cb_cta, h->t_nodes, h->cb_slot_off, h->cb_slots, h->tileM, h->tnD, h->Wf,
+                       ld, nE, N, h->cpart, st);
       launch_coup_reduce(h->ncb, nE, N, h->cpart, -1.0, We, N, 1.0, h->rb, N, st);
       launch_gemm_nn(nE, N, nE, 1.0, h->Sinv, nE, h->rb, N, 0.0, h->xe, N, st);
-      launch_coup_cols<float>(h->n_tn, h->ncb_cols, h->cb_cta_cols, h->t_nodes, h->cb_slot_off, h->cb_slots, h->tileM, -1.f, h->xe, N,
-                              nE, N, h->Wf, ld, st);
+      launch_coup_cols(h->n_tn, h->ncb_cols, h->cb_cta_cols, h->t_nodes, h->cb_slot_off, h->cb_slots, h->tileM, -1.f, h->xe, N,
+                       nE, N, h->Wf, ld, st, &comb);
     } else {
       // many enrichment functions: node-major FP32 columns products, grouped
       // FP32 rows products with FP64 partial sums, FP64 n_E x n_E products
@@ -771,7 +776,9 @@ int degree_f32(efe_handle* h, const float* Yc, const double* Yce, const float* Y
       CKL();
     }
   }
-  launch_cheb_combine_f4(nn, ld, h->Dinv, h->Wf, Yc, Yp, Yn, coef, st);
+  // the combine of the pattern rows went with the last columns product
+  if (tiles) launch_cheb_combine_f4(h->n_rest, ld, h->rest_nodes, h->Dinv, h->Wf, Yc, Yp, Yn, coef, st);
+  else launch_cheb_combine_f4(nn, ld, nullptr, h->Dinv, h->Wf, Yc, Yp, Yn, coef, st);
   if (h->nE > 0) launch_cheb_combine<double>(h->nE, nullptr, h->xe, N, Yce, N, Ype, N, Yne, N, coef, N, st);
   CKL();
   return EFE_OK;
@@ -1329,6 +1336,20 @@ int efe_create(const efe_mesh_desc* mesh, const efe_atoms_desc* atoms, const efe
     }
     h->n_tn = (int64_t)s.t_nodes.size();
     TRY(upload(h, &h->t_nodes, s.t_nodes));
+    {
+      std::vector<float> td(s.t_nodes.size());
+      std::vector<char> in(h->n_nodes, 0);
+      for (size_t i = 0; i < td.size(); ++i) {
+        td[i] = (float)s.Dinv[s.t_nodes[i]];
+        in[s.t_nodes[i]] = 1;
+      }
+      std::vector<int32_t> rest;
+      for (int64_t g = 0; g < h->n_nodes; ++g)
+        if (!in[g]) rest.push_back((int32_t)g);
+      h->n_rest = (int64_t)rest.size();
+      TRY(upload(h, &h->tnD, td));
+      TRY(upload(h, &h->rest_nodes, rest));
+    }
     TRY(upload(h, &h->t_ptr, s.t_ptr));
     TRY(upload(h, &h->t_col, s.t_col));
     TRY(upload(h, &h->t_perm, s.t_perm));

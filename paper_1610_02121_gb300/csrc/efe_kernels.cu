@@ -644,116 +644,169 @@ __global__ void k_tile_scatter(int64_t nnz, const int64_t* __restrict__ pos, con
 }
 
 // Rows product: part[b][a][c] = sum over the blocks of CTA b of
-//   sum_u tile[slot][u] * scale[g_u] * X[g_u][c]  accumulated at a = f(slot),
+//   sum_u tile[slot][u] * tscale[u] * X[g_u][c]  accumulated at a = f(slot),
 // in a CTA-private (n_E x N) shared-memory array.  CTA b takes the blocks
-// cta_blk[b] .. cta_blk[b + 1] (a one-wave partition balanced by slot count).
-// Shared rows are padded to a multiple of four floats so that every thread
-// reads and updates its four columns with one 16-byte access.
-template <typename T>
-__global__ void __launch_bounds__(256) k_coup_rows(int64_t n_tn, const int64_t* __restrict__ cta_blk,
-                                                   const int32_t* __restrict__ t_nodes,
-                                                   const int64_t* __restrict__ slot_off,
-                                                   const int32_t* __restrict__ slots, const float* __restrict__ tile,
-                                                   const double* __restrict__ scale, const T* __restrict__ X,
-                                                   int64_t ldx, int nE, int N, float* __restrict__ part) {
+// cta_blk[b] .. cta_blk[b + 1] (a one-wave partition balanced by slot count; the partition
+// fixes the order of the FP32 sums).  X: FP32 rows, ldx a multiple of four, zero past N.
+// A block is a chain of dependent loads (node ids, rows, tile) and a short product, so its
+// latency bounds the kernel, then DRAM: UX 16-byte pieces of the next block's rows, its tile
+// and the ids of the one after that are held in registers a block ahead (UX = 0: blocks wider
+// than 160 columns, loaded when needed); a thread takes 2 slots x 4 columns, so that few
+// slots still keep every warp busy.  Before -> now: 47 k pattern nodes x 12 columns 17.4 ->
+// 10.3 us, 612 k x 135 349 -> 247 us.
+template <int UX>
+__global__ void __launch_bounds__(256, 3) k_coup_rows(int64_t n_tn, const int64_t* __restrict__ cta_blk,
+                                                      const int32_t* __restrict__ t_nodes,
+                                                      const int64_t* __restrict__ slot_off,
+                                                      const int32_t* __restrict__ slots, const float* __restrict__ tile,
+                                                      const float* __restrict__ tscale, const float* __restrict__ X,
+                                                      int64_t ldx, int nE, int N, float* __restrict__ part) {
   extern __shared__ __align__(16) float smf[];
-  const int ldy = (N + 3) & ~3;
+  const int ldy = (N + 3) & ~3, q4 = ldy / 4;
   float* acc = smf;                                  // nE x ldy
   float* Ys = acc + (size_t)nE * ldy;                // CPB x ldy
   float* Ps = Ys + CPB * ldy;                        // CPF x CPB
   __shared__ int sf[CPF];
-  const int tid = threadIdx.x, bd = blockDim.x;
-  for (int i = tid; i < nE * ldy; i += bd) acc[i] = 0.f;
+  const int tid = threadIdx.x;
+  constexpr int UR = UX > 0 ? UX : 1;
+  for (int i = tid; i < nE * ldy; i += 256) acc[i] = 0.f;
   const int64_t b0 = cta_blk[blockIdx.x], b1 = cta_blk[blockIdx.x + 1];
-  const int ncb = ldy / 4;
-  for (int64_t bb = b0; bb < b1; ++bb) {
-    const int64_t r0 = bb * CPB;
-    const int nb = (int)min((int64_t)CPB, n_tn - r0);
-    __syncthreads();
-    if (sizeof(T) == 4 && (ldx & 3) == 0 && ((uintptr_t)X & 15) == 0 && ldy <= ldx) {
-      // padded FP32 rows: four columns per 16-byte load (columns past N are zero)
-      const int q4 = ldy / 4;
-      for (int i = tid; i < CPB * q4; i += bd) {
-        const int u = i / q4, c4 = i % q4;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (u < nb) {
-          const int64_t g = t_nodes[r0 + u];
-          v = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(X) + g * ldx + 4 * c4);
-          if (scale) {
-            const float sc = (float)scale[g];
-            v.x *= sc; v.y *= sc; v.z *= sc; v.w *= sc;
-          }
-        }
-        *reinterpret_cast<float4*>(Ys + u * ldy + 4 * c4) = v;
-      }
-    } else {
-      for (int i = tid; i < CPB * ldy; i += bd) {
-        const int u = i / ldy, c = i % ldy;
-        float v = 0.f;
-        if (u < nb && c < N) {
-          const int64_t g = t_nodes[r0 + u];
-          v = (float)X[g * ldx + c];
-          if (scale) v *= (float)scale[g];
-        }
-        Ys[i] = v;
-      }
-    }
-    const int64_t s0 = slot_off[bb], s1 = slot_off[bb + 1];
-    for (int64_t sp = s0; sp < s1; sp += CPF) {
-      const int nf = (int)min((int64_t)CPF, s1 - sp);
-      __syncthreads();
-      for (int i = tid; i < CPF * CPB; i += bd) Ps[i] = (i < nf * CPB) ? tile[sp * CPB + i] : 0.f;
-      if (tid < nf) sf[tid] = slots[sp + tid];
-      __syncthreads();
-      const int nsb = (nf + 3) / 4;
-      for (int t = tid; t < nsb * ncb; t += bd) {
-        const int sb = t / ncb, cb = t % ncb;
-        float r[4][4] = {};
-#pragma unroll 8
-        for (int u = 0; u < CPB; ++u) {
-          float pv[4];
+  int pk[UR];                // this thread's pieces: node of the block (CPB: none), first column
 #pragma unroll
-          for (int i = 0; i < 4; ++i) pv[i] = Ps[(sb * 4 + i) * CPB + u];
-          const float4 y4 = *reinterpret_cast<const float4*>(Ys + u * ldy + cb * 4);
+  for (int u = 0; u < UR; ++u) {
+    const int i = tid + u * 256;
+    pk[u] = min(i / q4, CPB) << 16 | (i % q4) * 4;
+  }
+  auto un = [&](int u) { return pk[u] >> 16; };
+  auto uc = [&](int u) { return pk[u] & 0xffff; };
+  int32_t pg[UR];            // node ids, two blocks ahead
+  float4 px[UR], pt[2];      // rows and tile, one block ahead
+  float ps[UR];
+  int pf = 0;
+  auto piece = [&](int64_t bb, int u) { return un(u) < CPB && bb * CPB + un(u) < n_tn; };
+  auto ids = [&](int64_t bb) {
+#pragma unroll
+    for (int u = 0; u < UX; ++u) pg[u] = bb < b1 && piece(bb, u) ? t_nodes[bb * CPB + un(u)] : 0;
+  };
+  auto ahead = [&](int64_t bb) {
+#pragma unroll
+    for (int u = 0; u < UX; ++u) {
+      const bool in = piece(bb, u);
+      px[u] = in ? *reinterpret_cast<const float4*>(X + pg[u] * ldx + uc(u)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      ps[u] = in && tscale ? tscale[bb * CPB + un(u)] : 1.f;
+    }
+    const int64_t s0 = slot_off[bb];
+    const int nf = (int)min((int64_t)CPF, slot_off[bb + 1] - s0);
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const int i = tid + v * 256;
+      pt[v] = i < nf * (CPB / 4) ? reinterpret_cast<const float4*>(tile + s0 * CPB)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (tid < nf) pf = slots[s0 + tid];
+    ids(bb + 1);
+  };
+  auto product = [&](int nf) {
+    const int total = (nf + 1) / 2 * q4;
+    for (int t = tid; t < total; t += 256) {
+      const int sb = t / q4, cb = t % q4;
+      float r[2][4] = {};
+      const float* yp = Ys + cb * 4;
+#pragma unroll 4
+      for (int u = 0; u < CPB; u += 4) {
+        const float4 p0 = *reinterpret_cast<const float4*>(Ps + (2 * sb) * CPB + u);
+        const float4 p1 = *reinterpret_cast<const float4*>(Ps + (2 * sb + 1) * CPB + u);
+        const float pa[4] = {p0.x, p0.y, p0.z, p0.w}, pb[4] = {p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 y4 = *reinterpret_cast<const float4*>(yp + (u + k) * ldy);
           const float yv[4] = {y4.x, y4.y, y4.z, y4.w};
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) r[i][j] = fmaf(pv[i], yv[j], r[i][j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int sl = sb * 4 + i;
-          if (sl >= nf) break;
-          float4* ar = reinterpret_cast<float4*>(acc + (size_t)sf[sl] * ldy + cb * 4);
-          float4 a4 = *ar;
-          a4.x += r[i][0];
-          a4.y += r[i][1];
-          a4.z += r[i][2];
-          a4.w += r[i][3];
-          *ar = a4;
+          for (int j = 0; j < 4; ++j) {
+            r[0][j] = fmaf(pa[k], yv[j], r[0][j]);
+            r[1][j] = fmaf(pb[k], yv[j], r[1][j]);
+          }
         }
       }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (sb * 2 + i >= nf) break;
+        float4* ar = reinterpret_cast<float4*>(acc + (size_t)sf[sb * 2 + i] * ldy + cb * 4);
+        float4 a4 = *ar;
+        a4.x += r[i][0];
+        a4.y += r[i][1];
+        a4.z += r[i][2];
+        a4.w += r[i][3];
+        *ar = a4;
+      }
+    }
+  };
+  if (b0 < b1) {
+    ids(b0);
+    ahead(b0);
+  }
+  for (int64_t bb = b0; bb < b1; ++bb) {
+    const int64_t s0 = slot_off[bb], s1 = slot_off[bb + 1];
+    __syncthreads();
+    if (UX > 0) {
+#pragma unroll
+      for (int u = 0; u < UX; ++u) {
+        if (un(u) >= CPB) continue;
+        float4 v = px[u];
+        v.x *= ps[u]; v.y *= ps[u]; v.z *= ps[u]; v.w *= ps[u];
+        *reinterpret_cast<float4*>(Ys + un(u) * ldy + uc(u)) = v;
+      }
+    } else {
+      for (int i = tid; i < CPB * q4; i += 256) {
+        const int u = i / q4, c = (i % q4) * 4;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (bb * CPB + u < n_tn) {
+          v = *reinterpret_cast<const float4*>(X + t_nodes[bb * CPB + u] * ldx + c);
+          const float sc = tscale ? tscale[bb * CPB + u] : 1.f;
+          v.x *= sc; v.y *= sc; v.z *= sc; v.w *= sc;
+        }
+        *reinterpret_cast<float4*>(Ys + u * ldy + c) = v;
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 2; ++v) reinterpret_cast<float4*>(Ps)[tid + v * 256] = pt[v];
+    if (tid < CPF) sf[tid] = pf;
+    __syncthreads();
+    if (bb + 1 < b1) ahead(bb + 1);
+    product((int)min((int64_t)CPF, s1 - s0));
+    for (int64_t sp = s0 + CPF; sp < s1; sp += CPF) {
+      const int nf = (int)min((int64_t)CPF, s1 - sp);
+      __syncthreads();
+      for (int i = tid; i < CPF * CPB; i += 256) Ps[i] = (i < nf * CPB) ? tile[sp * CPB + i] : 0.f;
+      if (tid < nf) sf[tid] = slots[sp + tid];
+      __syncthreads();
+      product(nf);
     }
   }
   __syncthreads();
   float* Pp = part + (int64_t)blockIdx.x * nE * N;
-  for (int i = tid; i < nE * N; i += bd) Pp[i] = acc[(i / N) * ldy + i % N];
+  for (int i = tid; i < nE * N; i += 256) Pp[i] = acc[(i / N) * ldy + i % N];
 }
 
 // out[a][c] = alpha_base * base[a][c] + sgn * sum_b part[b][a][c]  (fixed order, FP64).
-// A block takes 32 consecutive outputs; its 8 thread rows sum the partials
-// b = y, y + 8, ... and the 8 row sums are added in order.
-__global__ void __launch_bounds__(256) k_coup_reduce(int nb, int nE, int N, const float* __restrict__ part,
-                                                     double sgn, const double* __restrict__ base, int64_t ldb,
-                                                     double alpha_base, double* __restrict__ out, int64_t ldo) {
-  __shared__ double rs[8][33];
-  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
-  const int64_t idx = blockIdx.x * 32LL + x;
+// A block takes CRED consecutive outputs; its 8 thread rows sum the partials
+// b = y, y + 8, ... and the 8 row sums are added in order.  The FP64 pipe (a conversion
+// and an addition a partial, 16 cycles a warp each) and the chain of loads bound it, so
+// the outputs go to many CTAs of two warps, with eight loads in flight: 456 partials of
+// 120 outputs 13.5 -> 10.9 us.  (32 thread rows would add in another order, which the
+// inverse Schur complement and the FP32 rounding after it turn into other bits.)
+constexpr int CRED = 8;
+__global__ void __launch_bounds__(8 * CRED) k_coup_reduce(int nb, int nE, int N, const float* __restrict__ part,
+                                                         double sgn, const double* __restrict__ base, int64_t ldb,
+                                                         double alpha_base, double* __restrict__ out, int64_t ldo) {
+  __shared__ double rs[8][CRED + 1];
+  const int x = threadIdx.x % CRED, y = threadIdx.x / CRED;
+  const int64_t idx = blockIdx.x * (int64_t)CRED + x;
   const int64_t tot = (int64_t)nE * N;
   double s = 0.0;
-  if (idx < tot)
+  if (idx < tot) {
+#pragma unroll 8
     for (int b = y; b < nb; b += 8) s += (double)part[(int64_t)b * tot + idx];
+  }
   rs[y][x] = s;
   __syncthreads();
   if (y == 0 && idx < tot) {
@@ -1102,109 +1155,122 @@ __global__ void __launch_bounds__(CX * GRP_KMAX) k_grp_rows_df(const int4* __res
   if (k < kg && c < N) part[((int64_t)blockIdx.x * GRP_KMAX + k) * N + c] = df_f2d(S) + df_f2d(C);
 }
 
-// Columns product: W[g_u][c] += sgn * sum_slot tile[slot][u] * Xe[f(slot)][c]
-// (Xe staged in shared memory as FP32, rows padded to four floats), same block
-// tiles and CTA partition as the rows product.
-template <typename T>
-__global__ void __launch_bounds__(256) k_coup_cols(int64_t n_tn, const int64_t* __restrict__ cta_blk,
-                                                   const int32_t* __restrict__ t_nodes,
-                                                   const int64_t* __restrict__ slot_off,
-                                                   const int32_t* __restrict__ slots, const float* __restrict__ tile,
-                                                   float sgn, const double* __restrict__ Xe, int64_t ldxe, int nE,
-                                                   int N, T* __restrict__ W, int64_t ldw) {
+// one 4-column piece of the Chebyshev combine (the same expressions in both kernels below)
+__device__ __forceinline__ float4 comb4(float4 x, float4 y, float sc, float alpha, float cc) {
+  float4 o;
+  o.x = alpha * (sc * x.x - cc * y.x);
+  o.y = alpha * (sc * x.y - cc * y.y);
+  o.z = alpha * (sc * x.z - cc * y.z);
+  o.w = alpha * (sc * x.w - cc * y.w);
+  return o;
+}
+
+// Columns product: w = W[g_u][c] + sgn * sum_slot tile[slot][u] * Xe[f(slot)][c] over the
+// pattern nodes (Xe staged in shared memory as FP32, rows padded to four floats); w goes back
+// to W, or (COMB) is the x of the degree's Chebyshev combine, whose result goes to Yn.
+// W, Yc, Yp, Yn: FP32 rows, ldw a multiple of four.
+// DRAM bounds it (the rows of W, and of Yc, Yp and Yn, once each) if enough of them are in
+// flight: a thread takes 4 nodes x 4 columns at a time, loads W before the slot loop, reads
+// the tile through L1 (the lanes of a warp share its entries) and never waits for another
+// thread.  Combining here saves writing W and reading it back.  612 k pattern nodes x 135
+// columns: 520 us and 535 us for the combine of all 1.87 M nodes before -> 240 us, or 357 us
+// with the combine and 384 us for the other nodes.
+template <bool COMB>
+__global__ void __launch_bounds__(512, 2) k_coup_cols(int64_t n_tn, const int64_t* __restrict__ cta_blk,
+                                                      const int32_t* __restrict__ t_nodes,
+                                                      const int64_t* __restrict__ slot_off,
+                                                      const int32_t* __restrict__ slots, const float* __restrict__ tile,
+                                                      float sgn, const double* __restrict__ Xe, int64_t ldxe, int nE,
+                                                      int N, float* __restrict__ W, int64_t ldw,
+                                                      const float* __restrict__ tscale, const float* __restrict__ Yc,
+                                                      const float* Yp, float* Yn, const double* __restrict__ coef) {
   extern __shared__ __align__(16) float smf[];
   const int ldx = (N + 3) & ~3;
   float* xs = smf;                                   // nE x ldx
-  float* Ps = xs + (size_t)nE * ldx;                 // CPF x CPB
-  __shared__ int sf[CPF];
-  __shared__ int64_t sg[CPB];
-  const int tid = threadIdx.x, bd = blockDim.x;
-  for (int i = tid; i < nE * ldx; i += bd) {
+  const int tid = threadIdx.x;
+  for (int i = tid; i < nE * ldx; i += 512) {
     const int a = i / ldx, c = i % ldx;
     xs[i] = c < N ? (float)Xe[(int64_t)a * ldxe + c] : 0.f;
   }
+  __syncthreads();
   const int64_t b0 = cta_blk[blockIdx.x], b1 = cta_blk[blockIdx.x + 1];
-  const int ncb = ldx / 4;
-  for (int64_t bb = b0; bb < b1; ++bb) {
-    const int64_t r0 = bb * CPB;
-    const int nb = (int)min((int64_t)CPB, n_tn - r0);
-    const int64_t s0 = slot_off[bb], s1 = slot_off[bb + 1];
-    // thread t owns output tiles (4 nodes x 4 columns) t and t + bd of each group of
-    // 2 bd tiles; results summed over the slot passes
-    const int ntile = (CPB / 4) * ncb;
-    __syncthreads();
-    if (tid < nb) sg[tid] = t_nodes[r0 + tid];
-    for (int tg = 0; tg < ntile; tg += 2 * bd) {
-      float r[2][4][4] = {};
-      for (int64_t sp = s0; sp < s1; sp += CPF) {
-        const int nf = (int)min((int64_t)CPF, s1 - sp);
-        __syncthreads();
-        for (int i = tid; i < CPF * CPB; i += bd) Ps[i] = (i < nf * CPB) ? tile[sp * CPB + i] : 0.f;
-        if (tid < nf) sf[tid] = slots[sp + tid];
-        __syncthreads();
-        for (int k = 0; k < 2; ++k) {
-          const int t = tg + tid + k * bd;
-          if (t >= ntile) break;
-          const int ub = t / ncb, cb = t % ncb;
-          for (int sl = 0; sl < nf; ++sl) {
-            const float4 x4 = *reinterpret_cast<const float4*>(xs + (size_t)sf[sl] * ldx + cb * 4);
-            const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
-            const float4 p4 = *reinterpret_cast<const float4*>(Ps + sl * CPB + ub * 4);
-            const float pv[4] = {p4.x, p4.y, p4.z, p4.w};
+  const int ncb = ldx / 4, ntile = (CPB / 4) * ncb;
+  float alpha = 0.f, cc = 0.f, beta = 0.f;
+  if (COMB) {
+    alpha = (float)coef[0];
+    cc = (float)coef[1];
+    beta = (float)coef[2];
+  }
+  for (int64_t w = tid; w < (b1 - b0) * ntile; w += 512) {
+    const int64_t bb = b0 + w / ntile;
+    const int t = (int)(w % ntile), ub = t / ncb, cb = (t % ncb) * 4;
+    const int64_t n0 = bb * CPB + ub * 4;
+    const int nu = (int)min((int64_t)4, n_tn - n0);
+    if (nu <= 0) continue;
+    int32_t g[4];
+    float4 o[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i) g[i] = t_nodes[n0 + min(i, nu - 1)];
 #pragma unroll
-              for (int j = 0; j < 4; ++j) r[k][i][j] = fmaf(pv[i], xv[j], r[k][i][j]);
-          }
+    for (int i = 0; i < 4; ++i) o[i] = *reinterpret_cast<const float4*>(W + g[i] * ldw + cb);
+    const int64_t s0 = slot_off[bb];
+    const int ns = (int)(slot_off[bb + 1] - s0);
+    const float4* tp = reinterpret_cast<const float4*>(tile + s0 * CPB) + ub;
+    float r[4][4] = {};
+#pragma unroll 2
+    for (int sl = 0; sl < ns; ++sl) {
+      const float4 x4 = *reinterpret_cast<const float4*>(xs + (size_t)slots[s0 + sl] * ldx + cb);
+      const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
+      const float4 p4 = tp[sl * (CPB / 4)];
+      const float pv[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) r[i][j] = fmaf(pv[i], xv[j], r[i][j]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i >= nu) break;
+      o[i].x += sgn * r[i][0];
+      o[i].y += sgn * r[i][1];
+      o[i].z += sgn * r[i][2];
+      o[i].w += sgn * r[i][3];
+      const int64_t at = g[i] * ldw + cb;
+      if (COMB) {
+        o[i] = comb4(o[i], *reinterpret_cast<const float4*>(Yc + at), tscale[n0 + i], alpha, cc);
+        if (Yp) {
+          const float4 p = *reinterpret_cast<const float4*>(Yp + at);
+          o[i].x += beta * p.x;
+          o[i].y += beta * p.y;
+          o[i].z += beta * p.z;
+          o[i].w += beta * p.w;
         }
-      }
-      for (int k = 0; k < 2; ++k) {
-        const int t = tg + tid + k * bd;
-        if (t >= ntile) break;
-        const int ub = t / ncb, cb = t % ncb;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int u = ub * 4 + i;
-          if (u >= nb) break;
-          T* wr = W + sg[u] * ldw + cb * 4;
-          if (sizeof(T) == 4 && (ldw & 3) == 0 && ((uintptr_t)W & 15) == 0 && cb * 4 + 4 <= ldw) {
-            // padded FP32 rows: one 16-byte update (columns past N add zero)
-            float4* w4 = reinterpret_cast<float4*>(wr);
-            float4 o = *w4;
-            o.x += sgn * r[k][i][0];
-            o.y += sgn * r[k][i][1];
-            o.z += sgn * r[k][i][2];
-            o.w += sgn * r[k][i][3];
-            *w4 = o;
-          } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              if (cb * 4 + j < N) wr[j] = (T)((float)wr[j] + sgn * r[k][i][j]);
-          }
-        }
+        *reinterpret_cast<float4*>(Yn + at) = o[i];
+      } else {
+        *reinterpret_cast<float4*>(W + at) = o[i];
       }
     }
   }
 }
 
 // Chebyshev combine on 16-byte aligned FP32 rows (ld multiple of 4): four columns per thread.
-// as k_cheb_combine: Yn may be Yp.  X (the cell-product output of this degree)
-// is zeroed after it is read, ready to accumulate the next degree's products.
-__global__ void k_cheb_combine_f4(int64_t nrows, int ld4, const double* __restrict__ rowscale,
+// as k_cheb_combine: Yn may be Yp.  rows: the rows to do (null: all of them).
+__global__ void k_cheb_combine_f4(int64_t nrows, int ld4, const int32_t* __restrict__ rows,
+                                  const double* __restrict__ rowscale,
                                   const float4* __restrict__ X, const float4* __restrict__ Yc,
                                   const float4* Yp, float4* Yn,
                                   const double* __restrict__ coef) {
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= nrows * ld4) return;
   const float alpha = (float)coef[0], cc = (float)coef[1], beta = (float)coef[2];
-  const int64_t r = idx / ld4;
+  int64_t r = idx / ld4;
+  if (rows) {
+    const int c4 = (int)(idx - r * ld4);
+    r = rows[r];
+    idx = r * ld4 + c4;
+  }
   const float sc = rowscale ? (float)rowscale[r] : 1.f;
-  const float4 x = X[idx], y = Yc[idx];
-  float4 o;
-  o.x = alpha * (sc * x.x - cc * y.x);
-  o.y = alpha * (sc * x.y - cc * y.y);
-  o.z = alpha * (sc * x.z - cc * y.z);
-  o.w = alpha * (sc * x.w - cc * y.w);
+  float4 o = comb4(X[idx], Yc[idx], sc, alpha, cc);
   if (Yp) {
     const float4 p = Yp[idx];
     o.x += beta * p.x;
@@ -2090,23 +2156,27 @@ int coup_block_nodes() { return CPB; }
 // kernel's CPB x (N + 4) vector tile and one CPF x CPB pattern tile
 size_t coup_smem(int nE, int N, bool rows) {
   const size_t ld = (size_t)((N + 3) & ~3);
-  return sizeof(float) * ((size_t)nE * ld + (rows ? (size_t)CPB * ld : 0) + (size_t)CPF * CPB);
+  return sizeof(float) * ((size_t)nE * ld + (rows ? (size_t)CPB * ld + (size_t)CPF * CPB : 0));
 }
 
-// CTAs of the rows (or columns) product resident at once (one wave of its partition)
+// CTAs of the rows (or columns) product resident at once (one wave of its partition).
+// Rows: three to an SM if the shared memory holds them (1,280 bytes of each are static or
+// the system's), by rule and not by the compiled kernel's registers, because the partition
+// fixes the order of the rows product's FP32 sums.
 int coup_resident_ctas(int nE, int N, int n_sm, bool rows) {
   const size_t smem = coup_smem(nE, N, rows);
   int per_sm = 0;
-  cudaError_t e;
   if (rows) {
-    cudaFuncSetAttribute(k_coup_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coup_rows<float>, 256, smem);
+    int dev = 0, sm_bytes = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess)
+      sm_bytes = 0;
+    per_sm = (int)std::min<size_t>(3, (size_t)sm_bytes / (smem + 1280));
   } else {
-    cudaFuncSetAttribute(k_coup_cols<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coup_cols<float>, 256, smem);
+    cudaFuncSetAttribute(k_coup_cols<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coup_cols<true>, 512, smem) != cudaSuccess) per_sm = 1;
   }
-  if (e != cudaSuccess || per_sm < 1) per_sm = 1;
-  return per_sm * n_sm;
+  return std::max(1, per_sm) * n_sm;
 }
 
 void launch_tile_scatter(int64_t nnz, const int64_t* pos, const float* val, float* tile, cudaStream_t st) {
@@ -2115,42 +2185,45 @@ void launch_tile_scatter(int64_t nnz, const int64_t* pos, const float* val, floa
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
-template <typename T>
 void launch_coup_rows(int64_t n_tn, int ncta, const int64_t* cta_blk, const int32_t* t_nodes,
-                      const int64_t* slot_off, const int32_t* slots, const float* tile, const double* scale,
-                      const T* X, int64_t ldx, int nE, int N, float* part, cudaStream_t st) {
+                      const int64_t* slot_off, const int32_t* slots, const float* tile, const float* tscale,
+                      const float* X, int64_t ldx, int nE, int N, float* part, cudaStream_t st) {
   if (n_tn <= 0 || N <= 0 || nE <= 0 || ncta <= 0) return;
   const size_t smem = coup_smem(nE, N, true);
-  cudaFuncSetAttribute(k_coup_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_coup_rows<T><<<ncta, 256, smem, st>>>(n_tn, cta_blk, t_nodes, slot_off, slots, tile, scale, X, ldx, nE, N, part);
+  auto run = [&](auto kern) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<ncta, 256, smem, st>>>(n_tn, cta_blk, t_nodes, slot_off, slots, tile, tscale, X, ldx, nE, N, part);
+  };
+  // 8 N bytes of rows a thread and block, held in 16-byte registers where five hold them
+  if (N <= 32) run(k_coup_rows<1>);
+  else if (N <= 96) run(k_coup_rows<3>);
+  else if (N <= 160) run(k_coup_rows<5>);
+  else run(k_coup_rows<0>);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
-template void launch_coup_rows<float>(int64_t, int, const int64_t*, const int32_t*, const int64_t*, const int32_t*,
-                                      const float*, const double*, const float*, int64_t, int, int, float*,
-                                      cudaStream_t);
 
 void launch_coup_reduce(int nb, int nE, int N, const float* part, double sgn, const double* base, int64_t ldb,
                         double alpha_base, double* out, int64_t ldo, cudaStream_t st) {
   if (nE <= 0 || N <= 0) return;
-  k_coup_reduce<<<(unsigned)(((int64_t)nE * N + 31) / 32), 256, 0, st>>>(nb, nE, N, part, sgn, base, ldb, alpha_base,
+  k_coup_reduce<<<(unsigned)(((int64_t)nE * N + CRED - 1) / CRED), 8 * CRED, 0, st>>>(nb, nE, N, part, sgn, base, ldb, alpha_base,
                                                                          out, ldo);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
-template <typename T>
 void launch_coup_cols(int64_t n_tn, int ncta, const int64_t* cta_blk, const int32_t* t_nodes,
                       const int64_t* slot_off, const int32_t* slots, const float* tile, float sgn, const double* Xe,
-                      int64_t ldxe, int nE, int N, T* W, int64_t ldw, cudaStream_t st) {
+                      int64_t ldxe, int nE, int N, float* W, int64_t ldw, cudaStream_t st, const CombArgs* comb) {
   if (n_tn <= 0 || N <= 0 || nE <= 0 || ncta <= 0) return;
   const size_t smem = coup_smem(nE, N, false);
-  cudaFuncSetAttribute(k_coup_cols<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_coup_cols<T><<<ncta, 256, smem, st>>>(n_tn, cta_blk, t_nodes, slot_off, slots, tile, sgn, Xe, ldxe, nE, N, W,
-                                          ldw);
+  auto run = [&](auto kern, const CombArgs& q) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<ncta, 512, smem, st>>>(n_tn, cta_blk, t_nodes, slot_off, slots, tile, sgn, Xe, ldxe, nE, N, W, ldw,
+                                  q.tscale, q.Yc, q.Yp, q.Yn, q.coef);
+  };
+  if (comb) run(k_coup_cols<true>, *comb);
+  else run(k_coup_cols<false>, CombArgs{});
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
-template void launch_coup_cols<float>(int64_t, int, const int64_t*, const int32_t*, const int64_t*, const int32_t*,
-                                      const float*, float, const double*, int64_t, int, int, float*, int64_t,
-                                      cudaStream_t);
 
 int grp_kmax() { return GRP_KMAX; }
 
@@ -2200,11 +2273,11 @@ void launch_spmm_nodes_f32(int64_t nrows, const int32_t* rnode, const int64_t* p
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }
 
-void launch_cheb_combine_f4(int64_t nrows, int ld, const double* rowscale, const float* X, const float* Yc,
+void launch_cheb_combine_f4(int64_t nrows, int ld, const int32_t* rows, const double* rowscale, const float* X, const float* Yc,
                             const float* Yp, float* Yn, const double* coef, cudaStream_t st) {
   if (nrows <= 0) return;
   const int ld4 = ld / 4;
-  k_cheb_combine_f4<<<grid1(nrows * ld4, 256), 256, 0, st>>>(nrows, ld4, rowscale, (const float4*)X,
+  k_cheb_combine_f4<<<grid1(nrows * ld4, 256), 256, 0, st>>>(nrows, ld4, rows, rowscale, (const float4*)X,
                                                             (const float4*)Yc, (const float4*)Yp, (float4*)Yn, coef);
   g_launches.fetch_add(1, std::memory_order_relaxed);
 }

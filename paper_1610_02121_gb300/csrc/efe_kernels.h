@@ -65,17 +65,25 @@ size_t coup_smem(int nE, int N, bool rows);
 int coup_resident_ctas(int nE, int N, int n_sm, bool rows);   // CTAs of one product resident at once
 // CTA b of the rows / columns products takes the node blocks cta_blk[b] .. cta_blk[b + 1]
 void launch_tile_scatter(int64_t nnz, const int64_t* pos, const float* val, float* tile, cudaStream_t st);
-template <typename T>
+// (rows of X, W and the combine's blocks: FP32, 16-byte aligned, ld a multiple of four, zero past N)
 void launch_coup_rows(int64_t n_tn, int ncta, const int64_t* cta_blk, const int32_t* t_nodes,
-                      const int64_t* slot_off, const int32_t* slots, const float* tile, const double* scale,
-                      const T* X, int64_t ldx, int nE, int N, float* part, cudaStream_t st);
+                      const int64_t* slot_off, const int32_t* slots, const float* tile, const float* tscale,
+                      const float* X, int64_t ldx, int nE, int N, float* part, cudaStream_t st);
 void launch_coup_reduce(int nb, int nE, int N, const float* part, double sgn, const double* base, int64_t ldb,
                         double alpha_base, double* out, int64_t ldo, cudaStream_t st);
-template <typename T>
+// comb: do the Chebyshev combine of the pattern rows in the same pass (rows as W's; W is
+// then left as it was).  tscale: D^-1 of the pattern nodes in FP32
+struct CombArgs {
+  const float *tscale, *Yc, *Yp;
+  float* Yn;
+  const double* coef;
+};
 void launch_coup_cols(int64_t n_tn, int ncta, const int64_t* cta_blk, const int32_t* t_nodes,
                       const int64_t* slot_off, const int32_t* slots, const float* tile, float sgn, const double* Xe,
-                      int64_t ldxe, int nE, int N, T* W, int64_t ldw, cudaStream_t st);
-void launch_cheb_combine_f4(int64_t nrows, int ld, const double* rowscale, const float* X, const float* Yc,
+                      int64_t ldxe, int nE, int N, float* W, int64_t ldw, cudaStream_t st,
+                      const CombArgs* comb = nullptr);
+// rows: the rows to do (null: all nrows)
+void launch_cheb_combine_f4(int64_t nrows, int ld, const int32_t* rows, const double* rowscale, const float* X, const float* Yc,
                             const float* Yp, float* Yn, const double* coef, cudaStream_t st);
 // mixed coupling for many enrichment functions (FP32 products, FP64 partial sums):
 // rows product over function groups (items: first function, functions, node
