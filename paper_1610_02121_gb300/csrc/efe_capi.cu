@@ -51,6 +51,7 @@ struct efe_handle {
   float* Hcc32 = nullptr;
   float* Aimg32 = nullptr;  // FP32 images of H^cc_e in the tensor-core layout (chunk-major)
   int tc_mode = 0;          // 1: TF32 tcgen05 cell products, 2: 3-term split TF32 (FP32-grade), 3: BF16
+  float* cellP32 = nullptr;        // tensor-core cell products of all cells at once (small problems)
   int tc_tile = 0, tc_tile_N = 0;  // autotuned column tile of the tensor-core cell kernel for N
   int n_sm = 148;
   int grid_cap = 0;         // test/tuning cap on the persistent tensor-core grids (0: one CTA per SM)
@@ -276,6 +277,13 @@ constexpr int64_t WHOLE_RR_MAX_BYTES = 16ll << 30;
 // cells of one colour are enough to fill the chip.
 constexpr int64_t CELLP_MAX_BYTES = 256ll << 20;
 
+// Largest scratch array of the tensor-core cell products (reserve32): all cells in one
+// launch and a gather instead of eight coloured launches that scatter into W and leave
+// each SM one cell or none.  The line lies where the scratch stops paying beside the other
+// vectors in L2: 1,200 cells, mixed filter of degree 24, 12 columns (9 MB) 4.68 -> 3.57 ms,
+// 48 (29 MB) 5.22 -> 4.37, 104 (62 MB) 7.23 either way.
+constexpr int64_t CELLP32_MAX_BYTES = 40ll << 20;
+
 // FP32 blocks of the mixed degrees (see efe_handle): dropped before the FP64
 // workspace they may live in is reallocated
 void free32(efe_handle* h) {
@@ -288,6 +296,8 @@ void free32(efe_handle* h) {
     h->Yf[i] = nullptr;
     h->Ye[i] = nullptr;
   }
+  dfree(h, h->cellP32);
+  h->cellP32 = nullptr;
   dfree(h, h->cpart);
   dfree(h, h->We);
   dfree(h, h->gpart);
@@ -372,6 +382,8 @@ int reserve32(efe_handle* h, int N) {
     TRY(dalloc(h, &h->Wf, n32));
     CK(cudaMemset(h->Wf, 0, sizeof(float) * n32));
   }
+  if (tc3_scratch_elems(h->n_cell, ld) * (int64_t)sizeof(float) <= CELLP32_MAX_BYTES)
+    TRY(dalloc(h, &h->cellP32, tc3_scratch_elems(h->n_cell, ld)));
   for (int i = 0; i < 2; ++i) TRY(dalloc(h, &h->Ye[i], std::max<int64_t>(1, h->nE) * N));
   TRY(dalloc(h, &h->We, std::max<int64_t>(1, h->nE) * N));
   // coupling products: one wave of CTAs each, node blocks split so that every
@@ -527,10 +539,45 @@ int cell_apply_engine(efe_handle* h, const double* Y, int64_t ldy, double* Wc, i
   return EFE_OK;
 }
 
+// One tensor-core launch of the classical cell products (mode as launch_cell_tc3) and,
+// over all cells at once, their gather
+int tc3_launch_cells(efe_handle* h, const int32_t* cells, int64_t nc, const float* Y, int64_t ldy, float* W,
+                     int64_t ldw, int N, int mode, int tile, int stall, cudaStream_t st) {
+  if (launch_cell_tc3(h->Aimg32, cells, nc, h->mesh, Y, ldy, cells ? W : h->cellP32, ldw, N, mode, tc_grid(h),
+                      h->info + 4, st, tile, stall)) {
+    h->err = "tensor-core cell kernel needs 16-byte aligned rows";
+    return EFE_ERR_ARG;
+  }
+  if (!cells) launch_tc3_gather(h->mesh, h->cellP32, ldw, N, W, ldw, st);
+  CKL();
+  return EFE_OK;
+}
+
+// --- classical cell products of the FP32 filter on the tensor cores: W_c = H^cc Y_c ---
+// (ld32 rows; eight coloured launches add into W, which is zeroed first)
+int tc3_cells(efe_handle* h, const float* Y, float* W, int N, int mode, int tile, int stall, cudaStream_t st) {
+  const int ld = h->ld32;
+  if (h->cellP32) {
+    int slot;
+    TRY(timed_begin(h, st, &slot));
+    TRY(tc3_launch_cells(h, nullptr, h->n_cell, Y, ld, W, ld, N, mode, tile, stall, st));
+    return timed_end(h, st, slot, (double)(h->n_cell * (int64_t)N));
+  }
+  CK(cudaMemsetAsync(W, 0, sizeof(float) * h->n_nodes * ld, st));
+  for (int c = 0; c < 8; ++c) {
+    const int64_t nc = h->colour_off[c + 1] - h->colour_off[c];
+    if (nc == 0) continue;
+    int slot;
+    TRY(timed_begin(h, st, &slot));
+    TRY(tc3_launch_cells(h, h->colour_cells + h->colour_off[c], nc, Y, ld, W, ld, N, mode, tile, stall, st));
+    TRY(timed_end(h, st, slot, (double)(nc * (int64_t)N)));
+  }
+  return EFE_OK;
+}
+
 // --- classical cell products, all 8 parity colours: W_c += H^cc Y_c ---
 template <typename T>
-int cell_apply_all(efe_handle* h, const T* Hc, const T* Y, int64_t ldy, T* Wc, int64_t ldw, int N, cudaStream_t st,
-                   bool tc = false) {
+int cell_apply_all(efe_handle* h, const T* Hc, const T* Y, int64_t ldy, T* Wc, int64_t ldw, int N, cudaStream_t st) {
   for (int c = 0; c < 8; ++c) {
     const int64_t nc = h->colour_off[c + 1] - h->colour_off[c];
     if (nc == 0) continue;
@@ -540,15 +587,7 @@ int cell_apply_all(efe_handle* h, const T* Hc, const T* Y, int64_t ldy, T* Wc, i
     if constexpr (sizeof(T) == 8) {
       launch_cell_apply_f64((const double*)Hc, cl, nc, h->mesh, (const double*)Y, ldy, (double*)Wc, ldw, N, st);
     } else {
-      if (tc) {
-        if (launch_cell_tc3(h->Aimg32, cl, nc, h->mesh, (const float*)Y, ldy, (float*)Wc, ldw, N,
-                            h->tc_mode - 1, tc_grid(h), h->info + 4, st, h->tc_tile_N == N ? h->tc_tile : 0,
-                            h->opt_test_stall)) {
-          h->err = "tensor-core cell kernel needs 16-byte aligned rows";
-          return EFE_ERR_ARG;
-        }
-      }
-      else if (N <= 8)
+      if (N <= 8)
         launch_cell_apply_narrow_f32((const float*)Hc, cl, nc, h->mesh, (const float*)Y, ldy, (float*)Wc, ldw, N, st);
       else
         launch_cell_apply_f32((const float*)Hc, cl, nc, h->mesh, (const float*)Y, ldy, (float*)Wc, ldw, N, st);
@@ -728,9 +767,13 @@ int degree_f32(efe_handle* h, const float* Yc, const double* Yce, const float* Y
   const int64_t nn = h->n_nodes;
   const int ld = h->ld32;
   double* We = h->We;  // nE x N FP64 scratch (W may hold the FP32 slots)
-  CK(cudaMemsetAsync(h->Wf, 0, sizeof(float) * nn * ld, st));
   h->time_this = true;
-  TRY(cell_apply_all<float>(h, h->Hcc32, Yc, ld, h->Wf, ld, N, st, h->tc_mode != 0));
+  if (h->tc_mode) {
+    TRY(tc3_cells(h, Yc, h->Wf, N, h->tc_mode - 1, h->tc_tile_N == N ? h->tc_tile : 0, h->opt_test_stall, st));
+  } else {
+    CK(cudaMemsetAsync(h->Wf, 0, sizeof(float) * nn * ld, st));
+    TRY(cell_apply_all<float>(h, h->Hcc32, Yc, ld, h->Wf, ld, N, st));
+  }
   h->time_this = false;
   const bool tiles = h->nE > 0 && coup_tiles_fit(h, N);
   if (h->nE > 0) {
@@ -2893,16 +2936,8 @@ int efe_autotune(efe_handle* h, int32_t N, int32_t precision, int32_t* tile_out,
     float ms = 0.f;
     for (int rep = 0; rep < 3; ++rep) {  // rep 0 warms up
       CK(cudaEventRecord(e0, st));
-      for (int c = 0; c < 8; ++c) {
-        const int64_t nc = h->colour_off[c + 1] - h->colour_off[c];
-        if (nc == 0) continue;
-        if (launch_cell_tc3(h->Aimg32, h->colour_cells + h->colour_off[c], nc, h->mesh, h->Yf[0], h->ld32, h->Wf,
-                            h->ld32, N, precision == EFE_PREC_TF32X3 ? 1 : (precision == EFE_PREC_BF16 ? 2 : 0),
-                            tc_grid(h), h->info + 4, st, tiles[i])) {
-          h->err = "tensor-core cell kernel needs 16-byte aligned rows";
-          return EFE_ERR_ARG;
-        }
-      }
+      TRY(tc3_cells(h, h->Yf[0], h->Wf, N, precision == EFE_PREC_TF32X3 ? 1 : (precision == EFE_PREC_BF16 ? 2 : 0),
+                    tiles[i], 0, st));
       CK(cudaEventRecord(e1, st));
       CK(cudaEventSynchronize(e1));
       float t = 0.f;

@@ -1,4 +1,4 @@
-// Warp-specialised tensor-core cell products (tcgen05 + bulk async copies, sm_103a).
+// Warp-specialised tensor-core cell products (tcgen05 + asynchronous copies, sm_103a).
 //
 // Paper, Sec. V (last paragraph): W_c(e) += H^cc_e Y_c(e) for every cell of
 // one parity colour (cells of a colour share no node, so the scatter needs no
@@ -161,7 +161,7 @@ template <int MODE, int TW>
 __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
     k_cell_tc3(const float* __restrict__ Ag, const int32_t* __restrict__ cells, int64_t ncells, MeshDev m,
                const float* __restrict__ Y, int64_t ldy, float* __restrict__ W, int64_t ldw, int N, int ntiles,
-               int* __restrict__ err, int stall) {
+               int* __restrict__ err, int stall) {   // cells: null for all cells, their products to W's rows (e, r)
   using L = T3Layout<TW>;
   constexpr int ST = L::STAGES;
   extern __shared__ __align__(1024) unsigned char sm[];
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
       if (ft < my_items) {
         if (fk < 2) {
           const int64_t item = blockIdx.x + ft * gridDim.x;
-          const int64_t e = cells[item / ntiles];
+          const int64_t e = cells ? cells[item / ntiles] : item / ntiles;
           const int c0 = (int)(item % ntiles) * TW, col = c0 + cg + (lane & 7) * 4;
           fa = Ag + e * (int64_t)(T3_M * T3_K) + gt * 4;
           fcol = col < min(N, c0 + TW);
@@ -404,16 +404,16 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
     const int sub = lane & 3;
     for (int64_t t = 0; t < my_items && !*abort_flag; ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
-      const int64_t e = cells[item / ntiles];
+      const int64_t e = cells ? cells[item / ntiles] : item / ntiles;
       const int c0 = (int)(item % ntiles) * TW;
       const int ncol = min(TW, N - c0);
       const int b = (int)(t & 1);
       // after the exchange below this lane holds 16 bytes of each of the four rows of its lane quad
       const int r0 = quarter * 32 + (lane & ~3);
-      float* wr = W + cell_corner(m, e) * ldw + c0;
+      float* wr = W + (cells ? cell_corner(m, e) : e * NL) * ldw + c0;
       int64_t ro[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) ro[i] = (int64_t)lut[r0 + i] * ldw;
+      for (int i = 0; i < 4; ++i) ro[i] = (int64_t)(cells ? lut[r0 + i] : r0 + i) * ldw;
       if (!bar_wait(accf + b, (uint32_t)((t / 2) & 1))) {
         *abort_flag = 1;
         atomicExch(err, 1);
@@ -451,7 +451,16 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
         for (int i = 0; i < 4; ++i) {
           if (r0 + i >= NL) continue;
           float* o = wr + ro[i] + c;
-          if (c + 4 <= ncol) {
+          if (!cells) {
+            if (c + 4 <= ncol) {
+              *reinterpret_cast<float4*>(o) = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
+                                                          __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+            } else {
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (c + q < ncol) o[q] = __uint_as_float(v[4 * i + q]);
+            }
+          } else if (c + 4 <= ncol) {
             asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(o),
                          "f"(__uint_as_float(v[4 * i])), "f"(__uint_as_float(v[4 * i + 1])),
                          "f"(__uint_as_float(v[4 * i + 2])), "f"(__uint_as_float(v[4 * i + 3]))
@@ -481,6 +490,49 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
   }
 }
 
+// W row of a node = the rows (e, r) of P that meet it, added in the order of the cells'
+// parity colours (as the coloured launches add them); columns N .. 4 q4 of W are zero
+__global__ void k_tc3_gather(MeshDev m, int64_t n_nodes, const float* __restrict__ Pc, int64_t ldp, int N, int q4,
+                             float* __restrict__ W, int64_t ldw) {
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (idx >= n_nodes * q4) return;
+  const int64_t g = idx / q4;
+  const int c = (int)(idx % q4) * 4;
+  const int G[3] = {(int)(g % m.nn[0]), (int)((g / m.nn[0]) % m.nn[1]), (int)(g / ((int64_t)m.nn[0] * m.nn[1]))};
+  int hi[3], cnt[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    hi[d] = min(G[d] / P, m.nc[d] - 1);
+    cnt[d] = (G[d] % P == 0 && G[d] > 0 && G[d] / P < m.nc[d]) ? 2 : 1;
+  }
+  float4 v[8];
+  bool ok[8];
+#pragma unroll
+  for (int col = 0; col < 8; ++col) {
+    int cc[3], l[3];
+    ok[col] = c < N;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int par = (col >> d) & 1;
+      cc[d] = (hi[d] & 1) == par ? hi[d] : hi[d] - 1;
+      ok[col] = ok[col] && (cc[d] == hi[d] || cnt[d] == 2);
+      l[d] = G[d] - P * cc[d];
+    }
+    const int64_t e = cc[0] + (int64_t)m.nc[0] * (cc[1] + (int64_t)m.nc[1] * cc[2]);
+    if (ok[col]) v[col] = *reinterpret_cast<const float4*>(Pc + (e * NL + l[0] + NP1 * (l[1] + NP1 * l[2])) * ldp + c);
+  }
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int col = 0; col < 8; ++col) {
+    if (!ok[col]) continue;
+    s.x += v[col].x;
+    if (c + 1 < N) s.y += v[col].y;
+    if (c + 2 < N) s.z += v[col].z;
+    if (c + 3 < N) s.w += v[col].w;
+  }
+  *reinterpret_cast<float4*>(W + g * ldw + c) = s;
+}
+
 // FP32 images of H^cc_e, [cell][16-wide chunk], each in the K-major core-matrix layout
 __global__ void k_build_aimg(const double* __restrict__ Hcc, int64_t n_cell, float* __restrict__ A) {
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // (cell, row, K quad)
@@ -506,7 +558,17 @@ void launch_build_aimg(const double* Hcc, int64_t n_cell, float* A, cudaStream_t
   }
 }
 
-// W += H_e Y_e over the cells of one colour.  Y / W: FP32 rows, ld a multiple of 4
+int64_t tc3_scratch_elems(int64_t n_cell, int64_t ld) { return n_cell * NL * ld; }
+
+void launch_tc3_gather(const MeshDev& m, const float* Pc, int64_t ldp, int N, float* W, int64_t ldw, cudaStream_t st) {
+  const int64_t nn = (int64_t)m.nn[0] * m.nn[1] * m.nn[2];
+  const int q4 = (int)(ldw / 4);
+  k_tc3_gather<<<(unsigned)((nn * q4 + 255) / 256), 256, 0, st>>>(m, nn, Pc, ldp, N, q4, W, ldw);
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+}
+
+// W += H_e Y_e over the cells of one colour; cells == nullptr: rows (e, r) of W = row r of
+// H_e Y_e over all ncells cells.  Y / W: FP32 rows, ld a multiple of 4
 // elements and rows 16-byte aligned (the 16-byte copies and reductions).
 namespace {
 template <int TW>

@@ -158,6 +158,10 @@ void launch_build_aimg(const double* Hcc, int64_t n_cell, float* A, cudaStream_t
 // tile: column tile width (64, 96 or 160; 0 = default 160)
 // stall (tests only): the MMA warp first waits on a barrier nothing completes, so the
 // bounded wait runs out and the launch takes its abort path
+// cells null: all cells at once, their products to W as (n_cell x 125) x ldw scratch, which
+// launch_tc3_gather adds per node (W's columns N .. ldw become zero)
+int64_t tc3_scratch_elems(int64_t n_cell, int64_t ld);
+void launch_tc3_gather(const MeshDev& m, const float* Pc, int64_t ldp, int N, float* W, int64_t ldw, cudaStream_t st);
 // mode 0: one TF32 pass; 1: 3-term TF32 split (FP32-grade); 2: BF16 operands (FP32 accumulate)
 int launch_cell_tc3(const float* A, const int32_t* cells, int64_t ncells, const MeshDev& m,
                     const float* Y, int64_t ldy, float* W, int64_t ldw, int N, int mode, int n_sm, int* err,
