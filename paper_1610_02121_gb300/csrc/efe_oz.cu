@@ -50,21 +50,38 @@ constexpr int OZ_EPI_W0 = 4, OZ_EPI_WN = 12;   // epilogue warps
 constexpr int OZ_THREADS = 16 * 32;            // 16 warps: 128 registers a thread
 
 struct OzL {
-  static constexpr uint32_t ASL = OZ_M * OZ_KC * 2;        // one A slice, 4 KB
-  static constexpr uint32_t BSL = OZ_TW * OZ_KC * 2;       // one B slice, 3 KB
-  static constexpr uint32_t STAGE = OZ_S * (ASL + BSL);    // 49 KB
+  static constexpr uint32_t ASL = OZ_M * OZ_KC * 2;        // one slice of 128 rows, 4 KB
+  static constexpr uint32_t GRP = OZ_S * 256;              // eight rows (columns) of a chunk: seven slices of 256 B
+  static constexpr uint32_t A = OZ_M / 8 * GRP;            // 28 KB
+  static constexpr uint32_t STAGE = A + OZ_TW / 8 * GRP;   // 49 KB
   static constexpr uint32_t BARS = OZ_STAGES * STAGE;
   static constexpr uint32_t STG = BARS + 256;                // epilogue staging: up to 12 warps x 32 rows x 9 doubles
   static constexpr size_t TOTAL = (size_t)STG + 12 * 32 * 9 * 8;
 };
 
-// K-major, no swizzle, BF16: core matrix 8 rows x 16 B; LBO = 128 B (next 8 K), SBO = 256 B (next 8 rows)
+// cell images, K-major, no swizzle, BF16: core matrix 8 rows x 16 B, the next 8 K 128 B and
+// the next 8 rows 256 B further
 __device__ __forceinline__ uint32_t bo(int row, int k) {
   return (uint32_t)(row >> 3) * 256u + (uint32_t)(k >> 3) * 128u + (uint32_t)(row & 7) * 16u + (uint32_t)(k & 7) * 2u;
 }
+// operand images of this file: [chunk][8 rows][slice][8 K][row of 16 B], so that any run of
+// rows of a chunk is one contiguous piece with all its slices and one bulk copy brings an
+// operand's chunk.  (Slice-major 128-column tiles took 8 or, across two tiles, 15 copies a
+// chunk, and their issue, about 120 cycles each, outlasted the chunk's 28 MMAs.  The products
+// of a Rayleigh-Ritz of 559 k rows x 640 columns, with the segment rule of the Gram products
+// below: 83 -> 69 ms, of 559 k x 135: 8.4 -> 5.8 ms.)  Slice i of row r, K octet o:
+__device__ __forceinline__ uint32_t go(int row, int i, int oct) {
+  return (uint32_t)(row >> 3) * OzL::GRP + (uint32_t)i * 256u + (uint32_t)oct * 128u + (uint32_t)(row & 7) * 16u;
+}
+// LBO = 128 B (next 8 K), SBO = GRP (next 8 rows)
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(256u >> 4) << 32) |
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(OzL::GRP >> 4) << 32) |
          ((uint64_t)1 << 46);
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
 }
 __device__ __forceinline__ uint32_t idesc_bf16(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
@@ -117,11 +134,11 @@ struct OzArgs {
   const int2* pairs;        // (M tile, N tile) of every item pair
   double* part;
   // pre-sliced operand images (k_oz_img_rows / k_oz_img_cols).  ROWS: Aimg = row image
-  // of A, Bimg = column image of B; GRAM: both column images.  img_nch: 16-wide K chunks
-  // per 128-wide tile of a column image.
+  // of A, Bimg = column image of B; GRAM: both column images.  astep, bstep: bytes of a
+  // chunk of a column image.
   const unsigned char* Aimg;
   const unsigned char* Bimg;
-  int64_t img_nch;
+  int64_t astep, bstep;
   int stall;                // tests only: the MMA warp first waits on a barrier nothing completes
 };
 
@@ -157,7 +174,8 @@ __device__ __forceinline__ OzItem oz_item(const OzArgs& g, int64_t item) {
 
 __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
   extern __shared__ __align__(1024) unsigned char sm[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   __shared__ int s_skip;
   if (tid == 0) s_skip = *(volatile int*)g.err;
   __syncthreads();
@@ -226,9 +244,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
         ok = bar_wait(afull + s, (uint32_t)((ch / OZ_STAGES) & 1));
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!ok) break;
-        if (lane == 0) {
-          const uint32_t sA = su32(sm + s * OzL::STAGE);
-          const uint32_t sB = sA + OZ_S * OzL::ASL;
+        const uint32_t sA = su32(sm) + (uint32_t)s * OzL::STAGE, sB = sA + OzL::A;
+        if (elect_one()) {
           const uint32_t id = idesc_bf16(nmma);
           bool first[OZ_NACC] = {true, true, true, true, true};
 #pragma unroll
@@ -240,8 +257,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
               if (i > OZ_S || j > OZ_S) continue;
               const uint32_t acc = (kc % gsz > 0 || !first[a]) ? 1u : 0u;
               first[a] = false;
-              mma_bf16(tmem + (uint32_t)(a * OZ_TW), sdesc(sA + (uint32_t)(i - 1) * OzL::ASL),
-                       sdesc(sB + (uint32_t)(j - 1) * OzL::BSL), id, acc);
+              mma_bf16(tmem + (uint32_t)(a * OZ_TW), sdesc(sA + (uint32_t)(i - 1) * 256u),
+                       sdesc(sB + (uint32_t)(j - 1) * 256u), id, acc);
             }
           }
           mma_commit(empty + s);
@@ -269,32 +286,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
           if (!ok) break;
         }
         unsigned char* SA = sm + s * OzL::STAGE;
-        unsigned char* SB = SA + OZ_S * OzL::ASL;
-        // operand chunks: bulk copies of 256-byte row groups into the stage
+        // one bulk copy an operand and chunk: rows m0 .. of A's, columns c0 .. of B's image
         const int64_t kA = (g.mode == 2) ? it.kb / OZ_KC + kc : kc;
-        const int ga = (g.mode == 2) ? (int)((min((int64_t)OZ_M, (int64_t)g.Na - it.m0) + 7) / 8) : 16;
-        const int gb = nmma / 8;
-        bar_expect_tx(afull + s, (uint32_t)(OZ_S * (ga + gb) * 256));
-        // ROWS: image of row tile ia; GRAM: of column tile m0 / 128
-        const int64_t img = (g.mode == 1) ? it.ia * (int64_t)nch + kA : (it.m0 / OZ_M) * g.img_nch + kA;
-        const unsigned char* srcA = g.Aimg + img * OZ_S * (int64_t)OzL::ASL;
-        if (ga == 16) {
-          bulk_g2s(SA, srcA, OZ_S * OzL::ASL, afull + s);
-        } else {
-          for (int i2 = 0; i2 < OZ_S; ++i2)
-            bulk_g2s(SA + i2 * OzL::ASL, srcA + i2 * OzL::ASL, (uint32_t)(ga * 256), afull + s);
-        }
-        // columns c0 .. c0 + nmma of B: row groups of the 128-wide column tiles
-        const int64_t nchB = (g.mode == 2) ? g.img_nch : nch;
-        for (int j = 0; j < gb;) {
-          const int G = c0 / 8 + j;
-          const int tile = G >> 4, gi = G & 15;
-          const int run = min(gb - j, 16 - gi);
-          const unsigned char* src = g.Bimg + ((tile * nchB + kA) * OZ_S) * (int64_t)OzL::ASL + gi * 256;
-          for (int i2 = 0; i2 < OZ_S; ++i2)
-            bulk_g2s(SB + i2 * OzL::BSL + j * 256, src + i2 * OzL::ASL, (uint32_t)(run * 256), afull + s);
-          j += run;
-        }
+        const uint32_t la = (g.mode == 2) ? (uint32_t)((min((int64_t)OZ_M, (int64_t)g.Na - it.m0) + 7) / 8) * OzL::GRP
+                                          : OzL::A;
+        const uint32_t lb = (uint32_t)(nmma / 8) * OzL::GRP;
+        bar_expect_tx(afull + s, la + lb);
+        bulk_g2s(SA, (g.mode == 2) ? g.Aimg + kA * g.astep + (it.m0 / 8) * OzL::GRP
+                                   : g.Aimg + (it.ia * (int64_t)nch + kA) * OzL::A, la, afull + s);
+        bulk_g2s(SA + OzL::A, g.Bimg + kA * g.bstep + (int64_t)(c0 / 8) * OzL::GRP, lb, afull + s);
         last_copy = ch;
       }
       if (!ok) {
@@ -482,7 +482,7 @@ __global__ void k_oz_preslice(const double* __restrict__ H, const int* __restric
 }
 
 // Row image of a tall A (rows x K, the A operand of ROWS): per 128-row tile and
-// 16-wide K chunk the seven 4 KB BF16 slices in the shared-memory layout of
+// 16-wide K chunk the seven BF16 slices of its rows in the shared-memory layout of
 // the MMA operand (row exponents aexp); rows past `rows` are zero.  One thread
 // per (tile row, K octet); a warp covers 32 rows of one octet.
 __global__ void k_oz_img_rows(const double* __restrict__ A, int64_t lda, int64_t rows, int K,
@@ -505,15 +505,15 @@ __global__ void k_oz_img_rows(const double* __restrict__ A, int64_t lda, int64_t
   }
   uint32_t pk[OZ_S][4];
   oz_pack8(x, E, pk);
-  unsigned char* base = img + tc * OZ_S * (int64_t)OzL::ASL + bo(rr, oct * 8);
+  unsigned char* base = img + tc * (int64_t)OzL::A + go(rr, 0, oct);
 #pragma unroll
   for (int i = 0; i < OZ_S; ++i)
-    *reinterpret_cast<uint4*>(base + (int64_t)i * OzL::ASL) = make_uint4(pk[i][0], pk[i][1], pk[i][2], pk[i][3]);
+    *reinterpret_cast<uint4*>(base + i * 256) = make_uint4(pk[i][0], pk[i][1], pk[i][2], pk[i][3]);
 }
 
 // Column image of A (Krows x ncols): the K-major operand A^T, element (m, k) =
-// A[k][m], per 128-column tile and 16-row chunk (nch chunks per tile, rows past
-// Krows zero), seven 4 KB slices in the MMA layout (column exponents cexp).
+// A[k][m], per 16-row chunk (nch of them, rows past Krows zero) all columns, padded to
+// 128, with their seven slices in the MMA layout (column exponents cexp).
 // Columns past ncols rounded up to 16 are not written.  A warp reads 32
 // consecutive columns of one row.
 __global__ void k_oz_img_cols(const double* __restrict__ A, int64_t lda, int64_t Krows, int ncols,
@@ -523,9 +523,9 @@ __global__ void k_oz_img_cols(const double* __restrict__ A, int64_t lda, int64_t
   if (t >= (int64_t)ntile * nch * 2 * OZ_M) return;
   const int m = (int)(t % OZ_M);
   const int oct = (int)((t / OZ_M) & 1);
-  const int64_t tc = t / (2 * OZ_M);   // tile * nch + chunk
-  const int64_t c = tc % nch;
-  const int col = (int)(tc / nch) * OZ_M + m;
+  const int64_t tc = t / (2 * OZ_M);   // chunk * ntile + tile
+  const int64_t c = tc / ntile;
+  const int col = (int)(tc % ntile) * OZ_M + m;
   if (col >= ((ncols + 15) & ~15)) return;
   const int E = col < ncols ? cexp[col] : -2000;
   double x[8];
@@ -536,10 +536,10 @@ __global__ void k_oz_img_cols(const double* __restrict__ A, int64_t lda, int64_t
   }
   uint32_t pk[OZ_S][4];
   oz_pack8(x, E, pk);
-  unsigned char* base = img + tc * OZ_S * (int64_t)OzL::ASL + bo(m, oct * 8);
+  unsigned char* base = img + c * (int64_t)ntile * OzL::A + go(col, 0, oct);
 #pragma unroll
   for (int i = 0; i < OZ_S; ++i)
-    *reinterpret_cast<uint4*>(base + (int64_t)i * OzL::ASL) = make_uint4(pk[i][0], pk[i][1], pk[i][2], pk[i][3]);
+    *reinterpret_cast<uint4*>(base + i * 256) = make_uint4(pk[i][0], pk[i][1], pk[i][2], pk[i][3]);
 }
 
 // per-row scale exponents of an FP64 matrix (one warp per row)
@@ -676,6 +676,7 @@ int launch_oz_rows(int64_t rows, int K, const int* aexp, const int* bexp, double
   a.ldo = ldc;
   a.N = N;
   a.ntiles = (N + OZ_TW - 1) / OZ_TW;
+  a.bstep = oz_img_cols_bytes(1, N);
   a.err = err;
   a.stall = stall;
   return oz_launch(a, n_sm, st);
@@ -688,10 +689,25 @@ int launch_oz_rows(int64_t rows, int K, const int* aexp, const int* bexp, double
 // C is symmetric, only tiles that meet the upper triangle are formed and the
 // rest is mirrored.  aexp / bexp: launch_oz_colexp of A and B.  work: at least
 // oz_gram_work_elems doubles; pairs_dev: at least oz_gram_max_pairs int2.
-int64_t oz_gram_segments(int64_t K, int npairs, int n_sm) {
-  int64_t nseg = std::max<int64_t>(1, (2 * (int64_t)n_sm + npairs - 1) / npairs);
-  nseg = std::min<int64_t>(nseg, (K + 255) / 256);
-  return std::max<int64_t>(nseg, 1);
+//
+// Segment length, in 256-row groups: the one that ends first when the (tile pair, segment)
+// items run n_sm at a time, an item costing its groups and half a group to fill and drain the
+// pipeline (about two items a CTA before: 135 columns 306 items, 640 columns 320, in three
+// rounds of 152).  Partials of at most max_seg segments fit the work array; more than 2 n_sm
+// segments gain nothing.
+int64_t oz_gram_seg_groups(int64_t groups, int npairs, int n_sm, int64_t max_seg) {
+  int64_t best = groups;
+  double best_cost = 1e300;
+  max_seg = std::max<int64_t>(1, std::min<int64_t>(max_seg, 2 * (int64_t)n_sm));
+  for (int64_t ns = std::min(groups, max_seg); ns >= 1; --ns) {
+    const int64_t len = (groups + ns - 1) / ns, items = (groups + len - 1) / len * npairs;
+    const double cost = (double)((items + n_sm - 1) / n_sm) * ((double)len + 0.5);
+    if (cost <= best_cost) {
+      best_cost = cost;
+      best = len;
+    }
+  }
+  return best;
 }
 
 int oz_gram_pairs(int Na, int N, bool sym, int2* pairs_host) {
@@ -728,11 +744,10 @@ int launch_oz_gram(int64_t K, int Na, int N, const double* A, int64_t lda, const
   if (sym && Na != N) return 1;
   std::vector<int2> pairs(oz_gram_pairs(Na, N, sym, nullptr));
   const int np = oz_gram_pairs(Na, N, sym, pairs.data());
-  int64_t nseg = oz_gram_segments(K, np, n_sm);
-  while (nseg > 1 && nseg * (int64_t)Na * N > work_elems) --nseg;
-  if (nseg * (int64_t)Na * N > work_elems) return 1;
-  const int64_t seg_len = ((K + nseg - 1) / nseg + 255) / 256 * 256;
-  nseg = (K + seg_len - 1) / seg_len;
+  if ((int64_t)Na * N > work_elems) return 1;
+  const int64_t groups = (K + 255) / 256;
+  const int64_t seg_len = 256 * oz_gram_seg_groups(groups, np, n_sm, work_elems / ((int64_t)Na * N));
+  const int64_t nseg = (K + seg_len - 1) / seg_len;
   if (cudaMemcpyAsync(pairs_dev, pairs.data(), sizeof(int2) * np, cudaMemcpyHostToDevice, st) != cudaSuccess) return 1;
   OzArgs a{};
   a.mode = 2;
@@ -757,7 +772,8 @@ int launch_oz_gram(int64_t K, int Na, int N, const double* A, int64_t lda, const
   if (B != A) launch_oz_img_cols(B, ldb, K, N, bexp, nch, img_b, st);
   a.Aimg = img_a;
   a.Bimg = (B == A) ? img_a : img_b;
-  a.img_nch = nch;
+  a.astep = oz_img_cols_bytes(1, Na);
+  a.bstep = oz_img_cols_bytes(1, N);
   if (oz_launch(a, n_sm, st)) return 1;
   k_oz_gram_reduce<<<(unsigned)(((int64_t)Na * N + 255) / 256), 256, 0, st>>>((int)nseg, Na, N, work, sym ? 1 : 0,
                                                                              accumulate ? 1 : 0, C, ldc);

@@ -142,3 +142,74 @@ def test_split_cell_tiles(tiny_pair, prec, tol, N):
         out.append(Xd)
     assert rel_err(out[0], ref) < tol
     assert torch.equal(out[0], out[1])
+
+
+# FP64 engine's tall products where the operand pieces of 128 rows and 96 columns and the
+# 256-row groups of the segments end, against the oracle (figures of the blocked case)
+@pytest.mark.parametrize("cap", [0, 3])
+@pytest.mark.parametrize("N", [95, 96, 97, 127, 128, 129, 191, 193, 224])
+def test_engine_tall_products(tiny_pair, cap, N):
+    from oracle.chfsi import cholqr, rayleigh_ritz
+    d, G = tiny_pair
+    X = W.random_block(d.system, N, seed=900 + N)
+    eps_ref, _, _ = rayleigh_ritz(d.apply_H_assembled, d.apply_M_assembled, cholqr(X)[0])
+    G.set_fp64_engine("tensor")
+    G.set_grid_cap(cap)
+    try:
+        Xd = to_dev(X)
+        eps, _ = G.rayleigh_ritz(Xd)
+    finally:
+        G.set_grid_cap(0)
+        G.set_fp64_engine("dfma")
+    np.testing.assert_allclose(eps, eps_ref, atol=1e-8, rtol=1e-8)
+    gram = (Xd.T @ G.apply_M(Xd)).cpu().numpy()
+    np.testing.assert_allclose(gram, np.eye(N), atol=1e-8)
+
+
+# descriptors: fewest and most Gaussians, widths at which most terms fall out of an FP32 sum
+# and at which all stay, several atoms of a species; FP64 to rounding (arguments up to a few
+# hundred: 1e-12 of the largest entry), FP32 to a few roundings of the largest entry (1e-6)
+@pytest.mark.parametrize("width", [0.02, 0.45, 5.0, 1e-160])
+@pytest.mark.parametrize("nr,nang", [(1, 0), (12, 4), (16, 8)])
+def test_descriptor_sums(nr, nang, width):
+    from paper_1610_02121_gb300 import learned as LR
+    s = dict(W.tiny(seed=11))
+    s["Z"] = np.ones(len(s["Z"]))
+    G = gpu_system(s)
+    p = LR.desc_params()
+    p.n_radial, p.n_ang, p.radial_sigma, p.ang_sigma = nr, nang, width, max(width, 0.1)
+    mu = np.linspace(0.3, 7.5, 16)
+    for i in range(16):
+        p.radial_mu[i] = mu[i]
+    for i in range(8):
+        p.ang_mu[i] = mu[2 * i]
+    q = G.qpoints().cpu().numpy()[:, :3]
+    ref = np.zeros((len(q), 4 * (nr + nang)))
+    vec = np.zeros((len(q), nang, 3))
+    with np.errstate(over="ignore", divide="ignore", invalid="ignore"):
+        for a in np.asarray(s["atoms"]):
+            d = q - a
+            r = np.sqrt((d * d).sum(axis=1))
+            fc = np.where(r < p.r_cut, 0.5 * (1 + np.cos(np.pi * r / p.r_cut)), 0.0)
+            ref[:, :nr] += np.exp(-(r[:, None] - mu[None, :nr]) ** 2 / (2 * width * width)) * fc[:, None]
+            g = np.exp(-(r[:, None] - mu[None, :2 * nang:2]) ** 2 / (2 * p.ang_sigma ** 2)) * fc[:, None]
+            vec += g[:, :, None] * (d / np.maximum(r, 1e-12)[:, None])[:, None, :]
+    ref[:, 4 * nr:4 * nr + nang] = (vec * vec).sum(axis=2)
+    for prec, tol in (("fp64", 1e-12), ("fp32", 1e-6)):
+        D = G.descriptors(p, precision=prec).double().cpu().numpy()
+        assert D.shape == ref.shape
+        assert np.abs(D - ref).max() <= tol * max(1.0, np.abs(ref).max())
+
+
+# superposed atoms with one to three shells: every point to 1e-11 of its own value (the
+# exponents reach a few hundred, at 2^-53 each; shells are left out below 2^-58 of the sum)
+@pytest.mark.parametrize("Z", [(1, 1), (14, 1), (14, 14), (8, 14)])
+def test_sad_points(tiny_pair, Z):
+    from oracle import learned as OL
+    d, G = tiny_pair
+    q = G.qpoints().cpu().numpy()
+    atoms = np.asarray(d.system["atoms"])
+    shells = [W.sad_shells(Z[i % 2]) for i in range(len(atoms))]
+    rho = G.sad_density(shells).cpu().numpy()
+    ref = OL.sad_density(q[:, :3], atoms, shells)
+    np.testing.assert_allclose(rho, ref, rtol=1e-11)
