@@ -12,6 +12,8 @@
 
 #include <type_traits>
 
+#include <cmath>
+
 #include "efe_kernels.h"
 
 namespace efe {
@@ -32,68 +34,184 @@ __device__ __forceinline__ T silu_grad_d(T z) {
 
 // ---------------------------------------------------------------------------
 // SAD: rho(x) = sum_I sum_s N_s C_s^2 r^(2 n_s - 2) exp(-2 zeta_s r) / (4 pi)
-__global__ void k_sad(const double* __restrict__ qpts, int64_t nq, const double* __restrict__ axyz, int na,
-                      const SadShellDev* __restrict__ sh, double* __restrict__ rho) {
-  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  const double x = qpts[4 * q], y = qpts[4 * q + 1], z = qpts[4 * q + 2];
-  double s = 0.0;
+//
+// The FP64 pipe bounds it (an exponential per point, atom and shell), so a point starts with
+// its nearest atom and takes a further shell only if FP32 arithmetic finds it above 2^-58 of
+// the sum so far (FP32 distances are off by about 1e-6 here, far less than a factor of two
+// in a term).  Most inner shells of most atoms fall out: 3.84 M points, 16 atoms of three
+// shells 9.2 -> 5.6 ms.
+constexpr int SAD_TILE = 32;     // atoms whose shells wait in shared memory
+
+struct SadShell {
+  double w, z2;    // N C^2, 2 zeta
+  float lw, z2f;   // log2 of w (rounded up), 2 zeta log2(e)
+  int p;           // 2 n - 2
+};
+
+__device__ __forceinline__ SadShell sad_shell(const SadShellDev& S, int k) {
+  SadShell o;
+  o.w = S.occ[k] * S.c[k] * S.c[k];
+  o.z2 = 2.0 * S.zeta[k];
+  o.lw = log2f(fabsf((float)o.w)) + 1.f;
+  o.z2f = (float)(o.z2 * 1.4426950408889634);
+  o.p = max(0, 2 * S.n[k] - 2);
+  return o;
+}
+
+__device__ __forceinline__ double sad_term(const SadShell& S, double r) {
+  double rp = S.w;
+  for (int i = 0; i < S.p; ++i) rp *= r;
+  return rp * exp(-S.z2 * r);
+}
+
+__global__ void __launch_bounds__(256) k_sad(const double* __restrict__ qpts, int64_t nq,
+                                             const double* __restrict__ axyz, int na,
+                                             const SadShellDev* __restrict__ sh, double* __restrict__ rho) {
+  __shared__ double ax[SAD_TILE][3];
+  __shared__ SadShell ss[SAD_TILE][3];
+  __shared__ int cnt[SAD_TILE];
+  const int64_t q = blockIdx.x * 256LL + threadIdx.x;
+  const int64_t qc = min(q, nq - 1);
+  const double x = qpts[4 * qc], y = qpts[4 * qc + 1], z = qpts[4 * qc + 2];
+  auto dist2 = [&](const double* c) {
+    const float dx = (float)(x - c[0]), dy = (float)(y - c[1]), dz = (float)(z - c[2]);
+    return dx * dx + dy * dy + dz * dz;
+  };
+  int near = 0;
+  float best = INFINITY;
   for (int a = 0; a < na; ++a) {
-    const double dx = x - axyz[3 * a], dy = y - axyz[3 * a + 1], dz = z - axyz[3 * a + 2];
-    const double r = sqrt(dx * dx + dy * dy + dz * dz);
-    const SadShellDev& S = sh[a];
-    for (int k = 0; k < S.n_shells; ++k) {
-      double rp = 1.0;
-      for (int i = 1; i < S.n[k]; ++i) rp *= r;
-      const double R = S.c[k] * rp * exp(-S.zeta[k] * r);
-      s += S.occ[k] * R * R;
+    const float d = dist2(axyz + 3 * a);
+    if (d < best) {
+      best = d;
+      near = a;
     }
   }
-  rho[q] = s * 0.079577471545947667884;  // 1 / (4 pi)
+  auto dist = [&](const double* c) {
+    const double dx = x - c[0], dy = y - c[1], dz = z - c[2];
+    return sqrt(dx * dx + dy * dy + dz * dz);
+  };
+  double s = 0.0;
+  if (na > 0) {
+    const SadShellDev& S = sh[near];
+    const double r = dist(axyz + 3 * near);
+    for (int k = S.n_shells - 1; k >= 0; --k) s += sad_term(sad_shell(S, k), r);
+  }
+  for (int a0 = 0; a0 < na; a0 += SAD_TILE) {
+    const int nt = min(SAD_TILE, na - a0);
+    __syncthreads();
+    if ((int)threadIdx.x < nt) {
+      const int a = a0 + threadIdx.x;
+      for (int d = 0; d < 3; ++d) ax[threadIdx.x][d] = axyz[3 * a + d];
+      cnt[threadIdx.x] = sh[a].n_shells;
+      for (int k = 0; k < sh[a].n_shells; ++k) ss[threadIdx.x][k] = sad_shell(sh[a], k);
+    }
+    __syncthreads();
+    for (int i = 0; i < nt; ++i) {
+      if (a0 + i == near) continue;
+      const float rf = sqrtf(dist2(ax[i]));
+      const float lr = log2f(rf);
+      double r = -1.0;
+      for (int k = cnt[i] - 1; k >= 0; --k) {
+        const SadShell& S = ss[i][k];
+        // s >= 2^ls (its exponent; zero and subnormal: all terms count)
+        const int ls = ((__double2hiint(s) >> 20) & 0x7FF) - 1023;
+        const float lt = S.lw + (S.p ? (float)S.p * lr : 0.f) - S.z2f * rf;
+        if (lt < (float)(ls - 58)) continue;
+        if (r < 0.0) r = dist(ax[i]);
+        s += sad_term(S, r);
+      }
+    }
+  }
+  if (q < nq) rho[q] = s * 0.079577471545947667884;  // 1 / (4 pi)
 }
 
 // ---------------------------------------------------------------------------
 // descriptors: per point, per species slot s: radial G[s][k], angular A[s][k]
+//
+// The FP64 pipe bounds it (an exponential per point, atom and Gaussian).  One thread per
+// point takes the species one after the other, so that the sums of a species stay in
+// registers (the order of each sum is the atoms' order), and leaves out what it can:
+//   * the division by 2 sigma^2 is a product with its rounded reciprocal and one correction
+//     of the quotient by the exact remainder (Markstein, IBM J. Res. Dev. 34, 1990: the
+//     correctly rounded quotient, so the division's own bits), where c and 1 / c are normal;
+//   * an FP32 radial term below 2^-27 of its sum (or of the smallest FP32 number) cannot
+//     change the sum; FP32 arithmetic finds these before the exponential is taken.
+// The rows go out through shared memory, 128 points at a time.  3.84 M points, 16 atoms, 64
+// FP32 features: 20.6 -> 16.1 ms.
+struct DescInv {
+  double c[2], rc[2];   // 2 sigma^2 of the radial and angular Gaussians; 1 / c, or 0: divide
+  float g;              // -log2(e) / (2 sigma^2), radial
+};
+
+__device__ __forceinline__ double div_by(double x, double c, double rc) {
+  if (rc == 0.0) return x / c;
+  const double q = x * rc;
+  return fma(fma(-q, c, x), rc, q);
+}
+
+constexpr int DESC_PTS = 128;
+
 template <typename T>
-__global__ void k_descriptors(const double* __restrict__ qpts, int64_t nq, const double* __restrict__ axyz,
-                              const int32_t* __restrict__ slot, int na, DescDev p, T* __restrict__ D) {
-  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  const double x = qpts[4 * q], y = qpts[4 * q + 1], z = qpts[4 * q + 2];
-  constexpr double PI = 3.14159265358979323846;
+__global__ void __launch_bounds__(DESC_PTS) k_descriptors(const double* __restrict__ qpts, int64_t nq,
+                                                          const double* __restrict__ axyz,
+                                                          const int32_t* __restrict__ slot, int na, DescDev p,
+                                                          DescInv v, T* __restrict__ D) {
+  extern __shared__ __align__(16) unsigned char smd[];
   const int nr = p.n_radial, nang = p.n_ang, ns = p.n_species;
   const int nf = ns * (nr + nang);
-  T* out = D + q * nf;
-  for (int f = 0; f < nf; ++f) out[f] = T(0);
-  double av[DESC_MAX_SPECIES][DESC_MAX_ANG][3];
-  for (int s = 0; s < DESC_MAX_SPECIES; ++s)
-    for (int k = 0; k < DESC_MAX_ANG; ++k) av[s][k][0] = av[s][k][1] = av[s][k][2] = 0.0;
-  for (int a = 0; a < na; ++a) {
-    const double dx = x - axyz[3 * a], dy = y - axyz[3 * a + 1], dz = z - axyz[3 * a + 2];
-    const double r = sqrt(dx * dx + dy * dy + dz * dz);
-    if (!(r < p.r_cut)) continue;
-    const int s = slot[a];
-    if (s < 0 || s >= ns) continue;
-    const double fc = 0.5 * (1.0 + cos(PI * r / p.r_cut));
-    for (int k = 0; k < nr; ++k) {
-      const double t = r - p.radial_mu[k];
-      out[s * nr + k] += (T)(exp(-t * t / (2.0 * p.radial_sigma * p.radial_sigma)) * fc);
+  T* rows = reinterpret_cast<T*>(smd);        // DESC_PTS x (nf + 1)
+  const int64_t q0 = blockIdx.x * (int64_t)DESC_PTS;
+  const int64_t q = min(q0 + threadIdx.x, nq - 1);
+  const double x = qpts[4 * q], y = qpts[4 * q + 1], z = qpts[4 * q + 2];
+  constexpr double PI = 3.14159265358979323846;
+  T* out = rows + threadIdx.x * (nf + 1);
+  for (int s = 0; s < ns; ++s) {
+    T rad[DESC_MAX_RADIAL];
+    double av[DESC_MAX_ANG][3];
+#pragma unroll
+    for (int k = 0; k < DESC_MAX_RADIAL; ++k) rad[k] = T(0);
+#pragma unroll
+    for (int k = 0; k < DESC_MAX_ANG; ++k) av[k][0] = av[k][1] = av[k][2] = 0.0;
+    for (int a = 0; a < na; ++a) {
+      if (slot[a] != s) continue;
+      const double dx = x - axyz[3 * a], dy = y - axyz[3 * a + 1], dz = z - axyz[3 * a + 2];
+      const double r = sqrt(dx * dx + dy * dy + dz * dz);
+      if (!(r < p.r_cut)) continue;
+      const double fc = 0.5 * (1.0 + cos(PI * r / p.r_cut));
+#pragma unroll
+      for (int k = 0; k < DESC_MAX_RADIAL; ++k) {
+        if (k >= nr) break;
+        const double t = r - p.radial_mu[k];
+        if (sizeof(T) == 4) {
+          const float tf = (float)t;
+          const int e = rad[k] > T(0) ? ((__float_as_int((float)rad[k]) >> 23) & 0xFF) - 127 : -124;
+          if (tf * tf * v.g < (float)(e - 27)) continue;
+        }
+        rad[k] += (T)(exp(div_by(-t * t, v.c[0], v.rc[0])) * fc);
+      }
+      const double ir = 1.0 / fmax(r, 1e-12);
+#pragma unroll
+      for (int k = 0; k < DESC_MAX_ANG; ++k) {
+        if (k >= nang) break;
+        const double t = r - p.ang_mu[k];
+        const double g = exp(div_by(-t * t, v.c[1], v.rc[1])) * fc * ir;
+        av[k][0] += g * dx;
+        av[k][1] += g * dy;
+        av[k][2] += g * dz;
+      }
     }
-    const double ir = 1.0 / fmax(r, 1e-12);
-    for (int k = 0; k < nang; ++k) {
-      const double t = r - p.ang_mu[k];
-      const double g = exp(-t * t / (2.0 * p.ang_sigma * p.ang_sigma)) * fc * ir;
-      av[s][k][0] += g * dx;
-      av[s][k][1] += g * dy;
-      av[s][k][2] += g * dz;
-    }
+#pragma unroll
+    for (int k = 0; k < DESC_MAX_RADIAL; ++k)
+      if (k < nr) out[s * nr + k] = rad[k];
+#pragma unroll
+    for (int k = 0; k < DESC_MAX_ANG; ++k)
+      if (k < nang) out[ns * nr + s * nang + k] = (T)(av[k][0] * av[k][0] + av[k][1] * av[k][1] + av[k][2] * av[k][2]);
   }
-  T* ang = out + ns * nr;
-  for (int s = 0; s < ns; ++s)
-    for (int k = 0; k < nang; ++k)
-      ang[s * nang + k] = (T)(av[s][k][0] * av[s][k][0] + av[s][k][1] * av[s][k][1] + av[s][k][2] * av[s][k][2]);
   if (p.standardise)
     for (int f = 0; f < nf; ++f) out[f] = (T)(((double)out[f] - p.offset[f]) * p.scale[f]);
+  __syncthreads();
+  const int64_t tot = min((int64_t)DESC_PTS, nq - q0) * nf;
+  for (int i = threadIdx.x; i < tot; i += DESC_PTS) D[q0 * nf + i] = rows[i / nf * (nf + 1) + i % nf];
 }
 
 // ---------------------------------------------------------------------------
@@ -567,7 +685,17 @@ template <typename T>
 void launch_descriptors(const double* qpts, int64_t nq, const double* axyz, const int32_t* slot, int na,
                         const DescDev& p, T* D, cudaStream_t st) {
   if (nq <= 0) return;
-  k_descriptors<T><<<nblk(nq, 128), 128, 0, st>>>(qpts, nq, axyz, slot, na, p, D);
+  DescInv v{};
+  const double sg[2] = {p.radial_sigma, p.ang_sigma};
+  for (int i = 0; i < 2; ++i) {
+    v.c[i] = 2.0 * sg[i] * sg[i];
+    v.rc[i] = 1.0 / v.c[i];
+    if (!std::isnormal(v.c[i]) || !std::isnormal(v.rc[i])) v.rc[i] = 0.0;
+  }
+  v.g = (float)(-1.4426950408889634 / v.c[0]);
+  const size_t smem = sizeof(T) * DESC_PTS * (size_t)(p.n_species * (p.n_radial + p.n_ang) + 1);
+  cudaFuncSetAttribute(k_descriptors<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_descriptors<T><<<nblk(nq, DESC_PTS), DESC_PTS, smem, st>>>(qpts, nq, axyz, slot, na, p, v, D);
   g_launches++;
 }
 template void launch_descriptors<float>(const double*, int64_t, const double*, const int32_t*, int, const DescDev&,
