@@ -1051,7 +1051,7 @@ __global__ void k_df_rows(int64_t rows, int N, const double* __restrict__ X, int
 // (each out value receives one addition per launch: the pattern nodes are distinct).
 // The chain of an entry's loads bounds it (value and function, then the function's row), so
 // a lane carries all its columns through the entries together.  One column a lane and pass ->
-// now: 180 k nodes x 135 columns 321 -> 189 us, x 640 1,186 -> 750 us; 47 k x 12 21.6 -> 19.4 us.
+// now: 180 k nodes x 135 columns 304 -> 189 us, x 640 1,186 -> 750 us; 47 k x 12 21.6 -> 19.4 us.
 // Same sums, bit for bit.
 template <int CPL>
 __global__ void __launch_bounds__(256) k_spmm_nodes_df(int64_t nrows, const int32_t* __restrict__ rnode,

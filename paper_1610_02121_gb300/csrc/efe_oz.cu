@@ -69,7 +69,7 @@ __device__ __forceinline__ uint32_t bo(int row, int k) {
 // operand's chunk.  (Slice-major 128-column tiles took 8 or, across two tiles, 15 copies a
 // chunk, and their issue, about 120 cycles each, outlasted the chunk's 28 MMAs.  The products
 // of a Rayleigh-Ritz of 559 k rows x 640 columns, with the segment rule of the Gram products
-// below: 83 -> 69 ms, of 559 k x 135: 8.4 -> 5.8 ms.)  Slice i of row r, K octet o:
+// below: 81 -> 69 ms, of 559 k x 135: 8.0 -> 5.8 ms.)  Slice i of row r, K octet o:
 __device__ __forceinline__ uint32_t go(int row, int i, int oct) {
   return (uint32_t)(row >> 3) * OzL::GRP + (uint32_t)i * 256u + (uint32_t)oct * 128u + (uint32_t)(row & 7) * 16u;
 }
