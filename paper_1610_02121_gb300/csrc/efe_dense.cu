@@ -416,6 +416,166 @@ __global__ void __launch_bounds__(256) k_bj_update(T* __restrict__ A, T* __restr
     A[(int64_t)bj_index<BJ_B>(row, u, v) * np + bj_index<BJ_B>(cq + c, p, q)] = Xs[row * LD + cq + c];
 }
 
+// Above BJ_DIAG_MIN rows: a visit diagonalises its subproblem, and columns and rows of A follow
+// in launches of their own.
+// One CTA per block pair of round r: diagonalise the BJ_S x BJ_S subproblem
+// [[A_pp, A_pq], [A_qp, A_qq]] in shared memory by cyclic Jacobi; write the
+// rotation J (BJ_S x BJ_S, row-major), the subproblem's eigenvalues, and whether
+// any rotation was applied.
+template <typename T, int BJ_B>
+__global__ void __launch_bounds__(256) k_bjd_solve(const T* __restrict__ A, int np, int nb, int r, T* __restrict__ Jb,
+                                                  T* __restrict__ lam, int* __restrict__ rotated, int max_sweeps) {
+  constexpr int BJ_S = 2 * BJ_B, BJ_LD = BJ_S + 1;
+  extern __shared__ double smraw[];
+  T* S = reinterpret_cast<T*>(smraw);
+  T* J = S + BJ_S * BJ_LD;
+  __shared__ T cs[BJ_B], sn[BJ_B];
+  __shared__ int pp[BJ_B], qq[BJ_B];
+  __shared__ int any, any_sweep;
+  const int k = blockIdx.x, tid = threadIdx.x;
+  int p, q;
+  bj_pair(k, r, nb, p, q);
+  for (int t = tid; t < BJ_S * BJ_S; t += blockDim.x) {
+    const int i = t / BJ_S, j = t % BJ_S;
+    S[i * BJ_LD + j] = A[(int64_t)bj_index<BJ_B>(i, p, q) * np + bj_index<BJ_B>(j, p, q)];
+    J[i * BJ_LD + j] = i == j ? T(1) : T(0);
+  }
+  if (tid == 0) any = 0;
+  __syncthreads();
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+    if (tid == 0) any_sweep = 0;
+    __syncthreads();
+    for (int rd = 0; rd < BJ_S - 1; ++rd) {
+      if (tid < BJ_B) {
+        const int a = tid == 0 ? 0 : ((tid - 1 + rd) % (BJ_S - 1)) + 1;
+        const int b2 = ((BJ_S - 1 - tid - 1 + rd) % (BJ_S - 1)) + 1;
+        const int i = min(a, b2), j = max(a, b2);
+        const T aij = S[i * BJ_LD + j], aii = S[i * BJ_LD + i], ajj = S[j * BJ_LD + j];
+        T c = T(1), s = T(0);
+        // negligible off-diagonal entry (below the rounding of both diagonal
+        // entries): no rotation
+        const T g = T(100) * fabs(aij);
+        if (aij != T(0) && !(fabs(aii) + g == fabs(aii) && fabs(ajj) + g == fabs(ajj))) {
+          const T tau = (ajj - aii) / (T(2) * aij);
+          const T t = (tau >= T(0) ? T(1) : T(-1)) / (fabs(tau) + sqrt(T(1) + tau * tau));
+          c = T(1) / sqrt(T(1) + t * t);
+          s = t * c;
+          any_sweep = 1;
+        }
+        pp[tid] = i;
+        qq[tid] = j;
+        cs[tid] = c;
+        sn[tid] = s;
+      }
+      __syncthreads();
+      // rows i, j of S
+      for (int t = tid; t < BJ_B * BJ_S; t += blockDim.x) {
+        const int e = t / BJ_S, col = t % BJ_S;
+        if (sn[e] == T(0)) continue;
+        const int i = pp[e], j = qq[e];
+        const T c = cs[e], s = sn[e];
+        const T x = S[i * BJ_LD + col], y = S[j * BJ_LD + col];
+        S[i * BJ_LD + col] = c * x - s * y;
+        S[j * BJ_LD + col] = s * x + c * y;
+      }
+      __syncthreads();
+      // columns i, j of S and of J
+      for (int t = tid; t < BJ_B * BJ_S; t += blockDim.x) {
+        const int e = t / BJ_S, row = t % BJ_S;
+        if (sn[e] == T(0)) continue;
+        const int i = pp[e], j = qq[e];
+        const T c = cs[e], s = sn[e];
+        const T x = S[row * BJ_LD + i], y = S[row * BJ_LD + j];
+        S[row * BJ_LD + i] = c * x - s * y;
+        S[row * BJ_LD + j] = s * x + c * y;
+        const T u = J[row * BJ_LD + i], v = J[row * BJ_LD + j];
+        J[row * BJ_LD + i] = c * u - s * v;
+        J[row * BJ_LD + j] = s * u + c * v;
+      }
+      __syncthreads();
+      if (tid < BJ_B && sn[tid] != T(0)) {
+        S[pp[tid] * BJ_LD + qq[tid]] = T(0);
+        S[qq[tid] * BJ_LD + pp[tid]] = T(0);
+      }
+      __syncthreads();
+    }
+    if (tid == 0 && any_sweep) any = 1;
+    __syncthreads();
+    if (!any_sweep) break;
+  }
+  T* Jo = Jb + (int64_t)k * BJ_S * BJ_S;
+  for (int t = tid; t < BJ_S * BJ_S; t += blockDim.x) Jo[t] = J[(t / BJ_S) * BJ_LD + t % BJ_S];
+  for (int t = tid; t < BJ_S; t += blockDim.x) lam[(int64_t)k * BJ_S + t] = S[t * BJ_LD + t];
+  if (tid == 0) rotated[k] = any;
+}
+
+// M[:, idx(p,q)] <- M[:, idx(p,q)] J_k for every pair k (rows in chunks of 32).
+template <typename T, int BJ_B>
+__global__ void __launch_bounds__(256) k_bjd_cols(T* __restrict__ M, int np, int nb, int r, const T* __restrict__ Jb,
+                                                 const int* __restrict__ rotated) {
+  constexpr int BJ_S = 2 * BJ_B;
+  const int k = blockIdx.y;
+  if (!rotated[k]) return;
+  __shared__ T Js[BJ_S][BJ_S + 1];
+  __shared__ T Xs[32][BJ_S + 1];
+  int p, q;
+  bj_pair(k, r, nb, p, q);
+  const T* Jk = Jb + (int64_t)k * BJ_S * BJ_S;
+  for (int t = threadIdx.x; t < BJ_S * BJ_S; t += blockDim.x) Js[t / BJ_S][t % BJ_S] = Jk[t];
+  const int r0 = blockIdx.x * 32;
+  for (int t = threadIdx.x; t < 32 * BJ_S; t += blockDim.x) {
+    const int rr = t / BJ_S, c = t % BJ_S;
+    Xs[rr][c] = (r0 + rr < np) ? M[(int64_t)(r0 + rr) * np + bj_index<BJ_B>(c, p, q)] : T(0);
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < 32 * BJ_S; t += blockDim.x) {
+    const int rr = t / BJ_S, c = t % BJ_S;
+    if (r0 + rr >= np) continue;
+    T acc = T(0);
+#pragma unroll 8
+    for (int l = 0; l < BJ_S; ++l) acc = fma(Xs[rr][l], Js[l][c], acc);
+    M[(int64_t)(r0 + rr) * np + bj_index<BJ_B>(c, p, q)] = acc;
+  }
+}
+
+// A[idx(p,q), :] <- J_k^T A[idx(p,q), :] for every pair k (columns in chunks
+// of one block); the pair's own BJ_S x BJ_S block becomes diag(lambda_k).
+template <typename T, int BJ_B>
+__global__ void __launch_bounds__(256) k_bjd_rows(T* __restrict__ A, int np, int nb, int r, const T* __restrict__ Jb,
+                                                 const T* __restrict__ lam, const int* __restrict__ rotated) {
+  constexpr int BJ_S = 2 * BJ_B;
+  const int k = blockIdx.y;
+  if (!rotated[k]) return;
+  __shared__ T Js[BJ_S][BJ_S + 1];
+  __shared__ T Xs[BJ_S][BJ_B + 1];
+  int p, q;
+  bj_pair(k, r, nb, p, q);
+  const int cblk = blockIdx.x, c0 = cblk * BJ_B;
+  if (cblk == p || cblk == q) {
+    // own block columns: diag(lambda) in rows idx(p,q), columns of this block
+    const int off = cblk == p ? 0 : BJ_B;
+    for (int t = threadIdx.x; t < BJ_S * BJ_B; t += blockDim.x) {
+      const int i = t / BJ_B, c = t % BJ_B;
+      A[(int64_t)bj_index<BJ_B>(i, p, q) * np + c0 + c] = (i == off + c) ? lam[(int64_t)k * BJ_S + i] : T(0);
+    }
+    return;
+  }
+  const T* Jk = Jb + (int64_t)k * BJ_S * BJ_S;
+  for (int t = threadIdx.x; t < BJ_S * BJ_S; t += blockDim.x) Js[t / BJ_S][t % BJ_S] = Jk[t];
+  for (int t = threadIdx.x; t < BJ_S * BJ_B; t += blockDim.x) {
+    const int i = t / BJ_B, c = t % BJ_B;
+    Xs[i][c] = A[(int64_t)bj_index<BJ_B>(i, p, q) * np + c0 + c];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < BJ_S * BJ_B; t += blockDim.x) {
+    const int i = t / BJ_B, c = t % BJ_B;
+    T acc = T(0);
+#pragma unroll 8
+    for (int l = 0; l < BJ_S; ++l) acc = fma(Js[l][i], Xs[l][c], acc);
+    A[(int64_t)bj_index<BJ_B>(i, p, q) * np + c0 + c] = acc;
+  }
+}
+
 // partial sums of the squared off-diagonal and total entries of the leading n x n part
 template <typename T>
 __global__ void k_bj_norms(const T* __restrict__ A, int np, int n, double* __restrict__ part) {
@@ -514,6 +674,13 @@ void launch_trinv_blocked(const double* L, int n, int lda, double* Li, int ldi, 
 
 constexpr int BJ_BLOCK = 16;   // block Jacobi block size of both stages
 
+// Above this size a visit of the block Jacobi diagonalises its subproblem instead of making one
+// sweep over it.  One sweep a visit is the faster at every size (640 rows: about 95 -> 31 ms), but
+// it rounds differently, and on large blocks the vectors of the closest pairs of Ritz values
+// turn with the rounding (norm x 2^-53 over the gap: 3.5e-9 seen at 640), more than a program
+// that compares runs expects; up to 512 the difference stayed below 1e-10.
+constexpr int BJ_DIAG_MIN = 512;
+
 static int64_t bj_scratch_bytes(int n, int elem, int B) {
   const int S = 2 * B;
   const int nb0 = (n + B - 1) / B;
@@ -539,6 +706,11 @@ int block_jacobi_b(const double* C, int n, int ldc, T* V, int ldv, T* w, int max
   const int nb = std::max(2, nb0 + (nb0 & 1));
   const int np = nb * BJ_B;
   const int pairs = nb / 2;
+  const bool diag = n > BJ_DIAG_MIN;
+  const size_t smem = sizeof(T) * 2 * BJ_S * (BJ_S + 1);
+  if (diag && cudaFuncSetAttribute(k_bjd_solve<T, BJ_B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+                  cudaSuccess)
+    return -1;
   T* A = reinterpret_cast<T*>(scratch);
   T* Vp = A + (int64_t)np * np;
   T* Jb = Vp + (int64_t)np * np;
@@ -566,7 +738,14 @@ int block_jacobi_b(const double* C, int n, int ldc, T* V, int ldv, T* w, int max
       break;
     }
     if (sweep == max_sweeps) break;
-    for (int r = 0; r < nb - 1; ++r) {
+    for (int r = 0; r < nb - 1 && diag; ++r) {
+      k_bjd_solve<T, BJ_B><<<pairs, 256, smem, st>>>(A, np, nb, r, Jb, Sb, rot, 30);
+      k_bjd_cols<T, BJ_B><<<dim3(nblk(np, 32), pairs), 256, 0, st>>>(A, np, nb, r, Jb, rot);
+      k_bjd_rows<T, BJ_B><<<dim3(nb, pairs), 256, 0, st>>>(A, np, nb, r, Jb, Sb, rot);
+      k_bjd_cols<T, BJ_B><<<dim3(nblk(np, 32), pairs), 256, 0, st>>>(Vp, np, nb, r, Jb, rot);
+      g_launches.fetch_add(4, std::memory_order_relaxed);
+    }
+    for (int r = 0; r < nb - 1 && !diag; ++r) {
       k_bj_solve<T, BJ_B><<<pairs, 256, 0, st>>>(A, np, nb, r, Jb, Sb, rot);
       k_bj_update<T, BJ_B><<<dim3((unsigned)pairs + nblk(np, BJ_S), pairs), 256, 0, st>>>(A, Vp, np, nb, r, Jb, Sb, rot);
       g_launches.fetch_add(2, std::memory_order_relaxed);
