@@ -1973,17 +1973,13 @@ int dense_scratch(efe_handle* h, int64_t bytes) {
 // the blocked ones, of 48 the same, of 12 2.36 and 2.39.  DENSE_SMALL_MAX: the N x N
 // products go to the tensor-core FP64 engine above it.
 constexpr int CHOL_ONE_CTA_MAX = 64;
-// From 513 to 2,048 columns the one-CTA factor again, although the blocked one is the faster:
-// it adds in another order, and on blocks this large the vectors of the closest pairs of Ritz
-// values turn with that rounding (3.7e-9 seen at 640 columns, against 5e-12 with the same order).
-constexpr int CHOL_BLOCKED_MAX = 512, CHOL_BLOCKED_FROM = 2049;
 constexpr int EIG_ONE_CTA_MAX = 48;
 constexpr int DENSE_SMALL_MAX = 512;
 
 // A = L L^T in place (lower, n x n, ld n); *info: 0 or j + 1 of the first breakdown
 int chol_lower(efe_handle* h, double* A, int n, cudaStream_t st, double* min_ratio, int* info = nullptr) {
   if (!info) info = h->info;
-  if ((n <= CHOL_ONE_CTA_MAX || (n > CHOL_BLOCKED_MAX && n < CHOL_BLOCKED_FROM)) && !h->opt_dense_blocked) {
+  if (n <= CHOL_ONE_CTA_MAX && !h->opt_dense_blocked) {
     launch_chol(A, n, n, info, st, min_ratio);
   } else {
     TRY(dense_scratch(h, (int64_t)sizeof(double) * chol_blocked_scratch(n)));

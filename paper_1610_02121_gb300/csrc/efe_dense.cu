@@ -92,6 +92,56 @@ __global__ void __launch_bounds__(128) k_chol_panel(double* A, int lda, int j0, 
   for (int k = 0; k < b; ++k) row[k] = x[k];
 }
 
+// A22 -= L21 L21^T, lower triangle: every entry takes the panel's products one after the other
+// in column order, as the one-CTA factor does (k_chol; the diagonal and panel kernels above
+// keep that order too), so that both give the same bits.  64 x 64 tiles, 4 x 4 a thread; the
+// panel's 64 terms a tile bound it (FP64 pipe).  640 columns, Rayleigh-Ritz call: one-CTA factor
+// 278 ms, this 201 ms.
+__global__ void __launch_bounds__(256) k_chol_update(double* A, int lda, int j0, int b, int n) {
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ double Pr[64][33], Pc[64][33];
+  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16, o = j0 + b;
+  const int i0 = o + blockIdx.y * 64, c0 = o + blockIdx.x * 64;
+  double v[4][4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int i = i0 + ty + 16 * u, c = c0 + tx + 16 * w;
+      v[u][w] = i < n && c <= i ? A[(int64_t)i * lda + c] : 0.0;
+    }
+  for (int k0 = 0; k0 < b; k0 += 32) {
+    __syncthreads();
+    for (int t = tid; t < 64 * 32; t += 256) {
+      const int r = t / 32, k = t % 32;
+      const bool in = k0 + k < b;
+      Pr[r][k] = in && i0 + r < n ? A[(int64_t)(i0 + r) * lda + j0 + k0 + k] : 0.0;
+      Pc[r][k] = in && c0 + r < n ? A[(int64_t)(c0 + r) * lda + j0 + k0 + k] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < 32; ++k) {
+      double p[4], q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        p[u] = Pr[ty + 16 * u][k];
+        q[u] = Pc[tx + 16 * u][k];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int w = 0; w < 4; ++w) v[u][w] = fma(-p[u], q[w], v[u][w]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int i = i0 + ty + 16 * u, c = c0 + tx + 16 * w;
+      if (i < n && c <= i) A[(int64_t)i * lda + c] = v[u][w];
+    }
+}
+
 // T (b x m, ld m) = transpose of the panel rows j0+b .. n-1, columns j0 .. j0+b-1
 __global__ void k_panel_transpose(const double* A, int lda, int j0, int b, int n, double* T) {
   const int m = n - j0 - b;
@@ -619,6 +669,10 @@ constexpr int BJ_NORM_BLOCKS = 128;
 }  // namespace
 
 // ------------------------------------------------------------------ host side
+// up to the one-CTA kernel's largest size the trailing update keeps that kernel's order
+// of sums (close pairs of Ritz vectors turn with the rounding); a tiled product above
+constexpr int CHOL_ORDERED_MAX = 2048;
+
 void launch_chol_blocked(double* A, int n, int lda, int* info, double* min_ratio, double* scratch,
                          cudaStream_t st) {
   // scratch: n (original diagonal) + CB * n (transposed panel) doubles
@@ -636,6 +690,11 @@ void launch_chol_blocked(double* A, int n, int lda, int* info, double* min_ratio
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (m <= 0) break;
     k_chol_panel<<<nblk(m, 128), 128, 0, st>>>(A, lda, j0, b, n);
+    if (n <= CHOL_ORDERED_MAX) {
+      k_chol_update<<<dim3(nblk(m, 64), nblk(m, 64)), 256, 0, st>>>(A, lda, j0, b, n);
+      g_launches.fetch_add(2, std::memory_order_relaxed);
+      continue;
+    }
     k_panel_transpose<<<nblk((int64_t)m * b, 256), 256, 0, st>>>(A, lda, j0, b, n, T);
     g_launches.fetch_add(2, std::memory_order_relaxed);
     // A22 -= L21 L21^T (the whole square; only its lower triangle is used)
@@ -677,7 +736,8 @@ constexpr int BJ_BLOCK = 16;   // block Jacobi block size of both stages
 // Above this size a visit of the block Jacobi diagonalises its subproblem instead of making one
 // sweep over it.  One sweep a visit is the faster at every size (640 rows: about 95 -> 31 ms), but
 // it rounds differently, and on large blocks the vectors of the closest pairs of Ritz values
-// turn with the rounding (norm x 2^-53 over the gap: 3.5e-9 seen at 640), more than a program
+// turn with the rounding (norm x 2^-53 over the gap: 3.5e-9 seen at 640, 5e-12 with both the
+// diagonalising visits and the ordered Cholesky), more than a program
 // that compares runs expects; up to 512 the difference stayed below 1e-10.
 constexpr int BJ_DIAG_MIN = 512;
 
