@@ -66,7 +66,9 @@ struct efe_handle {
   unsigned char* ozc_digits = nullptr;   // FP64 engine's cell products: digit planes of a column panel,
   double* ozc_products = nullptr;        // its products (grow-only)
   int64_t ozc_digits_bytes = 0, ozc_products_bytes = 0;
-  int64_t ws_gen = 0;       // counts reallocations of workspace that a recorded graph may point to
+  // counts everything a recorded batch graph depends on: reallocated workspace, the FP64
+  // engine, options that pick kernels, the tuned column tile
+  int64_t graph_gen = 0;
   int* oz_fexp = nullptr;   // per-column exponents (N, readable up to a multiple of 16)
   int* oz_bexp = nullptr;   // per-column exponents of small right-hand matrices (N)
   int* oz_aexp = nullptr;   // per-row exponents of tall left-hand matrices (rows)
@@ -313,7 +315,7 @@ void free32(efe_handle* h) {
 
 int reserve(efe_handle* h, int N) {
   if (N <= h->Nres) return EFE_OK;
-  h->ws_gen++;
+  h->graph_gen++;
   free32(h);
   for (void* p : {(void*)h->B1, (void*)h->B2, (void*)h->W, (void*)h->xe, (void*)h->rb, (void*)h->part,
                   (void*)h->small, (void*)h->tnwork, (void*)h->rpart})
@@ -361,7 +363,7 @@ int reserve(efe_handle* h, int N) {
 int reserve32(efe_handle* h, int N) {
   if (N <= h->Nres32) return EFE_OK;
   TRY(reserve(h, std::max(N, h->Nres)));
-  h->ws_gen++;
+  h->graph_gen++;
   free32(h);
   // classical rows padded to a multiple of 8 elements: 16-byte aligned rows for
   // vector loads and bulk copies; the padding columns are zero and stay zero
@@ -503,7 +505,7 @@ int oz_cell_scratch(efe_handle* h, int N, int* panel) {
     dfree(h, h->ozc_digits);
     h->ozc_digits = nullptr;
     h->ozc_digits_bytes = 0;
-    h->ws_gen++;
+    h->graph_gen++;
     TRY(dalloc(h, &h->ozc_digits, db));
     h->ozc_digits_bytes = db;
   }
@@ -511,7 +513,7 @@ int oz_cell_scratch(efe_handle* h, int N, int* panel) {
     dfree(h, h->ozc_products);
     h->ozc_products = nullptr;
     h->ozc_products_bytes = 0;
-    h->ws_gen++;
+    h->graph_gen++;
     TRY(dalloc(h, &h->ozc_products, pb / (int64_t)sizeof(double)));
     h->ozc_products_bytes = pb;
   }
@@ -2330,12 +2332,14 @@ int efe_rayleigh_ritz(efe_handle* h, double* X, int64_t ldx, int32_t N, double* 
 
 int efe_set_fp64_engine(efe_handle* h, int32_t engine) {
   if (!h || (engine != 0 && engine != 1)) return EFE_ERR_ARG;
+  if (h->fp64_engine != engine) h->graph_gen++;
   h->fp64_engine = engine;
   return EFE_OK;
 }
 
 int efe_set_option(efe_handle* h, int32_t option, int64_t value) {
   if (!h || value < 0) return EFE_ERR_ARG;
+  h->graph_gen++;
   switch (option) {
     case EFE_OPT_GRID_CAP:
       if (value > (1 << 20)) return EFE_ERR_ARG;
@@ -2960,6 +2964,7 @@ int efe_autotune(efe_handle* h, int32_t N, int32_t precision, int32_t* tile_out,
   }
   h->tc_tile = best;
   h->tc_tile_N = N;
+  h->graph_gen++;
   if (tile_out) *tile_out = best;
   return EFE_OK;
 }
@@ -2979,8 +2984,8 @@ struct efe_batch {
   std::vector<double*> X;
   std::vector<int64_t> ldx;
   std::vector<int32_t> N;
-  std::vector<int64_t> gen;   // workspace generation of every handle (efe_handle::ws_gen)
-  int m = 0, precision = -1, fp64_tail = -1, engine = -1;
+  std::vector<int64_t> gen;   // of every handle (efe_handle::graph_gen)
+  int m = 0, precision = -1, fp64_tail = -1;
   std::string err;
 };
 
@@ -3087,9 +3092,9 @@ int efe_batch_chfsi_step(efe_batch* b, double* const* X, const int64_t* ldx, con
     h->coef_pending = false;
   }
   bool same = b->exec && b->m == m && b->precision == precision && b->fp64_tail == fp64_tail &&
-              (int)b->X.size() == n && b->engine == b->hs[0]->fp64_engine;
+              (int)b->X.size() == n;
   for (int i = 0; same && i < n; ++i)
-    same = b->X[i] == X[i] && b->ldx[i] == ldx[i] && b->N[i] == N[i] && b->gen[i] == b->hs[i]->ws_gen;
+    same = b->X[i] == X[i] && b->ldx[i] == ldx[i] && b->N[i] == N[i] && b->gen[i] == b->hs[i]->graph_gen;
   if (!same) {
     batch_clear_graph(b);
     const int64_t l0 = g_launches.load();
@@ -3147,11 +3152,10 @@ int efe_batch_chfsi_step(efe_batch* b, double* const* X, const int64_t* ldx, con
     b->ldx.assign(ldx, ldx + n);
     b->N.assign(N, N + n);
     b->gen.resize(n);
-    for (int i = 0; i < n; ++i) b->gen[i] = b->hs[i]->ws_gen;
+    for (int i = 0; i < n; ++i) b->gen[i] = b->hs[i]->graph_gen;
     b->m = m;
     b->precision = precision;
     b->fp64_tail = fp64_tail;
-    b->engine = b->hs[0]->fp64_engine;
   }
   // refresh the staged coefficients (read by the graph's copy nodes), then replay
   for (int i = 0; i < n; ++i) {

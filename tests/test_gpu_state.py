@@ -1,0 +1,69 @@
+"""Handles and batches whose settings or workspaces change between calls: a recorded graph
+must follow them, and no call may meet freed or stale memory."""
+import pytest
+
+import workloads as W
+from tests.gpu_util import cuda_available, gpu_system, to_dev, torch
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")]
+
+
+@pytest.fixture()
+def members():
+    from paper_1610_02121_gb300 import Batch
+    ss = [W.tiny(seed=11), W.tiny(seed=12, cells=(3, 2, 2))]
+    Gs = [gpu_system(s) for s in ss]
+    Xs = [to_dev(W.initial_block(s, N, seed=3 + i)) for i, (s, N) in enumerate(zip(ss, (12, 20)))]
+    bounds = [[], [], []]
+    for G, X in zip(Gs, Xs):
+        e, _ = G.rayleigh_ritz(X)
+        for v, x in zip(bounds, (e.max(), G.upper_bound(X[:, -1].contiguous(), 10), e.min())):
+            v.append(x)
+    B = Batch(Gs)
+    yield Gs, Xs, bounds, B
+    B.close()
+    for G in Gs:
+        G.close()
+
+
+def _same_as_sequential(members, m, precision, tail):
+    """One replayed or newly recorded step against the same step without a graph, bit for bit;
+    the blocks' addresses stay those of the fixture."""
+    Gs, Xs, (a, b, a0), B = members
+    keep = [X.clone() for X in Xs]
+    B.chfsi_step(Xs, m, a, b, a0, precision=precision, fp64_tail=tail, graph=True)
+    got = [X.clone() for X in Xs]
+    for X, k in zip(Xs, keep):
+        X.copy_(k)
+    B.chfsi_step(Xs, m, a, b, a0, precision=precision, fp64_tail=tail, graph=False)
+    for g, X, k in zip(got, Xs, keep):
+        assert torch.equal(g, X)
+        X.copy_(k)
+
+
+@pytest.mark.parametrize("precision,tail", [("fp64", 0), ("tf32x3", 2)])
+def test_replayed_graph_follows_each_members_engine(members, precision, tail):
+    """The recorded FP64 kernels are those of every member's engine, and the digit images of
+    H are remade for the members that use them: a member that changes its engine and gets a
+    new potential is recorded anew."""
+    Gs = members[0]
+    for G in Gs:
+        G.set_fp64_engine("tensor")
+    _same_as_sequential(members, 6, precision, tail)
+    Gs[1].set_fp64_engine("dfma")
+    q = Gs[1].qpoints()
+    Gs[1].set_potential((-1.0 / (0.5 + (q[:, :3] ** 2).sum(dim=1).sqrt())).contiguous())
+    _same_as_sequential(members, 6, precision, tail)
+    Gs[1].set_fp64_engine("tensor")
+    _same_as_sequential(members, 6, precision, tail)
+
+
+@pytest.mark.parametrize("name,value", [("coupling_cols", 1), ("coupling_sparse", 1), ("grid_cap", 3)])
+def test_replayed_graph_follows_options(members, name, value):
+    Gs = members[0]
+    Gs[1].set_option("coupling_sparse", int(name == "coupling_cols"))
+    _same_as_sequential(members, 6, "tf32x3", 1)
+    Gs[1].set_option(name, value)
+    _same_as_sequential(members, 6, "tf32x3", 1)
+    Gs[1].set_option(name, 0)
+    _same_as_sequential(members, 6, "tf32x3", 1)
