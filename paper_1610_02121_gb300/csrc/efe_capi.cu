@@ -1722,9 +1722,11 @@ static int stage_coefs(efe_handle* h, int m, double a, double b, double a0, cuda
       return EFE_ERR_STATE;
     }
     if (h->coef_ev) CK(cudaEventSynchronize(h->coef_ev));
+    h->graph_gen++;   // a recorded graph copies from and to the buffers that go
+    h->coef_cap = 0;
     if (h->coefh) cudaFreeHost(h->coefh);
     dfree(h, h->coefd);
-    h->coefh = nullptr;
+    h->coefh = h->coefd = nullptr;
     CK(cudaMallocHost(&h->coefh, sizeof(double) * 3 * m));
     TRY(dalloc(h, &h->coefd, 3 * (int64_t)m));
     h->coef_cap = m;

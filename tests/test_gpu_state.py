@@ -67,3 +67,14 @@ def test_replayed_graph_follows_options(members, name, value):
     _same_as_sequential(members, 6, "tf32x3", 1)
     Gs[1].set_option(name, 0)
     _same_as_sequential(members, 6, "tf32x3", 1)
+
+
+def test_replayed_graph_follows_longer_recurrences(members):
+    """A filter of a higher degree on one member remakes its coefficient buffers, which the
+    recorded graph copies from: the batch records again."""
+    Gs, Xs, (a, b, a0), B = members
+    _same_as_sequential(members, 6, "tf32x3", 2)
+    first = B.graph_nodes()
+    Gs[1].chfsi_step(Xs[1].clone(), 40, a[1], b[1], a0[1])
+    _same_as_sequential(members, 6, "tf32x3", 2)
+    assert B.graph_nodes() == first
