@@ -2362,7 +2362,7 @@ int efe_set_option(efe_handle* h, int32_t option, int64_t value) {
       h->opt_dense_blocked = (int)value;
       return EFE_OK;
     case EFE_OPT_TEST_STALL:
-      if (value > 1) return EFE_ERR_ARG;
+      if (value > 3) return EFE_ERR_ARG;
       h->opt_test_stall = (int)value;
       return EFE_OK;
     case EFE_OPT_COUPLING_SPARSE:

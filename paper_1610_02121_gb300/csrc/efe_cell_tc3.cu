@@ -101,19 +101,42 @@ __device__ __forceinline__ void bar_arrive(uint64_t* b) {
   asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(su32(b)) : "memory");
 }
 
-__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
+__device__ __forceinline__ bool bar_try(uint64_t* b, uint32_t parity) {
   uint32_t done = 0;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(su32(b)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// one thread's bounded wait
+__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
   const long long t0 = clock64();
   do {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(su32(b)), "r"(parity)
-        : "memory");
-    if (done) return true;
+    if (bar_try(b, parity)) return true;
   } while (clock64() - t0 < T3_WAIT);
   return false;
+}
+// the same for a warp that goes on together.  Every lane has its own clock and its own view of
+// the barrier, so the lanes vote: one that left alone could not take part in the warp's next
+// collective step, and the others would wait for it there without a bound.
+__device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
+  if (__all_sync(0xffffffffu, bar_try(b, parity))) return true;
+  const long long t0 = clock64();
+  do {
+    if (__all_sync(0xffffffffu, bar_try(b, parity))) return true;
+  } while (__all_sync(0xffffffffu, clock64() - t0 < T3_WAIT));
+  return false;
+}
+// the abort flag, one answer for the whole warp
+__device__ __forceinline__ bool warp_aborted(const volatile int* flag) {
+  return __any_sync(0xffffffffu, *flag != 0);
+}
+// tests only: the lanes of `mine` wait on a barrier that nothing completes
+__device__ __forceinline__ bool stall_passed(uint64_t* never, bool mine) {
+  return __all_sync(0xffffffffu, !mine || bar_wait(never, 0u));
 }
 
 __device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
@@ -215,13 +238,12 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
-    if (stall && my_items > 0 && !bar_wait(never, 0u)) {
-      // test stall: a wait that nothing completes runs out like a real one
-      if (lane == 0) { *abort_flag = 1; atomicExch(err, 1); }
-    }
+    // test stall: a wait that nothing completes runs out like a real one
+    const bool go = my_items == 0 || stall_passed(never, stall == 1 || (stall == 2 && (lane & 1)));
+    if (!go && lane == 0) { *abort_flag = 1; atomicExch(err, 1); }
     int s = 0;
     uint32_t ph = 0;
-    for (int64_t t = 0; t < my_items && !*abort_flag; ++t) {
+    for (int64_t t = 0; go && t < my_items && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % ntiles) * TW;
       const int ncol = min(TW, N - c0);
@@ -229,11 +251,11 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
       const uint32_t id = MODE == 2 ? idesc_bf16(nmma) : idesc_tf32(nmma);
       const int b = (int)(t & 1);
       bool ok = true;
-      if (t >= 2) ok = bar_wait(acce + b, (uint32_t)((t / 2 - 1) & 1));
+      if (t >= 2) ok = warp_wait(acce + b, (uint32_t)((t / 2 - 1) & 1));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t d = tmem + (uint32_t)(b * 256);
       for (int kc = 0; kc < T3_NCH && ok; ++kc) {
-        ok = bar_wait(conv + s, ph);
+        ok = warp_wait(conv + s, ph);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!ok) break;
         const uint32_t a1 = su32(sm) + (uint32_t)s * L::STAGE, b1 = a1 + L::A;
@@ -313,7 +335,12 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
     for (int i = 0; i < L::DEPTH; ++i) fetch();
     int s = g, rs = 0;
     uint32_t ph = 0;
-    for (int64_t t = 0; t < my_items && !*abort_flag; ++t) {
+    const bool go = stall != 3 || my_items == 0 || stall_passed(never, lane & 1);
+    if (!go) {
+      *abort_flag = 1;
+      atomicExch(err, 1);
+    }
+    for (int64_t t = 0; go && t < my_items && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % ntiles) * TW;
       const int ncol = min(TW, N - c0);
@@ -337,7 +364,7 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
         __syncwarp();
         fetch();   // into the slot just read
         if (++rs == L::DEPTH) rs = 0;
-        if (t * T3_NCH + kc >= ST) ok = bar_wait(empty + s, ph ^ 1u);
+        if (t * T3_NCH + kc >= ST) ok = warp_wait(empty + s, ph ^ 1u);
         if (!ok) break;
         unsigned char* A1 = sm + (uint32_t)s * L::STAGE;
         unsigned char* B1 = A1 + L::A;
@@ -402,7 +429,12 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
     // ------------------------------------------------------------ epilogue
     const int quarter = warp & 3;         // TMEM lane quarter accessible to this warp
     const int sub = lane & 3;
-    for (int64_t t = 0; t < my_items && !*abort_flag; ++t) {
+    const bool go = stall != 3 || my_items == 0 || stall_passed(never, lane & 1);
+    if (!go) {
+      *abort_flag = 1;
+      atomicExch(err, 1);
+    }
+    for (int64_t t = 0; go && t < my_items && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int64_t e = cells ? cells[item / ntiles] : item / ntiles;
       const int c0 = (int)(item % ntiles) * TW;
@@ -414,7 +446,7 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
       int64_t ro[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) ro[i] = (int64_t)(cells ? lut[r0 + i] : r0 + i) * ldw;
-      if (!bar_wait(accf + b, (uint32_t)((t / 2) & 1))) {
+      if (!warp_wait(accf + b, (uint32_t)((t / 2) & 1))) {
         *abort_flag = 1;
         atomicExch(err, 1);
         break;
@@ -485,6 +517,7 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
+    __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(T3_TMEM_COLS) : "memory");
   }

@@ -139,7 +139,7 @@ struct OzArgs {
   const unsigned char* Aimg;
   const unsigned char* Bimg;
   int64_t astep, bstep;
-  int stall;                // tests only: the MMA warp first waits on a barrier nothing completes
+  int stall;                // tests only (EFE_OPT_TEST_STALL): waits on a barrier that nothing completes
 };
 
 // work item of a CTA: row block / tile pair and its K range
@@ -223,11 +223,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
 
   if (warp == 0) {
     // ---------------------------------------------------------------- MMA issuer
-    if (g.stall && my > 0 && !bar_wait(never, 0u)) {
-      // test stall: a wait that nothing completes runs out like a real one
-      if (lane == 0) { *abort_flag = 1; atomicExch(g.err, 1); }
-    }
-    for (int64_t t = 0; t < my && !*abort_flag; ++t) {
+    // test stall: a wait that nothing completes runs out like a real one
+    const bool go = my == 0 || stall_passed(never, g.stall == 1 || (g.stall == 2 && (lane & 1)));
+    if (!go && lane == 0) { *abort_flag = 1; atomicExch(g.err, 1); }
+    for (int64_t t = 0; go && t < my && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const OzItem it = oz_item(g, item);
       const int nmma = it.nmma;
@@ -235,13 +234,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
       for (int kc = 0; kc < nch && ok; ++kc) {
         const int64_t gc = t * ngrp + kc / gsz;   // accumulator group counter
         if (kc % gsz == 0) {
-          if (gc >= 1) ok = bar_wait(acce, (uint32_t)((gc - 1) & 1));
+          if (gc >= 1) ok = warp_wait(acce, (uint32_t)((gc - 1) & 1));
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           if (!ok) break;
         }
         const int64_t ch = t * nch + kc;
         const int s = (int)(ch % OZ_STAGES);
-        ok = bar_wait(afull + s, (uint32_t)((ch / OZ_STAGES) & 1));
+        ok = warp_wait(afull + s, (uint32_t)((ch / OZ_STAGES) & 1));
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!ok) break;
         const uint32_t sA = su32(sm) + (uint32_t)s * OzL::STAGE, sB = sA + OzL::A;
@@ -313,7 +312,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
     const int r = quarter * 32 + lane;
     const int ew = warp - OZ_EPI_W0, part = ew >> 2, nparts = OZ_EPI_WN >> 2;   // column blocks part, part + nparts, ...
     double* stg = reinterpret_cast<double*>(sm + OzL::STG) + ew * (32 * 9);
-    for (int64_t t = 0; t < my && !*abort_flag; ++t) {
+    const bool go = g.stall != 3 || my == 0 || stall_passed(never, lane & 1);
+    if (!go) {
+      *abort_flag = 1;
+      atomicExch(g.err, 1);
+    }
+    for (int64_t t = 0; go && t < my && !warp_aborted(abort_flag); ++t) {
       const OzItem it = oz_item(g, blockIdx.x + t * gridDim.x);
       const int c0 = it.c0, ncol = it.ncol;
       bool live;
@@ -341,7 +345,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
       bool stop = false;
       for (int grp = 0; grp < ngrp; ++grp) {
         const int64_t gc = t * ngrp + grp;
-        if (!bar_wait(accf, (uint32_t)(gc & 1))) {
+        if (!warp_wait(accf, (uint32_t)(gc & 1))) {
           *abort_flag = 1;
           atomicExch(g.err, 1);
           stop = true;
@@ -432,6 +436,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
+    __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_TMEM_COLS) : "memory");
   }

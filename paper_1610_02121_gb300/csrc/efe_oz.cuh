@@ -25,19 +25,42 @@ __device__ __forceinline__ void bar_init(uint64_t* b, uint32_t n) {
 __device__ __forceinline__ void bar_arrive(uint64_t* b) {
   asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(su32(b)) : "memory");
 }
-__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
+__device__ __forceinline__ bool bar_try(uint64_t* b, uint32_t parity) {
   uint32_t done = 0;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(su32(b)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// one thread's bounded wait
+__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
   const long long t0 = clock64();
   do {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(su32(b)), "r"(parity)
-        : "memory");
-    if (done) return true;
+    if (bar_try(b, parity)) return true;
   } while (clock64() - t0 < OZ_WAIT);
   return false;
+}
+// the same for a warp that goes on together.  Every lane has its own clock and its own view of
+// the barrier, so the lanes vote: one that left alone could not take part in the warp's next
+// collective step, and the others would wait for it there without a bound.
+__device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
+  if (__all_sync(0xffffffffu, bar_try(b, parity))) return true;
+  const long long t0 = clock64();
+  do {
+    if (__all_sync(0xffffffffu, bar_try(b, parity))) return true;
+  } while (__all_sync(0xffffffffu, clock64() - t0 < OZ_WAIT));
+  return false;
+}
+// the abort flag, one answer for the whole warp
+__device__ __forceinline__ bool warp_aborted(const volatile int* flag) {
+  return __any_sync(0xffffffffu, *flag != 0);
+}
+// tests only: the lanes of `mine` wait on a barrier that nothing completes
+__device__ __forceinline__ bool stall_passed(uint64_t* never, bool mine) {
+  return __all_sync(0xffffffffu, !mine || bar_wait(never, 0u));
 }
 __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
   asm volatile(

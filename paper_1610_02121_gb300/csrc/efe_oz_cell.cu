@@ -189,23 +189,22 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
 
   if (warp == 0) {
     // ---------------------------------------------------------------- MMA issuer
-    if (g.stall && my > 0 && !bar_wait(never, 0u)) {
-      // test stall: a wait that nothing completes runs out like a real one
-      if (lane == 0) { *abort_flag = 1; atomicExch(g.err, 1); }
-    }
+    // test stall: a wait that nothing completes runs out like a real one
+    const bool go = my == 0 || stall_passed(never, g.stall == 1 || (g.stall == 2 && (lane & 1)));
+    if (!go && lane == 0) { *abort_flag = 1; atomicExch(g.err, 1); }
     int s = 0;
     uint32_t ph = 0;
-    for (int64_t t = 0; t < my && !*abort_flag; ++t) {
+    for (int64_t t = 0; go && t < my && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % g.ntiles) * OC_TW;
       const uint32_t id = idesc_cell(min(OC_TW, g.ldn - c0));
       const int b = (int)(t & 1);
       bool ok = true;
-      if (t >= 2) ok = bar_wait(acce + b, (uint32_t)((t / 2 - 1) & 1));
+      if (t >= 2) ok = warp_wait(acce + b, (uint32_t)((t / 2 - 1) & 1));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t d = tmem + (uint32_t)(b * OZ_NACC * OC_TW);
       for (int kc = 0; kc < OC_NCH && ok; ++kc) {
-        ok = bar_wait(full + s, ph);
+        ok = warp_wait(full + s, ph);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!ok) break;
         const uint32_t sA = su32(sm) + (uint32_t)s * OC_STAGE;
@@ -301,7 +300,12 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
     const int quarter = warp & 3;   // the TMEM lane quarter this warp may read
     const int part = (warp - OC_EPI_W0) >> 2;
     const int r = quarter * 32 + lane;
-    for (int64_t t = 0; t < my && !*abort_flag; ++t) {
+    const bool go = g.stall != 3 || my == 0 || stall_passed(never, lane & 1);
+    if (!go) {
+      *abort_flag = 1;
+      atomicExch(g.err, 1);
+    }
+    for (int64_t t = 0; go && t < my && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int64_t e = item / g.ntiles;
       const int c0 = (int)(item % g.ntiles) * OC_TW;
@@ -309,7 +313,7 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
       const int b = (int)(t & 1);
       const int Er = g.hexp[e * OZ_M + r];
       double* out = g.P + (e * NL + r) * (int64_t)g.ldn + c0;
-      if (!bar_wait(accf + b, (uint32_t)((t / 2) & 1))) {
+      if (!warp_wait(accf + b, (uint32_t)((t / 2) & 1))) {
         *abort_flag = 1;
         atomicExch(g.err, 1);
         break;
@@ -369,6 +373,7 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
+    __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_TMEM_COLS) : "memory");
   }

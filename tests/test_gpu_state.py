@@ -78,3 +78,38 @@ def test_replayed_graph_follows_longer_recurrences(members):
     Gs[1].chfsi_step(Xs[1].clone(), 40, a[1], b[1], a0[1])
     _same_as_sequential(members, 6, "tf32x3", 2)
     assert B.graph_nodes() == first
+
+
+@pytest.mark.parametrize("stall", [2, 3])
+@pytest.mark.parametrize("what,precision,engine", [("filter", "tf32x3", "dfma"), ("filter", "fp64", "tensor"),
+                                                   ("ritz", "fp64", "tensor")])
+def test_wait_that_runs_out_on_part_of_a_warp(what, precision, engine, stall):
+    """Lanes of one warp may disagree about whether a bounded wait ran out.  The whole warp then
+    takes the abort path (lanes that went on would wait for the others for ever): the call
+    returns EFE_ERR_TIMEOUT, and the next one gives the bits of the one before."""
+    from paper_1610_02121_gb300 import EfeError
+    s = W.tiny(seed=11)
+    G = gpu_system(s)
+    X = to_dev(W.initial_block(s, 20, seed=2))
+    e, _ = G.rayleigh_ritz(X)
+    b = G.upper_bound(X[:, -1].contiguous(), 10)
+    G.set_fp64_engine(engine)
+
+    def call():
+        Y = X.clone()
+        if what == "ritz":
+            G.rayleigh_ritz(Y)
+        else:
+            G.chfsi_step(Y, 3, e.max(), b, e.min(), precision=precision)
+        return Y
+
+    before = call()
+    G.set_option("test_stall", stall)
+    try:
+        with pytest.raises(EfeError) as err:
+            call()
+        assert err.value.code == 5
+    finally:
+        G.set_option("test_stall", 0)
+    assert torch.equal(before, call())
+    G.close()
