@@ -213,3 +213,15 @@ def test_sad_points(tiny_pair, Z):
     rho = G.sad_density(shells).cpu().numpy()
     ref = OL.sad_density(q[:, :3], atoms, shells)
     np.testing.assert_allclose(rho, ref, rtol=1e-11)
+
+
+# superposed atoms far from their usual size: a density is linear in its occupations down to
+# the smallest numbers, whatever part of it FP32 arithmetic can hold (2^-160 is exact in FP64
+# and below FP32's range), so every point scales to rounding
+@pytest.mark.parametrize("scale", [2.0 ** -160, 2.0 ** 160])
+def test_sad_points_scale(tiny_pair, scale):
+    d, G = tiny_pair
+    shells = [W.sad_shells(z) for z in (14, 8)][:len(d.system["atoms"])]
+    one = G.sad_density(shells)
+    few = G.sad_density([[(n, z, o * scale) for n, z, o in s] for s in shells])
+    torch.testing.assert_close(few / scale, one, rtol=1e-14, atol=0.0)
