@@ -1979,6 +1979,7 @@ int dense_scratch(efe_handle* h, int64_t bytes) {
 constexpr int CHOL_ONE_CTA_MAX = 64;
 constexpr int EIG_ONE_CTA_MAX = 48;
 constexpr int DENSE_SMALL_MAX = 512;
+constexpr int BJ_EXACT_MAX = 512;
 
 // A = L L^T in place (lower, n x n, ld n); *info: 0 or j + 1 of the first breakdown
 int chol_lower(efe_handle* h, double* A, int n, cudaStream_t st, double* min_ratio, int* info = nullptr) {
@@ -2119,11 +2120,14 @@ int sym_eig_blocked(efe_handle* h, const double* C, int N, double* V, double* w,
     launch_symmetrize(C2, N, N, st);
     C64 = C2;
   }
-  // FP64 stage: on the nearly diagonal C2, or on C itself if the FP32 stage failed
-  // off-diagonal Frobenius norm <= 1e-13 of the total: eigenvalue errors of
-  // order 1e-26 relative, far below FP64 rounding of the projected matrix
-  const int r64 = block_jacobi<double>(C64, N, N, C64 == C ? V : V2, N, w, C64 == C ? 60 : 20, 1e-26, h->dsc, st,
-                                       &ratio);
+  // FP64 stage: on the nearly diagonal C2, or on C itself if the FP32 stage failed.
+  // Eigenvalues would be exact to FP64 rounding at an off-diagonal norm of 1e-13 of the
+  // total; the vectors of a close pair turn by what is left over their gap, so up to
+  // BJ_EXACT_MAX rows, as the one-CTA solver, the sweeps go on to 1e-15 (135 rows from core levels
+  // at -90 to gaps of 1e-4: vectors off by 1.2e-10 at 1e-13, 9e-13 at 1e-15, for one more
+  // sweep of 0.9 ms on about half of the blocks; 2.2e-12 by the one-CTA solver).
+  const int r64 = block_jacobi<double>(C64, N, N, C64 == C ? V : V2, N, w, C64 == C ? 60 : 20,
+                                       N <= BJ_EXACT_MAX ? 1e-30 : 1e-26, h->dsc, st, &ratio);
   if (r64 < 0) {
     h->err = "block Jacobi (FP64 stage): CUDA error";
     return EFE_ERR_CUDA;

@@ -225,3 +225,36 @@ def test_sad_points_scale(tiny_pair, scale):
     one = G.sad_density(shells)
     few = G.sad_density([[(n, z, o * scale) for n, z, o in s] for s in shells])
     torch.testing.assert_close(few / scale, one, rtol=1e-14, atol=0.0)
+
+
+# dense eigenproblem of Rayleigh-Ritz on spectra from core levels (-90) to pairs 1e-4 apart: what
+# is left off the diagonal of V^T C V turns a pair by itself over the gap.  The sweeps stop at
+# 1e-15 of the norm; a product's sum of N terms adds a few sqrt(N) roundings of it.  (V^T C V
+# and V^T V in extended precision; the mean value times V^T V - 1 belongs to the vectors' lengths.)
+@pytest.mark.parametrize("N", [40, 49, 96, 135, 200])
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_eigenvectors_of_close_pairs(tiny_pair, N, seed):
+    import ctypes as C
+    from paper_1610_02121_gb300._lib import lib
+    G = tiny_pair[1]
+    rng = np.random.default_rng(seed + N)
+    core = -90 + rng.uniform(-1, 1, N // 10)
+    ev = rng.uniform(-1, 3, N - len(core))
+    ev[1::8] = ev[0::8][:len(ev[1::8])] + 1e-4
+    ev[2], ev[3] = 1e-7, -1e-7
+    ev = np.concatenate([core, ev])
+    Q, _ = np.linalg.qr(rng.standard_normal((N, N)))
+    A = (Q * ev) @ Q.T
+    A = (A + A.T) / 2
+    G.reserve(N)
+    Ad, V, w, E = to_dev(A), *(torch.empty(n, dtype=torch.float64, device="cuda") for n in (N * N, N, 9 * N * N))
+    eig = lib().sym_eig
+    eig.argtypes, eig.restype = [C.c_void_p, C.c_void_p, C.c_int] + [C.c_void_p] * 4, C.c_int
+    assert eig(G.h, Ad.data_ptr(), N, V.data_ptr(), w.data_ptr(), E.data_ptr(),
+               torch.cuda.current_stream().cuda_stream) == 0
+    V = V.view(N, N).cpu().numpy().astype(np.longdouble)
+    T, L = V.T @ (A.astype(np.longdouble) @ V), V.T @ V
+    d = np.diag(T).copy()
+    left = T - np.diag(d) - (d[:, None] + d[None, :]) / 2 * (L - np.diag(np.diag(L)))
+    norm = np.linalg.norm(A)
+    assert np.abs(left).max() <= (1e-15 + 4 * np.sqrt(N) * 2.0 ** -53) * norm
