@@ -107,7 +107,7 @@ struct efe_handle {
   double *B1 = nullptr, *B2 = nullptr, *W = nullptr, *xe = nullptr, *rb = nullptr, *part = nullptr;
   double* small = nullptr;    // 16 N x N blocks + vectors
   double* tnwork = nullptr;
-  int64_t tnwork_elems = 0;
+  int64_t tnwork_elems = 0, gram_elems = 0;   // of it for the DFMA / the tensor-core products
   double* rpart = nullptr;
   double* cellP = nullptr;    // FP64 cell products of up to cellP_cols columns, all cells
   int cellP_cols = 0;
@@ -334,10 +334,11 @@ int reserve(efe_handle* h, int N) {
   h->xe2 = nullptr;
   TRY(dalloc(h, &h->xe2, std::max<int64_t>(1, h->nE) * N));
   TRY(dalloc(h, &h->small, 24 * (int64_t)N * N + 8 * (int64_t)N));
-  // split-K partials of the DFMA A^T B products and the segment partials of the
-  // tensor-core ones (both fit their split counts to this size)
+  // split-K partials of the DFMA A^T B products and, in the same array, the segment partials of
+  // the tensor-core ones, each as many as its own rule asks for
   h->tnwork_elems = std::max<int64_t>(gemm_tn_work_elems(R, N, N), 4 * (int64_t)N * N);
-  TRY(dalloc(h, &h->tnwork, h->tnwork_elems));
+  h->gram_elems = oz_gram_work_elems(N, N, h->n_sm);
+  TRY(dalloc(h, &h->tnwork, std::max(h->tnwork_elems, h->gram_elems)));
   TRY(dalloc(h, &h->rpart, ((R + 2047) / 2048 + 1) * (int64_t)N));
   // scratch of the FP64 cell products: as many columns as the kernel takes at once
   // and CELLP_MAX_BYTES hold (narrow blocks on large meshes, wider ones on small)
@@ -1934,13 +1935,14 @@ int gemm_gram(efe_handle* h, int64_t rows, int Na, int Nb, const double* A, int6
     const int64_t nch = (std::min(kp, rows) + 15) / 16 + 16 * (2 * (int64_t)tc_grid(h) + 1);
     TRY(oz_img_buf(h, 0, oz_img_cols_bytes(nch, Na)));
     if (B != A) TRY(oz_img_buf(h, 1, oz_img_cols_bytes(nch, Nb)));
+    const int64_t work = std::min(h->gram_elems, oz_gram_work_elems(Na, Nb, h->n_sm));
     bool ok = true;
     for (int64_t k0 = 0; k0 < rows && ok; k0 += kp) {
       const int64_t kn = std::min(kp, rows - k0);
       int slot;
       TRY(timed_begin(h, st, &slot, 1));
       ok = launch_oz_gram(kn, Na, Nb, A + k0 * lda, lda, h->oz_fexp, B + k0 * ldb, ldb, bexp, C, ldc, sym, h->tnwork,
-                          h->tnwork_elems, h->oz_pairs, tc_grid(h), h->info + 4, st, h->oz_img[0],
+                          work, h->oz_pairs, tc_grid(h), h->info + 4, st, h->oz_img[0],
                           h->oz_img_bytes[0], h->oz_img[1], h->oz_img_bytes[1], k0 > 0, h->opt_test_stall) == 0;
       TRY(timed_end(h, st, slot, ok ? (sym ? 1.0 : 2.0) * (double)kn * Na * (Nb + (sym ? 1 : 0)) : 0.0, 1));
     }

@@ -205,6 +205,7 @@ int launch_oz_gram(int64_t K, int Na, int N, const double* A, int64_t lda, const
                    int64_t img_a_bytes = 0, unsigned char* img_b = nullptr, int64_t img_b_bytes = 0,
                    bool accumulate = false, int stall = 0);
 int oz_gram_max_pairs(int Na, int N);
+int64_t oz_gram_work_elems(int Na, int N, int n_sm);
 
 // ---- dense FP64 ----
 // C[M x Nc] = alpha * A[M x K] B[K x Nc] + beta * C   (row-major, lda/ldb/ldc)

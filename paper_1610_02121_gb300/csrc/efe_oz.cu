@@ -697,9 +697,8 @@ int launch_oz_rows(int64_t rows, int K, const int* aexp, const int* bexp, double
 //
 // Segment length, in 256-row groups: the one that ends first when the (tile pair, segment)
 // items run n_sm at a time, an item costing its groups and half a group to fill and drain the
-// pipeline (about two items a CTA before: 135 columns 306 items, 640 columns 320, in three
-// rounds of 152).  Partials of at most max_seg segments fit the work array; more than 2 n_sm
-// segments gain nothing.
+// pipeline.  Partials of at most max_seg segments fit the work array; more than 2 n_sm segments
+// gain nothing.
 int64_t oz_gram_seg_groups(int64_t groups, int npairs, int n_sm, int64_t max_seg) {
   int64_t best = groups;
   double best_cost = 1e300;
@@ -713,6 +712,18 @@ int64_t oz_gram_seg_groups(int64_t groups, int npairs, int n_sm, int64_t max_seg
     }
   }
   return best;
+}
+
+// Doubles for the segment partials of an Na x N product: room for four 48 x 48 blocks an SM
+// (11 MB on 152 SMs) or four whole products, whichever is more.  The first keeps the SMs busy up
+// to about 300 columns, where one product's tile pairs are few: 559 k rows x 100 columns 6.34 ms
+// in 7 segments, 0.91 in 76; x 200 11.1 ms in 4, 2.0 in 30; x 300 11.3 in 4, 3.5 in 16.
+// Wider blocks keep four segments and idle SMs: at 640 columns 13 segments would take 8.0 ms for
+// 12.0, at 400 4.8 for 5.7, but add the rows in another order, with which the vectors of the
+// closest Ritz pairs turn.
+int64_t oz_gram_work_elems(int Na, int N, int n_sm) {
+  const int64_t one = (int64_t)Na * N;
+  return std::max<int64_t>(4LL * n_sm * 48 * 48 + one, 4 * one);
 }
 
 int oz_gram_pairs(int Na, int N, bool sym, int2* pairs_host) {
