@@ -1393,7 +1393,7 @@ __global__ void __launch_bounds__(256) k_gemm_nn_small(int64_t M, int Nc, int K,
 
 // A^T B (split K): each CTA forms one (16 TM) x (16 TM) output tile over a range of
 // rows, TM x TM outputs a thread.  The FP64 pipe bounds it (about two FMAs a clock
-// and SM), so the tile is the one that pads the block least (gemm_tn_tile) and K is
+// and SM), so the tile is the one that pads the block least (gemm_tn_tm) and K is
 // split until every SM has work.  49,005 rows: 12 vectors in one 48 x 48 tile over
 // six 8192-row splits took 3.1 ms, in 16 x 16 tiles over 294 splits 29 us.
 constexpr int64_t TN_KC = 64;    // fewest rows of a split
@@ -2054,23 +2054,36 @@ int gemm_tn_tm(int Na, int Nb) {
 }
 }  // namespace
 
-// K splits of an A^T B product: about two CTAs per SM over the output tiles (four
-// for 48 x 48 tiles), none shorter than TN_KC rows
-int64_t gemm_tn_splits(int64_t K, int Na, int Nb) {
+// K splits of an A^T B product: about two CTAs per SM over the output tiles (four for 48 x 48
+// tiles), none shorter than TN_KC rows.  Of a symmetric product only about half of the tiles are
+// formed: narrow tiles then take the count, up to about four CTAs per SM, with which the busiest SM
+// has the least to do (559 k rows: one split of the 210 tiles of 640 columns gives some SMs two
+// and others one, 433 ms, two splits 284; 200 columns 54.8 -> 36.0, 80 8.4 -> 7.3; 60 columns, three
+// tiles, 76 splits 3.80, 152 3.79, but 102 with their last two CTAs alone 4.27).
+int64_t gemm_tn_splits(int64_t K, int Na, int Nb, bool sym, int n_sm) {
   const int tm = gemm_tn_tm(Na, Nb);
-  const int64_t t = 16 * tm;
-  const int64_t tiles = (int64_t)((Na + t - 1) / t) * ((Nb + t - 1) / t);
-  const int64_t want = ((tm == 3 ? 4 : 2) * (int64_t)current_sm_count() + tiles - 1) / tiles;
+  const int64_t t = 16 * tm, ta = (Na + t - 1) / t;
+  const int64_t tiles = ta * ((Nb + t - 1) / t);
+  int64_t want = ((tm == 3 ? 4 : 2) * (int64_t)n_sm + tiles - 1) / tiles;
+  if (sym && Na == Nb && tm < 3) {
+    const int64_t formed = ta * (ta + 1) / 2, most = (4 * (int64_t)n_sm + formed - 1) / formed;
+    // tiles x rows of the busiest SM, in units of a tile's K: rounds(s) / s
+    auto rounds = [&](int64_t s) { return (formed * s + n_sm - 1) / n_sm; };
+    for (int64_t s = want + 1; s <= most; ++s)
+      if (rounds(s) * want < rounds(want) * s) want = s;
+  }
   const int64_t most = (K + TN_KC - 1) / TN_KC;
   return std::max<int64_t>(1, std::min(want, most));
 }
 
-int64_t gemm_tn_work_elems(int64_t K, int Na, int Nb) { return gemm_tn_splits(K, Na, Nb) * (int64_t)Na * Nb; }
+int64_t gemm_tn_work_elems(int64_t K, int Na, int Nb) {
+  return gemm_tn_splits(K, Na, Nb, true, current_sm_count()) * (int64_t)Na * Nb;
+}
 
 void launch_gemm_tn(int64_t K, int Na, int Nb, const double* A, int64_t lda, const double* B, int64_t ldb,
                     double* C, int64_t ldc, double* work, int64_t work_elems, cudaStream_t st, bool sym) {
   if (Na <= 0 || Nb <= 0) return;
-  int64_t nsplit = gemm_tn_splits(K, Na, Nb);
+  int64_t nsplit = gemm_tn_splits(K, Na, Nb, sym, current_sm_count());
   nsplit = std::max<int64_t>(1, std::min(nsplit, work_elems / ((int64_t)Na * Nb)));
   const int64_t kc = ((K + nsplit - 1) / nsplit + 15) / 16 * 16;
   nsplit = std::max<int64_t>(1, (K + kc - 1) / kc);

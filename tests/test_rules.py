@@ -40,3 +40,20 @@ def test_gram_segments_fill_the_sms(rule, N, groups):
     assert -(-total // seg) * N * N <= work
     # a narrower block's partials fit the array of a wider one
     assert rule("_ZN3efe18oz_gram_work_elemsEiii", I, I, I)(N, N // 2, n_sm) <= work
+
+
+# DFMA A^T A of a tall block: of a symmetric product only the tiles on and above the diagonal
+# are formed.  Work of the busiest SM over the average, for the widths that take 16- and 32-wide
+# tiles: 1.25 at most (153 tiles on 152 SMs are the worst), 1.69 by a rule that counts all tiles.
+def test_symmetric_splits_count_the_tiles_they_form(rule):
+    n_sm, rows = 152, 559625
+    splits = rule("_ZN3efe14gemm_tn_splitsEliibi", L, I, I, C.c_bool, I)
+    for N in range(1, 1200):
+        pad = {t: -(-N // t) * t for t in (48, 32, 16)}
+        t = min(pad, key=lambda k: (pad[k], -k))
+        n = pad[t] // t
+        s, formed = splits(rows, N, N, True, n_sm), n * (n + 1) // 2
+        assert s >= splits(rows, N, N, False, n_sm)
+        if t < 48:
+            assert -(-formed * s // n_sm) / s <= 1.25 * formed / n_sm, N
+        assert splits(100, N, N, True, n_sm) <= 2          # no split is shorter than 64 rows
