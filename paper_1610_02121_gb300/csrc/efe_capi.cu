@@ -317,10 +317,11 @@ int reserve(efe_handle* h, int N) {
   if (N <= h->Nres) return EFE_OK;
   h->graph_gen++;
   free32(h);
-  for (void* p : {(void*)h->B1, (void*)h->B2, (void*)h->W, (void*)h->xe, (void*)h->rb, (void*)h->part,
-                  (void*)h->small, (void*)h->tnwork, (void*)h->rpart})
-    dfree(h, p);
-  h->B2 = nullptr;
+  h->Nres = 0;   // until all of it is there again: an allocation below may fail
+  for (double** p : {&h->B1, &h->B2, &h->W, &h->xe, &h->rb, &h->part, &h->small, &h->tnwork, &h->rpart}) {
+    dfree(h, *p);
+    *p = nullptr;
+  }
   const int64_t R = h->rows;
   h->whole_rr = (int64_t)sizeof(double) * R * N <= WHOLE_RR_MAX_BYTES && !h->opt_rr_panels;
   TRY(dalloc(h, &h->B1, R * N));
@@ -354,6 +355,8 @@ int reserve(efe_handle* h, int N) {
   dfree(h, h->oz_fexp);
   dfree(h, h->oz_bexp);
   dfree(h, h->oz_pairs);
+  h->oz_fexp = h->oz_bexp = nullptr;
+  h->oz_pairs = nullptr;
   TRY(dalloc(h, &h->oz_fexp, N + 16));
   TRY(dalloc(h, &h->oz_bexp, N));
   TRY(dalloc(h, &h->oz_pairs, oz_gram_max_pairs(N, N)));
@@ -2570,6 +2573,7 @@ int efe_scf_step(efe_handle* h, double* X, int64_t ldx, int32_t N, int32_t m, in
   }
   if (h->occ_cap < N) {
     if (h->occ_dev) dfree(h, h->occ_dev);
+    h->occ_cap = 0;
     TRY(dalloc(h, &h->occ_dev, N));
     h->occ_cap = N;
   }

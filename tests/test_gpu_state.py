@@ -113,3 +113,23 @@ def test_wait_that_runs_out_on_part_of_a_warp(what, precision, engine, stall):
         G.set_option("test_stall", 0)
     assert torch.equal(before, call())
     G.close()
+
+
+def test_handle_after_a_refused_reservation():
+    """A reservation that the device has no memory for (50 million columns, 424 GB) is an error;
+    the workspace that it gave up is not used again, and the next calls reserve their own."""
+    from paper_1610_02121_gb300 import EfeError
+    G = gpu_system(W.tiny(seed=11))
+    X = to_dev(W.initial_block(G.system, 20, seed=2))
+    e, _ = G.rayleigh_ritz(X)
+    b = G.upper_bound(X[:, -1].contiguous(), 10)
+    before = G.chfsi_step(X.clone(), 5, e.max(), b, e.min(), precision="tf32x3", fp64_tail=2)
+    for _ in range(2):
+        with pytest.raises(EfeError) as err:
+            G.reserve(50_000_000)
+        assert err.value.code == 7
+    for N in (7, 20):
+        Y = X[:, :N].clone()
+        G.chfsi_step(Y, 5, e.max(), b, e.min(), precision="tf32x3", fp64_tail=2)
+        assert N < 20 or torch.equal(before, Y)
+    G.close()
