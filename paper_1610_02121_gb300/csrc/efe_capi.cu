@@ -1845,6 +1845,7 @@ int efe_chfsi_step(efe_handle* h, double* X, int64_t ldx, int32_t N, int32_t m, 
 int oz_img_buf(efe_handle* h, int i, int64_t bytes) {
   if (bytes <= h->oz_img_bytes[i]) return EFE_OK;
   dfree(h, h->oz_img[i]);
+  h->graph_gen++;   // the n_E x n_E products of many-function filters use it (gemm_ee)
   h->oz_img[i] = nullptr;
   h->oz_img_bytes[i] = 0;
   TRY(dalloc(h, &h->oz_img[i], bytes));
