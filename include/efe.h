@@ -243,6 +243,10 @@ int efe_set_fp64_engine(efe_handle* h, int32_t engine);
 #define EFE_OPT_COUPLING_COLS 7   /* the columns product W_c += (H^ec)^T Y_e of the many-function coupling:
                                     0 (default): dense tiles of 32-node blocks; 1: each node's own entries only.
                                     Same products, FP32 sums in another order */
+#define EFE_OPT_CELL_SCRATCH 8    /* scratch arrays of the cell products above this many bytes count as refused by the
+                                    device (0: no such limit).  The FP64 engine then takes narrower column panels
+                                    and, below one 48-column tile, the DFMA products; the FP32 and DFMA products go
+                                    colour by colour.  Same results but for the engine's change to DFMA */
 int efe_set_option(efe_handle* h, int32_t option, int64_t value);
 
 /* Kernel timing: when enabled, the library brackets every launch of its

@@ -481,13 +481,14 @@ class System:
         return t.value, ms
 
     OPTIONS = {"grid_cap": 1, "image_rows": 2, "rr_panels": 3, "dense_blocked": 4, "coupling_sparse": 5,
-               "test_stall": 6, "coupling_cols": 7}
+               "test_stall": 6, "coupling_cols": 7, "cell_scratch": 8}
 
     def set_option(self, name, value):
         """Test/tuning control of the library (EFE_OPT_*): grid_cap (CTAs of the
         persistent tensor-core kernels), image_rows (FP64-engine image panel rows),
         rr_panels (1: panelled Rayleigh-Ritz), dense_blocked (1: multi-CTA dense
-        kernels), coupling_sparse (1: many-function mixed coupling); 0 restores
+        kernels), coupling_sparse (1: many-function mixed coupling), cell_scratch
+        (largest scratch array of the cell products in bytes); 0 restores
         the size-based default."""
         self._check(self.L.efe_set_option(self.h, self.OPTIONS[name], int(value)))
 

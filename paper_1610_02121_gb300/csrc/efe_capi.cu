@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -66,9 +67,11 @@ struct efe_handle {
   unsigned char* ozc_digits = nullptr;   // FP64 engine's cell products: digit planes of a column panel,
   double* ozc_products = nullptr;        // its products (grow-only)
   int64_t ozc_digits_bytes = 0, ozc_products_bytes = 0;
+  int ozc_cols = INT_MAX;   // widest panel the device had memory for (0: none)
   // counts everything a recorded batch graph depends on: reallocated workspace, the FP64
   // engine, options that pick kernels, the tuned column tile
   int64_t graph_gen = 0;
+  bool capturing = false;   // a batch is recording this handle's launches
   int* oz_fexp = nullptr;   // per-column exponents (N, readable up to a multiple of 16)
   int* oz_bexp = nullptr;   // per-column exponents of small right-hand matrices (N)
   int* oz_aexp = nullptr;   // per-row exponents of tall left-hand matrices (rows)
@@ -141,6 +144,7 @@ struct efe_handle {
   int opt_coup_sparse = 0;                    // 1: grouped sparse coupling whatever the size
   int opt_coup_cols = 0;                      // columns product: 0 dense tiles, 1 per-node entries
   int opt_test_stall = 0;                     // tests: tensor-core launches take their abort path
+  int64_t opt_cell_scratch = 0;               // largest scratch array of the cell products (bytes; 0: by their rules)
   // dense FP32 tiles of the pattern over blocks of pattern nodes (mixed filter)
   int64_t cb_nblk = 0, cb_nslots = 0;
   int64_t *cb_slot_off = nullptr, *cb_pos = nullptr, *cb_cta = nullptr, *cb_cta_cols = nullptr;
@@ -221,12 +225,51 @@ namespace {
     if (_r != EFE_OK) return _r; \
   } while (0)
 
+void dfree(efe_handle* h, void* p) {
+  if (!p) return;
+  auto it = std::find(h->allocs.begin(), h->allocs.end(), p);
+  if (it != h->allocs.end()) h->allocs.erase(it);
+  cudaFree(p);
+}
+
+// Scratch of the cell products makes them faster and is not needed for any: it is allocated
+// where the device has the room, and the FP64 engine's (up to 16 GiB) goes when memory that a
+// call cannot do without would not fit beside it.
+bool release_cell_scratch(efe_handle* h) {
+  if (h->capturing || (!h->ozc_digits && !h->ozc_products)) return false;
+  dfree(h, h->ozc_digits);
+  dfree(h, h->ozc_products);
+  h->ozc_digits = nullptr;
+  h->ozc_products = nullptr;
+  h->ozc_digits_bytes = h->ozc_products_bytes = 0;
+  h->graph_gen++;
+  return true;
+}
+
+template <typename T>
+bool dalloc_scratch(efe_handle* h, T** p, int64_t n) {
+  *p = nullptr;
+  if (h->opt_cell_scratch > 0 && (int64_t)sizeof(T) * n > h->opt_cell_scratch) return false;
+  void* q = nullptr;
+  if (cudaMalloc(&q, sizeof(T) * (size_t)n) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  h->allocs.push_back(q);
+  *p = (T*)q;
+  return true;
+}
+
 template <typename T>
 int dalloc(efe_handle* h, T** p, int64_t n) {
   *p = nullptr;
   if (n <= 0) n = 1;
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, sizeof(T) * (size_t)n);
+  if (e == cudaErrorMemoryAllocation && release_cell_scratch(h)) {
+    cudaGetLastError();
+    e = cudaMalloc(&q, sizeof(T) * (size_t)n);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     h->err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
@@ -242,13 +285,6 @@ int upload(efe_handle* h, T** p, const std::vector<T>& v) {
   TRY(dalloc(h, p, (int64_t)v.size()));
   if (!v.empty()) CK(cudaMemcpy(*p, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
   return EFE_OK;
-}
-
-void dfree(efe_handle* h, void* p) {
-  if (!p) return;
-  auto it = std::find(h->allocs.begin(), h->allocs.end(), p);
-  if (it != h->allocs.end()) h->allocs.erase(it);
-  cudaFree(p);
 }
 
 int set_dev(efe_handle* h) {
@@ -349,9 +385,9 @@ int reserve(efe_handle* h, int N) {
   {
     const int64_t per = (int64_t)sizeof(double) * cell_f64_scratch_elems(h->n_cell, 1);
     const int nc = (int)std::min<int64_t>({N, cell_f64_max_cols(), CELLP_MAX_BYTES / std::max<int64_t>(1, per)});
-    if (nc > 0) TRY(dalloc(h, &h->cellP, cell_f64_scratch_elems(h->n_cell, nc)));
-    h->cellP_cols = nc;
+    if (nc > 0 && dalloc_scratch(h, &h->cellP, cell_f64_scratch_elems(h->n_cell, nc))) h->cellP_cols = nc;
   }
+  h->ozc_cols = INT_MAX;
   dfree(h, h->oz_fexp);
   dfree(h, h->oz_bexp);
   dfree(h, h->oz_pairs);
@@ -389,7 +425,7 @@ int reserve32(efe_handle* h, int N) {
     CK(cudaMemset(h->Wf, 0, sizeof(float) * n32));
   }
   if (tc3_scratch_elems(h->n_cell, ld) * (int64_t)sizeof(float) <= CELLP32_MAX_BYTES)
-    TRY(dalloc(h, &h->cellP32, tc3_scratch_elems(h->n_cell, ld)));
+    dalloc_scratch(h, &h->cellP32, tc3_scratch_elems(h->n_cell, ld));
   for (int i = 0; i < 2; ++i) TRY(dalloc(h, &h->Ye[i], std::max<int64_t>(1, h->nE) * N));
   TRY(dalloc(h, &h->We, std::max<int64_t>(1, h->nE) * N));
   // coupling products: one wave of CTAs each, node blocks split so that every
@@ -500,35 +536,33 @@ int ensure_oz_aimg(efe_handle* h, cudaStream_t st) {
 // panel (2.9 and 3.3 GB), the 280-atom mesh 144 columns at a time (6.1 and 6.7 GB).
 constexpr int64_t OZ_CELL_BUDGET = 8ll << 30;
 
-// scratch of the FP64 engine's cell products for blocks of N columns (grow-only)
-int oz_cell_scratch(efe_handle* h, int N, int* panel) {
-  const int w = ozc_panel_cols(h->n_nodes, h->n_cell, N, OZ_CELL_BUDGET, OZ_CELL_BUDGET);
+// scratch of the FP64 engine's cell products for blocks of N columns (grow-only); *panel: the
+// columns it holds, halved until the device has the memory; 0: not even one 48-column tile, the
+// products then run on the DFMA pipe, which needs none
+void oz_cell_scratch(efe_handle* h, int N, int* panel) {
+  auto grow = [&](auto** p, int64_t* have, int64_t bytes) {
+    if (bytes <= *have) return true;
+    dfree(h, *p);
+    *have = 0;
+    h->graph_gen++;
+    if (!dalloc_scratch(h, p, bytes / (int64_t)sizeof(**p))) return false;
+    *have = bytes;
+    return true;
+  };
+  int w = std::min(ozc_panel_cols(h->n_nodes, h->n_cell, N, OZ_CELL_BUDGET, OZ_CELL_BUDGET), h->ozc_cols);
+  while (w > 0 && !(grow(&h->ozc_digits, &h->ozc_digits_bytes, ozc_digit_bytes(h->n_nodes, w)) &&
+                    grow(&h->ozc_products, &h->ozc_products_bytes, ozc_product_bytes(h->n_cell, w)))) {
+    release_cell_scratch(h);
+    w = h->ozc_cols = w > 48 ? std::max(48, w / 2 / 48 * 48) : 0;
+  }
   *panel = w;
-  const int64_t db = ozc_digit_bytes(h->n_nodes, w), pb = ozc_product_bytes(h->n_cell, w);
-  if (db > h->ozc_digits_bytes) {
-    dfree(h, h->ozc_digits);
-    h->ozc_digits = nullptr;
-    h->ozc_digits_bytes = 0;
-    h->graph_gen++;
-    TRY(dalloc(h, &h->ozc_digits, db));
-    h->ozc_digits_bytes = db;
-  }
-  if (pb > h->ozc_products_bytes) {
-    dfree(h, h->ozc_products);
-    h->ozc_products = nullptr;
-    h->ozc_products_bytes = 0;
-    h->graph_gen++;
-    TRY(dalloc(h, &h->ozc_products, pb / (int64_t)sizeof(double)));
-    h->ozc_products_bytes = pb;
-  }
-  return EFE_OK;
 }
 
 // --- FP64 engine: W_c = H^cc Y_c over all cells, in column panels ---
-int cell_apply_engine(efe_handle* h, const double* Y, int64_t ldy, double* Wc, int64_t ldw, int N, cudaStream_t st) {
+// of w columns (oz_cell_scratch)
+int cell_apply_engine(efe_handle* h, const double* Y, int64_t ldy, double* Wc, int64_t ldw, int N, int w,
+                      cudaStream_t st) {
   TRY(ensure_oz_aimg(h, st));
-  int w;
-  TRY(oz_cell_scratch(h, N, &w));
   launch_oz_colexp(Y, ldy, h->n_nodes, N, h->oz_fexp, st);
   for (int c0 = 0; c0 < N; c0 += w) {
     const int nc = std::min(w, N - c0);
@@ -609,13 +643,6 @@ int cell_apply_all(efe_handle* h, const T* Hc, const T* Y, int64_t ldy, T* Wc, i
 // vectors; the plain FP64 kernels otherwise.
 bool use_df(const efe_handle* h, int N) { return h->fp64_engine == 1 && h->nE > 0 && N > 8; }
 
-// The FP64 cell products run over all cells at once, through a scratch array, where
-// that array was reserved for this many columns (reserve()) and the DFMA kernel is
-// the one that runs.
-bool cells_at_once(const efe_handle* h, int N) {
-  return N <= h->cellP_cols && (h->fp64_engine == 0 || N <= 8);
-}
-
 template <typename T>
 int couple_H(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, int64_t ldxe, T* Wc, int64_t ldw, double* We,
              int64_t ldwe, int N, cudaStream_t st);
@@ -625,11 +652,15 @@ int couple_H(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, int64_t 
 template <typename T>
 int apply_H_generic(efe_handle* h, const T* Xc, int64_t ldx, const double* Xe, int64_t ldxe, T* Wc, int64_t ldw,
                     double* We, int64_t ldwe, int N, cudaStream_t st, const T* Hc) {
-  if (sizeof(T) == 8 && h->fp64_engine == 1 && N > 8) {
-    TRY(cell_apply_engine(h, (const double*)Xc, ldx, (double*)Wc, ldw, N, st));
+  int w = 0;
+  if (sizeof(T) == 8 && h->fp64_engine == 1 && N > 8) oz_cell_scratch(h, N, &w);
+  if (w > 0) {
+    TRY(cell_apply_engine(h, (const double*)Xc, ldx, (double*)Wc, ldw, N, w, st));
     return couple_H<T>(h, Xc, ldx, Xe, ldxe, Wc, ldw, We, ldwe, N, st);
   }
-  if (sizeof(T) == 8 && cells_at_once(h, N)) {
+  // DFMA products over all cells at once, through a scratch array, where it was reserved for
+  // this many columns (reserve()); colour by colour otherwise
+  if (sizeof(T) == 8 && N <= h->cellP_cols) {
     launch_cell_apply_f64_all((const double*)Hc, h->n_cell, h->mesh, (const double*)Xc, ldx, h->cellP, (double*)Wc, ldw,
                               N, st);
     CKL();
@@ -2382,6 +2413,13 @@ int efe_set_option(efe_handle* h, int32_t option, int64_t value) {
         h->Nres32 = 0;   // the mixed workspace is remade at the next filter call
       }
       return EFE_OK;
+    case EFE_OPT_CELL_SCRATCH:
+      if (h->opt_cell_scratch != value) {
+        h->opt_cell_scratch = value;
+        release_cell_scratch(h);
+        h->Nres = h->Nres32 = 0;   // reserved again, with the new limit
+      }
+      return EFE_OK;
     case EFE_OPT_COUPLING_COLS:
       if (value > 1) return EFE_ERR_ARG;
       h->opt_coup_cols = (int)value;
@@ -3085,25 +3123,28 @@ int efe_batch_chfsi_step(efe_batch* b, double* const* X, const int64_t* ldx, con
     return EFE_OK;
   }
   const int n_low = (precision == EFE_PREC_FP64) ? 0 : std::max(0, m - fp64_tail);
-  // workspaces and coefficient buffers exist before any capture
-  for (int i = 0; i < n; ++i) {
+  // workspaces, digit images (they follow the potential, not the recorded graph) and coefficient
+  // buffers exist before any capture; first what the members cannot do without
+  auto engine_cells = [&](int i) { return n_low < m && b->hs[i]->fp64_engine == 1 && N[i] > 8; };
+  auto prepare = [&](int i) {
     efe_handle* h = b->hs[i];
-    int rc = reserve(h, N[i]);
-    if (rc == EFE_OK && n_low > 0) rc = reserve32(h, N[i]);
-    // the digit images follow the potential, not the recorded graph
-    if (rc == EFE_OK && n_low < m && h->fp64_engine == 1 && N[i] > 8) {
-      int w;
-      rc = oz_cell_scratch(h, N[i], &w);
-      if (rc == EFE_OK) rc = ensure_oz_aimg(h, caller);
+    TRY(reserve(h, N[i]));
+    if (n_low > 0) TRY(reserve32(h, N[i]));
+    if (engine_cells(i)) TRY(ensure_oz_aimg(h, caller));
+    return h->coef_cap < m ? stage_coefs(h, m, a[i], bnd[i], a0[i], caller, false) : EFE_OK;
+  };
+  for (int i = 0; i < n; ++i) {
+    int rc = prepare(i);
+    if (rc == EFE_ERR_ALLOC) {
+      for (efe_handle* h : b->hs) release_cell_scratch(h);
+      rc = prepare(i);
     }
     if (rc != EFE_OK) return fail(i, rc);
-    if (h->coef_cap < m) {
-      rc = stage_coefs(h, m, a[i], bnd[i], a0[i], caller, false);
-      if (rc != EFE_OK) return fail(i, rc);
-    }
-    if (h->coef_pending) cudaEventSynchronize(h->coef_ev);
-    h->coef_pending = false;
+    if (b->hs[i]->coef_pending) cudaEventSynchronize(b->hs[i]->coef_ev);
+    b->hs[i]->coef_pending = false;
   }
+  for (int i = 0, w; i < n; ++i)
+    if (engine_cells(i)) oz_cell_scratch(b->hs[i], N[i], &w);
   bool same = b->exec && b->m == m && b->precision == precision && b->fp64_tail == fp64_tail &&
               (int)b->X.size() == n;
   for (int i = 0; same && i < n; ++i)
@@ -3111,14 +3152,15 @@ int efe_batch_chfsi_step(efe_batch* b, double* const* X, const int64_t* ldx, con
   if (!same) {
     batch_clear_graph(b);
     const int64_t l0 = g_launches.load();
+    if (cudaStreamBeginCapture(b->s0, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
+      b->err = "cudaStreamBeginCapture failed";
+      return EFE_ERR_CUDA;
+    }
     std::vector<bool> timing(n);
     for (int i = 0; i < n; ++i) {
       timing[i] = b->hs[i]->timing;
       b->hs[i]->timing = false;
-    }
-    if (cudaStreamBeginCapture(b->s0, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
-      b->err = "cudaStreamBeginCapture failed";
-      return EFE_ERR_CUDA;
+      b->hs[i]->capturing = true;
     }
     int rc = EFE_OK, bad = -1;
     cudaEventRecord(b->fork, b->s0);
@@ -3131,7 +3173,10 @@ int efe_batch_chfsi_step(efe_batch* b, double* const* X, const int64_t* ldx, con
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(b->s0, &graph);
-    for (int i = 0; i < n; ++i) b->hs[i]->timing = timing[i];
+    for (int i = 0; i < n; ++i) {
+      b->hs[i]->timing = timing[i];
+      b->hs[i]->capturing = false;
+    }
     g_launches.store(l0);  // capture records, it does not launch
     if (rc != EFE_OK) {
       if (graph) cudaGraphDestroy(graph);

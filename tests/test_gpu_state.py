@@ -58,9 +58,11 @@ def test_replayed_graph_follows_each_members_engine(members, precision, tail):
     _same_as_sequential(members, 6, precision, tail)
 
 
-@pytest.mark.parametrize("name,value", [("coupling_cols", 1), ("coupling_sparse", 1), ("grid_cap", 3)])
+@pytest.mark.parametrize("name,value", [("coupling_cols", 1), ("coupling_sparse", 1), ("grid_cap", 3),
+                                        ("cell_scratch", 1)])
 def test_replayed_graph_follows_options(members, name, value):
     Gs = members[0]
+    Gs[0].set_fp64_engine("tensor")
     Gs[1].set_option("coupling_sparse", int(name == "coupling_cols"))
     _same_as_sequential(members, 6, "tf32x3", 1)
     Gs[1].set_option(name, value)
@@ -132,4 +134,59 @@ def test_handle_after_a_refused_reservation():
         Y = X[:, :N].clone()
         G.chfsi_step(Y, 5, e.max(), b, e.min(), precision="tf32x3", fp64_tail=2)
         assert N < 20 or torch.equal(before, Y)
+    G.close()
+
+
+# 48 columns of the 1,053 nodes and 12 cells of the tiny mesh: 14 B a value of the digit planes,
+# 8 B a product
+ONE_TILE = max(14 * 1053 * 48, 8 * 12 * 125 * 48)
+
+
+@pytest.mark.parametrize("N", [20, 48, 49, 100, 145])
+def test_engine_cells_take_what_memory_there_is(N):
+    """The FP64 engine's cell products where the device refuses their scratch: in 48-column
+    panels the bits of one panel, and without any room the DFMA products, against the oracle
+    (the engine's figure, 1e-10 of the largest entry).  A filter, which keeps its panels from
+    degree to degree, and a call after the memory has come back."""
+    from oracle.operators import Discretisation
+    from tests.gpu_util import rel_err
+    G = gpu_system(W.tiny(seed=11))
+    assert (G.n_nodes, G.n_cells) == (1053, 12)
+    X = W.random_block(G.system, N, seed=700 + N)
+    Xd = to_dev(X)
+    ref = Discretisation(G.system).apply_H_assembled(X)
+    b = G.upper_bound(Xd[:, -1].contiguous(), 10)
+    G.set_fp64_engine("tensor")
+
+    def step():
+        return G.chfsi_step(Xd.clone(), 3, 0.2 * b, b, -1.0)
+
+    whole, filtered = G.apply_H(Xd), step()
+    G.set_option("cell_scratch", ONE_TILE)
+    assert torch.equal(G.apply_H(Xd), whole) and torch.equal(step(), filtered)
+    G.set_option("cell_scratch", 1)
+    assert rel_err(G.apply_H(Xd), ref) < 1e-10
+    none = step()
+    assert rel_err(none, filtered.cpu().numpy()) < 1e-9
+    G.set_option("cell_scratch", 0)
+    assert torch.equal(G.apply_H(Xd), whole) and torch.equal(step(), filtered)
+    G.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "tf32", "tf32x3", "bf16"])
+@pytest.mark.parametrize("N", [1, 5, 16, 33, 96, 159, 160, 161])
+def test_cells_colour_by_colour(precision, N):
+    """Without scratch the cell products go colour by colour and are added into the result in
+    the kernel: the bits of the launch over all cells and its gather."""
+    G = gpu_system(W.tiny(seed=11))
+    X = to_dev(W.random_block(G.system, N, seed=800 + N))
+    b = G.upper_bound(X[:, -1].contiguous(), 10)
+
+    def step(cap):
+        G.set_grid_cap(cap)
+        return G.chfsi_step(X.clone(), 3, 0.2 * b, b, -1.0, precision=precision)
+
+    at_once = step(0)
+    G.set_option("cell_scratch", 1)
+    assert torch.equal(step(0), at_once) and torch.equal(step(1), at_once)
     G.close()
