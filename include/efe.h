@@ -227,9 +227,11 @@ int efe_set_fp64_engine(efe_handle* h, int32_t engine);
 #define EFE_OPT_RR_PANELS 3      /* 1: Rayleigh-Ritz forms H Q and M Q in two column panels (and the residuals by
                                     fresh H and M applies) whatever the size; 0: only when a third R x N FP64 block
                                     would exceed 16 GiB.  Takes effect at the next workspace reservation */
-#define EFE_OPT_DENSE_BLOCKED 4  /* 1: the blocked multi-CTA dense N x N kernels (Cholesky, triangular inverse,
-                                    block Jacobi eigensolver) whatever the size; 0: for N > 48 (Cholesky:
-                                    N > 64; the triangular inverse always) */
+#define EFE_OPT_DENSE_BLOCKED 4  /* 1: the dense N x N kernels of the largest blocks (Cholesky with tiled trailing
+                                    updates, block Jacobi eigensolver whose visits diagonalise, N x N products on the
+                                    FP64 engine when it is on) whatever the size; 0: the blocked eigensolver for
+                                    N > 48, with such visits for N > 512; the blocked Cholesky for N > 64, with tiled
+                                    updates for N > 2048; engine products for N > 512 */
 #define EFE_OPT_COUPLING_SPARSE 5 /* 1: the mixed degrees take the many-function enrichment coupling (node-major FP32
                                     columns products, rows products over function groups with FP64 partial sums)
                                     whatever the size; 0: only when the dense-tile kernels' n_E x N FP32 array

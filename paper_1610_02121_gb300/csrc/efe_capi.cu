@@ -58,7 +58,7 @@ struct efe_handle {
   int grid_cap = 0;         // test/tuning cap on the persistent tensor-core grids (0: one CTA per SM)
   int64_t opt_image_rows = 0;   // rows per operand-image panel of the FP64 engine's tall products (0: by budget)
   int opt_rr_panels = 0;        // 1: Rayleigh-Ritz in column panels whatever the size
-  int opt_dense_blocked = 0;    // 1: blocked multi-CTA dense N x N kernels whatever the size
+  int opt_dense_blocked = 0;    // 1: the dense N x N kernels of the largest blocks whatever the size
   double* noalloc_part = nullptr;  // device address of the static scratch of efe_apply_M_noalloc
   int fp64_engine = 0;      // 0: FP64 DFMA products; 1: FP64-grade products on the BF16 tensor cores
   int* hexp = nullptr;      // per-cell row exponents of H^cc_e (tensor-core FP64 products)
@@ -2025,7 +2025,7 @@ int chol_lower(efe_handle* h, double* A, int n, cudaStream_t st, double* min_rat
     launch_chol(A, n, n, info, st, min_ratio);
   } else {
     TRY(dense_scratch(h, (int64_t)sizeof(double) * chol_blocked_scratch(n)));
-    launch_chol_blocked(A, n, n, info, min_ratio, (double*)h->dsc, st);
+    launch_chol_blocked(A, n, n, info, min_ratio, (double*)h->dsc, st, h->opt_dense_blocked != 0);
   }
   CKL();
   return EFE_OK;
@@ -2122,7 +2122,7 @@ int sym_eig_blocked(efe_handle* h, const double* C, int N, double* V, double* w,
   // as dense_nn: below that size the DFMA products are the faster ones
   const bool engine = h->fp64_engine == 1 && (N > DENSE_SMALL_MAX || h->opt_dense_blocked);
   double ratio = 0.0;
-  const int r32 = block_jacobi<float>(C, N, N, V32, N, w32, 40, 1e-12, h->dsc, st, &ratio);
+  const int r32 = block_jacobi<float>(C, N, N, V32, N, w32, 40, 1e-12, h->dsc, st, &ratio, h->opt_dense_blocked != 0);
   if (r32 < 0) {
     h->err = "block Jacobi (FP32 stage): CUDA error";
     return EFE_ERR_CUDA;
@@ -2164,7 +2164,8 @@ int sym_eig_blocked(efe_handle* h, const double* C, int N, double* V, double* w,
   // at -90 to gaps of 1e-4: vectors off by 1.2e-10 at 1e-13, 9e-13 at 1e-15, for one more
   // sweep of 0.9 ms on about half of the blocks; 2.2e-12 by the one-CTA solver).
   const int r64 = block_jacobi<double>(C64, N, N, C64 == C ? V : V2, N, w, C64 == C ? 60 : 20,
-                                       N <= BJ_EXACT_MAX ? 1e-30 : 1e-26, h->dsc, st, &ratio);
+                                       N <= BJ_EXACT_MAX ? 1e-30 : 1e-26, h->dsc, st, &ratio,
+                                       h->opt_dense_blocked != 0);
   if (r64 < 0) {
     h->err = "block Jacobi (FP64 stage): CUDA error";
     return EFE_ERR_CUDA;

@@ -669,12 +669,14 @@ constexpr int BJ_NORM_BLOCKS = 128;
 }  // namespace
 
 // ------------------------------------------------------------------ host side
-// up to the one-CTA kernel's largest size the trailing update keeps that kernel's order
-// of sums (close pairs of Ritz vectors turn with the rounding); a tiled product above
+// Up to this size the trailing update adds in the order of sums of the one-CTA factor (k_chol), which
+// served it before: close pairs of Ritz vectors turn with the rounding, and so they turn as they
+// did.  Above it, where the tiled product always ran, it still does.
 constexpr int CHOL_ORDERED_MAX = 2048;
 
+// tiled: the trailing update as a tiled product whatever the size (tests)
 void launch_chol_blocked(double* A, int n, int lda, int* info, double* min_ratio, double* scratch,
-                         cudaStream_t st) {
+                         cudaStream_t st, bool tiled) {
   // scratch: n (original diagonal) + CB * n (transposed panel) doubles
   double* d0 = scratch;
   double* T = scratch + n;
@@ -690,7 +692,7 @@ void launch_chol_blocked(double* A, int n, int lda, int* info, double* min_ratio
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (m <= 0) break;
     k_chol_panel<<<nblk(m, 128), 128, 0, st>>>(A, lda, j0, b, n);
-    if (n <= CHOL_ORDERED_MAX) {
+    if (n <= CHOL_ORDERED_MAX && !tiled) {
       k_chol_update<<<dim3(nblk(m, 64), nblk(m, 64)), 256, 0, st>>>(A, lda, j0, b, n);
       g_launches.fetch_add(2, std::memory_order_relaxed);
       continue;
@@ -734,11 +736,11 @@ void launch_trinv_blocked(const double* L, int n, int lda, double* Li, int ldi, 
 constexpr int BJ_BLOCK = 16;   // block Jacobi block size of both stages
 
 // Above this size a visit of the block Jacobi diagonalises its subproblem instead of making one
-// sweep over it.  One sweep a visit is the faster at every size (640 rows: about 95 -> 31 ms), but
-// it rounds differently, and on large blocks the vectors of the closest pairs of Ritz values
-// turn with the rounding (norm x 2^-53 over the gap: 3.5e-9 seen at 640, 5e-12 with both the
-// diagonalising visits and the ordered Cholesky), more than a program
-// that compares runs expects; up to 512 the difference stayed below 1e-10.
+// sweep over it.  One sweep a visit is the faster at every size (640 rows: about 95 -> 31 ms) and
+// as accurate, but rounds differently, and the vectors of the closest pairs of Ritz values turn
+// with the rounding (norm x 2^-53 over the gap: 3.5e-9 seen at 640, as far from a 64-bit result
+// either way).  So this is not a line between two fields of use: it is where the visits that
+// diagonalise were in use before, and a program that compares such vectors between runs keeps them.
 constexpr int BJ_DIAG_MIN = 512;
 
 static int64_t bj_scratch_bytes(int n, int elem, int B) {
@@ -760,13 +762,12 @@ int64_t block_jacobi_scratch_bytes(int n, int elem) { return bj_scratch_bytes(n,
 namespace {
 template <typename T, int BJ_B>
 int block_jacobi_b(const double* C, int n, int ldc, T* V, int ldv, T* w, int max_sweeps, double tol2, void* scratch,
-                   cudaStream_t st, double* ratio_out) {
+                   cudaStream_t st, double* ratio_out, bool diag) {
   constexpr int BJ_S = 2 * BJ_B;
   const int nb0 = (n + BJ_B - 1) / BJ_B;
   const int nb = std::max(2, nb0 + (nb0 & 1));
   const int np = nb * BJ_B;
   const int pairs = nb / 2;
-  const bool diag = n > BJ_DIAG_MIN;
   const size_t smem = sizeof(T) * 2 * BJ_S * (BJ_S + 1);
   if (diag && cudaFuncSetAttribute(k_bjd_solve<T, BJ_B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
                   cudaSuccess)
@@ -824,13 +825,14 @@ int block_jacobi_b(const double* C, int n, int ldc, T* V, int ldv, T* w, int max
 // 32-wide blocks, 4.95 s with 16)
 template <typename T>
 int block_jacobi(const double* C, int n, int ldc, T* V, int ldv, T* w, int max_sweeps, double tol2, void* scratch,
-                 cudaStream_t st, double* ratio_out) {
-  return block_jacobi_b<T, BJ_BLOCK>(C, n, ldc, V, ldv, w, max_sweeps, tol2, scratch, st, ratio_out);
+                 cudaStream_t st, double* ratio_out, bool diagonalise) {
+  return block_jacobi_b<T, BJ_BLOCK>(C, n, ldc, V, ldv, w, max_sweeps, tol2, scratch, st, ratio_out,
+                                     diagonalise || n > BJ_DIAG_MIN);
 }
 
 template int block_jacobi<float>(const double*, int, int, float*, int, float*, int, double, void*, cudaStream_t,
-                                 double*);
+                                 double*, bool);
 template int block_jacobi<double>(const double*, int, int, double*, int, double*, int, double, void*, cudaStream_t,
-                                  double*);
+                                  double*, bool);
 
 }  // namespace efe

@@ -231,16 +231,18 @@ void launch_mirror_upper(double* A, int n, int lda, cudaStream_t st);
 // ---- dense N x N kernels for large N (efe_dense.cu) ----
 // blocked Cholesky A = L L^T in place (lower; upper zeroed); info: 0 or j + 1 of the
 // first breakdown; min_ratio (optional): min_j L_jj^2 / A_jj; scratch: chol_blocked_scratch(n) doubles
-void launch_chol_blocked(double* A, int n, int lda, int* info, double* min_ratio, double* scratch, cudaStream_t st);
+void launch_chol_blocked(double* A, int n, int lda, int* info, double* min_ratio, double* scratch, cudaStream_t st,
+                         bool tiled);
 int64_t chol_blocked_scratch(int n);
 // Li = L^-1 by 2 x 2 block recursion; scratch: n * n / 4 + 64 n doubles
 void launch_trinv_blocked(const double* L, int n, int lda, double* Li, int ldi, double* scratch, cudaStream_t st);
 // symmetric C = V diag(w) V^T by multi-CTA block Jacobi in precision T (float or double);
 // 0: converged (off-diagonal square sum <= tol2 x total), 1: sweeps ran out, -1: CUDA error;
-// ratio_out (optional): the last off / total ratio.  scratch: block_jacobi_scratch_bytes(n, sizeof(T))
+// ratio_out (optional): the last off / total ratio.  scratch: block_jacobi_scratch_bytes(n, sizeof(T)).
+// diagonalise: visits diagonalise their subproblem whatever the size (tests)
 template <typename T>
 int block_jacobi(const double* C, int n, int ldc, T* V, int ldv, T* w, int max_sweeps, double tol2, void* scratch,
-                 cudaStream_t st, double* ratio_out);
+                 cudaStream_t st, double* ratio_out, bool diagonalise);
 int64_t block_jacobi_scratch_bytes(int n, int elem);
 void launch_jacobi(double* A, int n, int lda, double* V, int ldv, double* w, int max_sweeps, int* info,
                    cudaStream_t st);

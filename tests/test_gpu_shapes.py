@@ -258,3 +258,35 @@ def test_eigenvectors_of_close_pairs(tiny_pair, N, seed):
     left = T - np.diag(d) - (d[:, None] + d[None, :]) / 2 * (L - np.diag(np.diag(L)))
     norm = np.linalg.norm(A)
     assert np.abs(left).max() <= (1e-15 + 4 * np.sqrt(N) * 2.0 ** -53) * norm
+
+
+# Rayleigh-Ritz above 512 vectors (blocked Cholesky, block Jacobi with diagonalising visits, N x N
+# products on the engine) and with the kernels of the largest blocks forced on smaller ones, against
+# the oracle; the figures of the long tall products (1e-9 of the largest Ritz value; both engines)
+@pytest.fixture(scope="module")
+def wide_pair():
+    from oracle.operators import Discretisation
+    s = W.tiny(seed=11, cells=(3, 3, 3))
+    return Discretisation(s), gpu_system(s)
+
+
+@pytest.mark.parametrize("engine", ["dfma", "tensor"])
+@pytest.mark.parametrize("N,forced", [(513, 0), (513, 1), (600, 0), (65, 1), (97, 1), (129, 1)])
+def test_rayleigh_ritz_of_wide_blocks(wide_pair, engine, N, forced):
+    from oracle.chfsi import cholqr, rayleigh_ritz
+    d, G = wide_pair
+    X = W.random_block(d.system, N, seed=1000 + N)
+    eps_ref, _, res_ref = rayleigh_ritz(d.apply_H_assembled, d.apply_M_assembled, cholqr(X)[0])
+    top = np.abs(eps_ref).max()
+    G.set_fp64_engine(engine)
+    G.set_option("dense_blocked", forced)
+    try:
+        Xd = to_dev(X)
+        eps, res = G.rayleigh_ritz(Xd)
+    finally:
+        G.set_option("dense_blocked", 0)
+        G.set_fp64_engine("dfma")
+    np.testing.assert_allclose(eps, eps_ref, rtol=1e-9, atol=1e-9 * top)
+    np.testing.assert_allclose(res, res_ref, rtol=1e-6, atol=1e-8 * top)
+    gram = (Xd.T @ G.apply_M(Xd)).cpu().numpy()
+    np.testing.assert_allclose(gram, np.eye(N), atol=1e-8)

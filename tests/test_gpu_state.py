@@ -142,19 +142,24 @@ def test_handle_after_a_refused_reservation():
 ONE_TILE = max(14 * 1053 * 48, 8 * 12 * 125 * 48)
 
 
+@pytest.fixture(scope="module")
+def oracle_H():
+    from oracle.operators import Discretisation
+    return Discretisation(W.tiny(seed=11)).apply_H_assembled
+
+
 @pytest.mark.parametrize("N", [20, 48, 49, 100, 145])
-def test_engine_cells_take_what_memory_there_is(N):
+def test_engine_cells_take_what_memory_there_is(oracle_H, N):
     """The FP64 engine's cell products where the device refuses their scratch: in 48-column
     panels the bits of one panel, and without any room the DFMA products, against the oracle
     (the engine's figure, 1e-10 of the largest entry).  A filter, which keeps its panels from
     degree to degree, and a call after the memory has come back."""
-    from oracle.operators import Discretisation
     from tests.gpu_util import rel_err
     G = gpu_system(W.tiny(seed=11))
     assert (G.n_nodes, G.n_cells) == (1053, 12)
     X = W.random_block(G.system, N, seed=700 + N)
     Xd = to_dev(X)
-    ref = Discretisation(G.system).apply_H_assembled(X)
+    ref = oracle_H(X)
     b = G.upper_bound(Xd[:, -1].contiguous(), 10)
     G.set_fp64_engine("tensor")
 
