@@ -1646,6 +1646,8 @@ int efe_apply_H(efe_handle* h, const double* X, int64_t ldx, int32_t N, double* 
   TRY(check_disjoint(h, X, ldx, Y, ldy, N));
   TRY(set_dev(h));
   TRY(reserve(h, N));
+  // the engine's error flag: an earlier call may have timed out
+  if (h->fp64_engine == 1) CK(cudaMemsetAsync(h->info + 4, 0, sizeof(int), S(stream)));
   return apply_H_impl(h, X, ldx, N, Y, ldy, S(stream));
 }
 

@@ -195,3 +195,21 @@ def test_cells_colour_by_colour(precision, N):
     G.set_option("cell_scratch", 1)
     assert torch.equal(step(0), at_once) and torch.equal(step(1), at_once)
     G.close()
+
+
+def test_products_after_a_wait_that_ran_out():
+    """The error flag of a call that timed out belongs to that call: the engine's products of
+    the next one run."""
+    from paper_1610_02121_gb300 import EfeError
+    G = gpu_system(W.tiny(seed=11))
+    X = to_dev(W.initial_block(G.system, 20, seed=2))
+    b = G.upper_bound(X[:, -1].contiguous(), 10)
+    G.set_fp64_engine("tensor")
+    before = G.apply_H(X)
+    G.set_option("test_stall", 1)
+    with pytest.raises(EfeError):
+        G.chfsi_step(X.clone(), 1, 0.2 * b, b, -1.0)
+    G.set_option("test_stall", 0)
+    after = G.apply_H(2.0 * X)
+    assert torch.equal(after, 2.0 * before)
+    G.close()
