@@ -230,7 +230,7 @@ int efe_set_fp64_engine(efe_handle* h, int32_t engine);
 #define EFE_OPT_DENSE_BLOCKED 4  /* 1: the dense N x N kernels of the largest blocks (Cholesky with tiled trailing
                                     updates, block Jacobi eigensolver whose visits diagonalise, N x N products on the
                                     FP64 engine when it is on) whatever the size; 0: the blocked eigensolver for
-                                    N > 48, with such visits for N > 512; the blocked Cholesky for N > 64, with tiled
+                                    N > 48, with such visits for N > 512; the blocked Cholesky for N > 160, with tiled
                                     updates for N > 2048; engine products for N > 512 */
 #define EFE_OPT_COUPLING_SPARSE 5 /* 1: the mixed degrees take the many-function enrichment coupling (node-major FP32
                                     columns products, rows products over function groups with FP64 partial sums)

@@ -2009,13 +2009,13 @@ int dense_scratch(efe_handle* h, int64_t bytes) {
   return EFE_OK;
 }
 
-// the one-CTA dense kernels up to these sizes, the blocked multi-CTA ones above:
-// the one-CTA Cholesky took 410 us at n = 135 and 28 ms at 640 (blocked: 0.25 and 2.4
-// ms), the one-CTA Jacobi eigensolver 16 ms at 135 (blocked: 3.4); a whole
-// Rayleigh-Ritz call of 33 vectors takes 3.2 ms with the one-CTA kernels and 3.6 with
-// the blocked ones, of 48 the same, of 12 2.36 and 2.39.  DENSE_SMALL_MAX: the N x N
-// products go to the tensor-core FP64 engine above it.
-constexpr int CHOL_ONE_CTA_MAX = 64;
+// The one-CTA dense kernels up to these sizes, the blocked multi-CTA ones above.  Cholesky, one
+// CTA against blocked (the same bits; a 64-wide trailing tile alone takes 70 us of FP64 pipe):
+// 65 rows 0.14 and 0.31 ms, 128 0.40 and 0.41, 144 0.50 and 0.62, 160 0.62 and 0.64, 176 0.76 and
+// 0.68, 256 2.1 and 1.0, 640 28 and 2.8.  Eigensolver: 48 rows 2.0 ms by one CTA, 49 rows 1.5
+// blocked, 135 rows 16 and 5.1.  DENSE_SMALL_MAX: the N x N products go to the tensor-core
+// FP64 engine above it.
+constexpr int CHOL_ONE_CTA_MAX = 160;
 constexpr int EIG_ONE_CTA_MAX = 48;
 constexpr int DENSE_SMALL_MAX = 512;
 constexpr int BJ_EXACT_MAX = 512;
