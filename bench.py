@@ -549,7 +549,7 @@ def main():
         oz_tf = oz_flops / (oz_ms * 1e-3) / 1e12
         roof_oz = {"bound": "tensor", "achieved": 28.0 * oz_tf, "peak": bf16_peak, "unit": "TFLOP/s",
                    "frac": 28.0 * oz_tf / bf16_peak, "traffic": None,
-                   "kernel": "k_oz (FP64-grade products)", "launches": oz_launch, "avg_launch_ms": oz_ms / oz_launch,
+                   "kernel": "k_oz, and k_ozc_slice / _cell / _gather together (FP64-grade products)", "launches": oz_launch, "avg_launch_ms": oz_ms / oz_launch,
                    "fp64_grade_tflops": oz_tf, "algorithmic_fp64_flops_per_launch": oz_flops / oz_launch,
                    "note": "achieved = 28 BF16 digit products per FP64 product x algorithmic FP64 flops / time",
                    "peak_source": bf16_src}

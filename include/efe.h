@@ -251,9 +251,10 @@ int efe_set_fp64_engine(efe_handle* h, int32_t engine);
                                     colour by colour.  Same results but for the engine's change to DFMA */
 int efe_set_option(efe_handle* h, int32_t option, int64_t value);
 
-/* Kernel timing: when enabled, the library brackets every launch of its
- * classical cell-apply kernel (any precision) with CUDA events on the
- * launching stream.  efe_kernel_stats synchronises the device, then returns
+/* Kernel timing: when enabled, the library brackets the classical cell products
+ * of the mixed-precision filter degrees (one launch a colour, or one launch and
+ * its gather for all cells) with CUDA events on the launching stream.
+ * efe_kernel_stats synchronises the device, then returns
  * the number of launches, their summed duration (ms) and the number of cell
  * products they performed (cells x N-column blocks counted as cells * N), and
  * optionally resets the counters. */
@@ -262,8 +263,9 @@ int efe_kernel_stats(efe_handle* h, int64_t* launches, double* total_ms, int64_t
                      int32_t reset);
 
 /* Second timing channel: the FP64 tensor-engine products (efe_set_fp64_engine
- * 1: the FP64 cell products, tall rotations and A^T B products), bracketed by
- * events while timing is enabled.  Returns their launches, summed duration
+ * 1: the FP64 cell products -- slicing, products and gather of a column panel as
+ * one -- tall rotations and A^T B products), bracketed by events while timing is
+ * enabled.  Returns the number of such products, their summed duration
  * (ms) and algorithmic FP64 flops (2 * 125^2 * N per cell product, 2 rows N^2
  * per rotation, rows N (N + 1) per symmetric A^T B, 2 rows N^2 otherwise). */
 int efe_kernel_stats_fp64(efe_handle* h, int64_t* launches, double* total_ms, double* flops, int32_t reset);

@@ -2,17 +2,17 @@
 // vectors (N in the thousands, Sec. V on the 280-atom cluster), spread over
 // many SMs:
 //   * blocked right-looking Cholesky (64-column panels: one-CTA diagonal block,
-//     row-parallel triangular solve of the panel, trailing update as an FP64
-//     GEMM);
+//     row-parallel triangular solve of the panel, trailing update in tiles that keep
+//     the one-CTA factor's order of sums, as an FP64 GEMM above 2,048 rows);
 //   * the inverse of a lower triangle by 2 x 2 block recursion (two half-size
 //     inverses and two GEMMs);
 //   * a two-sided block Jacobi eigensolver for symmetric matrices: the matrix
 //     is cut into blocks of B rows/columns, a round-robin tournament pairs the
-//     blocks, every pair's 2B x 2B subproblem is diagonalised in shared memory
-//     by one CTA (cyclic Jacobi), and the pair's rotation is applied to its 2B
-//     rows and columns of the whole matrix and to the eigenvector matrix by
-//     many CTAs (row-times-2B x 2B products), B = 16.  Float (the fast first
-//     stage) and double (the refinement).
+//     blocks, one CTA rotates every pair's 2B x 2B subproblem in shared memory
+//     (one cyclic Jacobi sweep; above 512 rows until it is diagonal), and the pair's
+//     rotation is applied to its 2B rows and columns of the whole matrix and to the
+//     eigenvector matrix by many CTAs (row-times-2B x 2B products), B = 16.  Float
+//     (the fast first stage) and double (the refinement).
 // No atomics: every result has a fixed order of operations.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -95,8 +95,9 @@ __global__ void __launch_bounds__(128) k_chol_panel(double* A, int lda, int j0, 
 // A22 -= L21 L21^T, lower triangle: every entry takes the panel's products one after the other
 // in column order, as the one-CTA factor does (k_chol; the diagonal and panel kernels above
 // keep that order too), so that both give the same bits.  64 x 64 tiles, 4 x 4 a thread; the
-// panel's 64 terms a tile bound it (FP64 pipe).  640 columns, Rayleigh-Ritz call: one-CTA factor
-// 278 ms, this 201 ms.
+// panel's 64 terms a tile bound it (FP64 pipe: 70 us a tile, and the last tiles run alone).  The
+// whole factor of 640 rows: one CTA 28 ms, with this update 2.8, with tiled products (another order)
+// 2.4; of 135 rows 0.39, 0.62, 0.51.
 __global__ void __launch_bounds__(256) k_chol_update(double* A, int lda, int j0, int b, int n) {
   if (blockIdx.x > blockIdx.y) return;
   __shared__ double Pr[64][33], Pc[64][33];
@@ -276,9 +277,10 @@ __device__ __forceinline__ void bj_angle(double aii, double ajj, double aij, dou
 // subproblem [[A_pp, A_pq], [A_qp, A_qq]] in shared memory; writes the rotation J
 // (BJ_S x BJ_S, row-major), the rotated subproblem and whether any rotation was
 // applied.  One sweep a visit: the outer sweeps come back to the pair anyway, and
-// diagonalising it on every visit took three to eight sweeps on one SM (640 rows:
-// 100 us a round in FP32 and 237 us in FP64; now 25 and 84, with as many outer
-// sweeps: 9 and 3).
+// diagonalising it on every visit takes three to eight sweeps on one SM (timed at 640
+// rows, a round 100 us in FP32 and 237 in FP64; this 25, as at 135 rows, and 84, with as
+// many outer sweeps).  The whole eigenproblem, diagonalising visits -> this: 135 rows 13.0 ->
+// 5.1 ms, 300 30.6 -> 11.7, 512 56 -> 23.
 // The two-sided rotation of the pairs (e, f) acts on a 2 x 2 block of S: a thread
 // per block with e <= f (S is symmetric, the mirrored block is copied).
 template <typename T, int BJ_B>
@@ -380,7 +382,8 @@ __global__ void __launch_bounds__(256) k_bj_solve(const T* __restrict__ A, int n
 // one is the solved subproblem), its mirror image the transpose.  blockIdx.x >=
 // pairs: 32 rows of V, V[:, idx(k)] <- V[:, idx(k)] J_k.  Blocks are independent,
 // so A needs no separate row and column pass (three launches a round and twice the
-// products before: 640 rows 82 us in FP64 and 24 in FP32, now 69 and 12).
+// products before).  135 rows: 8.7 us in FP32; timed at 640 rows, above its use, 69 us
+// in FP64 and 12 in FP32 for 82 and 24.
 template <typename T, int BJ_B>
 __global__ void __launch_bounds__(256) k_bj_update(T* __restrict__ A, T* __restrict__ V, int np, int nb, int r,
                                                    const T* __restrict__ Jb, const T* __restrict__ Sb,

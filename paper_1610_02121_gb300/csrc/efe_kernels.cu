@@ -2225,7 +2225,8 @@ void launch_coup_rows(int64_t n_tn, int ncta, const int64_t* cta_blk, const int3
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kern<<<ncta, 256, smem, st>>>(n_tn, cta_blk, t_nodes, slot_off, slots, tile, tscale, X, ldx, nE, N, part);
   };
-  // 8 N bytes of rows a thread and block, held in 16-byte registers where five hold them
+  // N / 2 bytes of rows a thread and block (32 rows of 4 N bytes over 256 threads), held in
+  // 16-byte registers where five hold them: up to 160 columns
   if (N <= 32) run(k_coup_rows<1>);
   else if (N <= 96) run(k_coup_rows<3>);
   else if (N <= 160) run(k_coup_rows<5>);

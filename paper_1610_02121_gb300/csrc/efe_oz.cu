@@ -18,11 +18,14 @@
 //
 // Products of this file (the cell products are in efe_oz_cell.cu):
 //   ROWS  C = A B for a tall A (rows x K) and a small B (K x N); K is taken in
-//         groups of 256 (exact FP32 sums), each group's FP64 value added to C;
+//         groups of 256 (exact FP32 sums for t <= 5);
 //   GRAM  C = A^T B for tall A, B (K x Na, K x N, K large): items are (tile
-//         pair, K segment); each segment is formed in 256-row groups (exact
-//         FP32 sums for t <= 5) drained into FP64 partial tiles, which a
-//         fixed-order reduction adds up.
+//         pair, K segment); each segment is formed in such groups of 256 rows, and a
+//         fixed-order FP64 reduction adds the segments' partial tiles.
+// The groups of an item are added in FP32 (hi, lo) pairs in registers (error-free sum of the
+// high parts, renormalised): each addition rounds within 2^-45 of the sum so far (two FP32
+// roundings of a low part up to 2^-22 of it; a few 2^-48 in the mean), so a segment of G groups
+// within G 2^-45.  The FP64 value is formed once per item.
 // Both operands are cut once per product into digit images (k_oz_img_rows /
 // k_oz_img_cols) and arrive in the stages by bulk asynchronous copies; the digit
 // images of the cell matrices (k_oz_preslice, once per potential) are made here too.
