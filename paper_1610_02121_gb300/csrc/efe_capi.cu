@@ -428,17 +428,20 @@ int reserve32(efe_handle* h, int N) {
     dalloc_scratch(h, &h->cellP32, tc3_scratch_elems(h->n_cell, ld));
   for (int i = 0; i < 2; ++i) TRY(dalloc(h, &h->Ye[i], std::max<int64_t>(1, h->nE) * N));
   TRY(dalloc(h, &h->We, std::max<int64_t>(1, h->nE) * N));
+  // the widest block of this reservation that the dense-tile coupling kernels serve (its n_E x N
+  // array in shared memory): they and the many-function kernels are both set up where N is wider,
+  // since a later call may bring fewer columns
+  int Nt = h->nE > 0 ? N : 0;
+  while (Nt > 0 && !coup_tiles_fit(h, Nt)) --Nt;
   // coupling products: one wave of CTAs each, node blocks split so that every
   // CTA holds about the same number of tile slots (plus a share for staging rows)
   auto partition = [&](bool rows, int64_t** dev, int* ncta_out) -> int {
     dfree(h, *dev);
     *dev = nullptr;
     *ncta_out = 1;
-    // the dense-tile coupling kernels serve only blocks whose (n_E x N) array
-    // fits in shared memory (the mixed degrees take the sparse kernels otherwise)
-    if (h->nE <= 0 || h->cb_nblk <= 0 || !coup_tiles_fit(h, N)) return EFE_OK;
+    if (Nt == 0 || h->cb_nblk <= 0) return EFE_OK;
     const int64_t nblk = h->cb_nblk;
-    const int ncta = (int)std::min<int64_t>(nblk, coup_resident_ctas((int)h->nE, N, h->n_sm, rows));
+    const int ncta = (int)std::min<int64_t>(nblk, coup_resident_ctas((int)h->nE, Nt, h->n_sm, rows));
     const auto& so = h->cb_soff_host;
     const double wtot = (double)so[nblk] + 3.0 * (double)nblk;
     std::vector<int64_t> cb(ncta + 1, nblk);
@@ -455,8 +458,8 @@ int reserve32(efe_handle* h, int N) {
   };
   TRY(partition(true, &h->cb_cta, &h->ncb));
   TRY(partition(false, &h->cb_cta_cols, &h->ncb_cols));
-  TRY(dalloc(h, &h->cpart, coup_tiles_fit(h, N) ? (int64_t)h->ncb * std::max<int64_t>(1, h->nE) * N : 1));
-  if (h->nE > 0 && !coup_tiles_fit(h, N)) {
+  TRY(dalloc(h, &h->cpart, Nt > 0 ? (int64_t)h->ncb * h->nE * Nt : 1));
+  if (h->nE > 0 && Nt < N) {
     TRY(dalloc(h, &h->gpart, (int64_t)std::max(1, h->n_gitems) * grp_kmax() * N));
     TRY(dalloc(h, &h->Xe32, h->nE * N));
   }

@@ -213,3 +213,25 @@ def test_products_after_a_wait_that_ran_out():
     after = G.apply_H(2.0 * X)
     assert torch.equal(after, 2.0 * before)
     G.close()
+
+
+def test_narrow_filter_after_a_wide_one():
+    """A block too wide for the dense-tile coupling kernels takes the many-function ones; a
+    narrower block on the same handle takes the dense tiles again (mixed filter of degree 3,
+    FP32-grade: 5e-5 of the largest entry, as in the mixed cases against the oracle)."""
+    from tests.gpu_util import rel_err
+    s = W.tiny(seed=11)
+    wide, fresh = gpu_system(s), gpu_system(s)
+    # (n_E + 32) rows of N floats and the pattern tile in 200 KB
+    N = (200 * 1024 // 4 - 2048) // (wide.n_enrich + 32) // 4 * 4 + 8
+    X = to_dev(W.random_block(s, N, seed=9))
+    b = fresh.upper_bound(X[:, -1].contiguous(), 10)
+    many = wide.chfsi_step(X.clone(), 3, 0.2 * b, b, -1.0, precision="tf32x3")
+    for n in (20, N - 16, N):
+        got = wide.chfsi_step(X[:, :n].clone(), 3, 0.2 * b, b, -1.0, precision="tf32x3")
+        ref = fresh.chfsi_step(X[:, :n].clone(), 3, 0.2 * b, b, -1.0, precision="tf32x3")
+        assert rel_err(got, ref.cpu().numpy()) < 5e-5
+        assert rel_err(got, many[:, :n].cpu().numpy()) < 5e-5
+    assert torch.equal(got, many)
+    wide.close()
+    fresh.close()
