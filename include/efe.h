@@ -237,11 +237,11 @@ int efe_set_fp64_engine(efe_handle* h, int32_t engine);
                                     whatever the size; 0: only when the dense-tile kernels' n_E x N FP32 array
                                     exceeds 200 KB of shared memory */
 #define EFE_OPT_TEST_STALL 6      /* tests of the failure path only: in every tensor-core launch (tcgen05 cell kernel,
-                                    FP64 engine) some lanes first wait on a barrier that nothing completes, so their
-                                    bounded wait runs out; the launch drains its copies and MMAs, frees its TMEM and
-                                    the call returns EFE_ERR_TIMEOUT.  1: the warp that issues the MMAs; 2: only its
-                                    odd lanes (a wait that runs out on a part of a warp); 3: the odd lanes of the
-                                    converter and epilogue warps.  0 (default): off */
+                                    FP64 engine) a barrier of the pipeline expects one arrival more than it gets, so the
+                                    bounded waits on it run out; the launch drains its copies and MMAs, frees its TMEM
+                                    and the call returns EFE_ERR_TIMEOUT.  1: operands ready (the warp that issues the
+                                    MMAs), 2: stage empty (converters, copies), 3: accumulators complete (epilogue).
+                                    0 (default): off */
 #define EFE_OPT_COUPLING_COLS 7   /* the columns product W_c += (H^ec)^T Y_e of the many-function coupling:
                                     0 (default): dense tiles of 32-node blocks; 1: each node's own entries only.
                                     Same products, FP32 sums in another order */

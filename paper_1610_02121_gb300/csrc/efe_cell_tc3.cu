@@ -123,7 +123,6 @@ __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
 // the barrier, so the lanes vote: one that left alone could not take part in the warp's next
 // collective step, and the others would wait for it there without a bound.
 __device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
-  if (__all_sync(0xffffffffu, bar_try(b, parity))) return true;
   const long long t0 = clock64();
   do {
     if (__all_sync(0xffffffffu, bar_try(b, parity))) return true;
@@ -133,10 +132,6 @@ __device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
 // the abort flag, one answer for the whole warp
 __device__ __forceinline__ bool warp_aborted(const volatile int* flag) {
   return __any_sync(0xffffffffu, *flag != 0);
-}
-// tests only: the lanes of `mine` wait on a barrier that nothing completes
-__device__ __forceinline__ bool stall_passed(uint64_t* never, bool mine) {
-  return __all_sync(0xffffffffu, !mine || bar_wait(never, 0u));
 }
 
 __device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
@@ -194,7 +189,6 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
   uint64_t* empty = conv + ST;                                  // [ST]
   uint64_t* accf = conv + 2 * ST;                               // [2]
   uint64_t* acce = accf + 2;                                    // [2]
-  uint64_t* never = accf + 4;   // no thread ever arrives here (the test stall waits on it)
   uint32_t* tslot = reinterpret_cast<uint32_t*>(accf + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(accf + 6);
   int32_t* lut = reinterpret_cast<int32_t*>(sm + L::LUT);
@@ -212,14 +206,13 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
   }
   if (tid == 32) {
     for (int s = 0; s < ST; ++s) {
-      bar_init(conv + s, L::GW);
-      bar_init(empty + s, 1);
+      bar_init(conv + s, L::GW + (stall == 1));   // stall: see launch_cell_tc3
+      bar_init(empty + s, 1 + (stall == 2));
     }
     for (int b = 0; b < 2; ++b) {
-      bar_init(accf + b, 1);
+      bar_init(accf + b, 1 + (stall == 3));
       bar_init(acce + b, T3_EPI_WARPS);
     }
-    bar_init(never, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid >= 64 && tid < 64 + T3_M) {
@@ -238,12 +231,9 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
-    // test stall: a wait that nothing completes runs out like a real one
-    const bool go = my_items == 0 || stall_passed(never, stall == 1 || (stall == 2 && (lane & 1)));
-    if (!go && lane == 0) { *abort_flag = 1; atomicExch(err, 1); }
     int s = 0;
     uint32_t ph = 0;
-    for (int64_t t = 0; go && t < my_items && !warp_aborted(abort_flag); ++t) {
+    for (int64_t t = 0; t < my_items && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % ntiles) * TW;
       const int ncol = min(TW, N - c0);
@@ -335,12 +325,7 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
     for (int i = 0; i < L::DEPTH; ++i) fetch();
     int s = g, rs = 0;
     uint32_t ph = 0;
-    const bool go = stall != 3 || my_items == 0 || stall_passed(never, lane & 1);
-    if (!go) {
-      *abort_flag = 1;
-      atomicExch(err, 1);
-    }
-    for (int64_t t = 0; go && t < my_items && !warp_aborted(abort_flag); ++t) {
+    for (int64_t t = 0; t < my_items && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % ntiles) * TW;
       const int ncol = min(TW, N - c0);
@@ -429,12 +414,7 @@ __global__ void __launch_bounds__(T3Layout<TW>::THREADS, 1)
     // ------------------------------------------------------------ epilogue
     const int quarter = warp & 3;         // TMEM lane quarter accessible to this warp
     const int sub = lane & 3;
-    const bool go = stall != 3 || my_items == 0 || stall_passed(never, lane & 1);
-    if (!go) {
-      *abort_flag = 1;
-      atomicExch(err, 1);
-    }
-    for (int64_t t = 0; go && t < my_items && !warp_aborted(abort_flag); ++t) {
+    for (int64_t t = 0; t < my_items && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int64_t e = cells ? cells[item / ntiles] : item / ntiles;
       const int c0 = (int)(item % ntiles) * TW;

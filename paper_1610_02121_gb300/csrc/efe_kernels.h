@@ -156,8 +156,10 @@ int64_t tc3_image_elems(int64_t n_cell);
 // FP32 image of every H^cc_e in the MMA's core-matrix layout (split into TF32 parts in the kernel)
 void launch_build_aimg(const double* Hcc, int64_t n_cell, float* A, cudaStream_t st);
 // tile: column tile width (64, 96 or 160; 0 = default 160)
-// stall (tests only): the MMA warp first waits on a barrier nothing completes, so the
-// bounded wait runs out and the launch takes its abort path
+// stall (tests only): a barrier of the pipeline expects one arrival more than it gets, so the
+// waits on it run out and the launch takes its abort path.  1: operands ready (MMA warp), 2: stage
+// empty (converters), 3: accumulators complete (epilogue).  (A wait of its own at the head of a
+// role costs every launch 1 to 3 us and the digit products 1 to 3 % of their rate.)
 // cells null: all cells at once, their products to W as (n_cell x 125) x ldw scratch, which
 // launch_tc3_gather adds per node (W's columns N .. ldw become zero)
 int64_t tc3_scratch_elems(int64_t n_cell, int64_t ld);
@@ -169,9 +171,7 @@ int launch_cell_tc3(const float* A, const int32_t* cells, int64_t ncells, const 
 const int* tc3_tiles(int* count);
 
 // ---- FP64-grade products on the BF16 tensor cores (efe_oz.cu) ----
-// stall (tests only, every launcher below): the MMA warp first waits on a
-// barrier nothing completes, so the bounded wait runs out and the launch takes
-// its abort path
+// stall (tests only, every launcher below): as launch_cell_tc3, 2: the copies
 int64_t oz_hexp_elems(int64_t n_cell);
 void launch_oz_hexp(const double* Hcc, int64_t n_cell, int* hexp, cudaStream_t st);
 void launch_oz_colexp(const double* Y, int64_t ldy, int64_t rows, int N, int* fexp, cudaStream_t st);

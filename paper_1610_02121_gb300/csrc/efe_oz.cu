@@ -142,7 +142,7 @@ struct OzArgs {
   const unsigned char* Aimg;
   const unsigned char* Bimg;
   int64_t astep, bstep;
-  int stall;                // tests only (EFE_OPT_TEST_STALL): waits on a barrier that nothing completes
+  int stall;                // tests only (EFE_OPT_TEST_STALL)
 };
 
 // work item of a CTA: row block / tile pair and its K range
@@ -189,7 +189,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
   uint64_t* acce = accf + 1;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(accf + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(accf + 3);
-  uint64_t* never = accf + 4;                                    // no thread ever arrives here (test stall)
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)),
                  "r"(OZ_TMEM_COLS)
@@ -198,12 +197,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
   }
   if (tid == 32) {
     for (int s = 0; s < OZ_STAGES; ++s) {
-      bar_init(empty + s, 1);
-      bar_init(afull + s, 1);
+      bar_init(empty + s, 1 + (g.stall == 2));
+      bar_init(afull + s, 1 + (g.stall == 1));
     }
-    bar_init(accf, 1);
+    bar_init(accf, 1 + (g.stall == 3));
     bar_init(acce, OZ_EPI_WN * 32);
-    bar_init(never, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -226,10 +224,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
 
   if (warp == 0) {
     // ---------------------------------------------------------------- MMA issuer
-    // test stall: a wait that nothing completes runs out like a real one
-    const bool go = my == 0 || stall_passed(never, g.stall == 1 || (g.stall == 2 && (lane & 1)));
-    if (!go && lane == 0) { *abort_flag = 1; atomicExch(g.err, 1); }
-    for (int64_t t = 0; go && t < my && !warp_aborted(abort_flag); ++t) {
+    for (int64_t t = 0; t < my && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const OzItem it = oz_item(g, item);
       const int nmma = it.nmma;
@@ -315,12 +310,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
     const int r = quarter * 32 + lane;
     const int ew = warp - OZ_EPI_W0, part = ew >> 2, nparts = OZ_EPI_WN >> 2;   // column blocks part, part + nparts, ...
     double* stg = reinterpret_cast<double*>(sm + OzL::STG) + ew * (32 * 9);
-    const bool go = g.stall != 3 || my == 0 || stall_passed(never, lane & 1);
-    if (!go) {
-      *abort_flag = 1;
-      atomicExch(g.err, 1);
-    }
-    for (int64_t t = 0; go && t < my && !warp_aborted(abort_flag); ++t) {
+    for (int64_t t = 0; t < my && !warp_aborted(abort_flag); ++t) {
       const OzItem it = oz_item(g, blockIdx.x + t * gridDim.x);
       const int c0 = it.c0, ncol = it.ncol;
       bool live;
@@ -426,12 +416,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz(OzArgs g) {
   // are released: every bulk copy still in flight into the stage ring lands (the copy
   // thread issues into a stage only after its MMAs released it, so at most the last
   // OZ_STAGES chunks are outstanding), and the last MMA commit -- which covers every
-  // MMA this CTA issued -- arrives.  Each drain wait is bounded like the pipeline's own.
+  // MMA this CTA issued -- arrives.  Each drain wait is bounded like the pipeline's own;
+  // after one that ran out there is nothing left to wait for.
   __syncthreads();
   if (*abort_flag) {
     if (last_copy >= 0) {
       for (int64_t ch = last_copy - OZ_STAGES + 1; ch <= last_copy; ++ch)
-        if (ch >= 0) bar_wait(afull + (int)(ch % OZ_STAGES), (uint32_t)((ch / OZ_STAGES) & 1));
+        if (ch >= 0 && !bar_wait(afull + (int)(ch % OZ_STAGES), (uint32_t)((ch / OZ_STAGES) & 1))) break;
     }
     if (warp == 0 && lane == 0 && last_mma >= 0)
       bar_wait(empty + (int)(last_mma % OZ_STAGES), (uint32_t)((last_mma / OZ_STAGES) & 1));

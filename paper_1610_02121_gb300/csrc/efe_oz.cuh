@@ -47,7 +47,6 @@ __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
 // the barrier, so the lanes vote: one that left alone could not take part in the warp's next
 // collective step, and the others would wait for it there without a bound.
 __device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
-  if (__all_sync(0xffffffffu, bar_try(b, parity))) return true;
   const long long t0 = clock64();
   do {
     if (__all_sync(0xffffffffu, bar_try(b, parity))) return true;
@@ -57,10 +56,6 @@ __device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
 // the abort flag, one answer for the whole warp
 __device__ __forceinline__ bool warp_aborted(const volatile int* flag) {
   return __any_sync(0xffffffffu, *flag != 0);
-}
-// tests only: the lanes of `mine` wait on a barrier that nothing completes
-__device__ __forceinline__ bool stall_passed(uint64_t* never, bool mine) {
-  return __all_sync(0xffffffffu, !mine || bar_wait(never, 0u));
 }
 __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
   asm volatile(

@@ -134,7 +134,7 @@ struct OzCellArgs {
   double* P;                   // products, [cell][125][ldn]
   int ldn, ntiles;
   int* err;
-  int stall;
+  int stall;                   // tests only (EFE_OPT_TEST_STALL)
 };
 
 __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
@@ -155,7 +155,6 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
   uint64_t* empty = full + OC_STAGES;                           // [stages] its MMAs are done
   uint64_t* accf = full + 2 * OC_STAGES;                        // [2] accumulator set complete
   uint64_t* acce = accf + 2;                                    // [2] accumulator set read
-  uint64_t* never = accf + 4;                                   // no thread ever arrives here (test stall)
   uint32_t* tslot = reinterpret_cast<uint32_t*>(accf + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(accf + 6);
   if (warp == 0) {
@@ -166,14 +165,13 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
   }
   if (tid == 32) {
     for (int i = 0; i < OC_STAGES; ++i) {
-      bar_init(full + i, OC_CPY_T + 1);
-      bar_init(empty + i, 1);
+      bar_init(full + i, OC_CPY_T + 1 + (g.stall == 1));
+      bar_init(empty + i, 1 + (g.stall == 2));
     }
     for (int i = 0; i < 2; ++i) {
-      bar_init(accf + i, 1);
+      bar_init(accf + i, 1 + (g.stall == 3));
       bar_init(acce + i, OC_EPI_WN * 32);
     }
-    bar_init(never, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -189,12 +187,9 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
 
   if (warp == 0) {
     // ---------------------------------------------------------------- MMA issuer
-    // test stall: a wait that nothing completes runs out like a real one
-    const bool go = my == 0 || stall_passed(never, g.stall == 1 || (g.stall == 2 && (lane & 1)));
-    if (!go && lane == 0) { *abort_flag = 1; atomicExch(g.err, 1); }
     int s = 0;
     uint32_t ph = 0;
-    for (int64_t t = 0; go && t < my && !warp_aborted(abort_flag); ++t) {
+    for (int64_t t = 0; t < my && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int c0 = (int)(item % g.ntiles) * OC_TW;
       const uint32_t id = idesc_cell(min(OC_TW, g.ldn - c0));
@@ -300,12 +295,7 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
     const int quarter = warp & 3;   // the TMEM lane quarter this warp may read
     const int part = (warp - OC_EPI_W0) >> 2;
     const int r = quarter * 32 + lane;
-    const bool go = g.stall != 3 || my == 0 || stall_passed(never, lane & 1);
-    if (!go) {
-      *abort_flag = 1;
-      atomicExch(g.err, 1);
-    }
-    for (int64_t t = 0; go && t < my && !warp_aborted(abort_flag); ++t) {
+    for (int64_t t = 0; t < my && !warp_aborted(abort_flag); ++t) {
       const int64_t item = blockIdx.x + t * gridDim.x;
       const int64_t e = item / g.ntiles;
       const int c0 = (int)(item % g.ntiles) * OC_TW;
@@ -366,7 +356,7 @@ __global__ void __launch_bounds__(OC_THREADS, 1) k_ozc_cell(OzCellArgs g) {
   if (*abort_flag) {
     if (last_copy >= 0)
       for (int64_t ch = max(last_copy - OC_STAGES + 1, (int64_t)0); ch <= last_copy; ++ch)
-        bar_wait(full + (int)(ch % OC_STAGES), (uint32_t)((ch / OC_STAGES) & 1));
+        if (!bar_wait(full + (int)(ch % OC_STAGES), (uint32_t)((ch / OC_STAGES) & 1))) break;
     if (warp == 0 && lane == 0 && last_mma >= 0)
       bar_wait(empty + (int)(last_mma % OC_STAGES), (uint32_t)((last_mma / OC_STAGES) & 1));
   }

@@ -82,12 +82,12 @@ def test_replayed_graph_follows_longer_recurrences(members):
     assert B.graph_nodes() == first
 
 
-@pytest.mark.parametrize("stall", [2, 3])
+@pytest.mark.parametrize("stall", [1, 2, 3])
 @pytest.mark.parametrize("what,precision,engine", [("filter", "tf32x3", "dfma"), ("filter", "fp64", "tensor"),
                                                    ("ritz", "fp64", "tensor")])
-def test_wait_that_runs_out_on_part_of_a_warp(what, precision, engine, stall):
-    """Lanes of one warp may disagree about whether a bounded wait ran out.  The whole warp then
-    takes the abort path (lanes that went on would wait for the others for ever): the call
+def test_waits_that_run_out_in_each_role(what, precision, engine, stall):
+    """A barrier that never completes, for the MMA warp, the converters or copies, and the
+    epilogue: every lane's wait runs out by its own clock, the warps leave as a whole, the call
     returns EFE_ERR_TIMEOUT, and the next one gives the bits of the one before."""
     from paper_1610_02121_gb300 import EfeError
     s = W.tiny(seed=11)
